@@ -200,21 +200,27 @@ def _front(case, seed):
             "y": y, "accepted": torch.from_numpy(accepted).to(DEVICE)}
 
 
-def _device(case, seed):
+def _device_inputs(case, seed):
     wl = _workload(case, seed)
-    B, H, T, N = case["B"], case["H"], case["T"], case["budget"]
+    B, T = case["B"], case["T"]
     parents, _ = inputs.make_trees(wl)
     parents = np.where(np.arange(T)[None] == 0, -1, parents).astype(np.int32)
     gen = torch.Generator(device=DEVICE).manual_seed(seed % 1000003 + 1)
     p = torch.rand(B, T, generator=gen, device=DEVICE) * 0.9 + 0.1
-    par = torch.from_numpy(parents).to(DEVICE)
-    # an earlier round's selection: its buffers are kept, and the sampler accepts one of its nodes
-    selected = tv.budget_select(par, p, N)
-    accepted = (torch.rand(B, generator=gen, device=DEVICE) * selected["counts"]).to(torch.int32)
+    draw_accepted = lambda counts: (torch.rand(B, generator=gen, device=DEVICE) * counts).to(torch.int32)
     # the model's tensors for the kept nodes, already packed: planes [H, budget, d]
-    wide = inputs.make_tensors(dataclasses.replace(wl, B=1, T=N), device=DEVICE)
+    wide = inputs.make_tensors(dataclasses.replace(wl, B=1, T=case["budget"]), device=DEVICE)
     planes = {n: None if wide[n] is None else wide[n][0] for n in ("q", "k", "v", "alpha", "beta")}
     S = inputs.make_tensors(dataclasses.replace(wl, T=1), device=DEVICE)["S_pre"]
+    return torch.from_numpy(parents).to(DEVICE), p, draw_accepted, planes, S
+
+
+def _device(case, seed):
+    B, H, T, N = case["B"], case["H"], case["T"], case["budget"]
+    par, p, draw_accepted, planes, S = _device_inputs(case, seed)
+    # an earlier round's selection: its buffers are kept, and the sampler accepts one of its nodes
+    selected = tv.budget_select(par, p, N)
+    accepted = draw_accepted(selected["counts"])
     O = torch.zeros(H, N, case["dv"], device=DEVICE)
     return {"case": case, "parents": par, "p": p, "planes": planes, "S": S, "O": O,
             "U": torch.zeros_like(O) if case["rule"] == "delta" else None,
@@ -348,3 +354,141 @@ def tolerance(case):
     if case["rule"] == "delta":                      # states read as tf32: 3e-4, largest 1.6e-3
         return {"rel": 1.2e-3, "max": 6e-3}
     return {"rel": 4e-5, "max": 2.5e-4}              # states read as bf16 pairs: 8.6e-6, largest 5.7e-5
+
+
+# ---------------------------------------------------------------------------
+# The same results in 64 bits
+# ---------------------------------------------------------------------------
+def _paths(parents):
+    """[B, T, T] float64: row i is one at node i and at its ancestors."""
+    M = np.zeros(parents.shape + parents.shape[-1:])
+    for b, par in enumerate(parents):
+        for i, p in enumerate(par):
+            if p >= 0:
+                M[b, i] = M[b, p]
+            M[b, i, i] = 1.0
+    return torch.from_numpy(M).to(DEVICE)
+
+
+def _exact_layer(S, q, k, v, alpha, beta, parents, accepted):
+    """O, U and the committed states of one layer: every node's path sum, then (delta rule) one
+    triangular solve per (request, head)."""
+    wide = lambda x: None if x is None else x.to(DEVICE, torch.float64)
+    S, q, k, v, alpha, beta = (wide(x) for x in (S, q, k, v, alpha, beta))
+    G = S.shape[1] // k.shape[1]
+    q, k = q.repeat_interleave(G, 1), k.repeat_interleave(G, 1)
+    M = _paths(parents)[:, None]
+    logP = (M @ alpha.log()[..., None])[..., 0]
+    P = logP.exp()[..., None]
+    W = torch.where(M > 0, logP[..., :, None] - logP[..., None, :], -torch.inf).exp()   # P_i / P_j on the path
+    U = v
+    if beta is not None:
+        R = beta[..., None] * (v - P * (k @ S.mT))
+        A = beta[..., None] * (W * (k @ k.mT))
+        U = torch.linalg.solve_triangular(torch.tril(A, -1) + torch.eye(A.shape[-1], device=DEVICE, dtype=A.dtype), R,
+                                          upper=False)
+    O = P * (q @ S.mT) + (W * (q @ k.mT)) @ U
+    new = None
+    if accepted is not None:
+        acc = torch.as_tensor(accepted).to(DEVICE).long()
+        at = acc.clamp(min=0)
+        b = torch.arange(len(acc), device=DEVICE)
+        new = P[b, :, at][..., None] * S + (W[b, :, at][..., None] * U).mT @ k
+        new = torch.where((acc < 0)[:, None, None, None], S, new)
+    return O, U if beta is not None else None, new
+
+
+def _exact_round(case, seed, commit=True):
+    wl = _workload(case, seed)
+    parents, accepted = inputs.make_trees(wl)
+    t = _tensors(case, wl)
+    one = case["L"] == 1
+    layer = lambda x, l: None if x is None else x if one else x[l]
+    got = [_exact_layer(*[layer(t[n], l) for n in ("S_pre", "q", "k", "v", "alpha", "beta")], parents,
+                        accepted if commit else None) for l in range(case["L"])]
+    O, U, S = (None if x[0] is None else x[0] if one else torch.stack(x) for x in zip(*got))
+    return {"O": O, "U": U, "S": S} if commit else {"O": O, "U": U}
+
+
+def _exact_front(case, seed):
+    wl = _workload(case, seed)
+    parents, accepted = inputs.make_trees(wl)
+    g = {n: x.double() for n, x in inputs.make_conv_inputs(wl, device=DEVICE, W=WIDTH).items()}
+    S = inputs.make_tensors(dataclasses.replace(wl, T=1), device=DEVICE)["S_pre"]
+    B, H, T, dk, dv = (case[n] for n in ("B", "H", "T", "dk", "dv"))
+    rows = torch.cat([g["ctx"], g["x"]], 1)                     # context, oldest first, then the nodes
+    first = WIDTH - 1                                           # row of node 0; before it the newest context row
+    up = np.concatenate([np.broadcast_to(np.arange(-1, first - 1), (B, first)),
+                         np.where(parents >= 0, parents + first, first - 1)], 1)
+    up = torch.from_numpy(up).to(DEVICE).long()
+    b = torch.arange(B, device=DEVICE)[:, None]
+    at = torch.arange(T, device=DEVICE).expand(B, T) + first
+    z = g["bias"].expand(B, T, -1)
+    for r in range(WIDTH):
+        z = z + rows[b, at] * g["weight"][:, WIDTH - 1 - r]
+        at = up[b, at].clamp(min=0)
+    y = z * torch.sigmoid(z)
+    heads = lambda x: x.reshape(B, T, H, -1).transpose(1, 2)
+    norm = lambda x: x / (x.square().sum(-1, keepdim=True) + 1e-6).sqrt()
+    to = lambda x: x.to(wl.torch_dtype).double()                # what the next stage is given
+    q, k, v = to(norm(heads(y[..., :H * dk]))), to(norm(heads(y[..., H * dk:2 * H * dk]))), to(heads(y[..., 2 * H * dk:]))
+    alpha = (-g["A_log"].exp() * torch.nn.functional.softplus(g["gate_a"] + g["dt_bias"])).exp().transpose(1, 2)
+    beta = torch.sigmoid(g["gate_b"]).transpose(1, 2)
+    O, U, S = _exact_layer(S, q, k, v, alpha, beta if case["rule"] == "delta" else None, parents, accepted)
+    ctx = g["ctx"].clone()
+    for i, a in enumerate(accepted):
+        path = []
+        while a >= 0:
+            path.insert(0, int(a) + first)
+            a = parents[i, a]
+        ctx[i] = rows[i, (list(range(first)) + path)[-first:]]
+    return {"y": {"q": q, "k": k, "v": v, "alpha": alpha, "beta": beta}, "O": O, "U": U, "S": S, "ctx": ctx}
+
+
+def _exact_device(case, seed):
+    B, H, T, N = case["B"], case["H"], case["T"], case["budget"]
+    par, p, draw_accepted, planes, S = _device_inputs(case, seed)
+    par, p = par.cpu().numpy(), p.cpu().numpy()
+    rho = p.copy()
+    for i in range(T):
+        rho[:, i] *= np.where(par[:, i] >= 0, rho[np.arange(B), par[:, i]], np.float32(1))
+    rank = np.where(np.arange(T)[None] == 0, np.float32(np.inf), rho)
+    keep = np.zeros(B * T, dtype=bool)
+    keep[np.argsort(-rank.reshape(-1), kind="stable")[:N]] = True
+    keep = keep.reshape(B, T)
+    new = np.cumsum(keep, 1) - 1
+    local = np.full((B, T), -1)                                 # parents among the kept nodes; padding is a root
+    for b in range(B):
+        kept = np.nonzero(keep[b])[0]
+        local[b, :len(kept)] = np.where(par[b, kept] >= 0, new[b, par[b, kept]], -1)
+    counts = keep.sum(1)
+    accepted = draw_accepted(torch.from_numpy(counts.astype(np.int32)).to(DEVICE)).cpu().numpy()
+    row = np.cumsum(counts) - counts
+    own = np.concatenate([np.arange(c) for c in counts])
+    req = np.repeat(np.arange(B), counts)
+
+    def padded(x, fill):                                        # [H, N, ..] -> [B, H, T, ..]
+        if x is None:
+            return None
+        out = torch.full((B, T, H) + tuple(x.shape[2:]), fill, device=DEVICE, dtype=torch.float64)
+        out[req, own] = x.double().transpose(0, 1)
+        return out.transpose(1, 2)
+
+    O, U, S = _exact_layer(S, *[padded(planes[n], 1.0 if n == "alpha" else 0.0) for n in ("q", "k", "v", "alpha", "beta")],
+                           local, accepted)
+    packed = lambda x: None if x is None else x.transpose(1, 2)[req, own].transpose(0, 1).contiguous()
+    i32 = lambda x: torch.from_numpy(np.ascontiguousarray(x).astype(np.int32))
+    return {"O": packed(O), "U": packed(U), "S": S,
+            "selected": {"rho": torch.from_numpy(rho).double(), "counts": i32(counts),
+                         "offsets": i32(np.concatenate([row, [N]])), "parent_packed": i32(local),
+                         "node_id": i32(req * T + np.nonzero(keep)[1])}}
+
+
+def exact(case, seed):
+    """What the first pass returns, from plain torch in float64: the closed form over root paths."""
+    if case["kind"] == "front":
+        return _exact_front(case, seed)
+    if case["kind"] == "device":
+        return _exact_device(case, seed)
+    got = _exact_round(case, seed, commit=case["kind"] != "static")
+    return {"O": got["O"], "S": got["S"]} if case["kind"] == "session" else got
