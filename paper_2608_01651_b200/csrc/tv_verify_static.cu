@@ -80,6 +80,12 @@ unsigned char* scratch_address(int dev, cudaError_t* err) {
     unsigned char* ptr = nullptr;
     *err = cudaGetSymbolAddress((void**)&ptr, g_static_tree);
     if (*err != cudaSuccess) return nullptr;
+    // kernels load at their first use, which takes device memory: the ones this entry point may
+    // launch load here, whatever sizes come later
+    if (tv_prepare_verify_simt() != TV_OK) {
+      *err = (cudaError_t)tv_last_cuda_error();
+      return nullptr;
+    }
     table[dev] = ptr;
   }
   return table[dev];
