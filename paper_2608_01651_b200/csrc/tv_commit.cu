@@ -177,53 +177,68 @@ commit_factored_kernel(const CommitArgs a, const __grid_constant__ CommitLayers 
   }
 }
 
-// dk = 128 fast path.  A CTA of 4 warps owns 64 consecutive rows (value
-// channels) of one state; warp w owns rows 16w..16w+15 and a lane owns one
-// float4 column, so every load and store of a warp is one contiguous 512-byte
-// row and the key row k_j[4 lane .. 4 lane + 3] stays in registers across the
-// 16 rows.  All 16 loads of a thread are in flight before anything else
-// happens; several CTAs per SM keep the stream continuous.
+// dk = 64 and 128.  A CTA of 4 warps owns 4 * RPT * SUB consecutive rows (value channels) of one
+// state; DK / 4 lanes own one float4 column each (SUB = 128 / DK rows side by side in a warp), so every
+// load and store of a warp is whole rows of 256 or 512 bytes and the key row k_j[4 c .. 4 c + 3] stays in
+// registers across the thread's RPT rows.  All its loads are in flight before anything else happens.
+// Behind them is one chain of three dependent reads -- accepted node, its mask, the path's rows -- and
+// nothing in it is serial over the path: the thread of a node finds the node's place by counting mask
+// bits, a warp scan turns the gates into weights while the rows of up to 16 path nodes are on their way.
+// A chain that loaded those rows one by one and scanned the gates with one thread took 23.5 us where this
+// takes 21.7 (1024 items of 128 x 128, 20.5 at the copy peak), 4.2 against 2.4 at 16 items, and 24.1
+// against 16.8 on paths of 40 nodes (256 items).  A persistent form of it with double-buffered rows was
+// the slower one at every size too: 347 against 336 us on 16384 items.
 constexpr int kRowThreads = 128;
-constexpr int kRowsPerCta = 64;
 
-// Four keys of a path row, widened to float.
+// Four elements of a row, widened to float.
 template <bool BF16>
-__device__ __forceinline__ float4 load_key4(const void* kg, size_t idx) {
+__device__ __forceinline__ float4 widen4(const uint4& r) {
+  if (BF16)
+    return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16),
+                       __uint_as_float(r.y & 0xffff0000u));
+  return make_float4(__uint_as_float(r.x), __uint_as_float(r.y), __uint_as_float(r.z), __uint_as_float(r.w));
+}
+template <bool BF16>
+__device__ __forceinline__ uint4 load_raw4(const void* base, size_t idx) {
   if (BF16) {
-    const uint2 r = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(kg) + idx);
-    return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u),
-                       __uint_as_float(r.y << 16), __uint_as_float(r.y & 0xffff0000u));
+    const uint2 r = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(base) + idx);
+    return make_uint4(r.x, r.y, 0u, 0u);
   }
-  return *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(kg) + idx);
+  return *reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(base) + idx);
 }
 
-template <bool BF16>
-__global__ void __launch_bounds__(kRowThreads)
-commit_factored_dk128_kernel(const CommitArgs a, const __grid_constant__ CommitLayers tb) {
+template <bool BF16, int DK, int RPT, int CTAS>
+__global__ void __launch_bounds__(kRowThreads, CTAS)
+commit_rows_kernel(const CommitArgs a, const __grid_constant__ CommitLayers tb) {
+  constexpr int LPR = DK / 4, SUB = 32 / LPR, ROWS = 4 * RPT * SUB;
+  constexpr int KQ = kPathChunk * LPR / kRowThreads;              // a thread's key quads of a chunk
+  constexpr int UQ = kPathChunk * (ROWS / 4) / kRowThreads > 0 ? kPathChunk * (ROWS / 4) / kRowThreads : 1;
   __shared__ int path_s[TV_MAX_NODES];
-  __shared__ float w_s[TV_MAX_NODES];
+  __shared__ __align__(16) float w_s[TV_MAX_NODES];
+  __shared__ __align__(16) float al_s[TV_MAX_NODES];
   __shared__ float Pa_s;
-  __shared__ float al_s[TV_MAX_NODES];
-  __shared__ __align__(16) float k_s[kPathChunk][128];
-  __shared__ __align__(16) float cu_s[kPathChunk][kRowsPerCta];
+  __shared__ __align__(16) float k_s[kPathChunk][DK];
+  __shared__ __align__(16) float cu_s[kPathChunk][ROWS];
 
   const int dv = a.dv;
-  const int n_half = (dv + kRowsPerCta - 1) / kRowsPerCta;
-  const int item = blockIdx.x / n_half, half = blockIdx.x - item * n_half;
+  const int n_part = (dv + ROWS - 1) / ROWS;
+  const int item = blockIdx.x / n_part, part = blockIdx.x - item * n_part;
   const LayerItem li = layer_item(a, item);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int row0 = half * kRowsPerCta + warp * 16;
-  const size_t sbase = (size_t)li.it * dv * 128;
-  const float4* src = reinterpret_cast<const float4*>(tb.S_pre[li.l] + sbase) + (size_t)row0 * 32 + lane;
-  float4* dst = reinterpret_cast<float4*>(tb.S_new[li.l] + sbase) + (size_t)row0 * 32 + lane;
+  const int first = part * ROWS;                                  // of the CTA
+  const int own = (warp * SUB + lane / LPR) * RPT;                // of the thread, within the CTA
+  const int row0 = first + own;
+  const size_t sbase = (size_t)li.it * dv * DK;
+  const float4* src = reinterpret_cast<const float4*>(tb.S_pre[li.l] + sbase) + (size_t)row0 * LPR + lane % LPR;
+  float4* dst = reinterpret_cast<float4*>(tb.S_new[li.l] + sbase) + (size_t)row0 * LPR + lane % LPR;
 
   int acc = a.accepted[li.b];
   if (acc >= a.T) acc = -1;
   if (acc < 0 && a.in_place) return;
-  float4 s[16];
+  float4 s[RPT];
 #pragma unroll
-  for (int e = 0; e < 16; ++e)
-    if (row0 + e < dv) s[e] = ld_stream(src + e * 32);
+  for (int e = 0; e < RPT; ++e)
+    if (row0 + e < dv) s[e] = ld_stream(src + e * LPR);
   // Dependent launch: this grid may have started under the tail of the kernel in front of it
   // (a verify kernel, or the tree-metadata kernel when no verify call sits in between).  S_pre
   // and the accepted nodes are older than either; everything those kernels write -- U, and the
@@ -236,46 +251,92 @@ commit_factored_dk128_kernel(const CommitArgs a, const __grid_constant__ CommitL
   if (acc < 0) {
     if (a.in_place) return;
 #pragma unroll
-    for (int e = 0; e < 16; ++e)
-      if (row0 + e < dv) st_stream(dst + e * 32, s[e]);
+    for (int e = 0; e < RPT; ++e)
+      if (row0 + e < dv) st_stream(dst + e * LPR, s[e]);
     return;
   }
   const void* kg = tb.k[li.l];
   const void* vg = tb.v[li.l];
   const float* Ug = tb.U[li.l];
-  const int len = build_path(a.tree, rows.meta0, T, acc, tb.alpha[li.l], rows.g0, rows.g_rs, path_s, w_s, al_s, &Pa_s);
-  const float Pa = Pa_s;
-  bool scaled = false;
+
+  // the path: thread t is node t
+  int len;
+  {
+    const uint64_t* m = a.tree.anc + (rows.meta0 + acc) * 2;
+    const float al = tid < T ? tb.alpha[li.l][rows.g0 + (size_t)tid * rows.g_rs] : 1.f;
+    uint64_t m0 = m[0], m1 = m[1];
+    if (acc < 64) m0 |= 1ull << acc; else m1 |= 1ull << (acc - 64);
+    len = __popcll(m0) + __popcll(m1);
+    const uint64_t w = tid < 64 ? m0 : m1, bit = 1ull << (tid & 63);
+    const int pos = __popcll(w & (bit - 1)) + (tid < 64 ? 0 : __popcll(m0));
+    if (w & bit) {
+      path_s[pos] = tid;
+      al_s[pos] = al;
+    }
+    if (tid >= len) al_s[tid] = 1.f;
+  }
+  __syncthreads();
+
   for (int c0 = 0; c0 < len; c0 += kPathChunk) {
     const int nc = min(kPathChunk, len - c0);
-    if (c0) __syncthreads();
-    for (int i = tid; i < nc * 32; i += kRowThreads) {   // 4 keys per thread per step
-      const int p = i >> 5, k4 = i & 31;
-      *reinterpret_cast<float4*>(&k_s[p][k4 * 4]) =
-          load_key4<BF16>(kg, rows.qk0 + (size_t)path_s[c0 + p] * rows.qk_rs + k4 * 4);
-    }
-    for (int i = tid; i < nc * kRowsPerCta; i += kRowThreads) {
-      const int p = i >> 6, r = i & 63;
-      const int vrow = half * kRowsPerCta + r;
-      float u = 0.f;
-      if (vrow < dv)
-        u = a.has_U ? Ug[rows.o0 + (size_t)path_s[c0 + p] * rows.o_rs + vrow]
-                    : load_elem<BF16>(vg, rows.v0 + (size_t)path_s[c0 + p] * rows.v_rs + vrow);
-      cu_s[p][r] = w_s[c0 + p] * u;
-    }
-    __syncthreads();
-    if (!scaled) {   // first use of the state: the loads have had the path build to land
-      scaled = true;
+    uint4 kr[KQ], ur[UQ];
 #pragma unroll
-      for (int e = 0; e < 16; ++e) {
+    for (int q = 0; q < KQ; ++q) {
+      const int i = tid + q * kRowThreads, p = i / LPR;
+      if (p < nc) kr[q] = load_raw4<BF16>(kg, rows.qk0 + (size_t)((int64_t)path_s[c0 + p] * rows.qk_rs) + (i % LPR) * 4);
+    }
+#pragma unroll
+    for (int q = 0; q < UQ; ++q) {
+      const int i = tid + q * kRowThreads, p = i / (ROWS / 4), v = first + (i % (ROWS / 4)) * 4;
+      ur[q] = make_uint4(0u, 0u, 0u, 0u);
+      if (p < nc && v < dv)
+        ur[q] = a.has_U ? load_raw4<false>(Ug, rows.o0 + (size_t)((int64_t)path_s[c0 + p] * rows.o_rs) + v)
+                        : load_raw4<BF16>(vg, rows.v0 + (size_t)((int64_t)path_s[c0 + p] * rows.v_rs) + v);
+    }
+    if (c0 == 0) {
+      if (warp == 0) {   // weights P_a / P_j: the product of the gates behind a position, four positions per lane
+        const float4 x = *reinterpret_cast<const float4*>(&al_s[4 * lane]);
+        const float x3 = x.w, x2 = x.z * x3, x1 = x.y * x2, x0 = x.x * x1;
+        float behind = x0;   // product from this lane on
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const float y = __shfl_down_sync(0xffffffffu, behind, o);
+          if (lane + o < 32) behind *= y;
+        }
+        if (lane == 0) Pa_s = behind;
+        float next = __shfl_down_sync(0xffffffffu, behind, 1);
+        if (lane == 31) next = 1.f;
+        *reinterpret_cast<float4*>(&w_s[4 * lane]) = make_float4(x1 * next, x2 * next, x3 * next, next);
+      }
+      __syncthreads();
+      const float Pa = Pa_s;   // the first use of the state: its loads have had the path to land
+#pragma unroll
+      for (int e = 0; e < RPT; ++e) {
         s[e].x *= Pa; s[e].y *= Pa; s[e].z *= Pa; s[e].w *= Pa;
       }
+    } else {
+      __syncthreads();   // the chunk before has been read
     }
-    for (int p = 0; p < nc; ++p) {
-      const float4 kv = *reinterpret_cast<const float4*>(&k_s[p][lane * 4]);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float4 cu = *reinterpret_cast<const float4*>(&cu_s[p][warp * 16 + q * 4]);
+    for (int q = 0; q < KQ; ++q) {
+      const int i = tid + q * kRowThreads, p = i / LPR;
+      if (p < nc) *reinterpret_cast<float4*>(&k_s[p][(i % LPR) * 4]) = widen4<BF16>(kr[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < UQ; ++q) {
+      const int i = tid + q * kRowThreads, p = i / (ROWS / 4);
+      if (p < nc) {
+        const float w = w_s[c0 + p];
+        const float4 u = a.has_U ? widen4<false>(ur[q]) : widen4<BF16>(ur[q]);
+        *reinterpret_cast<float4*>(&cu_s[p][(i % (ROWS / 4)) * 4]) = make_float4(w * u.x, w * u.y, w * u.z, w * u.w);
+      }
+    }
+    __syncthreads();
+    for (int p = 0; p < nc; ++p) {
+      const float4 kv = *reinterpret_cast<const float4*>(&k_s[p][(lane % LPR) * 4]);
+#pragma unroll
+      for (int q = 0; q < RPT / 4; ++q) {
+        const float4 cu = *reinterpret_cast<const float4*>(&cu_s[p][own + q * 4]);
         const float c[4] = {cu.x, cu.y, cu.z, cu.w};
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -289,221 +350,8 @@ commit_factored_dk128_kernel(const CommitArgs a, const __grid_constant__ CommitL
     }
   }
 #pragma unroll
-  for (int e = 0; e < 16; ++e) {
-    if (row0 + e < dv) st_stream(dst + e * 32, s[e]);
-  }
-}
-
-// Persistent version of the dk = 128 row-owner kernel for accepted paths of at most 16 nodes
-// and batches of at most 256 requests.  A CTA walks units of 64 state rows; the accepted node
-// and path mask of every request are read once per CTA, and while the 16 loads of unit n are
-// in flight the path of unit n+1 is worked out (nodes from the mask bits, suffix products
-// P_a/P_j by a warp scan) and its key / value rows are fetched into registers, to be staged in
-// the other half of a double buffer after unit n has been updated.  No unit waits on a chain of
-// dependent global loads.
-#ifndef TV_STREAM_CTAS
-#define TV_STREAM_CTAS 5
-#endif
-constexpr int kStreamMaxB = 256;
-constexpr int kStreamMaxLen = 16;
-
-template <bool BF16>
-__global__ void __launch_bounds__(kRowThreads, TV_STREAM_CTAS)
-commit_stream_dk128_kernel(const CommitArgs a, const __grid_constant__ CommitLayers tb) {
-  __shared__ int acc_s[kStreamMaxB];
-  __shared__ uint64_t mask_s[kStreamMaxB][2];
-  __shared__ __align__(16) float k_s[2][kStreamMaxLen][128];
-  __shared__ __align__(16) float cu_s[2][kStreamMaxLen][kRowsPerCta];
-  __shared__ int node_s[2][kStreamMaxLen];
-  __shared__ float w_s[2][kStreamMaxLen];
-  __shared__ float Pa_s[2];
-  __shared__ int len_s[2];
-
-  const int dv = a.dv, T = a.T;
-  const int n_half = dv / kRowsPerCta;
-  const int n_units = a.L * a.B * a.H * n_half;
-  const int units_per_layer = a.B * a.H * n_half;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool in_place = a.in_place != 0;
-
-  for (int b = tid; b < a.B; b += kRowThreads) {
-    int acc = a.accepted[b];
-    const int nb = a.tree.offsets ? a.tree.offsets[b + 1] - a.tree.offsets[b] : T;
-    if (acc >= nb) acc = -1;
-    acc_s[b] = acc;
-    uint64_t m0 = 0, m1 = 0;
-    if (acc >= 0) {
-      const int tb_ = a.tree.n_trees == 1 ? 0 : b;
-      const uint64_t* m = a.tree.anc + ((size_t)tb_ * T + acc) * 2;
-      m0 = m[0];
-      m1 = m[1];
-      if (acc < 64) m0 |= 1ull << acc; else m1 |= 1ull << (acc - 64);
-    }
-    mask_s[b][0] = m0;
-    mask_s[b][1] = m1;
-  }
-  __syncthreads();
-
-  auto req_of = [&](int u) { return ((u / n_half) / a.H) % a.B; };
-  auto next_live = [&](int u) {   // first unit >= u (in this CTA's stride) that has work to do
-    while (u < n_units && in_place && acc_s[req_of(u)] < 0) u += gridDim.x;
-    return u;
-  };
-
-  // path of unit u into buffer nb: nodes, weights P_a/P_j, P_a, length (warp 0)
-  auto path_nodes = [&](int u, int nb) {
-    if (warp != 0) return;
-    const int b = req_of(u);
-    const uint64_t m0 = mask_s[b][0], m1 = mask_s[b][1];
-    const int c0 = __popcll(m0);
-    const int len = min(c0 + __popcll(m1), kStreamMaxLen);
-    int node = 0;
-    float al = 1.f;
-    if (lane < len) {
-      uint64_t w = lane < c0 ? m0 : m1;
-      const int r = lane < c0 ? lane : lane - c0;
-      for (int i = 0; i < r; ++i) w &= w - 1;
-      node = __ffsll((long long)w) - 1 + (lane < c0 ? 0 : 64);
-      const LayerItem li = layer_item(a, u / n_half);
-      const ItemRows rows = rows_of(a, li.it);
-      al = tb.alpha[li.l][rows.g0 + (size_t)node * rows.g_rs];
-    }
-    float incl = al;   // product of alpha over path positions >= lane
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const float up = __shfl_down_sync(0xffffffffu, incl, o);
-      if (lane + o < 32) incl *= up;
-    }
-    const float nxt = __shfl_down_sync(0xffffffffu, incl, 1);
-    if (lane < kStreamMaxLen) {
-      node_s[nb][lane] = node;
-      w_s[nb][lane] = lane + 1 < 32 ? nxt : 1.f;
-    }
-    if (lane == 0) {
-      Pa_s[nb] = incl;
-      len_s[nb] = len;
-    }
-  };
-
-  // key / value rows of unit u's path: 4 x 16 keys and 8 values per thread, in registers
-  uint2 kreg[4];
-  uint2 kreg2[4];
-  float ureg[8];
-  auto fetch_rows = [&](int u, int nb) {
-    const int item = u / n_half, half = u - item * n_half;
-    const LayerItem li = layer_item(a, item);
-    const ItemRows rows = rows_of(a, li.it);
-    const void* kg = tb.k[li.l];
-    const void* vg = tb.v[li.l];
-    const float* Ug = tb.U[li.l];
-    const int len = len_s[nb];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = tid + q * kRowThreads;          // (p, k4) = (i / 32, i % 32)
-      const int p = i >> 5, k4 = i & 31;
-      kreg[q] = make_uint2(0u, 0u);
-      kreg2[q] = make_uint2(0u, 0u);
-      if (p < len) {
-        const size_t idx = rows.qk0 + (size_t)node_s[nb][p] * rows.qk_rs + k4 * 4;
-        if (BF16) {
-          kreg[q] = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(kg) + idx);
-        } else {
-          const uint4 r = *reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(kg) + idx);
-          kreg[q] = make_uint2(r.x, r.y);
-          kreg2[q] = make_uint2(r.z, r.w);
-        }
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int i = tid + q * kRowThreads;          // (p, r) = (i / 64, i % 64)
-      const int p = i >> 6, r = i & 63;
-      ureg[q] = 0.f;
-      if (p < len) {
-        const int vrow = half * kRowsPerCta + r;
-        ureg[q] = a.has_U ? Ug[rows.o0 + (size_t)node_s[nb][p] * rows.o_rs + vrow]
-                          : load_elem<BF16>(vg, rows.v0 + (size_t)node_s[nb][p] * rows.v_rs + vrow);
-      }
-    }
-  };
-  auto stage_rows = [&](int nb) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = tid + q * kRowThreads;
-      const int p = i >> 5, k4 = i & 31;
-      float4 kv;
-      if (BF16) {
-        kv = make_float4(__uint_as_float(kreg[q].x << 16), __uint_as_float(kreg[q].x & 0xffff0000u),
-                         __uint_as_float(kreg[q].y << 16), __uint_as_float(kreg[q].y & 0xffff0000u));
-      } else {
-        kv = make_float4(__uint_as_float(kreg[q].x), __uint_as_float(kreg[q].y),
-                         __uint_as_float(kreg2[q].x), __uint_as_float(kreg2[q].y));
-      }
-      *reinterpret_cast<float4*>(&k_s[nb][p][k4 * 4]) = kv;
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int i = tid + q * kRowThreads;
-      const int p = i >> 6, r = i & 63;
-      cu_s[nb][p][r] = w_s[nb][p] * ureg[q];
-    }
-  };
-
-  int u = next_live(blockIdx.x);
-  if (u >= n_units) return;
-  path_nodes(u, 0);
-  __syncthreads();
-  fetch_rows(u, 0);
-  stage_rows(0);
-  __syncthreads();
-
-  for (int n = 0; u < n_units; ++n) {
-    const int cb = n & 1, nb = cb ^ 1;
-    const int un = next_live(u + gridDim.x);
-    // a. the 16 loads of this unit
-    const int row0 = warp * 16;
-    const int l = u / units_per_layer, ul = u - l * units_per_layer;
-    const float4* src = reinterpret_cast<const float4*>(tb.S_pre[l]) + ((size_t)ul * kRowsPerCta + row0) * 32 + lane;
-    float4* dst = reinterpret_cast<float4*>(tb.S_new[l]) + ((size_t)ul * kRowsPerCta + row0) * 32 + lane;
-    float4 s[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) s[e] = ld_stream(src + e * 32);
-    // b-d. the path of the next unit, and its rows into registers
-    if (un < n_units) path_nodes(un, nb);
-    __syncthreads();
-    if (un < n_units) fetch_rows(un, nb);
-    // e. update and store this unit
-    const float Pa = Pa_s[cb];
-    const int len = len_s[cb];
-    if (len > 0) {
-#pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        s[e].x *= Pa; s[e].y *= Pa; s[e].z *= Pa; s[e].w *= Pa;
-      }
-      for (int p = 0; p < len; ++p) {
-        const float4 kv = *reinterpret_cast<const float4*>(&k_s[cb][p][lane * 4]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float4 cu = *reinterpret_cast<const float4*>(&cu_s[cb][p][warp * 16 + q * 4]);
-          const float c[4] = {cu.x, cu.y, cu.z, cu.w};
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            float4& x = s[q * 4 + t];
-            x.x = fmaf(c[t], kv.x, x.x);
-            x.y = fmaf(c[t], kv.y, x.y);
-            x.z = fmaf(c[t], kv.z, x.z);
-            x.w = fmaf(c[t], kv.w, x.w);
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < 16; ++e) st_stream(dst + e * 32, s[e]);
-    // f. the next unit's rows into the other buffer
-    if (un < n_units) stage_rows(nb);
-    __syncthreads();
-    u = un;
-  }
+  for (int e = 0; e < RPT; ++e)
+    if (row0 + e < dv) st_stream(dst + e * LPR, s[e]);
 }
 
 // Delta rule without stored corrections: every row v of the [dv][dk] state
@@ -639,6 +487,29 @@ cudaError_t launch_after_verify(void (*kernel)(const CommitArgs, const CommitLay
   return cudaLaunchKernelEx(&cfg, kernel, a, tb);
 }
 
+// Rows per thread.  Four (and no limit on registers) while that puts at most four CTAs on an SM: nothing
+// but the chain counts there (16 items of 128 x 128: 2.4 us, 3.1 with sixteen rows).  Four, eight CTAs per
+// SM, while all of them are resident (128 items: 4.6 us against 5.2 with eight rows).  Beyond that
+// 64 rows per CTA -- sixteen per thread, eight for dk = 64: fewest paths to work out per byte (a round of
+// 1024 items 53.2 us against 55.8 with half as many rows, of 512 items 40.4 against 41.1).
+constexpr int kSMs = 148;
+template <bool BF16, int DK>
+cudaError_t launch_rows(const CommitArgs& a, const CommitLayers& tb, int items, cudaStream_t stream) {
+  constexpr int kRpt = DK == 128 ? 16 : 8, kCtas = DK == 128 ? 4 : BF16 ? 8 : 7;   // 64 rows per CTA
+  constexpr int rows4 = 16 * (128 / DK), rows = 64;
+  const int64_t ctas4 = (int64_t)items * ((a.dv + rows4 - 1) / rows4);
+  if (ctas4 <= 4 * kSMs) return launch_after_verify(commit_rows_kernel<BF16, DK, 4, 4>, (int)ctas4, stream, a, tb);
+  if (ctas4 <= 8 * kSMs) return launch_after_verify(commit_rows_kernel<BF16, DK, 4, 8>, (int)ctas4, stream, a, tb);
+  const int ctas = items * ((a.dv + rows - 1) / rows);
+  // From some seven waves on an ordinary launch: most CTAs start long after the kernel in front is done,
+  // and the dependent launch measured slower (a round of 24576 items 1612-1631 us against 1667).
+  if (ctas >= 30 * kSMs) {
+    commit_rows_kernel<BF16, DK, kRpt, kCtas><<<ctas, kRowThreads, 0, stream>>>(a, tb);
+    return cudaSuccess;   // the caller asks for the launch's error
+  }
+  return launch_after_verify(commit_rows_kernel<BF16, DK, kRpt, kCtas>, ctas, stream, a, tb);
+}
+
 }  // namespace
 
 int tv_launch_commit(const CommitArgs& a, const CommitLayers& tb, cudaStream_t stream) {
@@ -646,25 +517,10 @@ int tv_launch_commit(const CommitArgs& a, const CommitLayers& tb, cudaStream_t s
   const int items = a.L * a.B * a.H;
   if ((size_t)a.dk * a.dv > (size_t)kMaxVec * kThreads * 4) return TV_ERR_UNSUPPORTED;
   const bool recompute = a.rule == TV_GATED_DELTA && !a.has_U;
-  static thread_local int sm_count = 0;
-  if (!sm_count) {
-    int dev = 0;
-    TV_CUDA_TRY(cudaGetDevice(&dev));
-    TV_CUDA_TRY(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
-  }
-  const int units = a.dv % kRowsPerCta == 0 ? items * (a.dv / kRowsPerCta) : 0;
-  // the persistent kernel pays a prologue per CTA: worth it from about six units per CTA on
-  if (!recompute && a.dk == 128 && units >= 6 * TV_STREAM_CTAS * sm_count && a.B <= kStreamMaxB &&
-      a.tree.max_depth_all < kStreamMaxLen) {
-    const int ctas = TV_STREAM_CTAS * sm_count;
-    // ordinary launch: at this size the dependent launch measured slower (13.4 vs 12.7 ms per step
-    // on 48 layers of 128 requests)
-    if (a.bf16) commit_stream_dk128_kernel<true><<<ctas, kRowThreads, 0, stream>>>(a, tb);
-    else commit_stream_dk128_kernel<false><<<ctas, kRowThreads, 0, stream>>>(a, tb);
-  } else if (!recompute && a.dk == 128) {
-    const int ctas = items * ((a.dv + kRowsPerCta - 1) / kRowsPerCta);
-    TV_CUDA_TRY(a.bf16 ? launch_after_verify(commit_factored_dk128_kernel<true>, ctas, stream, a, tb)
-                       : launch_after_verify(commit_factored_dk128_kernel<false>, ctas, stream, a, tb));
+  if (!recompute && a.dk == 128) {
+    TV_CUDA_TRY((a.bf16 ? launch_rows<true, 128> : launch_rows<false, 128>)(a, tb, items, stream));
+  } else if (!recompute && a.dk == 64) {
+    TV_CUDA_TRY((a.bf16 ? launch_rows<true, 64> : launch_rows<false, 64>)(a, tb, items, stream));
   } else if (!recompute) {
     TV_CUDA_TRY(a.bf16 ? launch_after_verify(commit_factored_kernel<true>, items, stream, a, tb, kThreads)
                        : launch_after_verify(commit_factored_kernel<false>, items, stream, a, tb, kThreads));
