@@ -234,7 +234,13 @@ commit_rows_kernel(const CommitArgs a, const __grid_constant__ CommitLayers tb) 
 
   int acc = a.accepted[li.b];
   if (acc >= a.T) acc = -1;
-  if (acc < 0 && a.in_place) return;
+  if (acc < 0 && a.in_place) {
+    // Nothing to do, but not before the kernel in front is done: if every request is rejected these are all
+    // the grid's threads, and the kernel behind -- an upload, a convolution -- waits for this grid only
+    // before it overwrites what the kernel in front (verify) may still be reading.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   float4 s[RPT];
 #pragma unroll
   for (int e = 0; e < RPT; ++e)
@@ -470,8 +476,8 @@ commit_delta_rows_kernel(const CommitArgs a, const __grid_constant__ CommitLayer
 
 // Programmatic dependent launch behind the verify kernel (which releases its dependents once the
 // tree metadata it waited for is complete): the commit grid is scheduled as SMs drain, and every
-// kernel launched this way orders itself with griddepcontrol.wait.  Behind any other kernel this
-// is an ordinary launch.
+// thread of every kernel launched this way passes griddepcontrol.wait before it ends, so that a commit
+// never ends before the kernel in front of it.  Behind any other kernel this is an ordinary launch.
 cudaError_t launch_after_verify(void (*kernel)(const CommitArgs, const CommitLayers), int ctas, cudaStream_t stream,
                                 const CommitArgs& a, const CommitLayers& tb, int threads = kRowThreads) {
   cudaLaunchConfig_t cfg = {};

@@ -75,3 +75,37 @@ def test_unsynchronised_rounds_equal_synchronised_ones(name, B, H, T, rule, impl
                     assert x is None
                 else:
                     assert torch.equal(x, y), f"round {r}, output {i} differs (repeat {rep})"
+
+
+@pytest.mark.parametrize("rule", [tv.GATED, tv.DELTA])
+@pytest.mark.parametrize("d,T", [(64, 64), (128, 64), (64, 128), (128, 128)])
+def test_commit_that_rejects_every_request_keeps_the_order(d, T, rule):
+    """verify -> in-place commit in which no request accepts anything -> other trees -> verify, queued
+    without synchronisation.  The commit has nothing to do, and must still not end before the verify in
+    front of it: the upload behind it waits for the commit only and then overwrites the masks."""
+    wl = inputs.workload("c4", B=12, H=16, T=T, dk=d, dv=d, rule=rule, qkv_dtype=inputs.F32, seed=T + d)
+    t = {n: None if x is None else x.to(DEV) for n, x in inputs.make_tensors(wl).items()}
+    t["k"] = t["k"] * (8.0 / d ** 0.5)
+    trees = [inputs.make_trees(wl)[0], np.stack([inputs.tree_chain(T)] * wl.B)]
+    none = torch.full((wl.B,), -1, dtype=torch.int32, device=DEV)
+    tree = tv.tree_build(trees[0])
+
+    def run(sync):
+        pause = torch.cuda.synchronize if sync else (lambda: None)
+        S = t["S_pre"].clone()
+        outs = [torch.zeros(wl.B, wl.H, T, d, device=DEV) for _ in range(4)]
+        torch.cuda.synchronize()
+        for r in range(2):
+            tree.rebuild(trees[r]).upload(); pause()
+            tv.tree_verify(tree, S, t["q"], t["k"], t["v"], t["alpha"], t["beta"], rule=rule, O=outs[2 * r],
+                           U=outs[2 * r + 1], impl=tv.IMPL_SIMT); pause()
+            tv.commit_path(tree, none, S, t["k"], t["v"], t["alpha"], t["beta"], rule=rule, U=outs[2 * r + 1]); pause()
+        tree.rebuild(trees[0]).upload()      # over the masks of the last verify
+        torch.cuda.synchronize()
+        return [S] + outs
+
+    ref = run(sync=True)
+    assert torch.equal(ref[0], t["S_pre"]) and torch.isfinite(ref[3]).all()
+    for rep in range(3):
+        for i, (x, y) in enumerate(zip(run(sync=False), ref)):
+            assert torch.equal(x, y), (rep, i)
