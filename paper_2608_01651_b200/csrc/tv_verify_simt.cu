@@ -17,8 +17,9 @@
 //            substitution, 16 nodes at a time: one thread per column for the diagonal block, a
 //            product over all threads for the rows below.
 // The form is chosen per CTA from the masks (trees of up to 64 nodes) or by the launcher from the
-// depth it knows (up to 128 nodes, two row blocks).  Entries that are zero are skipped in both, so a
-// non-finite value stays on the paths through its node.
+// depth it knows (up to 128 nodes, two row blocks).  In both, a node's sums run over the nodes of its path,
+// whatever their coefficients are: a non-finite value stays on the paths through its node, and a zero gate,
+// key or query below it does not hide it (0 x NaN and 0 x inf are NaN).
 //
 // What bounds it: fp32 FMA issue in the state product, and the latency of the short phases behind it
 // with eight warps on an SM.  T = 63, 128 items, f32, delta: 27 us, of them 13 in the state product (8.6
@@ -36,6 +37,7 @@
 namespace {
 
 constexpr int kLD = TV_MAX_DIM + 4;  // floats between operand rows: 33 16-byte words, 8 consecutive rows miss each other's banks
+constexpr int kMaskParts = 8;         // 16-bit parts of a node's mask of 128 bits
 constexpr int kPath = 16;            // entries of a node's coefficient table: itself and 15 ancestors
 
 // 4 consecutive elements starting at idx (idx % 4 == 0) widened to float.
@@ -128,11 +130,15 @@ __device__ __forceinline__ void fma4(float4& o, float s, const float4& u) {
   o.w = fmaf(s, u.w, o.w);
 }
 
-// out[m][h] += sign * sum over the 16 nodes j of one block: w_m[j] * U[j][column quad h], for the row
-// tiles m >= m0.  w_m: row tile m of a coefficient matrix (16 rows of `wld` floats apart).
+// out[m][h] += sign * sum over the nodes j of one block of 16 that lie on the row's path: w_m[j] * U[j][column
+// quad h], for the row tiles m >= m0.  w_m: row tile m of a coefficient matrix (16 rows of `wld` floats apart);
+// on: the block's part of the path mask of the thread's first row.
 template <int MT, int NC>
-__device__ __forceinline__ void accumulate16(float4 (&out)[MT][NC], int m0, const float* w, int wld, const float* U,
-                                             int ustride, int hstep, float sign) {
+__device__ __forceinline__ void accumulate16(float4 (&out)[MT][NC], int m0, const float* w, int wld, const uint16_t* on,
+                                             const float* U, int ustride, int hstep, float sign) {
+  uint32_t path[MT];
+#pragma unroll
+  for (int m = 0; m < MT; ++m) path[m] = m < m0 ? 0u : on[16 * m * kMaskParts];
 #pragma unroll 2
   for (int j = 0; j < 16; j += 4) {
     float4 u[4][NC];
@@ -147,7 +153,7 @@ __device__ __forceinline__ void accumulate16(float4 (&out)[MT][NC], int m0, cons
       const float cj[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
       for (int x = 0; x < 4; ++x)
-        if (cj[x] != 0.f) {   // off the path: whatever U holds there stays out
+        if ((path[m] >> (j + x)) & 1) {   // whatever U and the coefficients hold off the path stays out
 #pragma unroll
           for (int h = 0; h < NC; ++h) fma4(out[m][h], sign * cj[x], u[x][h]);
         }
@@ -155,31 +161,37 @@ __device__ __forceinline__ void accumulate16(float4 (&out)[MT][NC], int m0, cons
   }
 }
 
-// Forward substitution of one diagonal block of 16 nodes, one thread per column.
-__device__ __forceinline__ void solve16(float* u, int ustride, const float* g, int gld) {
+// Forward substitution of one diagonal block of 16 nodes, one thread per column.  on: the block's part of
+// the path mask of its first node.
+__device__ __forceinline__ void solve16(float* u, int ustride, const float* g, int gld, const uint16_t* on) {
   float r[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) r[i] = u[i * ustride];
 #pragma unroll
   for (int i = 1; i < 16; ++i) {
+    const uint32_t path = on[i * kMaskParts];
 #pragma unroll
     for (int j = 0; j < i; j += 4) {
       const float4 w = *reinterpret_cast<const float4*>(g + i * gld + j);
       const float wj[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
       for (int x = 0; x < 4; ++x)
-        if (j + x < i && wj[x] != 0.f) r[i] = fmaf(-wj[x], r[j + x], r[i]);
+        if (j + x < i && ((path >> (j + x)) & 1)) r[i] = fmaf(-wj[x], r[j + x], r[i]);
     }
   }
 #pragma unroll
   for (int i = 1; i < 16; ++i) u[i * ustride] = r[i];
 }
 
-// Tables of an item in shared memory, entries past the tree included (no ancestors, alpha = beta = 0).
+// Tables of an item in shared memory, entries past the tree included (no path, alpha = beta = 0).
 struct Tables {
   float2* link;     // alpha and the parent (int bits, -1 at a root child) of every node
   float* beta;
-  uint64_t* anc;    // [2] per node
+  uint64_t* path;   // [2] per node: the node and its ancestors
+  // Part b of node i's mask: nodes 16 b .. 16 b + 15.
+  __device__ __forceinline__ const uint16_t* on(int i, int b) const {
+    return reinterpret_cast<const uint16_t*>(path) + i * kMaskParts + b;
+  }
 };
 
 // One node per thread: reads masks and gates, fills the tables, returns the node's ancestor count.
@@ -196,8 +208,9 @@ __device__ __forceinline__ int load_meta(const VerifyArgs& a, const ItemRows& ro
     if (DELTA) be = a.beta[rows.g0 + (size_t)tid * rows.g_rs];
   }
   const int parent = m1 ? 127 - __clzll((long long)m1) : m0 ? 63 - __clzll((long long)m0) : -1;
-  t.anc[2 * tid] = m0;
-  t.anc[2 * tid + 1] = m1;
+  const uint64_t self = tid < rows.n ? 1ull << (tid & 63) : 0;
+  t.path[2 * tid] = tid < 64 ? m0 | self : m0;
+  t.path[2 * tid + 1] = tid < 64 ? m1 : m1 | self;
   t.link[tid] = make_float2(al, __int_as_float(parent));
   t.beta[tid] = be;
   return __popcll(m0) + __popcll(m1);
@@ -283,6 +296,7 @@ struct Cfg {
   static constexpr int NB = 16 * MT;              // nodes of a row block
   static constexpr int N = NB * NBLK;
   static constexpr int DVC = 4 * CT * NC;         // value columns of the CTA
+  static constexpr bool kBlockForm = NBLK == 1 && N > kPath;   // 16 nodes have at most 15 ancestors
   // One row block: U and B0 take the state's place, C and G (block form) that of the operand rows.
   // Two: U takes the k rows' place and B0 the q rows', block by block.
   // shared memory, in floats: q rows and k rows of block 0 (, of block 1), state, tables
@@ -293,8 +307,8 @@ struct Cfg {
   static constexpr int oDep = oIdx + kPath * N / 4;  // uint8 [N]: depths
   static constexpr int oOrd = oDep + N / 4;          // uint8 [N]: nodes by depth
   static constexpr int oLev = oOrd + N / 4;          // int [kPath + 1]: first place of every depth
-  static constexpr int oAnc = oLev + 20;
-  static constexpr int oLink = oAnc + 4 * N;
+  static constexpr int oMask = oLev + 20;
+  static constexpr int oLink = oMask + 4 * N;
   static constexpr int oP = oLink + 2 * N;
   static constexpr int oBe = oP + N;
   static constexpr size_t kSmem = sizeof(float) * (oBe + N);
@@ -332,7 +346,7 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
   uint8_t* const dep_s = reinterpret_cast<uint8_t*>(sm + C::oDep);
   uint8_t* const ord_s = reinterpret_cast<uint8_t*>(sm + C::oOrd);
   int* const lev_s = reinterpret_cast<int*>(sm + C::oLev);
-  const Tables tab = {reinterpret_cast<float2*>(sm + C::oLink), sm + C::oBe, reinterpret_cast<uint64_t*>(sm + C::oAnc)};
+  const Tables tab = {reinterpret_cast<float2*>(sm + C::oLink), sm + C::oBe, reinterpret_cast<uint64_t*>(sm + C::oMask)};
   float* const P_s = sm + C::oP;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -373,7 +387,7 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
   if (tid < kPath + 2) lev_s[tid] = 0;
   const int n_anc = load_meta<DELTA>(a, rows, C::N, tab);
   if (tid < C::N) dep_s[tid] = tid < T ? (uint8_t)n_anc : 255;
-  const bool deep = __syncthreads_or(n_anc >= kPath) && NBLK == 1;
+  const bool deep = __syncthreads_or(n_anc >= kPath) && C::kBlockForm;
 
   if (!deep) {
     // path form: every node's thread lists its path with the decay ratios, and the nodes by depth
@@ -556,7 +570,7 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
     return;
   }
 
-  if constexpr (NBLK == 1) {
+  if constexpr (C::kBlockForm) {
     constexpr int NTS = C::NB / CT;   // a thread's score columns
     constexpr int ULD = C::DVC, GLD = C::NB + 4;   // floats between rows of U; of C and G
     float* const C_s = X;
@@ -570,13 +584,11 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
 #pragma unroll
       for (int m = 0; m < MT; ++m) {
         const int i = rt + 16 * m;
-        const uint64_t anc = tab.anc[2 * i];
 #pragma unroll
         for (int n = 0; n < NTS; ++n) {
           const int j = ct + CT * n;
-          const bool up = (anc >> j) & 1;
-          C_s[i * GLD + j] = up || (j == i && i < T) ? pair_sum(acc[m][n]) : 0.f;
-          if (DELTA) G_s[i * GLD + j] = up ? pair_sum(acc[MT + m][n]) : 0.f;
+          C_s[i * GLD + j] = pair_sum(acc[m][n]);
+          if (DELTA) G_s[i * GLD + j] = pair_sum(acc[MT + m][n]);
         }
       }
     }
@@ -588,7 +600,7 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
 #pragma unroll
       for (int b = 0; b < MT; ++b) {
         if (16 * b >= T) break;
-        if (tid < C::DVC) solve16(U_s + 16 * b * ULD + tid, ULD, G_s + 16 * b * GLD + 16 * b, GLD);
+        if (tid < C::DVC) solve16(U_s + 16 * b * ULD + tid, ULD, G_s + 16 * b * GLD + 16 * b, GLD, tab.on(16 * b, b));
         __syncthreads();
         if (b + 1 < MT && 16 * (b + 1) < T) {
           float4 r[MT][NC];
@@ -597,8 +609,8 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
 #pragma unroll
             for (int h = 0; h < NC; ++h)
               r[m][h] = *reinterpret_cast<const float4*>(U_s + (rt + 16 * m) * ULD + 4 * (ct + h * CT));
-          accumulate16<MT, NC>(r, b + 1, G_s + rt * GLD + 16 * b, GLD, U_s + 16 * b * ULD + 4 * ct, ULD,
-                               4 * CT, -1.f);
+          accumulate16<MT, NC>(r, b + 1, G_s + rt * GLD + 16 * b, GLD, tab.on(rt, b), U_s + 16 * b * ULD + 4 * ct,
+                               ULD, 4 * CT, -1.f);
 #pragma unroll
           for (int m = b + 1; m < MT; ++m)
 #pragma unroll
@@ -616,7 +628,8 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
       for (int h = 0; h < NC; ++h) o[m][h] = *reinterpret_cast<const float4*>(C::B0(sm, rt + 16 * m) + 4 * (ct + h * CT));
 #pragma unroll
     for (int b = 0; b < MT; ++b)
-      accumulate16<MT, NC>(o, b, C_s + rt * GLD + 16 * b, GLD, U_s + 16 * b * ULD + 4 * ct, ULD, 4 * CT, 1.f);
+      accumulate16<MT, NC>(o, b, C_s + rt * GLD + 16 * b, GLD, tab.on(rt, b), U_s + 16 * b * ULD + 4 * ct, ULD, 4 * CT,
+                           1.f);
 #pragma unroll
     for (int m = 0; m < MT; ++m)
 #pragma unroll
@@ -642,8 +655,8 @@ struct DeepCfg {
   static constexpr int oB0 = oU + N * DVC;
   static constexpr int oC = oB0 + NB * DVC;
   static constexpr int oG = oC + NB * GLD;
-  static constexpr int oAnc = oG + (DELTA ? NB * GLD : 0);
-  static constexpr int oLink = oAnc + 4 * N;
+  static constexpr int oMask = oG + (DELTA ? NB * GLD : 0);
+  static constexpr int oLink = oMask + 4 * N;
   static constexpr int oJump = oLink + 2 * N;
   static constexpr int oP = oJump + 2 * N;
   static constexpr int oBe = oP + N;
@@ -662,7 +675,7 @@ __global__ void __launch_bounds__(256) verify_simt_deep_kernel(const __grid_cons
   float* const B0_s = sm + C::oB0;
   float* const C_s = sm + C::oC;
   float* const G_s = sm + C::oG;
-  const Tables tab = {reinterpret_cast<float2*>(sm + C::oLink), sm + C::oBe, reinterpret_cast<uint64_t*>(sm + C::oAnc)};
+  const Tables tab = {reinterpret_cast<float2*>(sm + C::oLink), sm + C::oBe, reinterpret_cast<uint64_t*>(sm + C::oMask)};
   float2* const jump_s = reinterpret_cast<float2*>(sm + C::oJump);
   float* const P_s = sm + C::oP;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -725,13 +738,11 @@ __global__ void __launch_bounds__(256) verify_simt_deep_kernel(const __grid_cons
 #pragma unroll
       for (int m = 0; m < MT; ++m) {
         const int i = rt + 16 * m;
-        const uint64_t a0 = tab.anc[2 * (i0 + i)], a1 = tab.anc[2 * (i0 + i) + 1];
 #pragma unroll
         for (int n = 0; n < MT; ++n) {
           const int j = J * NB + ct + CT * n;
-          const bool up = ((j < 64 ? a0 : a1) >> (j & 63)) & 1;
-          C_s[i * C::GLD + j] = up || (j == i0 + i && j < T) ? pair_sum(acc[m][n]) : 0.f;
-          if (DELTA) G_s[i * C::GLD + j] = up ? pair_sum(acc[MT + m][n]) : 0.f;
+          C_s[i * C::GLD + j] = pair_sum(acc[m][n]);
+          if (DELTA) G_s[i * C::GLD + j] = pair_sum(acc[MT + m][n]);
         }
       }
     }
@@ -744,7 +755,8 @@ __global__ void __launch_bounds__(256) verify_simt_deep_kernel(const __grid_cons
         float4 r[MT][1];
 #pragma unroll
         for (int m = 0; m < MT; ++m) r[m][0] = *reinterpret_cast<const float4*>(U_s + (i0 + rt + 16 * m) * C::DVC + 4 * ct);
-        accumulate16<MT, 1>(r, m0, G_s + rt * C::GLD + j0, C::GLD, U_s + j0 * C::DVC + 4 * ct, C::DVC, 0, -1.f);
+        accumulate16<MT, 1>(r, m0, G_s + rt * C::GLD + j0, C::GLD, tab.on(i0 + rt, j0 / 16), U_s + j0 * C::DVC + 4 * ct,
+                            C::DVC, 0, -1.f);
 #pragma unroll
         for (int m = 0; m < MT; ++m)
           if (m >= m0) *reinterpret_cast<float4*>(U_s + (i0 + rt + 16 * m) * C::DVC + 4 * ct) = r[m][0];
@@ -758,7 +770,8 @@ __global__ void __launch_bounds__(256) verify_simt_deep_kernel(const __grid_cons
       for (int b = 0; b < MT; ++b) {
         if (i0 + 16 * b >= T) break;
         if (tid < C::DVC)
-          solve16(U_s + (i0 + 16 * b) * C::DVC + tid, C::DVC, G_s + 16 * b * C::GLD + i0 + 16 * b, C::GLD);
+          solve16(U_s + (i0 + 16 * b) * C::DVC + tid, C::DVC, G_s + 16 * b * C::GLD + i0 + 16 * b, C::GLD,
+                  tab.on(i0 + 16 * b, i0 / 16 + b));
         __syncthreads();
         if (b + 1 < MT && i0 + 16 * (b + 1) < T) {
           below(i0 + 16 * b, b + 1);
@@ -773,11 +786,13 @@ __global__ void __launch_bounds__(256) verify_simt_deep_kernel(const __grid_cons
     if (I > 0) {
 #pragma unroll 1
       for (int b = 0; b < MT; ++b)
-        accumulate16<MT, 1>(o, 0, C_s + rt * C::GLD + 16 * b, C::GLD, U_s + 16 * b * C::DVC + 4 * ct, C::DVC, 0, 1.f);
+        accumulate16<MT, 1>(o, 0, C_s + rt * C::GLD + 16 * b, C::GLD, tab.on(i0 + rt, b), U_s + 16 * b * C::DVC + 4 * ct,
+                            C::DVC, 0, 1.f);
     }
 #pragma unroll
     for (int b = 0; b < MT; ++b)
-      accumulate16<MT, 1>(o, b, C_s + rt * C::GLD + i0 + 16 * b, C::GLD, U_s + (i0 + 16 * b) * C::DVC + 4 * ct, C::DVC, 0, 1.f);
+      accumulate16<MT, 1>(o, b, C_s + rt * C::GLD + i0 + 16 * b, C::GLD, tab.on(i0 + rt, i0 / 16 + b),
+                          U_s + (i0 + 16 * b) * C::DVC + 4 * ct, C::DVC, 0, 1.f);
 #pragma unroll
     for (int m = 0; m < MT; ++m) {
       const int i = i0 + rt + 16 * m;

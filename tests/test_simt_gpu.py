@@ -98,3 +98,32 @@ def test_nan_stays_on_its_paths(T, tree):
     hit = np.array([bad in orc.path_to(parents[0], i) for i in range(T)])
     assert np.isnan(O[0][:, hit]).all()
     assert np.array_equal(O[0][:, ~hit], clean[0][:, ~hit]) and np.array_equal(O[1], clean[1])
+
+
+@pytest.mark.parametrize("zero", ["gate", "key"])
+@pytest.mark.parametrize("rule", [inputs.GATED, inputs.DELTA])
+@pytest.mark.parametrize("T,tree", [(30, "frontier"), (40, "chain"), (100, "frontier"), (100, "chain")])
+def test_a_zero_coefficient_does_not_hide_a_nan(T, tree, rule, zero):
+    """The coefficients below a non-finite value row are exactly zero, from a gate of zero or from the
+    row's own key: 0 x NaN is NaN for every node of the paths through it, in both forms."""
+    wl = inputs.workload("c4", B=2, H=2, T=T, rule=rule, tree=tree, qkv_dtype=inputs.F32, seed=T)
+    tens = inputs.make_tensors(wl)
+    tens["k"] = tens["k"] * (8.0 / wl.dk ** 0.5)
+    parents, accepted = inputs.make_trees(wl)
+    from oracle import tree_oracle as orc
+    below = [sum(n in orc.path_to(parents[0], i) for i in range(T)) for n in range(T)]
+    bad = max(range(1, T), key=lambda n: below[n] if n >= T // 8 else 0)   # a node with many below it
+    hit = np.array([bad in orc.path_to(parents[0], i) for i in range(T)])
+    assert hit.sum() > 1
+    if zero == "gate":
+        tens["alpha"][0][:, torch.from_numpy(parents[0] == bad)] = 0.0
+    else:
+        tens["k"][0, :, bad] = 0.0
+    O0, U0 = pu.gpu_round(wl, parents, accepted, tens, impl=tv.IMPL_SIMT)[:2]
+    assert np.isfinite(O0).all()
+    tens["v"][0, :, bad] = float("nan")
+    O, U = pu.gpu_round(wl, parents, accepted, tens, impl=tv.IMPL_SIMT)[:2]
+    assert np.isnan(O[0][:, hit]).all()
+    assert np.array_equal(O[0][:, ~hit], O0[0][:, ~hit]) and np.array_equal(O[1], O0[1])
+    if rule == inputs.DELTA:
+        assert np.isnan(U[0][:, hit]).all() and np.array_equal(U[0][:, ~hit], U0[0][:, ~hit])
