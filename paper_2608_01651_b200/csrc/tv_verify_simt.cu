@@ -9,6 +9,8 @@
 //            decay ratio is a running product of alpha along the path, never a division
 //   solve    delta rule: (I + G) U = R, which is triangular in topological order (Lemma 2)
 //   readout  O = B0 + C U
+// The sums over a path start from zero and meet R or B0 once, at the end: a term added to R itself rounds at
+// R's size, which on a chain of 128 nodes left U with an error of 2.1e-7 where this leaves 0.7e-7.
 // The state product is the same for every tree.  The rest has two forms:
 //   paths    (at most 15 ancestors per node: every drafted tree) only the pairs that exist: eight
 //            lanes walk up from a node and leave its coefficients in a table of 16 entries; nodes of
@@ -130,16 +132,23 @@ __device__ __forceinline__ void fma4(float4& o, float s, const float4& u) {
   o.w = fmaf(s, u.w, o.w);
 }
 
-// out[m][h] += sign * sum over the nodes j of one block of 16 that lie on the row's path: w_m[j] * U[j][column
+__device__ __forceinline__ float4 add4(const float4& a, const float4& b) {
+  return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+__device__ __forceinline__ float4 sub4(const float4& a, const float4& b) {
+  return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+}
+
+// out[m][h] += the sum over the nodes j of one block of 16 that lie on the row's path: w_m[j] * U[j][column
 // quad h], for the row tiles m >= m0.  w_m: row tile m of a coefficient matrix (16 rows of `wld` floats apart);
 // on: the block's part of the path mask of the thread's first row.
 template <int MT, int NC>
 __device__ __forceinline__ void accumulate16(float4 (&out)[MT][NC], int m0, const float* w, int wld, const uint16_t* on,
-                                             const float* U, int ustride, int hstep, float sign) {
+                                             const float* U, int ustride, int hstep) {
   uint32_t path[MT];
 #pragma unroll
   for (int m = 0; m < MT; ++m) path[m] = m < m0 ? 0u : on[16 * m * kMaskParts];
-#pragma unroll 2
+#pragma unroll (MT > 2 ? 2 : 1)   // MT = 2, unrolled: the kernel, at its limit of 128 registers, is 8 % slower
   for (int j = 0; j < 16; j += 4) {
     float4 u[4][NC];
 #pragma unroll
@@ -155,7 +164,7 @@ __device__ __forceinline__ void accumulate16(float4 (&out)[MT][NC], int m0, cons
       for (int x = 0; x < 4; ++x)
         if ((path[m] >> (j + x)) & 1) {   // whatever U and the coefficients hold off the path stays out
 #pragma unroll
-          for (int h = 0; h < NC; ++h) fma4(out[m][h], sign * cj[x], u[x][h]);
+          for (int h = 0; h < NC; ++h) fma4(out[m][h], cj[x], u[x][h]);
         }
     }
   }
@@ -170,14 +179,16 @@ __device__ __forceinline__ void solve16(float* u, int ustride, const float* g, i
 #pragma unroll
   for (int i = 1; i < 16; ++i) {
     const uint32_t path = on[i * kMaskParts];
+    float known = 0.f;
 #pragma unroll
     for (int j = 0; j < i; j += 4) {
       const float4 w = *reinterpret_cast<const float4*>(g + i * gld + j);
       const float wj[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
       for (int x = 0; x < 4; ++x)
-        if (j + x < i && ((path >> (j + x)) & 1)) r[i] = fmaf(-wj[x], r[j + x], r[i]);
+        if (j + x < i && ((path >> (j + x)) & 1)) known = fmaf(wj[x], r[j + x], known);
     }
+    r[i] -= known;
   }
 #pragma unroll
   for (int i = 1; i < 16; ++i) u[i * ustride] = r[i];
@@ -528,8 +539,9 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
     // solve and readout, path form: DVC / 4 lanes per node
     constexpr int LN = C::DVC / 4, NN = C::kThreads / LN;   // lanes per node, nodes at a time
     const int n0 = tid / LN, c = 4 * (tid % LN);
-    // r += sign * (entries first .. n of node i) times the U rows they belong to
-    auto along = [&](float4& r, const float* w, int i, int first, int n, float sign) {
+    // entries first .. n of node i times the U rows they belong to
+    auto along = [&](const float* w, int i, int first, int n) {
+      float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
       const uint4 iv = *reinterpret_cast<const uint4*>(idx_s + i * kPath);
       const uint32_t word[4] = {iv.x, iv.y, iv.z, iv.w};
 #pragma unroll
@@ -540,8 +552,9 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
 #pragma unroll
         for (int e = 0; e < 4; ++e)
           if (4 * e4 + e >= first && 4 * e4 + e <= n)
-            fma4(r, sign * xe[e], *reinterpret_cast<const float4*>(C::U(sm, (word[e4] >> (8 * e)) & 255) + c));
+            fma4(sum, xe[e], *reinterpret_cast<const float4*>(C::U(sm, (word[e4] >> (8 * e)) & 255) + c));
       }
+      return sum;
     };
     if (DELTA) {
       for (int lev = 1; lev < kPath; ++lev) {
@@ -550,17 +563,17 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
         __syncthreads();   // the level above
         for (int r = begin + n0; r < end; r += NN) {
           const int i = ord_s[r];
-          float4 u = *reinterpret_cast<const float4*>(C::U(sm, i) + c);
-          along(u, Gp_s, i, 1, lev, -1.f);
-          *reinterpret_cast<float4*>(C::U(sm, i) + c) = u;
+          float4* const at = reinterpret_cast<float4*>(C::U(sm, i) + c);
+          const float4 rhs = *at;
+          *at = sub4(rhs, along(Gp_s, i, 1, lev));
         }
       }
     }
     __syncthreads();
     for (int r = n0; r < T; r += NN) {
       const int i = ord_s[r];
-      float4 o = *reinterpret_cast<const float4*>(C::B0(sm, i) + c);
-      along(o, Cp_s, i, 0, dep_s[i], 1.f);
+      const float4 b0 = *reinterpret_cast<const float4*>(C::B0(sm, i) + c);
+      const float4 o = add4(b0, along(Cp_s, i, 0, dep_s[i]));
       if (v_first + c < dv) {
         const size_t at = rows.o0 + (size_t)((int64_t)i * rows.o_rs) + v_first + c;
         *reinterpret_cast<float4*>(a.O + at) = o;
@@ -595,41 +608,31 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
     __syncthreads();
     scale_rows<DELTA, C::kThreads>(tab, reinterpret_cast<const float2*>(Cp_s), C_s, G_s, GLD, 0, C::NB, MT);
     __syncthreads();
-    // solve, block form
+    // solve, block form: tile by tile, each after the sum of what the tiles above it explain
     if (DELTA) {
+      float4 known[MT][NC] = {};
 #pragma unroll
       for (int b = 0; b < MT; ++b) {
         if (16 * b >= T) break;
-        if (tid < C::DVC) solve16(U_s + 16 * b * ULD + tid, ULD, G_s + 16 * b * GLD + 16 * b, GLD, tab.on(16 * b, b));
-        __syncthreads();
-        if (b + 1 < MT && 16 * (b + 1) < T) {
-          float4 r[MT][NC];
+        if (b > 0) {
+          accumulate16<MT, NC>(known, b, G_s + rt * GLD + 16 * (b - 1), GLD, tab.on(rt, b - 1),
+                               U_s + 16 * (b - 1) * ULD + 4 * ct, ULD, 4 * CT);
 #pragma unroll
-          for (int m = b + 1; m < MT; ++m)
-#pragma unroll
-            for (int h = 0; h < NC; ++h)
-              r[m][h] = *reinterpret_cast<const float4*>(U_s + (rt + 16 * m) * ULD + 4 * (ct + h * CT));
-          accumulate16<MT, NC>(r, b + 1, G_s + rt * GLD + 16 * b, GLD, tab.on(rt, b), U_s + 16 * b * ULD + 4 * ct,
-                               ULD, 4 * CT, -1.f);
-#pragma unroll
-          for (int m = b + 1; m < MT; ++m)
-#pragma unroll
-            for (int h = 0; h < NC; ++h)
-              *reinterpret_cast<float4*>(U_s + (rt + 16 * m) * ULD + 4 * (ct + h * CT)) = r[m][h];
+          for (int h = 0; h < NC; ++h) {
+            float4* const at = reinterpret_cast<float4*>(U_s + (rt + 16 * b) * ULD + 4 * (ct + h * CT));
+            *at = sub4(*at, known[b][h]);
+          }
           __syncthreads();
         }
+        if (tid < C::DVC) solve16(U_s + 16 * b * ULD + tid, ULD, G_s + 16 * b * GLD + 16 * b, GLD, tab.on(16 * b, b));
+        __syncthreads();
       }
     }
     // readout, block form
-    float4 o[MT][NC];
-#pragma unroll
-    for (int m = 0; m < MT; ++m)
-#pragma unroll
-      for (int h = 0; h < NC; ++h) o[m][h] = *reinterpret_cast<const float4*>(C::B0(sm, rt + 16 * m) + 4 * (ct + h * CT));
+    float4 o[MT][NC] = {};
 #pragma unroll
     for (int b = 0; b < MT; ++b)
-      accumulate16<MT, NC>(o, b, C_s + rt * GLD + 16 * b, GLD, tab.on(rt, b), U_s + 16 * b * ULD + 4 * ct, ULD, 4 * CT,
-                           1.f);
+      accumulate16<MT, NC>(o, b, C_s + rt * GLD + 16 * b, GLD, tab.on(rt, b), U_s + 16 * b * ULD + 4 * ct, ULD, 4 * CT);
 #pragma unroll
     for (int m = 0; m < MT; ++m)
 #pragma unroll
@@ -637,7 +640,7 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
         const int i = rt + 16 * m, c = 4 * (ct + h * CT);
         if (i >= T || v_first + c >= dv) continue;
         const size_t at = rows.o0 + (size_t)((int64_t)i * rows.o_rs) + v_first + c;
-        *reinterpret_cast<float4*>(a.O + at) = o[m][h];
+        *reinterpret_cast<float4*>(a.O + at) = add4(*reinterpret_cast<const float4*>(C::B0(sm, i) + c), o[m][h]);
         if (a.U) *reinterpret_cast<float4*>(a.U + at) = *reinterpret_cast<const float4*>(U_s + i * ULD + c);
       }
   }
@@ -749,56 +752,51 @@ __global__ void __launch_bounds__(256) verify_simt_deep_kernel(const __grid_cons
     __syncthreads();
     scale_rows<DELTA, C::kThreads>(tab, jump_s, C_s, G_s, C::GLD, i0, NB, (I + 1) * MT);
     __syncthreads();
-    // solve
+    // solve: what the first block explains of this one, then tile by tile as above
     if (DELTA) {
-      auto below = [&](int j0, int m0) {   // the rows of tiles m >= m0 lose what the 16 nodes from j0 on explain
-        float4 r[MT][1];
-#pragma unroll
-        for (int m = 0; m < MT; ++m) r[m][0] = *reinterpret_cast<const float4*>(U_s + (i0 + rt + 16 * m) * C::DVC + 4 * ct);
-        accumulate16<MT, 1>(r, m0, G_s + rt * C::GLD + j0, C::GLD, tab.on(i0 + rt, j0 / 16), U_s + j0 * C::DVC + 4 * ct,
-                            C::DVC, 0, -1.f);
-#pragma unroll
-        for (int m = 0; m < MT; ++m)
-          if (m >= m0) *reinterpret_cast<float4*>(U_s + (i0 + rt + 16 * m) * C::DVC + 4 * ct) = r[m][0];
-      };
+      float4 known[MT][1] = {};
       if (I > 0) {
 #pragma unroll 1
-        for (int b = 0; b < MT; ++b) below(16 * b, 0);
-        __syncthreads();
+        for (int b = 0; b < MT; ++b)
+          accumulate16<MT, 1>(known, 0, G_s + rt * C::GLD + 16 * b, C::GLD, tab.on(i0 + rt, b),
+                              U_s + 16 * b * C::DVC + 4 * ct, C::DVC, 0);
       }
 #pragma unroll
       for (int b = 0; b < MT; ++b) {
         if (i0 + 16 * b >= T) break;
+        if (b > 0)
+          accumulate16<MT, 1>(known, b, G_s + rt * C::GLD + i0 + 16 * (b - 1), C::GLD, tab.on(i0 + rt, i0 / 16 + b - 1),
+                              U_s + (i0 + 16 * (b - 1)) * C::DVC + 4 * ct, C::DVC, 0);
+        if (I + b > 0) {
+          float4* const at = reinterpret_cast<float4*>(U_s + (i0 + rt + 16 * b) * C::DVC + 4 * ct);
+          *at = sub4(*at, known[b][0]);
+          __syncthreads();
+        }
         if (tid < C::DVC)
           solve16(U_s + (i0 + 16 * b) * C::DVC + tid, C::DVC, G_s + 16 * b * C::GLD + i0 + 16 * b, C::GLD,
                   tab.on(i0 + 16 * b, i0 / 16 + b));
         __syncthreads();
-        if (b + 1 < MT && i0 + 16 * (b + 1) < T) {
-          below(i0 + 16 * b, b + 1);
-          __syncthreads();
-        }
       }
     }
     // readout
-    float4 o[MT][1];
-#pragma unroll
-    for (int m = 0; m < MT; ++m) o[m][0] = *reinterpret_cast<const float4*>(B0_s + (rt + 16 * m) * C::DVC + 4 * ct);
+    float4 o[MT][1] = {};
     if (I > 0) {
 #pragma unroll 1
       for (int b = 0; b < MT; ++b)
         accumulate16<MT, 1>(o, 0, C_s + rt * C::GLD + 16 * b, C::GLD, tab.on(i0 + rt, b), U_s + 16 * b * C::DVC + 4 * ct,
-                            C::DVC, 0, 1.f);
+                            C::DVC, 0);
     }
 #pragma unroll
     for (int b = 0; b < MT; ++b)
       accumulate16<MT, 1>(o, b, C_s + rt * C::GLD + i0 + 16 * b, C::GLD, tab.on(i0 + rt, i0 / 16 + b),
-                          U_s + (i0 + 16 * b) * C::DVC + 4 * ct, C::DVC, 0, 1.f);
+                          U_s + (i0 + 16 * b) * C::DVC + 4 * ct, C::DVC, 0);
 #pragma unroll
     for (int m = 0; m < MT; ++m) {
       const int i = i0 + rt + 16 * m;
       if (i >= T || col >= dv) continue;
       const size_t at = rows.o0 + (size_t)((int64_t)i * rows.o_rs) + col;
-      *reinterpret_cast<float4*>(a.O + at) = o[m][0];
+      *reinterpret_cast<float4*>(a.O + at) =
+          add4(*reinterpret_cast<const float4*>(B0_s + (rt + 16 * m) * C::DVC + 4 * ct), o[m][0]);
       if (a.U) *reinterpret_cast<float4*>(a.U + at) = *reinterpret_cast<const float4*>(U_s + i * C::DVC + 4 * ct);
     }
   }
