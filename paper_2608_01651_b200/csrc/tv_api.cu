@@ -7,6 +7,19 @@
 static thread_local int g_last_cuda_error = 0;
 void tv_set_cuda_error(cudaError_t e) { g_last_cuda_error = (int)e; }
 
+int tv_sm_count() {
+  static thread_local int of_dev = -1, count = 0;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess && dev != of_dev) {
+    e = cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, dev);
+    of_dev = e == cudaSuccess ? dev : -1;
+  }
+  if (e == cudaSuccess) return count;
+  tv_set_cuda_error(e);
+  return 0;
+}
+
 #define TV_API __attribute__((visibility("default")))
 
 extern "C" {

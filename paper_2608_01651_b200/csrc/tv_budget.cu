@@ -4,14 +4,15 @@
 // parent slabs and offsets of a packed forest (Section V-B) -- all on the device, with fixed
 // shapes, so the selection can sit inside a GPU-resident round.
 //
-// Two small launches, each dependent on the one in front of it:
+// Up to 2048 candidates in at most as many requests as the GPU has SMs: two small launches, each dependent
+// on the one in front of it:
 //   budget_rho_kernel     one CTA per request: rho_i = rho_parent * p_i in float32, level by level
 //                         (parent before child, one rounding per edge), and a 32-bit sort key
 //   budget_choose_kernel  one CTA per request: every CTA finds the budget-th largest key of the batch
 //                         for itself (all keys in its registers, two bits of the threshold per step),
 //                         counts what the requests in front of its own keep, then compacts its own
 //                         request in order and renumbers the parents; ties go in (request, node) order
-// Batches of more than 8192 candidates do not fit a CTA's registers and take three launches:
+// Everything else takes three launches:
 //   budget_rho_kernel, then
 //   budget_select_kernel  one CTA: 4-pass radix select of the budget-th largest key, then per-request
 //                         counts and their prefix sums
@@ -19,6 +20,11 @@
 // The sizes are tiny (at most a few 10^4 candidates): what counts is the chain of launches and of
 // steps inside them.  A whole device-built round of 2048 candidates (32 requests, budget 1234) took 69.8 us
 // with three ordinary launches and takes 61.7 us with these two.
+// Every request's CTA of the two-launch form searches all keys: its work is requests x candidates.  Device
+// time of a selection, two launches against three: 2048 candidates in 16 / 148 / 300 / 1024 requests 7.5 / 7.7 /
+// 11.5 / 21.7 us against 10.4 / 10.9 / 10.3 / 10.5, 512 in 200 / 256 requests 8.9 / 10.4 against 8.9 / 9.2: up to
+// one CTA per SM.  With 32 keys per thread, which 2049 to 8192 candidates need, it was slower at any number of
+// requests: 4096 candidates in 32 / 1024 requests 14.5 / 64 us against 11.4 / 11.4.
 #include "tv_internal.h"
 #include "tv_tc_common.cuh"
 
@@ -108,8 +114,7 @@ __device__ __forceinline__ uint32_t block_sum(uint32_t x, uint32_t* buf) {
   return t;
 }
 
-// KPT: keys per thread, consecutive ones.  Counts stay below 65536: two of them share a word.
-template <int KPT>
+constexpr int KPT = 8;   // keys per thread, consecutive ones.  Counts stay below 65536: two of them share a word.
 __global__ void __launch_bounds__(kChooseThreads)
 budget_choose_kernel(const uint32_t* __restrict__ key, const int32_t* __restrict__ parent, int32_t N, int32_t K,
                      int32_t B, int32_t Tc, int32_t budget, int32_t* __restrict__ counts, int32_t* __restrict__ offsets,
@@ -326,12 +331,13 @@ TV_API int tv_budget_select(const int32_t* parent, const float* p_draft, int32_t
   uint32_t* key = reinterpret_cast<uint32_t*>(workspace);
   uint8_t* keep = reinterpret_cast<uint8_t*>(workspace) + (((size_t)N * sizeof(uint32_t) + 255) & ~(size_t)255);
   cudaStream_t s = (cudaStream_t)stream;
+  const int sms = tv_sm_count();
+  if (sms == 0) return TV_ERR_CUDA;
   TV_CUDA_TRY(tvtc::launch_dependent(budget_rho_kernel, n_req, TV_MAX_NODES, 0, s, parent, p_draft, n_cand, rho, key,
                                      status));
-  if (N <= 32 * kChooseThreads) {
-    TV_CUDA_TRY(tvtc::launch_dependent(N <= 8 * kChooseThreads ? budget_choose_kernel<8> : budget_choose_kernel<32>, n_req,
-                                       kChooseThreads, 0, s, (const uint32_t*)key, parent, N, K, n_req, n_cand, budget,
-                                       counts, offsets, parent_packed, node_id));
+  if (N <= KPT * kChooseThreads && n_req <= sms) {
+    TV_CUDA_TRY(tvtc::launch_dependent(budget_choose_kernel, n_req, kChooseThreads, 0, s, (const uint32_t*)key, parent, N,
+                                       K, n_req, n_cand, budget, counts, offsets, parent_packed, node_id));
     return TV_OK;
   }
   budget_select_kernel<<<1, kSelThreads, 0, s>>>(key, N, K, n_req, n_cand, keep, counts, offsets);

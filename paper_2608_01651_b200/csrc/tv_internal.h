@@ -159,6 +159,8 @@ __device__ inline ItemRows tv_item_rows(const TreeDev& t, const Layout& lay, int
 }
 
 void tv_set_cuda_error(cudaError_t e);
+// SMs of the current device, asked once per thread and device; 0 (and the error set) if CUDA refuses.
+int tv_sm_count();
 
 // Launchers (each returns a tv_status; all work is asynchronous on `stream`).
 int tv_launch_verify_simt(const VerifyArgs& a, cudaStream_t stream);

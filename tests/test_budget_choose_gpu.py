@@ -1,4 +1,4 @@
-"""The budget selector around the sizes where its kernels change (2048 and 8192 candidates) and with
+"""The budget selector around the sizes where its kernels change (2048 candidates, as many requests as SMs) and with
 scores that stress the threshold search: zeros, one value for everything, denormals, every budget from
 the roots alone to all nodes.  Bit for bit against the oracle, as whole numbers are."""
 import numpy as np
@@ -11,7 +11,7 @@ from oracle import budget_oracle as bo
 
 pytestmark = pytest.mark.gpu
 
-SIZES = [(2, 1), (16, 128), (683, 3), (64, 128), (65, 127), (1024, 8), (1000, 9), (7, 97)]
+SIZES = [(2, 1), (16, 128), (683, 3), (64, 128), (65, 127), (1024, 8), (1000, 9), (7, 97), (148, 13), (149, 13), (148, 1)]
 
 
 @pytest.mark.parametrize("scores", ["uniform", "few", "zeros", "ones", "denormal"])
@@ -32,3 +32,23 @@ def test_choose(B, Tc, scores):
             assert np.array_equal(got[n].cpu().numpy(), ref[n]), (n, budget)
         node_id = got["node_id"].cpu().numpy()
         assert np.array_equal(node_id[:K], ref["node_id"][:K]) and (node_id[K:] == -1).all()
+
+
+@pytest.mark.parametrize("B,Tc,few", [(16, 128, True), (0, 13, True), (1, 13, False), (17, 121, False), (1024, 2, False),
+                                      (683, 3, False), (1024, 8, False)])
+def test_launches(B, Tc, few):
+    """Every request's CTA of the two-launch form searches the whole batch's keys: it takes at most 2048
+    candidates and one CTA per SM (B = 0, 1: as many requests as SMs, one more)."""
+    import ctypes
+    if B < 2:
+        B += torch.cuda.get_device_properties(0).multi_processor_count
+    par = torch.full((B, Tc), -1, dtype=torch.int32, device="cuda")
+    p = torch.rand(B, Tc, device="cuda")
+    out = tv.budget_select(par, p, B)
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        tv.budget_select(par, p, B, out=out)
+    n = ctypes.c_size_t()
+    runtime = ctypes.CDLL("libcudart.so.12")
+    assert runtime.cudaGraphGetNodes(ctypes.c_void_p(graph.raw_cuda_graph()), None, ctypes.byref(n)) == 0
+    assert n.value == (2 if few else 3)
