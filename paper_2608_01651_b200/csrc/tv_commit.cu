@@ -185,7 +185,7 @@ commit_factored_kernel(const CommitArgs a, const __grid_constant__ CommitLayers 
 // nothing in it is serial over the path: the thread of a node finds the node's place by counting mask
 // bits, a warp scan turns the gates into weights while the rows of up to 16 path nodes are on their way.
 // A chain that loaded those rows one by one and scanned the gates with one thread took 23.5 us where this
-// takes 21.7 (1024 items of 128 x 128, 20.5 at the copy peak), 4.2 against 2.4 at 16 items, and 24.1
+// takes 21.7 (1024 items of 128 x 128, 20.5 at the copy peak), 4.2 against 2.3 at 16 items, and 24.1
 // against 16.8 on paths of 40 nodes (256 items).  A persistent form of it with double-buffered rows was
 // the slower one at every size too: 347 against 336 us on 16384 items.
 constexpr int kRowThreads = 128;
@@ -494,22 +494,24 @@ cudaError_t launch_after_verify(void (*kernel)(const CommitArgs, const CommitLay
 }
 
 // Rows per thread.  Four (and no limit on registers) while that puts at most four CTAs on an SM: nothing
-// but the chain counts there (16 items of 128 x 128: 2.4 us, 3.1 with sixteen rows).  Four, eight CTAs per
+// but the chain counts there (16 items of 128 x 128: 2.3 us, 3.1 with sixteen rows).  Four, eight CTAs per
 // SM, while all of them are resident (128 items: 4.6 us against 5.2 with eight rows).  Beyond that
 // 64 rows per CTA -- sixteen per thread, eight for dk = 64: fewest paths to work out per byte (a round of
-// 1024 items 53.2 us against 55.8 with half as many rows, of 512 items 40.4 against 41.1).
-constexpr int kSMs = 148;
+// 1024 items 53.2 us against 55.8 with half as many rows, of 512 items 40.4 against 41.1).  The register
+// limits of the dk = 64 kernels (8 CTAs per SM, 7 with f32 keys) cost 44 and 36 bytes of spills.
 template <bool BF16, int DK>
-cudaError_t launch_rows(const CommitArgs& a, const CommitLayers& tb, int items, cudaStream_t stream) {
+cudaError_t launch_rows(const CommitArgs& a, const CommitLayers& tb, int items, int sms, cudaStream_t stream) {
   constexpr int kRpt = DK == 128 ? 16 : 8, kCtas = DK == 128 ? 4 : BF16 ? 8 : 7;   // 64 rows per CTA
   constexpr int rows4 = 16 * (128 / DK), rows = 64;
   const int64_t ctas4 = (int64_t)items * ((a.dv + rows4 - 1) / rows4);
-  if (ctas4 <= 4 * kSMs) return launch_after_verify(commit_rows_kernel<BF16, DK, 4, 4>, (int)ctas4, stream, a, tb);
-  if (ctas4 <= 8 * kSMs) return launch_after_verify(commit_rows_kernel<BF16, DK, 4, 8>, (int)ctas4, stream, a, tb);
+  if (ctas4 <= 4 * sms) return launch_after_verify(commit_rows_kernel<BF16, DK, 4, 4>, (int)ctas4, stream, a, tb);
+  if (ctas4 <= 8 * sms) return launch_after_verify(commit_rows_kernel<BF16, DK, 4, 8>, (int)ctas4, stream, a, tb);
   const int ctas = items * ((a.dv + rows - 1) / rows);
-  // From some seven waves on an ordinary launch: most CTAs start long after the kernel in front is done,
-  // and the dependent launch measured slower (a round of 24576 items 1612-1631 us against 1667).
-  if (ctas >= 30 * kSMs) {
+  // From 30 CTAs per SM on an ordinary launch: most CTAs start long after the kernel in front is done, and
+  // the dependent launch is the slower one.  Rounds of 64-node trees, dependent against ordinary: 128 x 128
+  // states (two CTAs each) 1024 items 52.4 / 55.4 us, 2048 107.6 / 105.7, 4096 220 / 214, 24576 1290 / 1240;
+  // 64 x 64 states (one CTA each) 2048 items 47.6 / 50.8, 4096 94.1 / 95.6, 8192 186 / 183, 24576 552 / 533.
+  if (ctas >= 30 * sms) {
     commit_rows_kernel<BF16, DK, kRpt, kCtas><<<ctas, kRowThreads, 0, stream>>>(a, tb);
     return cudaSuccess;   // the caller asks for the launch's error
   }
@@ -523,10 +525,12 @@ int tv_launch_commit(const CommitArgs& a, const CommitLayers& tb, cudaStream_t s
   const int items = a.L * a.B * a.H;
   if ((size_t)a.dk * a.dv > (size_t)kMaxVec * kThreads * 4) return TV_ERR_UNSUPPORTED;
   const bool recompute = a.rule == TV_GATED_DELTA && !a.has_U;
+  const int sms = tv_sm_count();
+  if (sms == 0) return TV_ERR_CUDA;
   if (!recompute && a.dk == 128) {
-    TV_CUDA_TRY((a.bf16 ? launch_rows<true, 128> : launch_rows<false, 128>)(a, tb, items, stream));
+    TV_CUDA_TRY((a.bf16 ? launch_rows<true, 128> : launch_rows<false, 128>)(a, tb, items, sms, stream));
   } else if (!recompute && a.dk == 64) {
-    TV_CUDA_TRY((a.bf16 ? launch_rows<true, 64> : launch_rows<false, 64>)(a, tb, items, stream));
+    TV_CUDA_TRY((a.bf16 ? launch_rows<true, 64> : launch_rows<false, 64>)(a, tb, items, sms, stream));
   } else if (!recompute) {
     TV_CUDA_TRY(a.bf16 ? launch_after_verify(commit_factored_kernel<true>, items, stream, a, tb, kThreads)
                        : launch_after_verify(commit_factored_kernel<false>, items, stream, a, tb, kThreads));

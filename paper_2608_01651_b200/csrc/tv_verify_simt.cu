@@ -832,35 +832,36 @@ int launch_deep(const VerifyArgs& a, cudaStream_t stream) {
   return launch_kernel(verify_simt_deep_kernel<BF16, DELTA, MT>, C::kThreads, C::kSmem, C::DVC, configured_dev, a, stream);
 }
 
-constexpr int kSMs = 148;
-
 // Up to 64 nodes.  Every chunk of value columns computes the item's scores again, so a chunk is all 128
 // columns where there are enough items to fill the SMs, else 64 or 32 (T = 64, f32, delta: 128 items
 // 27.9 us in whole columns, 32.9 in halves; 64 items 25 us in halves).
 template <bool BF16, bool DELTA, int MT>
-int launch_one(const VerifyArgs& a, cudaStream_t stream) {
+int launch_one(const VerifyArgs& a, int sms, cudaStream_t stream) {
   const int64_t items = (int64_t)a.L * a.B * a.H;
-  if (a.dv <= 32 || items * ((a.dv + 31) / 32) <= kSMs) return launch<BF16, DELTA, MT, 8, 1, 1>(a, stream);
-  if (a.dv <= 64 || items * ((a.dv + 63) / 64) <= kSMs) return launch<BF16, DELTA, MT, 8, 2, 1>(a, stream);
+  if (a.dv <= 32 || items * ((a.dv + 31) / 32) <= sms) return launch<BF16, DELTA, MT, 8, 1, 1>(a, stream);
+  if (a.dv <= 64 || items * ((a.dv + 63) / 64) <= sms) return launch<BF16, DELTA, MT, 8, 2, 1>(a, stream);
   return launch<BF16, DELTA, MT, 16, 2, 1>(a, stream);
 }
 
 template <bool BF16, bool DELTA, int MT>
-int launch_two(const VerifyArgs& a, cudaStream_t stream) {
+int launch_two(const VerifyArgs& a, int sms, cudaStream_t stream) {
   const int64_t items = (int64_t)a.L * a.B * a.H;
-  if (a.dv <= 32 || items * ((a.dv + 31) / 32) <= kSMs) return launch<BF16, DELTA, MT, 8, 1, 2>(a, stream);
-  if (a.dv <= 64 || items * ((a.dv + 63) / 64) <= kSMs) return launch<BF16, DELTA, MT, 16, 1, 2>(a, stream);
+  if (a.dv <= 32 || items * ((a.dv + 31) / 32) <= sms) return launch<BF16, DELTA, MT, 8, 1, 2>(a, stream);
+  if (a.dv <= 64 || items * ((a.dv + 63) / 64) <= sms) return launch<BF16, DELTA, MT, 16, 1, 2>(a, stream);
   return launch<BF16, DELTA, MT, 16, 2, 2>(a, stream);
 }
 
 template <bool BF16, bool DELTA>
 int launch_nodes(const VerifyArgs& a, cudaStream_t stream) {
-  if (a.T <= 16) return launch_one<BF16, DELTA, 1>(a, stream);
-  if (a.T <= 32) return launch_one<BF16, DELTA, 2>(a, stream);
-  if (a.T <= 48) return launch_one<BF16, DELTA, 3>(a, stream);
-  if (a.T <= 64) return launch_one<BF16, DELTA, 4>(a, stream);
+  const int sms = tv_sm_count();
+  if (sms == 0) return TV_ERR_CUDA;
+  if (a.T <= 16) return launch_one<BF16, DELTA, 1>(a, sms, stream);
+  if (a.T <= 32) return launch_one<BF16, DELTA, 2>(a, sms, stream);
+  if (a.T <= 48) return launch_one<BF16, DELTA, 3>(a, sms, stream);
+  if (a.T <= 64) return launch_one<BF16, DELTA, 4>(a, sms, stream);
   // two row blocks of 48 or 64 nodes
-  if (a.tree.max_depth_all < kPath) return a.T <= 96 ? launch_two<BF16, DELTA, 3>(a, stream) : launch_two<BF16, DELTA, 4>(a, stream);
+  if (a.tree.max_depth_all < kPath)
+    return a.T <= 96 ? launch_two<BF16, DELTA, 3>(a, sms, stream) : launch_two<BF16, DELTA, 4>(a, sms, stream);
   return a.T <= 96 ? launch_deep<BF16, DELTA, 3>(a, stream) : launch_deep<BF16, DELTA, 4>(a, stream);
 }
 

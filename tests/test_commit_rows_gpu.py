@@ -46,3 +46,24 @@ def test_rows(B, H, T, tree, dk, dv, dtype):
                     assert pu.rel_fro(got[b, h], ref) <= 1e-5
             assert in_place or torch.equal(S, dev["S_pre"])
             assert torch.equal(out[accepted < 0], dev["S_pre"][accepted < 0])
+
+
+def test_many_64_wide_states():
+    """Enough of them that the commit is an ordinary launch (30 CTAs per SM), accepted and rejected requests."""
+    B, H, T, d = 160, 32, 20, 64
+    wl = inputs.workload("c3", B=B, H=H, T=T, dk=d, dv=d, tree="frontier", seed=17)
+    assert B * H >= 30 * torch.cuda.get_device_properties(0).multi_processor_count
+    tens = inputs.make_tensors(wl)
+    parents, accepted = inputs.make_trees(wl)
+    accepted[::7] = -1
+    dev = {n: None if x is None else x.cuda() for n, x in tens.items()}
+    tree_ = tv.tree_build(parents).upload()
+    out = tv.commit_path(tree_, torch.from_numpy(accepted).cuda(), dev["S_pre"].clone(), dev["k"], dev["v"], dev["alpha"])
+    got = inputs.to_f64(out)
+    f = {n: inputs.to_f64(x) for n, x in tens.items()}
+    for b in (0, 1, 7, 80, 159):
+        for h in (0, 31):
+            ref = orc.commit_walk(f["S_pre"][b, h].T, f["k"][b, h], f["v"][b, h], f["alpha"][b, h], None, parents[b],
+                                  int(accepted[b]), "gated").T
+            assert pu.rel_fro(got[b, h], ref) <= 1e-5
+    assert torch.equal(out[torch.from_numpy(accepted < 0)], dev["S_pre"][torch.from_numpy(accepted < 0)])
