@@ -109,3 +109,72 @@ def test_commit_that_rejects_every_request_keeps_the_order(d, T, rule):
     for rep in range(3):
         for i, (x, y) in enumerate(zip(run(sync=False), ref)):
             assert torch.equal(x, y), (rep, i)
+
+
+def _compare(run):
+    S_ref, ctx_ref, outs_ref = run(sync=True)
+    assert torch.isfinite(S_ref).all()
+    for rep in range(3):
+        S, ctx, outs = run(sync=False)
+        assert torch.equal(S, S_ref), rep
+        assert all(torch.equal(a, b) for a, b in zip(ctx, ctx_ref)), rep
+        for r, (got, ref) in enumerate(zip(outs, outs_ref)):
+            for i, (x, y) in enumerate(zip(got, ref)):
+                assert (x is None and y is None) or torch.equal(x, y), (rep, r, i)
+
+
+@pytest.mark.parametrize("rule", [tv.GATED, tv.DELTA])
+@pytest.mark.parametrize("tree,T,d,dtype,B,H", [
+    ("frontier", 63, 128, inputs.F32, 9, 16),     # path form, whole columns
+    ("frontier", 40, 64, inputs.F32, 5, 8),       # 64-wide states: column chunks, the commit kernel of dk = 64
+    ("chain", 40, 128, inputs.BF16, 9, 16),       # block form
+    ("chain", 40, 64, inputs.F32, 12, 16),
+    ("frontier", 100, 128, inputs.F32, 6, 16),    # two row blocks, path form
+    ("chain", 128, 128, inputs.BF16, 6, 16),      # two row blocks, block form: its second block is loaded late
+    ("chain", 90, 64, inputs.F32, 6, 16),
+])
+def test_queued_rounds_of_the_general_kernel(tree, T, d, dtype, B, H, rule):
+    """The fp32 kernel asks for the state before its wait, and so does the commit behind it."""
+    wl = inputs.workload("c4", B=B, H=H, T=T, dk=d, dv=d, tree=tree, qkv_dtype=dtype, rule=rule, seed=T + d)
+    _compare(_round_calls(wl, rule, tv.IMPL_SIMT))
+
+
+@pytest.mark.parametrize("B,Tc,rule,dtype", [
+    (32, 64, tv.GATED, inputs.BF16),    # 2048 candidates
+    (32, 64, tv.DELTA, inputs.BF16),
+    (24, 100, tv.DELTA, inputs.F32),    # 2400, general verify kernel
+    (100, 90, tv.GATED, inputs.BF16),   # 9000
+    (700, 3, tv.GATED, inputs.F32),     # many small requests
+])
+def test_queued_rounds_with_selection(B, Tc, rule, dtype):
+    """selection -> metadata from device memory -> verify -> commit in place, twice, with other candidates
+    the second time: the keys, the packed parents and the masks of one round are overwritten by the next."""
+    H, d, N = 4, 128, max(B, B * Tc * 6 // 10)
+    wl = inputs.workload("c4", B=1, H=H, T=N, rule=rule, qkv_dtype=dtype, seed=7)
+    rng = np.random.default_rng(B)
+    par = [torch.from_numpy(np.stack([inputs.tree_frontier(Tc, rng) for _ in range(B)])).to(DEV) for _ in range(2)]
+    p = [torch.from_numpy(rng.uniform(0.1, 1.0, (B, Tc)).astype(np.float32)).to(DEV) for _ in range(2)]
+    t = {n: None if x is None else x[0].to(DEV) for n, x in inputs.make_tensors(wl).items()}
+    if dtype == inputs.F32:
+        t["k"] = t["k"] * (8.0 / d ** 0.5)
+    S0 = inputs.make_tensors(inputs.workload("c4", B=B, H=H, T=1, seed=8))["S_pre"].to(DEV)
+    acc = torch.zeros(B, dtype=torch.int32, device=DEV)      # the root: every request keeps it
+    forest = tv.forest_build([np.array([-1], dtype=np.int32)] * B, n_max=Tc, capacity=N)
+    sel = tv.budget_select(par[0], p[0], N)
+
+    def run(sync):
+        pause = torch.cuda.synchronize if sync else (lambda: None)
+        S = S0.clone()
+        outs = [(torch.zeros(H, N, d, device=DEV), torch.zeros(H, N, d, device=DEV)) for _ in range(2)]
+        torch.cuda.synchronize()
+        for r in range(2):
+            O, U = outs[r]
+            tv.budget_select(par[r], p[r], N, out=sel); pause()
+            forest.upload_device(sel["parent_packed"], sel["offsets"], max_depth_bound=min(8, Tc - 1)); pause()
+            tv.tree_verify(forest, S, t["q"], t["k"], t["v"], t["alpha"], t["beta"], rule=rule, O=O, U=U); pause()
+            tv.commit_path(forest, acc, S, t["k"], t["v"], t["alpha"], t["beta"], rule=rule, U=U); pause()
+        torch.cuda.synchronize()
+        forest.device_status()
+        return S, [], outs
+
+    _compare(run)

@@ -180,8 +180,8 @@ def test_argument_errors_on_device():
 
 @pytest.mark.parametrize("rule", [inputs.GATED, inputs.DELTA])
 def test_commit_many_units_per_cta(rule):
-    """Enough states that the persistent commit kernel is the one that runs (several units per
-    CTA, mixed accepted / rejected requests, in place and out of place), checked on samples."""
+    """Enough states that the commit is an ordinary launch instead of a dependent one (mixed accepted /
+    rejected requests, in place and out of place), checked on samples."""
     wl = inputs.workload("c3", B=160, H=32, T=24, L=1, rule=rule, seed=321)
     parents, accepted = inputs.make_trees(wl)
     tens = inputs.make_tensors(wl)
@@ -200,7 +200,7 @@ def test_commit_many_units_per_cta(rule):
 def test_c5_all_48_layers_as_benchmarked():
     """The throughput workload as stated: 48 recurrent layers back to back at full batch, head and
     tree size -- 48 verify launches on one stream, then ONE in-place commit launch over all 48
-    layers (the persistent kernel, 393 216 units) -- in the launch configuration bench.py times.
+    layers (393 216 CTAs, an ordinary launch) -- in the launch configuration bench.py times.
     Layers 0, 23 and 47 are compared with the oracle on sampled (request, head) items; the values
     are drawn on the device and the oracle gets exactly what sits there."""
     import gc

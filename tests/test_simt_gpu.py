@@ -145,3 +145,51 @@ def test_corrections_of_long_chains_keep_their_precision(T, dtype):
     ver, _ = pu.oracle_round(wl, parents, accepted, tens)
     ref = np.stack([np.stack([ver[(b, h)][1] for h in range(wl.H)]) for b in range(wl.B)])
     assert pu.rel_fro(U, ref) <= 1e-7
+
+
+def _tree_of_depth(T, depth, rng):
+    """T nodes, the deepest with exactly `depth` ancestors (node `depth` is one of them)."""
+    return inputs.tree_frontier(T, rng, max_depth=depth, spine=depth + 1)
+
+
+@pytest.mark.parametrize("rule", [inputs.GATED, inputs.DELTA])
+@pytest.mark.parametrize("depth", [15, 16])
+@pytest.mark.parametrize("T", [17, 64, 65, 96, 97, 128])
+def test_the_depth_where_the_forms_change(T, depth, rule):
+    """15 ancestors fill the path form's tables; one more takes the block form."""
+    rng = np.random.default_rng(T)
+    for B, H in ((2, 3), (10, 6), (25, 8)):
+        wl = inputs.workload("c4", B=B, H=H, T=T, rule=rule, qkv_dtype=inputs.F32, seed=T + depth)
+        tens = inputs.make_tensors(wl)
+        tens["k"] = tens["k"] * (8.0 / wl.dk ** 0.5)
+        parents = np.stack([_tree_of_depth(T, depth, rng) for _ in range(B)])
+        assert inputs.node_depths(parents[0]).max() == depth
+        accepted = rng.integers(-1, T, size=B).astype(np.int32)
+        accepted[0], accepted[-1], accepted[B // 2] = depth, T - 1, depth
+        _check(wl, parents, accepted, tens, 1e-5)
+
+
+@pytest.mark.parametrize("rule", [inputs.GATED, inputs.DELTA])
+def test_forest_from_the_device_at_the_path_forms_depth(rule):
+    """A bound of 15 on more than 64 nodes selects the path form: the deepest trees it admits."""
+    from oracle import tree_oracle as orc
+    rng = np.random.default_rng(5)
+    B, H, n, d = 3, 2, 100, 128
+    par = np.stack([_tree_of_depth(n, 15, rng) for _ in range(B)])
+    forest = tv.forest_build([np.array([-1], dtype=np.int32)] * B, n_max=n, capacity=B * n)
+    forest.upload_device(torch.from_numpy(par).cuda(), torch.arange(0, (B + 1) * n, n, dtype=torch.int32, device="cuda"),
+                         max_depth_bound=15)
+    wl = inputs.workload("c4", B=1, H=H, T=B * n, rule=rule, qkv_dtype=inputs.F32, seed=9)
+    t = inputs.make_tensors(wl)
+    t["k"] = t["k"] * (8.0 / d ** 0.5)
+    S = inputs.make_tensors(inputs.workload("c4", B=B, H=H, T=1, seed=10))["S_pre"]
+    names = ("q", "k", "v", "alpha", "beta")
+    dev = {m: None if t[m] is None else t[m][0].cuda() for m in names}
+    O, U = tv.tree_verify(forest, S.cuda(), *[dev[m] for m in names], rule=rule, want_U=True, impl=tv.IMPL_SIMT)
+    forest.device_status()
+    for b in range(B):
+        cut = {m: None if t[m] is None else inputs.to_f64(t[m][:, :, b * n:(b + 1) * n]) for m in names}
+        ver = orc.verify_batch(inputs.to_f64(S[b:b + 1]), *[cut[m] for m in names], par[b][None], wl.rule_name)
+        for h in range(H):
+            assert pu.rel_l2_rows(inputs.to_f64(O[h, b * n:(b + 1) * n]), ver[(0, h)][0]) <= 1e-5
+            assert pu.rel_l2_rows(inputs.to_f64(U[h, b * n:(b + 1) * n]), ver[(0, h)][1]) <= 1e-5
