@@ -283,8 +283,9 @@ int tv_tree_verify(const tv_tree* tree, const tv_dims* dims,
  * TV_ERR_TOO_LARGE / TV_ERR_UNSUPPORTED is returned and nothing is launched.
  * The delta rule runs on the general fp32 kernel here (the tree depth is not
  * known on the host).
- * The first call on each device looks up the device address of that array
- * (with that device current); make that first call outside any stream capture.
+ * The first call on each device looks up the device address of that array and
+ * loads every kernel that any later call may launch (with that device current),
+ * whatever its own sizes are; make that first call outside any stream capture.
  * All calls share the array and it keeps the last call's metadata (the part a
  * call needs is rewritten, and its status word cleared, by the call itself):
  * two calls whose kernels may overlap on the GPU -- different streams without

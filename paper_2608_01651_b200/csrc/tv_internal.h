@@ -164,8 +164,10 @@ int tv_sm_count();
 
 // Launchers (each returns a tv_status; all work is asynchronous on `stream`).
 int tv_launch_verify_simt(const VerifyArgs& a, cudaStream_t stream);
-// Loads every kernel that a launch without known depth may pick, so that no later call loads one.
+// Load the kernels that tv_tree_verify_static may launch (no known depth, no packed forest), so that none of
+// its later calls loads one.
 int tv_prepare_verify_simt();
+int tv_prepare_verify_tc();
 int tv_launch_commit(const CommitArgs& a, const CommitLayers& layers, cudaStream_t stream);
 int tv_launch_tree_meta(const int32_t* parent_mapped, int32_t n_trees, int32_t n, uint64_t* anc,
                         int32_t* depth, int32_t* parent_dev, int32_t* status, const int32_t* offsets_mapped,

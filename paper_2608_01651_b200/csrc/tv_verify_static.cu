@@ -80,9 +80,12 @@ unsigned char* scratch_address(int dev, cudaError_t* err) {
     unsigned char* ptr = nullptr;
     *err = cudaGetSymbolAddress((void**)&ptr, g_static_tree);
     if (*err != cudaSuccess) return nullptr;
-    // kernels load at their first use, which takes device memory: the ones this entry point may
-    // launch load here, whatever sizes come later
-    if (tv_prepare_verify_simt() != TV_OK) {
+    // kernels load at their first use, which takes device memory: all that this entry point may
+    // launch load here, whatever sizes, types and rules come later
+    cudaFuncAttributes at;
+    if ((*err = cudaFuncGetAttributes(&at, tree_meta_static_kernel)) != cudaSuccess) return nullptr;
+    if ((*err = cudaFuncGetAttributes(&at, forward_status_kernel)) != cudaSuccess) return nullptr;
+    if (tv_prepare_verify_simt() != TV_OK || tv_prepare_verify_tc() != TV_OK) {
       *err = (cudaError_t)tv_last_cuda_error();
       return nullptr;
     }

@@ -1038,6 +1038,29 @@ extern "C" __attribute__((visibility("default"))) int tv_selftest_wait_timeout(i
   return TV_OK;
 }
 
+// Allows every form of the gated kernel its shared memory on the current device (which loads them).
+static int allow_shared_memory() {
+  TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<false, false, 128>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<false>::kSmemBytes));
+  TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<true, false, 128>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<false>::kSmemBytes));
+  TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<false, true, 128>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<true>::kSmemBytes));
+  TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<true, true, 128>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<true>::kSmemBytes));
+  TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<false, false, 64>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<false>::kSmemBytes));
+  TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<false, true, 64>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<true>::kSmemBytes));
+  return TV_OK;
+}
+
+int tv_prepare_verify_tc() {
+  cudaFuncAttributes at;
+  TV_CUDA_TRY(cudaFuncGetAttributes(&at, widen_rows_kernel));
+  return allow_shared_memory();
+}
+
 bool tv_verify_tc_supports(const VerifyArgs& a) {
   const bool d128 = a.dk == 128 && a.dv == 128;
   const bool d64 = a.dk == 64 && a.dv == 64 && a.tree.offsets == nullptr;   // dense layouts only
@@ -1110,18 +1133,8 @@ int tv_launch_verify_tc(const VerifyArgs& a, int32_t* status, cudaStream_t strea
   int dev = 0;
   TV_CUDA_TRY(cudaGetDevice(&dev));
   if (configured_dev != dev) {
-    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<false, false, 128>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<false>::kSmemBytes));
-    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<true, false, 128>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<false>::kSmemBytes));
-    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<false, true, 128>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<true>::kSmemBytes));
-    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<true, true, 128>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<true>::kSmemBytes));
-    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<false, false, 64>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<false>::kSmemBytes));
-    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<false, true, 64>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<true>::kSmemBytes));
+    const int st = allow_shared_memory();
+    if (st != TV_OK) return st;
     TV_CUDA_TRY(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
     configured_dev = dev;
   }

@@ -119,3 +119,45 @@ def test_static_call_allocates_nothing():
     torch.cuda.synchronize()
     free1, _ = torch.cuda.mem_get_info()
     assert free1 == free0 and torch.cuda.memory_allocated() == alloc0
+
+
+_FRESH = """
+import torch
+import paper_2608_01651_b200 as tv
+cases = []
+for dtype in (torch.float32, torch.bfloat16):
+    for rule in (tv.GATED, tv.DELTA):
+        for B, H, T, d in [(1, 1, 5, 8), (1, 2, 16, 64), (40, 4, 30, 128), (2, 8, 48, 128), (60, 4, 64, 64), (3, 4, 90, 128),
+                           (60, 4, 128, 128), (2, 2, 70, 16)]:
+            r = lambda *s: torch.rand(*s, device="cuda")
+            t = [r(B, H, d, d), r(B, H, T, d).to(dtype), r(B, H, T, d).to(dtype) / d, r(B, H, T, d).to(dtype), r(B, H, T),
+                 r(B, H, T) if rule == tv.DELTA else None]
+            O = torch.empty(B, H, T, d, device="cuda")
+            par = torch.arange(-1, T - 1, dtype=torch.int32, device="cuda").repeat(B, 1)
+            cases.append((par, t, rule, O, torch.empty_like(O)))
+status = torch.zeros(1, dtype=torch.int32, device="cuda")
+torch.cuda.synchronize()
+def call(c, U, status):
+    par, t, rule, O, _ = c
+    tv.tree_verify_static(par, *t, rule=rule, O=O, U=U, status=status)
+    torch.cuda.synchronize()
+call(cases[0], None, None)
+free = torch.cuda.mem_get_info()[0]
+for c in cases:
+    call(c, None, None)
+    call(c, c[4], status)
+    assert torch.cuda.mem_get_info()[0] == free, (c[1][1].shape, c[1][1].dtype, c[2], free - torch.cuda.mem_get_info()[0])
+assert int(status.item()) == 0
+print("ok")
+"""
+
+
+def test_first_call_loads_what_every_later_call_launches():
+    """In a process of its own, where no kernel is loaded yet: after one small call no other size, type,
+    rule or output takes device memory."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    p = subprocess.run([sys.executable, "-c", _FRESH], cwd=root, capture_output=True, text=True, timeout=300)
+    assert p.returncode == 0 and p.stdout.strip() == "ok", p.stderr[-2000:]
