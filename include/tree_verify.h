@@ -275,7 +275,7 @@ int tv_tree_verify(const tv_tree* tree, const tv_dims* dims,
  * This call does the same verification as tv_tree_verify but takes the parent
  * arrays straight from DEVICE memory (int32 [n_trees][T], n_trees = 1 or B, as
  * a drafter running on the GPU leaves them) and keeps the derived masks and
- * depths in a fixed array inside the library's device image: 384 KiB that
+ * depths in a fixed array inside the library's device image: 385 KiB that
  * every GPU which loads the library holds until the process exits.  It calls
  * no cudaMalloc/cudaFree and no allocating library routine.
  *

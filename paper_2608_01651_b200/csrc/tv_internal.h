@@ -76,6 +76,7 @@ struct VerifyArgs {
   const float* beta;
   float* O;
   float* U;
+  const int32_t* max_depth = nullptr;   // device [n_trees], where tree.max_depth_all is only the largest possible depth
 };
 
 // Commit: dimensions and flags; the tensors come layer by layer from a CommitLayers table, so that

@@ -18,10 +18,11 @@
 //   blocks   (deeper: chains) dense products [Q; K] K^T masked by the ancestor sets; block forward
 //            substitution, 16 nodes at a time: one thread per column for the diagonal block, a
 //            product over all threads for the rows below.
-// The form is chosen per CTA from the masks (trees of up to 64 nodes) or by the launcher from the
-// depth it knows (up to 128 nodes, two row blocks).  In both, a node's sums run over the nodes of its path,
-// whatever their coefficients are: a non-finite value stays on the paths through its node, and a zero gate,
-// key or query below it does not hide it (0 x NaN and 0 x inf are NaN).
+// The form is chosen per CTA from the masks (trees of up to 64 nodes), by the launcher from the depth it
+// knows (up to 128 nodes, two row blocks), or per CTA of two launches where it does not.  In both, a node's
+// sums run over the nodes of its path, whatever their coefficients are: a non-finite value stays on the
+// paths through its node, and a zero gate, key or query below it does not hide it (0 x NaN and 0 x inf are
+// NaN).
 //
 // What bounds it: fp32 FMA issue in the state product, and the latency of the short phases behind it
 // with eight warps on an SM.  T = 63, 128 items, f32, delta: 27 us, of them 13 in the state product (8.6
@@ -298,6 +299,11 @@ __device__ __forceinline__ void load_state(float* S_s, const float* Sg, int n_ro
   }
 }
 
+// The tree of a work item.
+__device__ __forceinline__ int tree_of(const VerifyArgs& a, int item) {
+  return a.tree.n_trees == 1 ? 0 : item / a.H % a.B;
+}
+
 // BF16, DELTA: operand type and rule.  MT: a thread's node rows (16 MT nodes in a row block).
 // CT, NC: column threads and column quads of a thread (4 CT NC value columns in the CTA's chunk, 16 CT
 // threads).  NBLK: row blocks (two: path form only).
@@ -366,6 +372,10 @@ verify_simt_kernel(const __grid_constant__ VerifyArgs a, int n_split) {
   const int dk = a.dk, dv = a.dv;
   const int item = blockIdx.x / n_split, v_first = (blockIdx.x - item * n_split) * C::DVC;
 
+  if (NBLK == 2 && a.max_depth != nullptr) {   // of unknown depth: the deeper trees are the kernel's below
+    tvtc::grid_dependency_wait();
+    if (a.max_depth[tree_of(a, item)] >= kPath) return;
+  }
   // The state is never the output of a kernel that releases its dependents early: its chunk is
   // requested before the dependency wait.
   load_state<CT, C::DVC, C::kWarps>(S_s, a.S_pre + ((size_t)item * dv + v_first) * dk, dv - v_first, dk);
@@ -686,6 +696,10 @@ __global__ void __launch_bounds__(256) verify_simt_deep_kernel(const __grid_cons
   const int dk = a.dk, dv = a.dv;
   const int item = blockIdx.x / n_split, v_first = (blockIdx.x - item * n_split) * C::DVC;
   // launch order: as in the kernel above
+  if (a.max_depth != nullptr) {
+    tvtc::grid_dependency_wait();
+    if (a.max_depth[tree_of(a, item)] < kPath) return;
+  }
   load_state<CT, C::DVC, C::kWarps>(S_s, a.S_pre + ((size_t)item * dv + v_first) * dk, dv - v_first, dk);
   tvtc::grid_dependency_wait();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -862,7 +876,19 @@ int launch_nodes(const VerifyArgs& a, cudaStream_t stream) {
   // two row blocks of 48 or 64 nodes
   if (a.tree.max_depth_all < kPath)
     return a.T <= 96 ? launch_two<BF16, DELTA, 3>(a, sms, stream) : launch_two<BF16, DELTA, 4>(a, sms, stream);
-  return a.T <= 96 ? launch_deep<BF16, DELTA, 3>(a, stream) : launch_deep<BF16, DELTA, 4>(a, stream);
+  // Depths that only the device knows: the block form serves every tree.  Under the gated rule with more items
+  // than SMs its dense scores cost a shallow tree more than a second launch, in which such trees take the path
+  // form (f32, depth 8, 160 / 512 items: 65 nodes 45 / 93 us against 68 / 167, 128 nodes 64 / 131 against 92 /
+  // 225), and a deep tree loses nothing by it (chains of 128 nodes, 512 items: 256 us against 255).  Elsewhere
+  // deep trees would: 65 nodes, 4 items 25.6 -> 27.3 us, delta rule, 512 items of 128 nodes 469 -> 475.
+  VerifyArgs b = a;
+  if (!DELTA && a.max_depth != nullptr && (int64_t)a.L * a.B * a.H > sms) {
+    const int st = a.T <= 96 ? launch_two<BF16, DELTA, 3>(a, sms, stream) : launch_two<BF16, DELTA, 4>(a, sms, stream);
+    if (st != TV_OK) return st;
+  } else {
+    b.max_depth = nullptr;   // every tree in one launch
+  }
+  return a.T <= 96 ? launch_deep<BF16, DELTA, 3>(b, stream) : launch_deep<BF16, DELTA, 4>(b, stream);
 }
 
 // Loads a kernel and allows its shared memory on the current device.
@@ -881,6 +907,13 @@ int prepare_one() {
   if (st == TV_OK) st = prepare<BF16, DELTA, MT, 16, 2, 1>();
   return st;
 }
+template <bool BF16, int MT>
+int prepare_two() {
+  int st = prepare<BF16, false, MT, 8, 1, 2>();
+  if (st == TV_OK) st = prepare<BF16, false, MT, 16, 1, 2>();
+  if (st == TV_OK) st = prepare<BF16, false, MT, 16, 2, 2>();
+  return st;
+}
 template <bool BF16, bool DELTA>
 int prepare_all() {
   int st = prepare_one<BF16, DELTA, 1>();
@@ -888,9 +921,13 @@ int prepare_all() {
   if (st == TV_OK) st = prepare_one<BF16, DELTA, 3>();
   if (st == TV_OK) st = prepare_one<BF16, DELTA, 4>();
   // the callers of tv_prepare_verify_simt do not know the depth: of the kernels for more than 64
-  // nodes they reach the block form only
+  // nodes they reach the block form and, under the gated rule, the path form
   if (st == TV_OK) st = prepare_kernel(verify_simt_deep_kernel<BF16, DELTA, 3>, DeepCfg<DELTA, 3>::kSmem);
   if (st == TV_OK) st = prepare_kernel(verify_simt_deep_kernel<BF16, DELTA, 4>, DeepCfg<DELTA, 4>::kSmem);
+  if constexpr (!DELTA) {
+    if (st == TV_OK) st = prepare_two<BF16, 3>();
+    if (st == TV_OK) st = prepare_two<BF16, 4>();
+  }
   return st;
 }
 

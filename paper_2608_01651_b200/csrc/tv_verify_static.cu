@@ -16,9 +16,10 @@ constexpr int kMaxTrees = TV_STATIC_MAX_TREES;
 constexpr size_t kNodes = (size_t)kMaxTrees * TV_MAX_NODES;
 constexpr size_t kAncBytes = kNodes * 2 * sizeof(uint64_t);
 constexpr size_t kI32Bytes = kNodes * sizeof(int32_t);
-constexpr size_t kScratchBytes = kAncBytes + 2 * kI32Bytes + 256;   // masks | depths | parents | status
+constexpr size_t kDepthBytes = kMaxTrees * sizeof(int32_t);
+constexpr size_t kScratchBytes = kAncBytes + 2 * kI32Bytes + kDepthBytes + 256;   // masks | depths | parents | max depths | status
 
-// The scratch.  Every GPU that loads the library holds these 384 KiB until the process exits.
+// The scratch.  Every GPU that loads the library holds these 385 KiB until the process exits.
 // In host code this name is only a stand-in for the symbol: the device address comes from
 // cudaGetSymbolAddress below and is what the kernels receive.
 static __device__ __align__(256) unsigned char g_static_tree[kScratchBytes];
@@ -29,13 +30,15 @@ static __device__ __align__(256) unsigned char g_static_tree[kScratchBytes];
 __global__ void __launch_bounds__(TV_MAX_NODES)
 tree_meta_static_kernel(const int32_t* __restrict__ parent, int32_t n, uint64_t* __restrict__ anc,
                         int32_t* __restrict__ depth, int32_t* __restrict__ parent_dev,
-                        int32_t* scratch_status, int32_t* user_status) {
+                        int32_t* __restrict__ max_depth, int32_t* scratch_status, int32_t* user_status) {
   __shared__ int32_t par_s[TV_MAX_NODES];
+  __shared__ int32_t max_s;
   const int t = blockIdx.x, i = threadIdx.x;
   // a verify kernel launched behind this one may be scheduled now and set itself up; it waits
   // for this grid to finish before it reads global memory
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   bool bad = false;
+  if (i == 0) max_s = 0;
   if (i < n) {
     int p = parent[(size_t)t * n + i];
     if (p < -1 || p >= i) {
@@ -47,13 +50,17 @@ tree_meta_static_kernel(const int32_t* __restrict__ parent, int32_t n, uint64_t*
   // the status word of the launch that is about to read this metadata starts at zero
   if (t == 0 && i == 0) *scratch_status = 0;
   if (__syncthreads_or(bad) && i == 0 && user_status) atomicExch(user_status, (int)TV_ERR_INVALID_TREE);
-  if (i >= n) return;
   uint64_t w0 = 0, w1 = 0;
   int d = 0;
-  for (int p = par_s[i]; p >= 0 && d < n; p = par_s[p]) {
+  for (int p = i < n ? par_s[i] : -1; p >= 0 && d < n; p = par_s[p]) {
     if (p < 64) w0 |= 1ull << p; else w1 |= 1ull << (p - 64);
     ++d;
   }
+  const int d_warp = __reduce_max_sync(0xffffffffu, d);
+  if ((i & 31) == 0) atomicMax(&max_s, d_warp);
+  __syncthreads();
+  if (i == 0) max_depth[t] = max_s;
+  if (i >= n) return;
   const size_t o = (size_t)t * n + i;
   anc[2 * o] = w0;
   anc[2 * o + 1] = w1;
@@ -132,7 +139,8 @@ int tv_tree_verify_static(const int32_t* parent, int32_t n_trees, const tv_dims*
   uint64_t* anc = reinterpret_cast<uint64_t*>(base);
   int32_t* depth = reinterpret_cast<int32_t*>(base + kAncBytes);
   int32_t* par_dev = reinterpret_cast<int32_t*>(base + kAncBytes + kI32Bytes);
-  int32_t* scratch_status = reinterpret_cast<int32_t*>(base + kAncBytes + 2 * kI32Bytes);
+  int32_t* max_depth = reinterpret_cast<int32_t*>(base + kAncBytes + 2 * kI32Bytes);
+  int32_t* scratch_status = max_depth + kMaxTrees;
 
   VerifyArgs a;
   a.tree.anc = anc;
@@ -140,6 +148,7 @@ int tv_tree_verify_static(const int32_t* parent, int32_t n_trees, const tv_dims*
   a.tree.parent = par_dev;
   a.tree.n_trees = n_trees;
   a.tree.max_depth_all = TV_MAX_NODES - 1;   // not known on the host
+  a.max_depth = max_depth;
   a.tree.offsets = nullptr;
   a.tree.capacity = 0;
   a.L = d->L; a.B = d->B; a.H = d->H; a.T = d->T; a.dk = d->dk; a.dv = d->dv;
@@ -154,7 +163,7 @@ int tv_tree_verify_static(const int32_t* parent, int32_t n_trees, const tv_dims*
 
   cudaStream_t s = (cudaStream_t)stream;
   tree_meta_static_kernel<<<n_trees, TV_MAX_NODES, 0, s>>>(parent, d->T, anc, depth, par_dev,
-                                                          scratch_status, status);
+                                                          max_depth, scratch_status, status);
   TV_CUDA_TRY(cudaGetLastError());
   int st;
   if (tc_gated && d->impl != TV_IMPL_SIMT) st = tv_launch_verify_tc(a, scratch_status, s);

@@ -161,3 +161,36 @@ def test_first_call_loads_what_every_later_call_launches():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     p = subprocess.run([sys.executable, "-c", _FRESH], cwd=root, capture_output=True, text=True, timeout=300)
     assert p.returncode == 0 and p.stdout.strip() == "ok", p.stderr[-2000:]
+
+
+@pytest.mark.parametrize("dtype", [inputs.F32, inputs.BF16])
+@pytest.mark.parametrize("T", [65, 96, 97, 128])
+def test_static_trees_of_unknown_depth(T, dtype):
+    """More than 64 nodes under the gated rule and more items than SMs: a shallow tree's items go to the path
+    form, a deep one's to the block form, in one call (dims that the tensor-core kernel does not take)."""
+    for B, H, d in ((12, 16, 72), (24, 8, 128)):
+        if d == 128 and dtype == inputs.BF16:
+            continue
+        wl = inputs.workload("c3", B=B, H=H, T=T, dk=d, dv=d, tree="frontier", qkv_dtype=dtype, seed=T)
+        parents, _ = inputs.make_trees(wl)
+        rng = np.random.default_rng(T)
+        parents[1] = inputs.tree_chain(T)
+        parents[2] = inputs.tree_frontier(T, rng, max_depth=15, spine=16)
+        parents[B - 1] = inputs.tree_frontier(T, rng, max_depth=16, spine=17)
+        t_cpu = inputs.make_tensors(wl)
+        if dtype == inputs.F32:
+            t_cpu["k"] = t_cpu["k"] * (8.0 / d ** 0.5)
+        t = {k: (None if v is None else v.cuda()) for k, v in t_cpu.items()}
+        O, U = _static(wl, torch.from_numpy(parents).cuda(), t, True)
+        items = [(b, h) for b in (0, 1, 2, 3, B - 1) for h in (0, H - 1)]
+        ver, _ = pu.oracle_round(wl, parents, np.full(B, -1), t_cpu, items=items)
+        On = O.cpu().double().numpy()
+        for (b, h), (Or, _) in ver.items():
+            assert pu.rel_l2_rows(On[b, h], Or) <= 5e-5       # fp32 sums over chains of up to 128 nodes
+        assert torch.equal(U, t["v"].float())
+        # one shared shallow tree, one shared deep tree
+        for par in (parents[2], parents[B - 1]):
+            O1, _ = _static(wl, torch.from_numpy(par[None]).cuda(), t, False)
+            ver, _ = pu.oracle_round(wl, np.stack([par] * B), np.full(B, -1), t_cpu, items=[(0, 0), (B - 1, H - 1)])
+            for (b, h), (Or, _) in ver.items():
+                assert pu.rel_l2_rows(O1[b, h].cpu().double().numpy(), Or) <= 5e-5
