@@ -234,17 +234,15 @@ commit_rows_kernel(const CommitArgs a, const __grid_constant__ CommitLayers tb) 
 
   int acc = a.accepted[li.b];
   if (acc >= a.T) acc = -1;
-  if (acc < 0 && a.in_place) {
-    // Nothing to do, but not before the kernel in front is done: if every request is rejected these are all
-    // the grid's threads, and the kernel behind -- an upload, a convolution -- waits for this grid only
-    // before it overwrites what the kernel in front (verify) may still be reading.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    return;
-  }
+  // A request rejected in place has nothing to do, but not before the kernel in front is done: if every
+  // request is rejected these are all the grid's threads, and the kernel behind -- an upload, a convolution --
+  // waits for this grid only before it overwrites what the kernel in front (verify) may still be reading.
   float4 s[RPT];
+  if (acc >= 0 || !a.in_place) {
 #pragma unroll
-  for (int e = 0; e < RPT; ++e)
-    if (row0 + e < dv) s[e] = ld_stream(src + e * LPR);
+    for (int e = 0; e < RPT; ++e)
+      if (row0 + e < dv) s[e] = ld_stream(src + e * LPR);
+  }
   // Dependent launch: this grid may have started under the tail of the kernel in front of it
   // (a verify kernel, or the tree-metadata kernel when no verify call sits in between).  S_pre
   // and the accepted nodes are older than either; everything those kernels write -- U, and the
@@ -498,7 +496,7 @@ cudaError_t launch_after_verify(void (*kernel)(const CommitArgs, const CommitLay
 // SM, while all of them are resident (128 items: 4.6 us against 5.2 with eight rows).  Beyond that
 // 64 rows per CTA -- sixteen per thread, eight for dk = 64: fewest paths to work out per byte (a round of
 // 1024 items 53.2 us against 55.8 with half as many rows, of 512 items 40.4 against 41.1).  The register
-// limits of the dk = 64 kernels (8 CTAs per SM, 7 with f32 keys) cost 44 and 36 bytes of spills.
+// limits of the dk = 64 kernels (8 CTAs per SM, 7 with f32 keys) cost up to 24 bytes of spills.
 template <bool BF16, int DK>
 cudaError_t launch_rows(const CommitArgs& a, const CommitLayers& tb, int items, int sms, cudaStream_t stream) {
   constexpr int kRpt = DK == 128 ? 16 : 8, kCtas = DK == 128 ? 4 : BF16 ? 8 : 7;   // 64 rows per CTA
