@@ -1,0 +1,826 @@
+// Tree verification of the gated delta rule on the tensor cores (tcgen05 + TMEM + TMA).
+//
+// Shapes: bf16 q/k/v, fp32 state, dk = dv = 128, tree depth <= 15, dense batches (any strides) and
+// packed forests.  NB = 1: up to 64 nodes, NB = 2: up to 128, worked on as two row blocks of 64.
+//
+// Algebra (Theorem 1, Eq. 2; Lemma 2/3).  With N = (I+G)^-1, A = N D_beta, W = C A, and
+// V' = V - D_P K S_pre^T (the part of the correction that the old state does not hold already):
+//     O = D_P Q S_pre^T + W V',     U = A V'
+// so the state is contracted once, with the raw [Q ; K], and nothing of that product waits for the
+// triangular systems.  G, C, N, A, W are T x T but ancestor-sparse: row i has entries only on the
+// root-to-node path p_0 < ... < p_d = i of node i, and slot s of node i and of any descendant refer
+// to the same node p_s.  Row i of W and of A come from ONE back-substitution each on the
+// path-restricted unit triangular system (w L = c, x L = e_d; L = I + G on the path).  All decay
+// factors are products of alpha over a stretch of the row's own path, never a quotient of two
+// numbers that may both underflow.
+//
+// Tile rows 0..63 carry the O problem of the block's nodes, rows 64..127 the U problem:
+//     Sc  = [Q_b ; K_b] K^T                   scores, columns = all nodes up to the block's last
+//     X   = [Q_b ; K_b] [S_hi + S_lo]^T       q/k exact, state as two bf16 (16 mantissa bits and more)
+//     X rows 0..63  *= P_i,  V' = V - P_i X rows 64..127 -> bf16 hi + lo, then those rows = 0
+//     X  += [W ; A]_hi V'_hi + [W ; A]_lo V'_hi + [W ; A]_hi V'_lo     rows 0..63 = O, 64..127 = U
+//
+// What bounds it and how it is laid out.  At the copy rate an SM's share of the memory moves an item
+// of 64 nodes in 4.1 us and one of 128 in 6.6; the dependent chain of one item is two to three times
+// that.  So the chain is cut between four groups of four warps, each busy for less than that time and
+// each working on a different item or block:
+//     warps 0..3    TMA producer | MMA issuer | metadata (paths, gates, P of the items to come) | -
+//     warps 4..7    state rows split in place into bf16 hi + lo, then V' and the scaling of X
+//     warps 8..11   thread = tile row: scores of its path, back-substitution, row of [W ; A]
+//     warps 12..15  finished rows of X to memory
+// and nothing of it is staged in a buffer that the next item needs: the coefficient rows are the A
+// operand in tensor memory, in the columns of the scores they came from; the state arrives in a ring
+// of four quarters of k (a quarter's fp32 rows of 128 bytes become [hi | lo] rows of the same bytes,
+// so one 128-wide tile feeds the hi and the lo product); outputs pass through 2 KiB per warp.
+// The thread that issues the MMAs takes whichever product is ready (outputs first), so that no item
+// waits for another one's operands.
+// Every wait is a bounded mbarrier wait (status word on expiry); every TMA load is a plain per-CTA copy.
+#pragma once
+#include "tv_tc_common.cuh"
+
+namespace tvdelta {
+
+using namespace tvtc;
+
+constexpr int kThreads = 512;
+constexpr int kSlots = 16;     // path slots per node: depth <= 15
+constexpr int kBlk = 64;       // nodes per row block
+constexpr int kLd = 17;        // row stride of the key-score table (floats): conflict-free per slot
+constexpr int kUnits = 4;      // quarters of k, ring slots of the state
+
+template <int NB>
+struct Map {
+  static constexpr int kNodes = kBlk * NB;
+  static constexpr int kMeta = NB == 1 ? 4 : 2;      // metadata buffers (items ahead of the slowest group)
+  // bytes from the 1024-aligned base
+  static constexpr uint32_t kOffQK = 0;              // two blocks of [Q ; K]: 2 k halves of [128][64] bf16 (NB = 1: two items)
+  static constexpr uint32_t kOffS = 4 * kTile;       // four units [128 v][32] fp32, after the split [128 v][32 hi | 32 lo] bf16
+  static constexpr uint32_t kOffV = 8 * kTile;       // V, then V'_hi in its place, and V'_lo: dv halves of [nodes][64] (NB = 1: two items)
+  static constexpr uint32_t kVHalf = kNodes * 128;   // one dv half
+  static constexpr uint32_t kVItem = 4 * kVHalf;     // hi, lo
+  static constexpr uint32_t kOffRow = 12 * kTile;    // 64 bytes per tile row, private to its thread (warps 8..11)
+  static constexpr uint32_t kOffOut = kOffRow + 8192;   // 2 KiB per warp (warps 12..15)
+  static constexpr uint32_t kOffGs = kOffOut + 8192;    // float Gs[kNodes][kLd]: K K^T on the path
+  static constexpr uint32_t kOffPath = kOffGs + kNodes * kLd * 4;          // kMeta x uint8[kNodes][16], path in slot order
+  static constexpr uint32_t kOffDepth = kOffPath + kMeta * kNodes * 16;    // kMeta x int8[kNodes], -1 = no node
+  static constexpr uint32_t kOffTab = kOffDepth + kMeta * kNodes;          // kMeta x {alpha, beta, P}[kNodes]
+  static constexpr uint32_t kOffItem = kOffTab + kMeta * kNodes * 12;      // kMeta x {nodes, first output element (2 words), -}
+  static constexpr uint32_t kOffBar = kOffItem + kMeta * 16;
+  static constexpr uint32_t kOffMisc = kOffBar + 8 * 48;
+  static constexpr uint32_t kSmemBytes = kOffMisc + 32;
+  static_assert(kOffBar % 8 == 0 && kSmemBytes <= 232448, "shared memory of one CTA");
+};
+
+// [2]: block g of the CTA (item * NB + row block) uses entry g & 1, in its phase g >> 1
+enum Bar {
+  QK_FULL = 0, QK_FREE = 2, GD = 4, SC_FREE = 6, COEF = 8, VP = 10, ACC = 12, X_FREE = 14,
+  V_FULL = 16, V_FREE = 18,          // [2]: NB = 1 as above, NB = 2 entry 0 per item
+  X_DONE = 20,                       // [2]: item & 1
+  S_FULL = 22, S_SPLIT = 26, S_FREE = 30,   // [4]: unit, phase = item
+  META_FULL = 34, META_FREE = 38,    // [kMeta]
+  E1_SYNC = 42, kNumBars = 43
+};
+static_assert(kNumBars <= 48, "barrier area");
+
+constexpr uint32_t kColX = 0, kColSc = 256;
+
+struct Params {
+  TreeDev tree;
+  int32_t n_items, B, H, T;
+  int32_t Hk;  // q/k heads (grouped key heads); H when not grouped
+  const float* alpha;
+  const float* beta;
+  int32_t* status;
+  float* O;
+  float* U;                  // null: corrections not wanted
+  const int32_t* offsets;    // packed forest only: row offsets of the requests, rows per (layer, head) plane
+  int32_t capacity;
+  ItemDiv div;               // divisions by H, B, H / Hk as multiply-shift
+  Str3 gate, out;            // strides of alpha / beta and of O / U (dense layouts)
+  // The q, k, v maps are 4-D, (channel, node, head, layer*request) or (channel, head, node, ...)
+  // whichever has ascending strides: bit 0 / 1 set = q,k / v take the node coordinate first.
+  int32_t node_first;
+};
+
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t idesc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 1, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d), "r"(a_tmem), "l"(b), "r"(idesc) : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+// Two fp32 -> one word of two bf16, rounded to nearest even (first argument in the low half).
+__device__ __forceinline__ uint32_t pack_rn(float lo_elem, float hi_elem) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi_elem), "f"(lo_elem));
+  return r;
+}
+// A pair of fp32 as bf16 hi (rounded to nearest) and lo (the exact remainder, rounded to nearest)
+__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hi, uint32_t& lo) {
+  hi = pack_rn(x0, x1);
+  lo = pack_rn(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u));
+}
+
+// DMAX: compile-time bound on the tree depth (8 covers draft trees, 15 the rest), so that the
+// per-row triangular solve is straight-line code whose loads all issue up front.
+// PACKED = packed forest: request b owns rows offsets[b] .. offsets[b+1]-1 of every plane; loads take
+// 64-row boxes at the request's offset.  Rows past the request's node count may hold anything: their
+// V' is set to zero, their scores are never selected and their outputs never stored.
+template <int NB, int DMAX, bool PACKED>
+__global__ void __launch_bounds__(kThreads, 1)
+verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                       const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmS,
+                       const Params p) {
+  using M = Map<NB>;
+  constexpr int kNodes = M::kNodes;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* sm = smem_raw;
+  const uint32_t sbase = smem_u32(sm);
+  if (sbase & 1023u) {   // the swizzled tiles need this alignment; refuse rather than compute garbage
+    if (threadIdx.x == 0 && p.status) atomicExch(p.status, (int)TV_ERR_CUDA);
+    return;
+  }
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + M::kOffMisc);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + M::kOffMisc + 4);
+  auto bar = [&](int i) { return sbase + M::kOffBar + 8u * (uint32_t)i; };
+  auto tab_of = [&](uint32_t buf) { return reinterpret_cast<float*>(sm + M::kOffTab) + buf * (3 * kNodes); };
+  auto item_of = [&](uint32_t buf) { return reinterpret_cast<int32_t*>(sm + M::kOffItem) + buf * 4; };
+  auto sc_col = [](int g) -> uint32_t { return kColSc + (uint32_t)(g & 1) * 64u; };   // NB = 2: block 1 has 128 columns from there
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int T = p.T;
+  const bool want_U = p.U != nullptr;
+  const uint32_t n_it = (int)blockIdx.x < p.n_items
+                            ? ((uint32_t)p.n_items - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u;
+
+  if (tid == 0) {
+    abort_flag[0] = 0;
+    abort_flag[1] = 0;
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar(QK_FULL + i), 1);  mbar_init(bar(QK_FREE + i), 1);
+      mbar_init(bar(GD + i), 1);       mbar_init(bar(SC_FREE + i), 1);
+      mbar_init(bar(COEF + i), 4);     mbar_init(bar(VP + i), 4);
+      mbar_init(bar(ACC + i), 1);      mbar_init(bar(X_FREE + i), 4);
+      mbar_init(bar(V_FULL + i), 1);   mbar_init(bar(V_FREE + i), 1);
+      mbar_init(bar(X_DONE + i), 1);
+    }
+    for (int i = 0; i < kUnits; ++i) {
+      mbar_init(bar(S_FULL + i), 1);
+      mbar_init(bar(S_SPLIT + i), 4);
+      mbar_init(bar(S_FREE + i), 1);
+    }
+    for (int i = 0; i < M::kMeta; ++i) {
+      mbar_init(bar(META_FULL + i), 1);
+      mbar_init(bar(META_FREE + i), 12);
+    }
+    mbar_init(bar(E1_SYNC), 4);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  // registers: 128 per thread at launch; the solving warps take what the first four give up
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    if (warp == 0 && lane == 0) {
+      // ===================== TMA producer =====================
+      grid_dependency_wait();   // inputs may come from the kernel in front (dependent launch)
+      uint32_t n_qk = 0, n_v = 0, n_s = 0;   // loads issued: blocks, items, units
+      for (uint32_t it = 0; it < n_it; ++it) {
+        const int item = (int)(blockIdx.x + it * gridDim.x);
+        // box coordinates: q/k head, v head, outermost index (layer*request, or the layer of a packed
+        // forest) and the first node row
+        const int lb = (int)fdiv((uint32_t)item, p.div.dH), h = item - lb * p.H;
+        const int hq = (int)fdiv((uint32_t)h, p.div.dG);
+        int z = lb, y0 = 0;
+        if constexpr (PACKED) {
+          z = (int)fdiv((uint32_t)lb, p.div.dB);
+          y0 = __ldg(p.offsets + (lb - z * p.B));
+        }
+        auto load_v = [&]() -> bool {
+          const uint32_t vb = NB == 1 ? it & 1 : 0, vph = NB == 1 ? it >> 1 : it;
+          if (!mbar_wait(bar(V_FREE + vb), (vph & 1) ^ 1, abort_flag)) return false;
+          mbar_expect_tx(bar(V_FULL + vb), 2 * M::kVHalf);
+#pragma unroll 1
+          for (int i = 0; i < 2 * NB; ++i)   // dv half i & 1, row block i >> 1
+            load_box(sbase + M::kOffV + vb * M::kVItem + (uint32_t)(i & 1) * M::kVHalf + (uint32_t)(i >> 1) * 8192u, &tmV,
+                     bar(V_FULL + vb), p.node_first & 2, 64 * (i & 1), y0 + kBlk * (i >> 1), h, z);
+          ++n_v;
+          return true;
+        };
+        bool ok = true;
+        for (int b = 0; b < NB; ++b) {
+          const uint32_t g = it * NB + b, gb = g & 1;
+          if (!(ok = mbar_wait(bar(QK_FREE + gb), ((g >> 1) & 1) ^ 1, abort_flag))) break;
+          mbar_expect_tx(bar(QK_FULL + gb), 4 * 8192);
+#pragma unroll 1
+          for (int i = 0; i < 4; ++i)   // k half i >> 1; Q rows, then K rows
+            load_box(sbase + M::kOffQK + gb * 2 * kTile + (uint32_t)(i >> 1) * kTile + (uint32_t)(i & 1) * 8192u,
+                     (i & 1) ? &tmK : &tmQ, bar(QK_FULL + gb), p.node_first & 1, 64 * (i >> 1), y0 + kBlk * b, hq, z);
+          ++n_qk;
+        }
+        if (!ok) break;
+        // NB = 1 has a second buffer for V, free long before the state's; NB = 2 has one, free last
+        if (NB == 1 && it > 0 && !load_v()) break;
+        for (int u = 0; ok && u < kUnits; ++u) {
+          if (!(ok = mbar_wait(bar(S_FREE + u), (it & 1) ^ 1, abort_flag))) break;
+          mbar_expect_tx(bar(S_FULL + u), kTile);
+          tma_load_3d(sbase + M::kOffS + (uint32_t)u * kTile, &tmS, bar(S_FULL + u), 32 * u, 0, item);
+          ++n_s;
+        }
+        if (!ok) break;
+        if ((NB == 2 || it == 0) && !load_v()) break;
+      }
+      if (*abort_flag) {
+        // Leave no copy of ours in flight: wait (bounded) for the last load issued into each buffer.
+        for (uint32_t g = n_qk > 2 ? n_qk - 2 : 0; g < n_qk; ++g) mbar_wait(bar(QK_FULL + (g & 1)), (g >> 1) & 1, abort_flag + 1);
+        for (uint32_t i = n_v > 2 ? n_v - 2 : 0; i < n_v; ++i)
+          mbar_wait(bar(V_FULL + (NB == 1 ? i & 1 : 0)), (NB == 1 ? i >> 1 : i) & 1, abort_flag + 1);
+        for (uint32_t i = n_s > 4 ? n_s - 4 : 0; i < n_s; ++i)
+          mbar_wait(bar(S_FULL + (i & 3)), (i >> 2) & 1, abort_flag + 1);
+      }
+    } else if (warp == 1 && lane == 0) {
+      // ===================== MMA issuer =====================
+      constexpr uint32_t kIdGram = idesc_bf16(64, false), kIdX = idesc_bf16(128, false), kIdAV = idesc_bf16(128, true);
+      const uint32_t n_g = n_it * NB, n_u = n_it * kUnits;
+      uint32_t ig = 0, iu = 0, ia = 0;   // next block's scores, next unit of the state product, next block's readout
+      const uint64_t dQK = desc_kmajor(sbase + M::kOffQK), dS = desc_kmajor(sbase + M::kOffS);
+      const uint64_t dV = desc_mnmajor(sbase + M::kOffV, M::kVHalf);
+      long long t_idle = clock64();
+      uint32_t spin = 0;
+      while (ia < n_g) {
+        bool progress = false;
+        // X += [W ; A] V' of block ia
+        if (mbar_test(bar(COEF + (ia & 1)), (ia >> 1) & 1) && mbar_test(bar(VP + (ia & 1)), (ia >> 1) & 1)) {
+          tc_fence_after();
+          const uint32_t b = NB == 1 ? 0u : ia & 1;
+          const uint32_t acc = tmem + kColX + (ia & 1) * 128u, chi = tmem + sc_col((int)ia), clo = chi + 32u * (b + 1);
+          const uint64_t dvi = dV + (NB == 1 ? ((ia & 1) * M::kVItem) >> 4 : 0u);
+#pragma unroll 1
+          for (uint32_t hb = 0; hb <= b; ++hb)   // 64 ancestors
+#pragma unroll
+            for (uint32_t s = 0; s < 4; ++s) {   // 16 ancestors per step
+              const uint64_t hi = dvi + ((hb * 8192u + s * 2048u) >> 4), lo = hi + ((2 * M::kVHalf) >> 4);
+              const uint32_t c = hb * 32u + s * 8u;
+              mma_bf16_ts(acc, chi + c, hi, kIdAV);
+              mma_bf16_ts(acc, clo + c, hi, kIdAV);
+              mma_bf16_ts(acc, chi + c, lo, kIdAV);
+            }
+          tc_commit(bar(ACC + (ia & 1)));
+          tc_commit(bar(SC_FREE + (ia & 1)));
+          if (NB == 1) tc_commit(bar(V_FREE + (ia & 1)));
+          else if (b == 1) tc_commit(bar(V_FREE));
+          ++ia;
+          progress = true;
+        }
+        // Sc = [Q ; K] K^T of block ig
+        if (ig < n_g && mbar_test(bar(QK_FULL + (ig & 1)), (ig >> 1) & 1) &&
+            mbar_test(bar(SC_FREE + (ig & 1)), ((ig >> 1) & 1) ^ 1)) {
+          tc_fence_after();
+          const uint32_t b = NB == 1 ? 0u : ig & 1;
+          const uint64_t dA = dQK + (((ig & 1) * 2 * kTile) >> 4);
+#pragma unroll 1
+          for (uint32_t hb = 0; hb <= b; ++hb) {   // K rows of block hb (NB = 1: of the block itself)
+            const uint64_t dB = (NB == 1 ? dA : dQK + ((hb * 2 * kTile) >> 4)) + (8192 >> 4);
+#pragma unroll
+            for (uint32_t i = 0; i < 8; ++i) {     // k half i >> 2, 32 bytes of k per step
+              const uint32_t off = ((i >> 2) * kTile + (i & 3u) * 32u) >> 4;
+              mma_bf16_ss(tmem + sc_col((int)ig) + 64u * hb, dA + off, dB + off, kIdGram, i);
+            }
+          }
+          tc_commit(bar(GD + (ig & 1)));
+          ++ig;
+          progress = true;
+        }
+        // X = [Q ; K] S_pre^T, one quarter of k for all blocks of the item
+        if (iu < n_u) {
+          const uint32_t it = iu / kUnits, u = iu % kUnits, g0 = it * NB;
+          bool ready = ig >= g0 + NB && mbar_test(bar(S_SPLIT + u), it & 1);
+          if (ready && u == 0)
+            for (uint32_t b = 0; b < NB; ++b)   // the block that had these columns before has been read out
+              ready = ready && mbar_test(bar(X_FREE + ((g0 + b) & 1)), (((g0 + b) >> 1) & 1) ^ 1);
+          if (ready) {
+            tc_fence_after();
+            const uint64_t dB = dS + ((u * kTile) >> 4);
+#pragma unroll
+            for (uint32_t b = 0; b < NB; ++b) {
+              const uint32_t gb = (g0 + b) & 1;
+              const uint64_t dA = dQK + ((gb * 2 * kTile + (u >> 1) * kTile + (u & 1) * 64u) >> 4);
+#pragma unroll
+              for (uint32_t i = 0; i < 4; ++i)   // hi: k 0..15, 16..31 of the quarter; lo: the same
+                mma_bf16_ss(tmem + kColX + gb * 128u, dA + (((i & 1u) * 32u) >> 4), dB + ((i * 32u) >> 4), kIdX, u | i);
+            }
+            tc_commit(bar(S_FREE + u));
+            if (u == kUnits - 1) {
+              tc_commit(bar(X_DONE + (it & 1)));
+              for (uint32_t b = 0; b < NB; ++b) tc_commit(bar(QK_FREE + ((g0 + b) & 1)));
+            }
+            ++iu;
+            progress = true;
+          }
+        }
+        if (progress) {
+          t_idle = clock64();
+          spin = 0;
+        } else if ((++spin & 255u) == 0) {   // the same limit as every other wait of the kernel
+          if (*abort_flag) break;
+          if (clock64() - t_idle > kWaitLimitCycles) {
+            *abort_flag = 1;
+            break;
+          }
+        }
+      }
+    } else if (warp == 2) {
+      // ===================== metadata =====================
+      grid_dependency_wait();   // tree metadata and gates may come from the kernels in front
+      for (uint32_t it = 0; it < n_it; ++it) {
+        const int item = (int)(blockIdx.x + it * gridDim.x);
+        const uint32_t buf = it % M::kMeta, use = it / M::kMeta;
+        if (!mbar_wait_warp(bar(META_FREE + buf), (use & 1) ^ 1, abort_flag)) break;
+        int n = T, tb = 0;
+        int64_t g0, gstep = 1;   // first gate of the item, step between nodes
+        size_t o0;               // element offset of the item's first output row
+        if constexpr (PACKED) {
+          const PackedItem pi = packed_item(p.offsets, p.B, p.H, p.Hk, item, p.div);
+          n = pi.n;
+          tb = pi.b;
+          g0 = (int64_t)pi.plane_v * p.capacity + pi.row0;
+          o0 = (size_t)g0 * 128;
+        } else {
+          const int lb = (int)fdiv((uint32_t)item, p.div.dH), h = item - lb * p.H;
+          tb = p.tree.n_trees == 1 ? 0 : request_of(item, p.B, p.div);
+          g0 = (int64_t)lb * p.gate.b + (int64_t)h * p.gate.h;
+          gstep = p.gate.t;
+          o0 = (size_t)((int64_t)lb * p.out.b + (int64_t)h * p.out.h);
+        }
+        // all loads first: one trip to memory, not one per table
+        ulonglong2 mk[2 * NB];
+        float al[2 * NB], be[2 * NB];
+#pragma unroll
+        for (int h = 0; h < 2 * NB; ++h) {
+          const int nd = lane + 32 * h;
+          mk[h] = make_ulonglong2(0ull, 0ull);
+          al[h] = 1.f;
+          be[h] = 0.f;
+          if (nd < n) {
+            mk[h] = __ldg(reinterpret_cast<const ulonglong2*>(p.tree.anc) + (size_t)tb * T + nd);
+            al[h] = __ldg(p.alpha + g0 + nd * gstep);
+            be[h] = __ldg(p.beta + g0 + nd * gstep);
+          }
+        }
+        float* tab = tab_of(buf);
+        uint8_t* paths = sm + M::kOffPath + (buf * kNodes) * 16;
+        int8_t* depths = reinterpret_cast<int8_t*>(sm + M::kOffDepth) + buf * kNodes;
+#pragma unroll
+        for (int h = 0; h < 2 * NB; ++h) {
+          tab[lane + 32 * h] = al[h];
+          tab[kNodes + lane + 32 * h] = be[h];
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int h = 0; h < 2 * NB; ++h) {
+          const int nd = lane + 32 * h;
+          // the node's path in slot order: the set bits of (ancestors | self) from the lowest up
+          // (nodes are numbered parent before child); slots past the node's depth name the node itself
+          uint64_t r0 = h == 0 ? mk[0].x : h == 1 ? mk[1].x : NB == 2 ? (h == 2 ? mk[2 * NB - 2].x : mk[2 * NB - 1].x) : 0ull;
+          uint64_t r1 = h == 0 ? mk[0].y : h == 1 ? mk[1].y : NB == 2 ? (h == 2 ? mk[2 * NB - 2].y : mk[2 * NB - 1].y) : 0ull;
+          const int d = __popcll(r0) + __popcll(r1);
+          float P = 1.f;
+          uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+          for (int s = 0; s < kSlots; ++s) {
+            int j = nd;
+            if (r0 != 0ull) {
+              j = __ffsll((long long)r0) - 1;
+              r0 &= r0 - 1;
+            } else if (NB == 2 && r1 != 0ull) {
+              j = 64 + __ffsll((long long)r1) - 1;
+              r1 &= r1 - 1;
+            }
+            w[s >> 2] |= (uint32_t)j << (8 * (s & 3));
+            if (s <= DMAX && s <= d) P *= tab[j];
+          }
+          *reinterpret_cast<uint4*>(paths + nd * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+          depths[nd] = nd < n ? (int8_t)d : (int8_t)-1;
+          tab[2 * kNodes + nd] = P;
+        }
+        if (lane == 0) {
+          int32_t* im = item_of(buf);
+          im[0] = n;
+          im[1] = (int32_t)(o0 & 0xffffffffu);
+          im[2] = (int32_t)(o0 >> 32);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(META_FULL + buf));
+      }
+    }
+  } else if (warp < 8) {
+    // ===================== state split, V', scaling of X =====================
+    const int quad = warp & 3, row = quad * 32 + lane;   // state row; TMEM lane
+    const int rn = row & 63;                             // node of this tile row within its block
+    const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
+    const uint32_t swz = (uint32_t)(row & 7);
+    bool ok = true;
+    for (uint32_t it = 0; ok && it < n_it; ++it) {
+#pragma unroll 1
+      for (int u = 0; u < kUnits; ++u) {
+        if (!(ok = mbar_wait_warp(bar(S_FULL + u), it & 1, abort_flag))) break;
+        // 32 fp32 of this row -> 32 bf16 hi | 32 bf16 lo in the same 128 bytes
+        unsigned char* r = sm + M::kOffS + (uint32_t)u * kTile + (uint32_t)row * 128u;
+        uint4 hi[4], lo[4];
+#pragma unroll
+        for (uint32_t c = 0; c < 4; ++c) {
+          const float4 a = *reinterpret_cast<const float4*>(r + (((2 * c) ^ swz) << 4));
+          const float4 e = *reinterpret_cast<const float4*>(r + (((2 * c + 1) ^ swz) << 4));
+          split_pair(a.x, a.y, hi[c].x, lo[c].x);
+          split_pair(a.z, a.w, hi[c].y, lo[c].y);
+          split_pair(e.x, e.y, hi[c].z, lo[c].z);
+          split_pair(e.z, e.w, hi[c].w, lo[c].w);
+        }
+#pragma unroll
+        for (uint32_t c = 0; c < 4; ++c) {
+          *reinterpret_cast<uint4*>(r + ((c ^ swz) << 4)) = hi[c];
+          *reinterpret_cast<uint4*>(r + (((c + 4) ^ swz) << 4)) = lo[c];
+        }
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(S_SPLIT + u));
+      }
+      if (!ok) break;
+      const uint32_t buf = it % M::kMeta, vb = NB == 1 ? it & 1 : 0;
+      if (!(ok = mbar_wait_warp(bar(META_FULL + buf), (it / M::kMeta) & 1, abort_flag))) break;
+      if (!(ok = mbar_wait_warp(bar(V_FULL + vb), (NB == 1 ? it >> 1 : it) & 1, abort_flag))) break;
+      if (!(ok = mbar_wait_warp(bar(X_DONE + (it & 1)), (it >> 1) & 1, abort_flag))) break;
+      tc_fence_after();
+      const int n = item_of(buf)[0];
+#pragma unroll 1
+      for (int b = 0; b < NB; ++b) {
+        const uint32_t g = it * NB + b;
+        const int nd = kBlk * b + rn;
+        const float P = tab_of(buf)[2 * kNodes + nd];
+        const uint32_t xcol = tmem + lane_addr + kColX + (g & 1) * 128u;
+        if (quad < 2) {
+          // O problem: the prefix term P_i q_i S_pre^T is where the accumulation starts
+          if (kBlk * b + quad * 32 < n) {
+#pragma unroll 1
+            for (int c = 0; c < 4; ++c) {
+              uint32_t x[32];
+              tmem_ld32(xcol + 32u * c, x);
+              tmem_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 32; ++i) x[i] = __float_as_uint(P * __uint_as_float(x[i]));
+              tmem_st32(xcol + 32u * c, x);
+            }
+          }
+        } else {
+          const bool alive = nd < n;
+#pragma unroll 1
+          for (int c = 0; c < 4; ++c) {   // 32 columns: half of dv half c >> 1
+            uint32_t x[32];
+            tmem_ld32(xcol + 32u * c, x);
+            unsigned char* vrow = sm + M::kOffV + vb * M::kVItem + (uint32_t)(c >> 1) * M::kVHalf + (uint32_t)nd * 128u;
+            uint4 v[4];
+#pragma unroll
+            for (uint32_t i = 0; i < 4; ++i)
+              v[i] = *reinterpret_cast<const uint4*>(vrow + ((((uint32_t)(c & 1) * 4 + i) ^ swz) << 4));
+            tmem_wait_ld();
+#pragma unroll
+            for (uint32_t i = 0; i < 4; ++i) {
+              const uint32_t vw[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+              uint32_t hi[4], lo[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const float a0 = fmaf(-P, __uint_as_float(x[8 * i + 2 * e]), __uint_as_float(vw[e] << 16));
+                const float a1 = fmaf(-P, __uint_as_float(x[8 * i + 2 * e + 1]), __uint_as_float(vw[e] & 0xffff0000u));
+                split_pair(a0, a1, hi[e], lo[e]);
+                hi[e] = alive ? hi[e] : 0u;   // select, never 0 * x: rows past the request may hold anything
+                lo[e] = alive ? lo[e] : 0u;
+              }
+              const uint32_t off = (((uint32_t)(c & 1) * 4 + i) ^ swz) << 4;
+              *reinterpret_cast<uint4*>(vrow + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+              *reinterpret_cast<uint4*>(vrow + 2 * M::kVHalf + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            }
+#pragma unroll
+            for (int i = 0; i < 32; ++i) x[i] = 0u;   // U problem: the accumulation starts from nothing
+            tmem_st32(xcol + 32u * c, x);
+          }
+          fence_async_smem();
+        }
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(VP + (g & 1)));
+      }
+      if (lane == 0) mbar_arrive(bar(META_FREE + buf));
+    }
+  } else if (warp < 12) {
+    // ===================== path systems =====================
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
+    constexpr int NS = DMAX + 1;            // path slots in use
+    const int quad = warp & 3, row = quad * 32 + lane;
+    const int rn = row & 63;
+    const int part = row >> 6;              // 0: O problem, 1: U problem
+    const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
+    float* Gs = reinterpret_cast<float*>(sm + M::kOffGs);
+    // 64 bytes of scratch per tile row, seen by its own thread only: values go in by column and come
+    // out by path node, or the other way round (registers cannot be indexed).  Chunks of 16 bytes are
+    // swizzled so that eight neighbouring rows cover all banks.
+    unsigned char* srow = sm + M::kOffRow + row * 64;
+    const uint32_t ssw = (uint32_t)(row >> 1) & 3u;
+    auto word = [&](uint32_t j) -> uint32_t { return (((j >> 2) ^ ssw) << 4) + ((j & 3u) << 2); };   // byte of column j < 16
+    bool ok = true;
+    for (uint32_t it = 0; ok && it < n_it; ++it) {
+      const uint32_t buf = it % M::kMeta;
+      if (!(ok = mbar_wait_warp(bar(META_FULL + buf), (it / M::kMeta) & 1, abort_flag))) break;
+      const float* al_s = tab_of(buf);
+      const float* be_s = al_s + kNodes;
+      const int n = item_of(buf)[0];
+#pragma unroll 1
+      for (int b = 0; b < NB; ++b) {
+        const uint32_t g = it * NB + b;
+        const int nd = kBlk * b + rn;
+        const uint4 pw = *reinterpret_cast<const uint4*>(sm + M::kOffPath + (buf * kNodes + nd) * 16);
+        const int depth = reinterpret_cast<const int8_t*>(sm + M::kOffDepth)[buf * kNodes + nd];   // -1: no node
+        const bool rows_live = kBlk * b + (quad & 1) * 32 < n;     // warp-uniform: some row of the warp is a node
+        const bool solves = rows_live && (part == 0 || want_U);    // warp-uniform: its rows carry problems
+        int path[NS];
+        float al[NS], bt[NS], vec[NS];
+        {
+          const uint32_t pword[4] = {pw.x, pw.y, pw.z, pw.w};
+#pragma unroll
+          for (int s = 0; s < NS; ++s) {
+            path[s] = (int)((pword[s >> 2] >> ((s & 3) * 8)) & 127u);
+            const float a2 = al_s[path[s]], b2 = be_s[path[s]];
+            al[s] = s <= depth ? a2 : 1.f;   // slots past the node count as no decay
+            bt[s] = s <= depth ? b2 : 0.f;
+            vec[s] = 0.f;
+          }
+        }
+        // ---- scores on the path: q_i . k_{p_s} (incl. the node), k_i . k_{p_s} ----
+        if (!(ok = mbar_wait_warp(bar(GD + (g & 1)), (g >> 1) & 1, abort_flag))) break;
+        // every warp has finished the solve of the block before, which read Gs
+        if (g > 0 && !(ok = mbar_wait_warp(bar(COEF + ((g - 1) & 1)), ((g - 1) >> 1) & 1, abort_flag))) break;
+        tc_fence_after();
+        const uint32_t col = tmem + lane_addr + sc_col((int)g);
+        // ancestors have smaller numbers than the node: nothing to select past the warp's last node
+        const int nch = 4 * b + (quad & 1) * 2 + 2;                // chunks of 16 columns
+        if (rows_live) {
+#pragma unroll 1
+          for (int c = 0; c < nch; c += 2) {
+            uint32_t r[32];
+            tmem_ld32(col + 16u * c, r);
+            tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+#pragma unroll
+              for (uint32_t i = 0; i < 4; ++i)
+                *reinterpret_cast<float4*>(srow + ((i ^ ssw) << 4)) =
+                    make_float4(__uint_as_float(r[16 * e + 4 * i]), __uint_as_float(r[16 * e + 4 * i + 1]),
+                                __uint_as_float(r[16 * e + 4 * i + 2]), __uint_as_float(r[16 * e + 4 * i + 3]));
+#pragma unroll
+              for (int s = 0; s < NS; ++s)
+                if ((path[s] >> 4) == c + e) vec[s] = *reinterpret_cast<const float*>(srow + word(path[s] & 15));
+            }
+          }
+          if (part == 1) {
+#pragma unroll
+            for (int s = 0; s < NS; ++s) Gs[nd * kLd + s] = vec[s];
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(E1_SYNC));
+        // C_{i,p_s} = (q_i . k_{p_s}) P_i / P_{p_s}: the ratio is the product of alpha over the slots
+        // after s, built up from the node's own slot backwards; x L = e_d for the U problem
+        {
+          float sfx = 1.f;
+#pragma unroll
+          for (int s = NS - 1; s >= 0; --s) {
+            if (part == 0) vec[s] = s <= depth ? vec[s] * sfx : 0.f;
+            else vec[s] = s == depth ? 1.f : 0.f;
+            sfx *= al[s];
+          }
+        }
+        if (!(ok = mbar_wait_warp(bar(E1_SYNC), g & 1, abort_flag))) break;
+        if (solves) {
+          // w_s = c_s - sum_{t > s} w_t G_{p_t,p_s},  G_{p_t,p_s} = beta_t (P_{p_t} / P_{p_s}) k_t.k_s;
+          // rr[t] holds P_{p_t} / P_{p_s} = alpha_{s+1} ... alpha_t for the current s and grows by one
+          // factor per step.  Slots past the node's depth carry vec = 0 and a deselected G, so nothing
+          // is predicated.
+          float rr[NS];
+#pragma unroll
+          for (int s = NS - 2; s >= 0; --s) {
+            float acc = vec[s];
+#pragma unroll
+            for (int t = s + 1; t < NS; ++t) {
+              rr[t] = t == s + 1 ? al[t] : rr[t] * al[s + 1];
+              const float gts = Gs[path[t] * kLd + s] * (bt[t] * rr[t]);
+              acc = fmaf(-vec[t], t <= depth ? gts : 0.f, acc);
+            }
+            if (s < depth) vec[s] = acc;
+          }
+          // ---- row of [W ; A] = (w or x) D_beta as bf16 hi and lo, into the columns of the scores ----
+#pragma unroll
+          for (int s = 0; s < NS; ++s) {
+            const float w = vec[s] * bt[s];
+            const uint32_t h = pack_rn(w, 0.f);
+            vec[s] = __uint_as_float(pack_rn(__uint_as_float(h << 16), w - __uint_as_float(h << 16)));   // hi | lo << 16, both exact roundings
+          }
+          const uint32_t lo_off = 32u * (b + 1);
+          const int n_all = 4 * (b + 1);
+#pragma unroll 1
+          for (int c = 0; c < n_all; ++c) {
+            uint32_t w[16];
+            if (c < nch) {
+#pragma unroll
+              for (uint32_t i = 0; i < 4; ++i) *reinterpret_cast<uint4*>(srow + (i << 4)) = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+              for (int s = 0; s < NS; ++s)
+                if (s <= depth && (path[s] >> 4) == c)
+                  *reinterpret_cast<uint32_t*>(srow + word(path[s] & 15)) = __float_as_uint(vec[s]);
+#pragma unroll
+              for (uint32_t i = 0; i < 4; ++i) {
+                const uint4 x = *reinterpret_cast<const uint4*>(srow + ((i ^ ssw) << 4));
+                w[4 * i] = x.x; w[4 * i + 1] = x.y; w[4 * i + 2] = x.z; w[4 * i + 3] = x.w;
+              }
+            } else {
+#pragma unroll
+              for (int i = 0; i < 16; ++i) w[i] = 0u;
+            }
+            uint32_t hi[8], lo[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              hi[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x5410);
+              lo[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x7632);
+            }
+            tmem_st8(col + 8u * c, hi);
+            tmem_st8(col + lo_off + 8u * c, lo);
+          }
+          tmem_wait_st();
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(COEF + (g & 1)));
+      }
+      if (ok && lane == 0) mbar_arrive(bar(META_FREE + buf));
+    }
+  } else {
+    // ===================== outputs =====================
+    const int quad = warp & 3, part = quad >> 1;
+    const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
+    unsigned char* stage = sm + M::kOffOut + (uint32_t)quad * 2048u;
+    const int64_t ostep = PACKED ? 128 : p.out.t;
+    grid_dependency_wait();   // O and U may still be read by a kernel in front
+    // the commit kernel behind this one may be scheduled as SMs drain (it orders itself)
+    if (warp == 12 && lane == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    bool ok = true;
+    for (uint32_t it = 0; ok && it < n_it; ++it) {
+      const uint32_t buf = it % M::kMeta;
+      if (!(ok = mbar_wait_warp(bar(META_FULL + buf), (it / M::kMeta) & 1, abort_flag))) break;
+      const int32_t* im = item_of(buf);
+      const int n = im[0];
+      float* out = (part == 0 ? p.O : p.U) + ((size_t)(uint32_t)im[1] | (size_t)(uint32_t)im[2] << 32);
+#pragma unroll 1
+      for (int b = 0; b < NB; ++b) {
+        const uint32_t g = it * NB + b;
+        if (!(ok = mbar_wait_warp(bar(ACC + (g & 1)), (g >> 1) & 1, abort_flag))) break;
+        tc_fence_after();
+        const int nd0 = kBlk * b + (quad & 1) * 32;   // first node of this warp
+        if (nd0 < n && (part == 0 || want_U)) {
+          // 32 rows x 32 columns at a time, 16 rows through the warp's 2 KiB: a store then covers whole
+          // 128-byte lines (eight lanes per row) where a lane with a row of its own touches 32 lines
+#pragma unroll 1
+          for (int c = 0; c < 4; ++c) {
+            uint32_t x[32];
+            tmem_ld32(tmem + lane_addr + kColX + (g & 1) * 128u + 32u * c, x);
+            tmem_wait_ld();
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              __syncwarp();
+              if ((lane >> 4) == h) {
+#pragma unroll
+                for (uint32_t i = 0; i < 8; ++i)
+                  *reinterpret_cast<uint4*>(stage + (lane & 15) * 128 + ((i ^ (uint32_t)(lane & 7)) << 4)) =
+                      make_uint4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+              }
+              __syncwarp();
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const int r = 4 * i + (lane >> 3);
+                const uint4 o4 = *reinterpret_cast<const uint4*>(stage + r * 128 + (((uint32_t)lane ^ (uint32_t)r) & 7u) * 16u);
+                const int nd = nd0 + 16 * h + r;
+                if (nd < n) *reinterpret_cast<uint4*>(out + (int64_t)nd * ostep + 32 * c + 4 * (lane & 7)) = o4;
+              }
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(X_FREE + (g & 1)));
+      }
+      if (ok && lane == 0) mbar_arrive(bar(META_FREE + buf));
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
+                 : "memory");
+  }
+  if (tid == 0 && *abort_flag && p.status) atomicExch(p.status, (int)TV_ERR_DEVICE_TIMEOUT);
+}
+
+template <int NB>
+inline bool supports(const VerifyArgs& a) {
+  return a.bf16 && a.dk == 128 && a.dv == 128 && a.rule == TV_GATED_DELTA && a.T > kBlk * (NB - 1) && a.T <= kBlk * NB &&
+         a.tree.max_depth_all < kSlots;
+}
+
+template <int NB>
+inline int launch(const VerifyArgs& a, int32_t* status, cudaStream_t stream) {
+  if (!supports<NB>(a)) return TV_ERR_UNSUPPORTED;
+  const bool packed = a.tree.offsets != nullptr;
+  const uint64_t items = (uint64_t)a.L * a.B * a.H;
+  const void* const ptrs[5] = {a.q, a.k, a.v, a.S_pre, nullptr};
+  // 4-D views: dense / strided layouts from the resolved strides, packed forests as planes
+  NodeView vq, vv;
+  if (!packed) {
+    const uint64_t lb = (uint64_t)a.L * a.B;
+    vq = NodeView{128, (uint64_t)a.T, (uint64_t)a.Hk, lb, a.lay.qk.b, a.lay.qk.h, a.lay.qk.t};
+    vv = NodeView{128, (uint64_t)a.T, (uint64_t)a.H, lb, a.lay.v.b, a.lay.v.h, a.lay.v.t};
+  } else {
+    const int64_t cap = a.tree.capacity;
+    vq = NodeView{128, (uint64_t)cap, (uint64_t)a.Hk, (uint64_t)a.L, (int64_t)a.Hk * cap * 128, cap * 128, 128};
+    vv = NodeView{128, (uint64_t)cap, (uint64_t)a.H, (uint64_t)a.L, (int64_t)a.H * cap * 128, cap * 128, 128};
+  }
+  const uint64_t key = view_key(vq) * 3 + view_key(vv) * 5 + items;
+  // q, k, v in boxes of 64 rows x 64 columns (rows past the tensor read as zero), S_pre in quarters of k
+  const MapSet* ms = cached_maps(ptrs, key, a.T, 9 | (a.Hk << 8), [&](CUtensorMap* m) {
+    return make_map4(&m[0], a.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, vq, 64, 64) &&
+           make_map4(&m[1], a.k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, vq, 64, 64) &&
+           make_map4(&m[2], a.v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, vv, 64, 64) &&
+           make_map(&m[3], a.S_pre, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, items, 128, 128, 32, 128);
+  });
+  if (!ms) return TV_ERR_CUDA;
+  constexpr uint32_t smem = Map<NB>::kSmemBytes;
+  static thread_local int configured_dev = -1;
+  int dev = 0;
+  TV_CUDA_TRY(cudaGetDevice(&dev));
+  if (configured_dev != dev) {
+    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_delta_kernel<NB, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_delta_kernel<NB, 15, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_delta_kernel<NB, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_delta_kernel<NB, 15, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    configured_dev = dev;
+  }
+  const int sm_count = tv_sm_count();
+  if (sm_count <= 0) return TV_ERR_CUDA;
+  Params p;
+  p.tree = a.tree;
+  p.n_items = (int32_t)items;
+  p.B = a.B; p.H = a.H; p.T = a.T; p.Hk = a.Hk;
+  p.alpha = a.alpha;
+  p.beta = a.beta;
+  p.status = status;
+  p.O = a.O;
+  p.U = a.U;
+  p.offsets = a.tree.offsets;
+  p.capacity = a.tree.capacity;
+  p.div = make_item_div(a.B, a.H, a.Hk);
+  p.gate = a.lay.gate;
+  p.out = a.lay.out;
+  p.node_first = (node_first_of(vq) ? 1 : 0) | (node_first_of(vv) ? 2 : 0);
+  // With a few items per CTA, as many CTAs as give every one the same number of items (512 items
+  // on 148 SMs: 128 CTAs of 4 rather than 148 of 3 or 4 -- the launch takes four item periods
+  // either way, and the CTAs that run share the memory system with fewer others).  With many items
+  // per CTA an idle SM costs more than the balance gains, so the rule stops at eight.
+  int grid = (int)(items < (uint64_t)sm_count ? items : (uint64_t)sm_count);
+  if (items > (uint64_t)sm_count) {
+    const uint64_t rounds = (items + sm_count - 1) / sm_count;
+    if (rounds <= 8) grid = (int)((items + rounds - 1) / rounds);
+  }
+  const bool shallow = a.tree.max_depth_all <= 8;
+  auto go = [&](auto kernel) {
+    return launch_dependent(kernel, grid, kThreads, smem, stream, ms->map[0], ms->map[1], ms->map[2], ms->map[3], p);
+  };
+  if (packed)
+    TV_CUDA_TRY(shallow ? go(verify_tc_delta_kernel<NB, 8, true>) : go(verify_tc_delta_kernel<NB, 15, true>));
+  else
+    TV_CUDA_TRY(shallow ? go(verify_tc_delta_kernel<NB, 8, false>) : go(verify_tc_delta_kernel<NB, 15, false>));
+  TV_CUDA_TRY(cudaGetLastError());
+  return TV_OK;
+}
+
+}  // namespace tvdelta
