@@ -86,19 +86,52 @@ __device__ __forceinline__ uint4 lds16(uint32_t addr) {
   return r;
 }
 
+// Two fp32 channels in one register pair.  The row loop is bound by instruction issue, and the packed
+// multiply and add of sm_100 do two channels with one instruction (same roundings as two scalar ones):
+// 20.5 -> 18.9 us on 16 requests of 64 nodes and 12288 bf16 channels.
+struct Pair {
+  uint64_t v;
+};
+__device__ __forceinline__ Pair pack(float a, float b) {
+  Pair r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack(Pair a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+  return r;
+}
+__device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c) {
+  Pair r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ Pair mul2(Pair a, Pair b) {
+  Pair r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ Pair add2(Pair a, Pair b) {
+  Pair r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+
 // The eight staged values of this lane for one tap row; a0 / a1 are the shared-memory byte
 // addresses of the lane's two channel groups in that row (bf16 reads both with one load).
-__device__ __forceinline__ void load8(const __nv_bfloat16*, uint32_t a0, uint32_t, float (&o)[8]) {
+__device__ __forceinline__ void load8(const __nv_bfloat16*, uint32_t a0, uint32_t, Pair (&o)[4]) {
   const uint4 t = lds16(a0);
-  o[0] = __uint_as_float(t.x << 16); o[1] = __uint_as_float(t.x & 0xffff0000u);
-  o[2] = __uint_as_float(t.y << 16); o[3] = __uint_as_float(t.y & 0xffff0000u);
-  o[4] = __uint_as_float(t.z << 16); o[5] = __uint_as_float(t.z & 0xffff0000u);
-  o[6] = __uint_as_float(t.w << 16); o[7] = __uint_as_float(t.w & 0xffff0000u);
+  const uint32_t w[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) o[e] = pack(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u));
 }
-__device__ __forceinline__ void load8(const float*, uint32_t a0, uint32_t a1, float (&o)[8]) {
+__device__ __forceinline__ void load8(const float*, uint32_t a0, uint32_t a1, Pair (&o)[4]) {
   const uint4 a = lds16(a0), b = lds16(a1);
-  o[0] = __uint_as_float(a.x); o[1] = __uint_as_float(a.y); o[2] = __uint_as_float(a.z); o[3] = __uint_as_float(a.w);
-  o[4] = __uint_as_float(b.x); o[5] = __uint_as_float(b.y); o[6] = __uint_as_float(b.z); o[7] = __uint_as_float(b.w);
+  o[0] = pack(__uint_as_float(a.x), __uint_as_float(a.y));
+  o[1] = pack(__uint_as_float(a.z), __uint_as_float(a.w));
+  o[2] = pack(__uint_as_float(b.x), __uint_as_float(b.y));
+  o[3] = pack(__uint_as_float(b.z), __uint_as_float(b.w));
 }
 __device__ __forceinline__ void store8(__nv_bfloat16* row, int g0, int, bool live0, bool, const float (&y)[8]) {
   uint32_t p[4];
@@ -123,13 +156,17 @@ __device__ __forceinline__ void store8(float* row, int g0, int g1, bool live0, b
                  : "memory");
 }
 
-// SiLU(z) = z / (1 + e^-z) in five instructions.  e^-z overflows to +inf for z < -88; its
-// reciprocal is then 0 and the product -0.
-__device__ __forceinline__ float silu(float z) {
-  float e, r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * -1.4426950408889634f));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
-  return z * r;
+// SiLU(z) = z / (1 + e^-z) of two channels in seven instructions.  e^-z overflows to +inf for z < -88;
+// its reciprocal is then 0 and the product -0.
+__device__ __forceinline__ Pair silu2(Pair z) {
+  const float2 x = unpack(mul2(z, pack(-1.4426950408889634f, -1.4426950408889634f)));
+  float e0, e1, r0, r1;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(x.x));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(x.y));
+  const float2 d = unpack(add2(pack(1.0f, 1.0f), pack(e0, e1)));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(d.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(d.y));
+  return mul2(z, pack(r0, r1));
 }
 __device__ __forceinline__ float rsqrt_fast(float x) {
   float r;
@@ -333,7 +370,7 @@ tree_conv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
 
   // Dead channel groups (past the slice's width) keep zero weights and read the row's first
   // bytes, so the row loop is straight-line code; only their store is predicated off.
-  float wreg[NJ][W][8], breg[NJ][8];
+  Pair wreg[NJ][W][4], breg[NJ][4];   // channels 2 e, 2 e + 1 of the lane's eight
   bool live0[NJ], live1[NJ];
   uint32_t off0[NJ], off1[NJ];
   int loaded_slice = -1;
@@ -365,13 +402,14 @@ tree_conv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         off0[j] = live0[j] ? (uint32_t)(g0 * sizeof(IO)) : 0u;
         off1[j] = live1[j] ? (uint32_t)(g1 * sizeof(IO)) : 0u;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const int c = e < 4 ? g0 + e : g1 + e - 4;
-          const bool live = e < 4 ? live0[j] : live1[j];
+        for (int e = 0; e < 4; ++e) {
+          const int c = e < 2 ? g0 + 2 * e : g1 + 2 * e - 4;   // even: both channels lie in one shifted group of 8
+          const bool live = e < 2 ? live0[j] : live1[j];
           const int shift = 2 * (c >> 3);
-          breg[j][e] = live && a.bias ? bf[c + shift] : 0.0f;
+          breg[j][e] = live && a.bias ? pack(bf[c + shift], bf[c + 1 + shift]) : pack(0.0f, 0.0f);
 #pragma unroll
-          for (int r = 0; r < W; ++r) wreg[j][r][e] = live ? wf[c * W + (W - 1 - r) + shift] : 0.0f;
+          for (int r = 0; r < W; ++r)
+            wreg[j][r][e] = live ? pack(wf[c * W + (W - 1 - r) + shift], wf[(c + 1) * W + (W - 1 - r) + shift]) : pack(0.0f, 0.0f);
         }
       }
     }
@@ -426,32 +464,39 @@ tree_conv_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
       uint32_t tap[W];
 #pragma unroll
       for (int r = 0; r < W; ++r) tap[r] = __shfl_sync(0xffffffffu, mytap[r], src_lane);
-      float y[NJ][8];
-      float ss = 0.0f;
+      Pair y[NJ][4];
+      Pair ss2 = pack(0.0f, 0.0f);
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
 #pragma unroll
         for (int r = 0; r < W; ++r) {
-          float in[8];
+          Pair in[4];
           load8((const IO*)nullptr, base0[j] + tap[r], base1[j] + tap[r], in);
 #pragma unroll
-          for (int e = 0; e < 8; ++e) y[j][e] = fmaf(wreg[j][r][e], in[e], r == 0 ? breg[j][e] : y[j][e]);
+          for (int e = 0; e < 4; ++e) y[j][e] = fma2(wreg[j][r][e], in[e], r == 0 ? breg[j][e] : y[j][e]);
         }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          y[j][e] = silu(y[j][e]);
-          ss = fmaf(y[j][e], y[j][e], ss);
+        for (int e = 0; e < 4; ++e) {
+          y[j][e] = silu2(y[j][e]);
+          ss2 = fma2(y[j][e], y[j][e], ss2);
         }
       }
+      const float2 sq = unpack(ss2);
+      float ss = sq.x + sq.y;
 #pragma unroll
       for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
       const float sc = norm ? rsqrt_fast(ss + eps) : 1.0f;
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
+        float o8[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) y[j][e] *= sc;
+        for (int e = 0; e < 4; ++e) {
+          const float2 s2 = unpack(mul2(y[j][e], pack(sc, sc)));
+          o8[2 * e] = s2.x;
+          o8[2 * e + 1] = s2.y;
+        }
         store8(out + (uint32_t)(i * d + 128 * j), Geo<IO>::g0(l16), Geo<IO>::g1(l16), row_live && live0[j],
-               row_live && live1[j], y[j]);
+               row_live && live1[j], o8);
       }
     }
     // this warp has read the slot
