@@ -305,19 +305,52 @@ def budget_select(parent, p_draft, budget, *, status=None, stream=None, out=None
     return out
 
 
+def _first_current_stream():
+    """Address of the current stream (0 where there is no GPU); settles how the later calls ask for it."""
+    global _current_stream
+    import torch
+    if not torch.cuda.is_available():
+        return 0
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
+    if raw is not None:
+        _current_stream = lambda: raw(device())
+    else:
+        _current_stream = lambda: torch.cuda.current_stream().cuda_stream
+    return _current_stream()
+
+
+_current_stream = _first_current_stream
+
+
 def _stream_ptr(stream):
     if stream is None:
-        import torch
-        if torch.cuda.is_available():
-            return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-        return ctypes.c_void_p(0)
+        return _current_stream()
     if hasattr(stream, "cuda_stream"):
-        return ctypes.c_void_p(stream.cuda_stream)
-    return ctypes.c_void_p(int(stream))
+        return stream.cuda_stream
+    return int(stream)
 
 
 def _ptr(t):
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# Arguments of calls that passed their checks, by everything that those look at: shapes, strides, types and
+# placement, never which tensor or address it is.  A serving loop repeats a few such forms.  Host time of a
+# round of upload, verify and commit, checked and marshalled from scratch / found here: 52 / 28 us, with
+# token-major tensors 55 / 24; a whole layer with its front end 88 / 44.
+_FORMS_KEPT = 256
+_forms = {}
+
+
+def _form(t):
+    return None if t is None else (t.shape, t.stride(), t.dtype, t.is_cuda)
+
+
+def _keep_form(key, args):
+    if len(_forms) >= _FORMS_KEPT:
+        _forms.clear()
+    _forms[key] = args
+    return args
 
 
 def _strides_of(t, tail, B):
@@ -395,22 +428,27 @@ def tree_verify(tree: Tree, S_pre, q, k, v, alpha, beta=None, *, rule=GATED, O=N
     Tensors are CUDA, contiguous, in the layout of ``tree_verify.h``.  Returns
     ``O`` or ``(O, U)``.
     """
-    import torch
-    _require(S_pre, "S_pre", torch.float32)
-    for t, n in ((alpha, "alpha"), (beta, "beta")):
-        _require(t, n, torch.float32, strided=True)
-    for t, n in ((q, "q"), (k, "k"), (v, "v")):
-        _require(t, n, k.dtype, strided=True)
-    if O is None:
-        O = torch.empty(*v.shape[:-1], v.shape[-1], device=v.device, dtype=torch.float32)
-    if U is None and want_U:
-        U = torch.empty_like(O)
-    _require(O, "O", torch.float32, strided=True)
-    _require(U, "U", torch.float32, strided=True)
-    d = _dims(S_pre, k, v, rule, impl, tree, q=q, gates=(alpha, beta), outs=(O, U))
-    _check(lib().tv_tree_verify(tree._h, ctypes.byref(d), _ptr(S_pre), _ptr(q), _ptr(k), _ptr(v),
-                                _ptr(alpha), _ptr(beta), _ptr(O), _ptr(U), _stream_ptr(stream)),
-           "tv_tree_verify")
+    if O is None or (U is None and want_U):
+        import torch
+        if O is None:
+            O = torch.empty(*v.shape[:-1], v.shape[-1], device=v.device, dtype=torch.float32)
+        if U is None and want_U:
+            U = torch.empty_like(O)
+    key = (tree_verify, tree.n, tree.capacity, type(rule), rule, type(impl), impl, _form(S_pre), _form(q), _form(k), _form(v),
+           _form(alpha), _form(beta), _form(O), _form(U))
+    d = _forms.get(key)
+    if d is None:
+        import torch
+        _require(S_pre, "S_pre", torch.float32)
+        for t, n in ((alpha, "alpha"), (beta, "beta")):
+            _require(t, n, torch.float32, strided=True)
+        for t, n in ((q, "q"), (k, "k"), (v, "v")):
+            _require(t, n, k.dtype, strided=True)
+        _require(O, "O", torch.float32, strided=True)
+        _require(U, "U", torch.float32, strided=True)
+        d = _keep_form(key, ctypes.byref(_dims(S_pre, k, v, rule, impl, tree, q=q, gates=(alpha, beta), outs=(O, U))))
+    _check(lib().tv_tree_verify(tree._h, d, _ptr(S_pre), _ptr(q), _ptr(k), _ptr(v), _ptr(alpha), _ptr(beta), _ptr(O),
+                                _ptr(U), _stream_ptr(stream)), "tv_tree_verify")
     return (O, U) if U is not None else O
 
 
@@ -421,19 +459,22 @@ def commit_path(tree: Tree, accepted, S_pre, k, v, alpha, beta=None, *, rule=GAT
     ``accepted`` is a CUDA int32 tensor [B].  ``S_new=None`` commits in place
     and returns ``S_pre``.
     """
-    import torch
-    _require(accepted, "accepted", torch.int32)
-    for t, n in ((S_pre, "S_pre"), (S_new, "S_new")):
-        _require(t, n, torch.float32)
-    for t, n in ((alpha, "alpha"), (beta, "beta"), (U, "U")):
-        _require(t, n, torch.float32, strided=True)
-    for t, n in ((k, "k"), (v, "v")):
-        _require(t, n, k.dtype, strided=True)
-    d = _dims(S_pre, k, v, rule, IMPL_AUTO, tree, gates=(alpha, beta), outs=(U,))
+    key = (commit_path, tree.n, tree.capacity, type(rule), rule, _form(accepted), _form(S_pre), _form(k), _form(v),
+           _form(alpha), _form(beta), _form(U), _form(S_new))
+    d = _forms.get(key)
+    if d is None:
+        import torch
+        _require(accepted, "accepted", torch.int32)
+        for t, n in ((S_pre, "S_pre"), (S_new, "S_new")):
+            _require(t, n, torch.float32)
+        for t, n in ((alpha, "alpha"), (beta, "beta"), (U, "U")):
+            _require(t, n, torch.float32, strided=True)
+        for t, n in ((k, "k"), (v, "v")):
+            _require(t, n, k.dtype, strided=True)
+        d = _keep_form(key, ctypes.byref(_dims(S_pre, k, v, rule, IMPL_AUTO, tree, gates=(alpha, beta), outs=(U,))))
     out = S_pre if S_new is None else S_new
-    _check(lib().tv_commit_path(tree._h, ctypes.byref(d), _ptr(accepted), _ptr(S_pre), _ptr(k),
-                                _ptr(v), _ptr(alpha), _ptr(beta), _ptr(U), _ptr(out),
-                                _stream_ptr(stream)), "tv_commit_path")
+    _check(lib().tv_commit_path(tree._h, d, _ptr(accepted), _ptr(S_pre), _ptr(k), _ptr(v), _ptr(alpha), _ptr(beta),
+                                _ptr(U), _ptr(out), _stream_ptr(stream)), "tv_commit_path")
     return out
 
 
@@ -483,22 +524,28 @@ def tree_verify_static(parent, S_pre, q, k, v, alpha, beta=None, *, rule=GATED, 
     ``status`` if wanted) are preallocated CUDA tensors.  Nothing is allocated here or in the
     library: the tree metadata lives in a fixed device array (at most 128 trees of 128 nodes).
     """
-    import torch
-    _require(parent, "parent", torch.int32)
-    _require(status, "status", torch.int32)
-    for t, n in ((S_pre, "S_pre"), (alpha, "alpha"), (beta, "beta"), (O, "O"), (U, "U")):
-        _require(t, n, torch.float32)
-    for t, n in ((q, "q"), (k, "k"), (v, "v")):
-        _require(t, n, k.dtype)
-    d = _dims(S_pre, k, v, rule, impl)
-    n_trees = parent.shape[0] if parent.dim() == 2 else 1
-    if parent.dim() not in (1, 2) or parent.shape[-1] != d.T:
-        raise ValueError("parent must be [T] or [n_trees, T] with T = the node count of q/k/v")
-    if n_trees not in (1, d.B):
-        raise ValueError("parent must hold one tree or one tree per request")
-    _check(lib().tv_tree_verify_static(_ptr(parent), n_trees, ctypes.byref(d), _ptr(S_pre), _ptr(q),
-                                       _ptr(k), _ptr(v), _ptr(alpha), _ptr(beta), _ptr(O), _ptr(U),
-                                       _ptr(status), _stream_ptr(stream)), "tv_tree_verify_static")
+    key = (tree_verify_static, type(rule), rule, type(impl), impl, _form(parent), _form(status), _form(S_pre), _form(q), _form(k),
+           _form(v), _form(alpha), _form(beta), _form(O), _form(U))
+    found = _forms.get(key)
+    if found is None:
+        import torch
+        _require(parent, "parent", torch.int32)
+        _require(status, "status", torch.int32)
+        for t, n in ((S_pre, "S_pre"), (alpha, "alpha"), (beta, "beta"), (O, "O"), (U, "U")):
+            _require(t, n, torch.float32)
+        for t, n in ((q, "q"), (k, "k"), (v, "v")):
+            _require(t, n, k.dtype)
+        d = _dims(S_pre, k, v, rule, impl)
+        n_trees = parent.shape[0] if parent.dim() == 2 else 1
+        if parent.dim() not in (1, 2) or parent.shape[-1] != d.T:
+            raise ValueError("parent must be [T] or [n_trees, T] with T = the node count of q/k/v")
+        if n_trees not in (1, d.B):
+            raise ValueError("parent must hold one tree or one tree per request")
+        found = _keep_form(key, (ctypes.byref(d), n_trees))
+    d, n_trees = found
+    _check(lib().tv_tree_verify_static(_ptr(parent), n_trees, d, _ptr(S_pre), _ptr(q), _ptr(k), _ptr(v), _ptr(alpha),
+                                       _ptr(beta), _ptr(O), _ptr(U), _ptr(status), _stream_ptr(stream)),
+           "tv_tree_verify_static")
     return O
 
 
@@ -525,20 +572,27 @@ def _conv_dims(x, H, dk, dv, W, normalize_qk, eps, tree=None, impl=IMPL_AUTO) ->
 
 def _conv_args(tree, x, ctx, weight, bias, H, dk, dv, gate_a, gate_b, A_log, dt_bias, normalize_qk, eps,
                q, k, v, alpha, beta, stream, impl=IMPL_AUTO):
-    import torch
-    for t, n in ((x, "x"), (ctx, "ctx"), (gate_a, "gate_a"), (gate_b, "gate_b"), (q, "q"), (k, "k"), (v, "v")):
-        _require(t, n, x.dtype)
-    for t, n in ((weight, "weight"), (bias, "bias"), (A_log, "A_log"), (dt_bias, "dt_bias"),
-                 (alpha, "alpha"), (beta, "beta")):
-        _require(t, n, torch.float32)
-    if weight.dim() != 2 or weight.shape[0] != x.shape[-1]:
-        raise ValueError("weight must be [C, W]")
-    W = weight.shape[1]
-    n_req = tree.n_trees if tree.capacity is not None else x.shape[0]
-    if W > 1 and (ctx is None or tuple(ctx.shape) != (n_req, W - 1, x.shape[-1])):
-        raise ValueError("ctx must be [B, W-1, C]")
-    d = _conv_dims(x, H, dk, dv, W, normalize_qk, eps, tree, impl)
-    args = (tree._h, ctypes.byref(d), _ptr(x), _ptr(ctx), _ptr(weight), _ptr(bias), _ptr(gate_a), _ptr(gate_b),
+    key = (_conv_args, tree.n, tree.n_trees, tree.capacity, type(H), H, type(dk), dk, type(dv), dv, type(impl), impl,
+           type(normalize_qk), normalize_qk, type(eps), eps, _form(x), _form(ctx), _form(weight), _form(bias),
+           _form(gate_a), _form(gate_b), _form(A_log), _form(dt_bias), _form(q), _form(k), _form(v), _form(alpha), _form(beta))
+    found = _forms.get(key)
+    if found is None:
+        import torch
+        for t, n in ((x, "x"), (ctx, "ctx"), (gate_a, "gate_a"), (gate_b, "gate_b"), (q, "q"), (k, "k"), (v, "v")):
+            _require(t, n, x.dtype)
+        for t, n in ((weight, "weight"), (bias, "bias"), (A_log, "A_log"), (dt_bias, "dt_bias"),
+                     (alpha, "alpha"), (beta, "beta")):
+            _require(t, n, torch.float32)
+        if weight.dim() != 2 or weight.shape[0] != x.shape[-1]:
+            raise ValueError("weight must be [C, W]")
+        W = weight.shape[1]
+        n_req = tree.n_trees if tree.capacity is not None else x.shape[0]
+        if W > 1 and (ctx is None or tuple(ctx.shape) != (n_req, W - 1, x.shape[-1])):
+            raise ValueError("ctx must be [B, W-1, C]")
+        d = _conv_dims(x, H, dk, dv, W, normalize_qk, eps, tree, impl)
+        found = _keep_form(key, (d, ctypes.byref(d)))
+    d, d_ref = found
+    args = (tree._h, d_ref, _ptr(x), _ptr(ctx), _ptr(weight), _ptr(bias), _ptr(gate_a), _ptr(gate_b),
             _ptr(A_log), _ptr(dt_bias), _ptr(q), _ptr(k), _ptr(v), _ptr(alpha), _ptr(beta), _stream_ptr(stream))
     keep = (tree, d, x, ctx, weight, bias, gate_a, gate_b, A_log, dt_bias, q, k, v, alpha, beta)
     return args, keep
@@ -552,15 +606,16 @@ def tree_conv(tree: Tree, x, ctx, weight, bias=None, *, H, dk, dv, gate_a=None, 
     ``x`` [B,T,C], ``ctx`` [B,W-1,C], ``weight`` f32 [C,W]; returns ``(q, k, v)`` head-major, and
     ``(q, k, v, alpha, beta)`` when ``gate_a`` is given (``beta`` None without ``gate_b``).
     """
-    import torch
-    lead = (H, tree.capacity) if tree.capacity is not None else (x.shape[0], H, x.shape[1])
-    q = torch.empty(*lead, dk, device=x.device, dtype=x.dtype) if q is None else q
-    k = torch.empty(*lead, dk, device=x.device, dtype=x.dtype) if k is None else k
-    v = torch.empty(*lead, dv, device=x.device, dtype=x.dtype) if v is None else v
-    if gate_a is not None and alpha is None:
-        alpha = torch.empty(*lead, device=x.device, dtype=torch.float32)
-    if gate_b is not None and beta is None:
-        beta = torch.empty(*lead, device=x.device, dtype=torch.float32)
+    if q is None or k is None or v is None or (gate_a is not None and alpha is None) or (gate_b is not None and beta is None):
+        import torch
+        lead = (H, tree.capacity) if tree.capacity is not None else (x.shape[0], H, x.shape[1])
+        q = torch.empty(*lead, dk, device=x.device, dtype=x.dtype) if q is None else q
+        k = torch.empty(*lead, dk, device=x.device, dtype=x.dtype) if k is None else k
+        v = torch.empty(*lead, dv, device=x.device, dtype=x.dtype) if v is None else v
+        if gate_a is not None and alpha is None:
+            alpha = torch.empty(*lead, device=x.device, dtype=torch.float32)
+        if gate_b is not None and beta is None:
+            beta = torch.empty(*lead, device=x.device, dtype=torch.float32)
     args, _keep = _conv_args(tree, x, ctx, weight, bias, H, dk, dv, gate_a, gate_b, A_log, dt_bias,
                              normalize_qk, eps, q, k, v, alpha, beta, stream, impl)
     _check(lib().tv_tree_conv(*args), "tv_tree_conv")
@@ -578,14 +633,18 @@ def prepare_tree_conv(tree: Tree, x, ctx, weight, bias=None, *, H, dk, dv, gate_
 
 def conv_commit(tree: Tree, accepted, x, ctx, *, H, dk, dv, ctx_new=None, stream=None):
     """``tv_conv_commit``: context rows after the accepted path (in place when ``ctx_new`` is None)."""
-    import torch
-    _require(accepted, "accepted", torch.int32)
-    for t, n in ((x, "x"), (ctx, "ctx"), (ctx_new, "ctx_new")):
-        _require(t, n, x.dtype)
+    key = (conv_commit, tree.n, tree.n_trees, tree.capacity, type(H), H, type(dk), dk, type(dv), dv, _form(accepted), _form(x),
+           _form(ctx), _form(ctx_new))
+    d = _forms.get(key)
+    if d is None:
+        import torch
+        _require(accepted, "accepted", torch.int32)
+        for t, n in ((x, "x"), (ctx, "ctx"), (ctx_new, "ctx_new")):
+            _require(t, n, x.dtype)
+        d = _keep_form(key, ctypes.byref(_conv_dims(x, H, dk, dv, ctx.shape[1] + 1, False, 0.0, tree)))
     out = ctx if ctx_new is None else ctx_new
-    d = _conv_dims(x, H, dk, dv, ctx.shape[1] + 1, False, 0.0, tree)
-    _check(lib().tv_conv_commit(tree._h, ctypes.byref(d), _ptr(accepted), _ptr(x), _ptr(ctx), _ptr(out),
-                                _stream_ptr(stream)), "tv_conv_commit")
+    _check(lib().tv_conv_commit(tree._h, d, _ptr(accepted), _ptr(x), _ptr(ctx), _ptr(out), _stream_ptr(stream)),
+           "tv_conv_commit")
     return out
 
 
