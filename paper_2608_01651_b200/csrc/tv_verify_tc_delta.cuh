@@ -14,26 +14,41 @@
 // factors are products of alpha over a stretch of the row's own path, never a quotient of two
 // numbers that may both underflow.
 //
-// Tile rows 0..63 carry the O problem of the block's nodes, rows 64..127 the U problem:
+// One half of a tile's 128 rows carries the O problem of the block's nodes (q rows), the other the U
+// problem (k rows):
 //     Sc  = [Q_b ; K_b] K^T                   scores, columns = all nodes up to the block's last
 //     X   = [Q_b ; K_b] [S_hi + S_lo]^T       q/k exact, state as two bf16 (16 mantissa bits and more)
-//     X rows 0..63  *= P_i,  V' = V - P_i X rows 64..127 -> bf16 hi + lo, then those rows = 0
-//     X  += [W ; A]_hi V'_hi + [W ; A]_lo V'_hi + [W ; A]_hi V'_lo     rows 0..63 = O, 64..127 = U
+//     q rows of X *= P_i,  V' = V - P_i (k rows of X) -> bf16 hi + lo, then those rows = 0
+//     X  += [W ; A]_hi V'_hi + [W ; A]_lo V'_hi + [W ; A]_hi V'_lo     q rows: O, k rows: U
+// Block 0 has the q rows in front, block 1 the k rows: in memory Q_0 K_0 K_1 Q_1, so that K_0 K_1 is one
+// operand of block 1's scores.
 //
 // What bounds it and how it is laid out.  At the copy rate an SM's share of the memory moves an item
 // of 64 nodes in 4.1 us and one of 128 in 6.6; the dependent chain of one item is two to three times
-// that.  So the chain is cut between four groups of four warps, each busy for less than that time and
+// that.  So the chain is cut between five groups of four warps, each busy for less than that time and
 // each working on a different item or block:
-//     warps 0..3    TMA producer | MMA issuer | metadata (paths, gates, P of the items to come) | -
-//     warps 4..7    state rows split in place into bf16 hi + lo, then V' and the scaling of X
+//     warps 0..3    TMA producer | MMAs of scores and readout | metadata (paths, gates, P of the items to
+//                   come) | MMAs of the state product
+//     warps 4..7    q and k rows into tensor memory, state rows split in place into bf16 hi + lo
 //     warps 8..11   thread = tile row: scores of its path, back-substitution, row of [W ; A]
 //     warps 12..15  finished rows of X to memory
+//     warps 16..19  V' and the scaling of X
 // and nothing of it is staged in a buffer that the next item needs: the coefficient rows are the A
 // operand in tensor memory, in the columns of the scores they came from; the state arrives in a ring
 // of four quarters of k (a quarter's fp32 rows of 128 bytes become [hi | lo] rows of the same bytes,
-// so one 128-wide tile feeds the hi and the lo product); outputs pass through 2 KiB per warp.
-// The thread that issues the MMAs takes whichever product is ready (outputs first), so that no item
-// waits for another one's operands.
+// so one 128-wide tile feeds the hi and the lo product); outputs pass through 2 or 4 KiB per warp.
+// The state product has an issuing thread of its own, so that no product waits for another one's operands; one
+// thread that polled for all three needed 150 ns per MMA.  Loops over columns stay rolled: all roles run at once
+// and share one instruction cache (unrolled, 512 items of 24 / 128 nodes took 22.2 / 43.1 us, rolled 20.6 / 41.2).
+//
+// Measured, back to back / in rounds of upload, verify and commit, before (one chain of phases over eight warps,
+// state as tf32, operand tiles and staged outputs sharing buffers) and now, us:
+//     items x nodes   512 x 24       512 x 64       2048 x 64       512 x 128      2048 x 128
+//     before          22.7 /  33.9   28.4 /  40.4   89.5 / 139.0    68.0 /  81.2   219 / 271
+//     now             20.6 /  31.8   23.9 /  36.3   78.5 / 133      41.2 /  55.4   133 / 198
+// Error against 64 bits 3e-4 before, 4.4e-6 now.  What is left: the four hops of an item (state product, V',
+// readout, stores) over two sets of columns, with shared memory half busy; without the stores 512 x 128 takes
+// 34 us, without V' 40, without the path systems 40.
 // Every wait is a bounded mbarrier wait (status word on expiry); every TMA load is a plain per-CTA copy.
 #pragma once
 #include "tv_tc_common.cuh"
@@ -42,30 +57,40 @@ namespace tvdelta {
 
 using namespace tvtc;
 
-constexpr int kThreads = 512;
+constexpr int kThreads = 640;
 constexpr int kSlots = 16;     // path slots per node: depth <= 15
 constexpr int kBlk = 64;       // nodes per row block
-constexpr int kLd = 17;        // row stride of the key-score table (floats): conflict-free per slot
+constexpr int kLd = 17;        // row stride of the table of G (floats): conflict-free per slot
 constexpr int kUnits = 4;      // quarters of k, ring slots of the state
 
 template <int NB>
 struct Map {
   static constexpr int kNodes = kBlk * NB;
-  static constexpr int kMeta = NB == 1 ? 4 : 2;      // metadata buffers (items ahead of the slowest group)
+  static constexpr int kMeta = NB == 1 ? 3 : 2;      // metadata buffers (items ahead of the slowest group)
   // bytes from the 1024-aligned base
-  static constexpr uint32_t kOffQK = 0;              // two blocks of [Q ; K]: 2 k halves of [128][64] bf16 (NB = 1: two items)
+  // NB = 1: two items, each 2 k halves of [Q ; K], [128][64] bf16.  NB = 2: 2 k halves of [Q_0 ; K_0 ; K_1 ; Q_1]
+  static constexpr uint32_t kOffQK = 0;
+  static constexpr uint32_t kBlkQK = NB == 1 ? 2 * kTile : kTile;    // from one block's operand to the next
+  static constexpr uint32_t kHalfQK = NB == 1 ? kTile : 2 * kTile;   // from one k half to the next
   static constexpr uint32_t kOffS = 4 * kTile;       // four units [128 v][32] fp32, after the split [128 v][32 hi | 32 lo] bf16
   static constexpr uint32_t kOffV = 8 * kTile;       // V, then V'_hi in its place, and V'_lo: dv halves of [nodes][64] (NB = 1: two items)
+  // [Q ; K] of the state product: from tensor memory where there is room for two items (columns kColA on; the
+  // next item's q and k then load while this one's product waits for its state), else from shared memory.  One
+  // set of columns, written block by block, was the slower way for NB = 2 (512 x 128: 45.5 against 45.0 us).
+  static constexpr bool kCopyA = NB == 1;
+  static constexpr uint32_t kColA = 384;
   static constexpr uint32_t kVHalf = kNodes * 128;   // one dv half
   static constexpr uint32_t kVItem = 4 * kVHalf;     // hi, lo
   static constexpr uint32_t kOffRow = 12 * kTile;    // 64 bytes per tile row, private to its thread (warps 8..11)
-  static constexpr uint32_t kOffOut = kOffRow + 8192;   // 2 KiB per warp (warps 12..15)
-  static constexpr uint32_t kOffGs = kOffOut + 8192;    // float Gs[kNodes][kLd]: K K^T on the path
+  static constexpr uint32_t kOffOut = kOffRow + 8192;   // staging of the outputs, per warp (warps 12..15)
+  static constexpr int kOutRows = NB == 1 ? 32 : 16;    // rows of 32 floats that an output warp stages at a time
+  static constexpr uint32_t kOffGs = kOffOut + 4 * kOutRows * 128;    // float Gs[kNodes][kLd]: rows of G, by path slot
   static constexpr uint32_t kOffPath = kOffGs + kNodes * kLd * 4;          // kMeta x uint8[kNodes][16], path in slot order
   static constexpr uint32_t kOffDepth = kOffPath + kMeta * kNodes * 16;    // kMeta x int8[kNodes], -1 = no node
-  static constexpr uint32_t kOffTab = kOffDepth + kMeta * kNodes;          // kMeta x {alpha, beta, P}[kNodes]
+  static constexpr uint32_t kOffTab = kOffDepth + kMeta * kNodes;          // kMeta x {{alpha, beta}[kNodes], P[kNodes]}
   static constexpr uint32_t kOffItem = kOffTab + kMeta * kNodes * 12;      // kMeta x {nodes, first output element (2 words), -}
-  static constexpr uint32_t kOffBar = kOffItem + kMeta * 16;
+  static constexpr uint32_t kOffLink = kOffItem + kMeta * 16;              // {alpha, parent}[kNodes], metadata warp only
+  static constexpr uint32_t kOffBar = kOffLink + kNodes * 8;
   static constexpr uint32_t kOffMisc = kOffBar + 8 * 48;
   static constexpr uint32_t kSmemBytes = kOffMisc + 32;
   static_assert(kOffBar % 8 == 0 && kSmemBytes <= 232448, "shared memory of one CTA");
@@ -75,13 +100,16 @@ struct Map {
 enum Bar {
   QK_FULL = 0, QK_FREE = 2, GD = 4, SC_FREE = 6, COEF = 8, VP = 10, ACC = 12, X_FREE = 14,
   V_FULL = 16, V_FREE = 18,          // [2]: NB = 1 as above, NB = 2 entry 0 per item
-  X_DONE = 20,                       // [2]: item & 1
+  X_DONE = 20,                       // [2]: as the first
   S_FULL = 22, S_SPLIT = 26, S_FREE = 30,   // [4]: unit, phase = item
   META_FULL = 34, META_FREE = 38,    // [kMeta]
-  E1_SYNC = 42, kNumBars = 43
+  E1_SYNC = 42,
+  A_READY = 43,                      // [2]: as the first
+  kNumBars = 45
 };
 static_assert(kNumBars <= 48, "barrier area");
 
+// TMEM columns: X of two blocks, scores (then coefficients), [Q ; K] as packed bf16 (NB = 1: of two items)
 constexpr uint32_t kColX = 0, kColSc = 256;
 
 struct Params {
@@ -102,11 +130,11 @@ struct Params {
   int32_t node_first;
 };
 
-__device__ __forceinline__ void mma_bf16_ts(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t idesc) {
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 1, 0;\n\t"
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d), "r"(a_tmem), "l"(b), "r"(idesc) : "memory");
+      ::"r"(d), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
 }
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
@@ -119,10 +147,28 @@ __device__ __forceinline__ uint32_t pack_rn(float lo_elem, float hi_elem) {
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi_elem), "f"(lo_elem));
   return r;
 }
+// Two fp32 in a register pair; a * b + c in both halves with one instruction.
+__device__ __forceinline__ uint64_t pair(float x0, float x1) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x0), "f"(x1));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ float2 halves(uint64_t a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+  return r;
+}
 // A pair of fp32 as bf16 hi (rounded to nearest) and lo (the exact remainder, rounded to nearest)
-__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hi, uint32_t& lo) {
-  hi = pack_rn(x0, x1);
-  lo = pack_rn(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u));
+__device__ __forceinline__ void split_pair(uint64_t x, uint32_t& hi, uint32_t& lo) {
+  const float2 v = halves(x);
+  hi = pack_rn(v.x, v.y);
+  const float2 r = halves(fma2(pair(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), pair(-1.f, -1.f), x));
+  lo = pack_rn(r.x, r.y);
 }
 
 // DMAX: compile-time bound on the tree depth (8 covers draft trees, 15 the rest), so that the
@@ -157,27 +203,20 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   const uint32_t n_it = (int)blockIdx.x < p.n_items
                             ? ((uint32_t)p.n_items - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u;
 
-  if (tid == 0) {
-    abort_flag[0] = 0;
-    abort_flag[1] = 0;
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(bar(QK_FULL + i), 1);  mbar_init(bar(QK_FREE + i), 1);
-      mbar_init(bar(GD + i), 1);       mbar_init(bar(SC_FREE + i), 1);
-      mbar_init(bar(COEF + i), 4);     mbar_init(bar(VP + i), 4);
-      mbar_init(bar(ACC + i), 1);      mbar_init(bar(X_FREE + i), 4);
-      mbar_init(bar(V_FULL + i), 1);   mbar_init(bar(V_FREE + i), 1);
-      mbar_init(bar(X_DONE + i), 1);
+  if (warp == 0) {
+    if (lane == 0) {
+      abort_flag[0] = 0;
+      abort_flag[1] = 0;
+      prefetch_map(&tmQ);
+      prefetch_map(&tmK);
+      prefetch_map(&tmS);
+      prefetch_map(&tmV);
     }
-    for (int i = 0; i < kUnits; ++i) {
-      mbar_init(bar(S_FULL + i), 1);
-      mbar_init(bar(S_SPLIT + i), 4);
-      mbar_init(bar(S_FREE + i), 1);
+    for (int i = lane; i < kNumBars; i += 32) {   // arrivals of a phase: one thread, unless it is four warps
+      const bool warps4 = (i >= COEF && i < ACC) || (i >= X_FREE && i < V_FULL) || (i >= S_SPLIT && i < S_FREE) || i >= E1_SYNC;
+      const bool qk = i >= QK_FREE && i < GD, meta = i >= META_FREE && i < E1_SYNC;
+      mbar_init(bar(i), qk ? (M::kCopyA ? 5 : 2) : meta ? 12 : warps4 ? 4 : 1);
     }
-    for (int i = 0; i < M::kMeta; ++i) {
-      mbar_init(bar(META_FULL + i), 1);
-      mbar_init(bar(META_FREE + i), 12);
-    }
-    mbar_init(bar(E1_SYNC), 4);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -190,57 +229,70 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  // registers: 128 per thread at launch; the solving warps take what the first four give up
+  // registers: 96 per thread at launch, moved to where the long rows are held
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
     if (warp == 0 && lane == 0) {
       // ===================== TMA producer =====================
       grid_dependency_wait();   // inputs may come from the kernel in front (dependent launch)
       uint32_t n_qk = 0, n_v = 0, n_s = 0;   // loads issued: blocks, items, units
-      for (uint32_t it = 0; it < n_it; ++it) {
-        const int item = (int)(blockIdx.x + it * gridDim.x);
-        // box coordinates: q/k head, v head, outermost index (layer*request, or the layer of a packed
-        // forest) and the first node row
-        const int lb = (int)fdiv((uint32_t)item, p.div.dH), h = item - lb * p.H;
-        const int hq = (int)fdiv((uint32_t)h, p.div.dG);
-        int z = lb, y0 = 0;
+      // Box coordinates: q/k head, v head, outermost index (layer*request, or the layer of a packed
+      // forest) and the first node row.
+      struct Coord {
+        int item, hq, h, z, y0;
+      };
+      auto coord_of = [&](uint32_t it) {
+        Coord c;
+        c.item = (int)(blockIdx.x + it * gridDim.x);
+        const int lb = (int)fdiv((uint32_t)c.item, p.div.dH);
+        c.h = c.item - lb * p.H;
+        c.hq = (int)fdiv((uint32_t)c.h, p.div.dG);
+        c.z = lb;
+        c.y0 = 0;
         if constexpr (PACKED) {
-          z = (int)fdiv((uint32_t)lb, p.div.dB);
-          y0 = __ldg(p.offsets + (lb - z * p.B));
+          c.z = (int)fdiv((uint32_t)lb, p.div.dB);
+          c.y0 = __ldg(p.offsets + (lb - c.z * p.B));
         }
-        auto load_v = [&]() -> bool {
-          const uint32_t vb = NB == 1 ? it & 1 : 0, vph = NB == 1 ? it >> 1 : it;
-          if (!mbar_wait(bar(V_FREE + vb), (vph & 1) ^ 1, abort_flag)) return false;
-          mbar_expect_tx(bar(V_FULL + vb), 2 * M::kVHalf);
-#pragma unroll 1
-          for (int i = 0; i < 2 * NB; ++i)   // dv half i & 1, row block i >> 1
-            load_box(sbase + M::kOffV + vb * M::kVItem + (uint32_t)(i & 1) * M::kVHalf + (uint32_t)(i >> 1) * 8192u, &tmV,
-                     bar(V_FULL + vb), p.node_first & 2, 64 * (i & 1), y0 + kBlk * (i >> 1), h, z);
-          ++n_v;
-          return true;
-        };
-        bool ok = true;
+        return c;
+      };
+      const bool nf_qk = p.node_first & 1, nf_v = p.node_first & 2;
+      auto load_qk = [&](uint32_t it, const Coord& co) -> bool {
         for (int b = 0; b < NB; ++b) {
           const uint32_t g = it * NB + b, gb = g & 1;
-          if (!(ok = mbar_wait(bar(QK_FREE + gb), ((g >> 1) & 1) ^ 1, abort_flag))) break;
+          if (!mbar_wait(bar(QK_FREE + gb), ((g >> 1) & 1) ^ 1, abort_flag)) return false;
           mbar_expect_tx(bar(QK_FULL + gb), 4 * 8192);
 #pragma unroll 1
           for (int i = 0; i < 4; ++i)   // k half i >> 1; Q rows, then K rows
-            load_box(sbase + M::kOffQK + gb * 2 * kTile + (uint32_t)(i >> 1) * kTile + (uint32_t)(i & 1) * 8192u,
-                     (i & 1) ? &tmK : &tmQ, bar(QK_FULL + gb), p.node_first & 1, 64 * (i >> 1), y0 + kBlk * b, hq, z);
+            load_box(sbase + M::kOffQK + gb * M::kBlkQK + (uint32_t)(i >> 1) * M::kHalfQK + (uint32_t)((i & 1) ^ b) * 8192u,
+                     (i & 1) ? &tmK : &tmQ, bar(QK_FULL + gb), nf_qk, 64 * (i >> 1), co.y0 + kBlk * b, co.hq, co.z);
           ++n_qk;
         }
-        if (!ok) break;
-        // NB = 1 has a second buffer for V, free long before the state's; NB = 2 has one, free last
-        if (NB == 1 && it > 0 && !load_v()) break;
-        for (int u = 0; ok && u < kUnits; ++u) {
-          if (!(ok = mbar_wait(bar(S_FREE + u), (it & 1) ^ 1, abort_flag))) break;
+        return true;
+      };
+      auto load_v = [&](uint32_t it, const Coord& co) -> bool {
+        const uint32_t vb = NB == 1 ? it & 1 : 0, vph = NB == 1 ? it >> 1 : it;
+        if (!mbar_wait(bar(V_FREE + vb), (vph & 1) ^ 1, abort_flag)) return false;
+        mbar_expect_tx(bar(V_FULL + vb), 2 * M::kVHalf);
+#pragma unroll 1
+        for (int i = 0; i < 2 * NB; ++i)   // dv half i & 1, row block i >> 1
+          load_box(sbase + M::kOffV + vb * M::kVItem + (uint32_t)(i & 1) * M::kVHalf + (uint32_t)(i >> 1) * 8192u, &tmV,
+                   bar(V_FULL + vb), nf_v, 64 * (i & 1), co.y0 + kBlk * (i >> 1), co.h, co.z);
+        ++n_v;
+        return true;
+      };
+      auto load_s = [&](uint32_t it, const Coord& co) -> bool {
+#pragma unroll 1
+        for (int u = 0; u < kUnits; ++u) {
+          if (!mbar_wait(bar(S_FREE + u), (it & 1) ^ 1, abort_flag)) return false;
           mbar_expect_tx(bar(S_FULL + u), kTile);
-          tma_load_3d(sbase + M::kOffS + (uint32_t)u * kTile, &tmS, bar(S_FULL + u), 32 * u, 0, item);
+          tma_load_3d(sbase + M::kOffS + (uint32_t)u * kTile, &tmS, bar(S_FULL + u), 32 * u, 0, co.item);
           ++n_s;
         }
-        if (!ok) break;
-        if ((NB == 2 || it == 0) && !load_v()) break;
+        return true;
+      };
+      for (uint32_t it = 0; it < n_it; ++it) {
+        const Coord co = coord_of(it);
+        if (!load_qk(it, co) || !load_s(it, co) || !load_v(it, co)) break;   // in the order in which they come free
       }
       if (*abort_flag) {
         // Leave no copy of ours in flight: wait (bounded) for the last load issued into each buffer.
@@ -251,31 +303,33 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           mbar_wait(bar(S_FULL + (i & 3)), (i >> 2) & 1, abort_flag + 1);
       }
     } else if (warp == 1 && lane == 0) {
-      // ===================== MMA issuer =====================
-      constexpr uint32_t kIdGram = idesc_bf16(64, false), kIdX = idesc_bf16(128, false), kIdAV = idesc_bf16(128, true);
-      const uint32_t n_g = n_it * NB, n_u = n_it * kUnits;
-      uint32_t ig = 0, iu = 0, ia = 0;   // next block's scores, next unit of the state product, next block's readout
-      const uint64_t dQK = desc_kmajor(sbase + M::kOffQK), dS = desc_kmajor(sbase + M::kOffS);
+      // ===================== MMAs: scores, readout =====================
+      constexpr uint32_t kIdGram = idesc_bf16(64, false), kIdGram2 = idesc_bf16(128, false), kIdAV = idesc_bf16(128, true);
+      const uint32_t n_g = n_it * NB;
+      uint32_t ig = 0, ia = 0;   // next block's scores, next block's readout
+      const uint64_t dQK = desc_kmajor(sbase + M::kOffQK);
       const uint64_t dV = desc_mnmajor(sbase + M::kOffV, M::kVHalf);
       long long t_idle = clock64();
       uint32_t spin = 0;
       while (ia < n_g) {
         bool progress = false;
         // X += [W ; A] V' of block ia
-        if (mbar_test(bar(COEF + (ia & 1)), (ia >> 1) & 1) && mbar_test(bar(VP + (ia & 1)), (ia >> 1) & 1)) {
+        if (mbar_test(bar(VP + (ia & 1)), (ia >> 1) & 1) && mbar_test(bar(COEF + (ia & 1)), (ia >> 1) & 1)) {
           tc_fence_after();
           const uint32_t b = NB == 1 ? 0u : ia & 1;
           const uint32_t acc = tmem + kColX + (ia & 1) * 128u, chi = tmem + sc_col((int)ia), clo = chi + 32u * (b + 1);
           const uint64_t dvi = dV + (NB == 1 ? ((ia & 1) * M::kVItem) >> 4 : 0u);
+          const int n = item_of((ia / NB) % M::kMeta)[0];   // the block's last steps may hold no node
 #pragma unroll 1
           for (uint32_t hb = 0; hb <= b; ++hb)   // 64 ancestors
 #pragma unroll
             for (uint32_t s = 0; s < 4; ++s) {   // 16 ancestors per step
+              if ((int)(64u * hb + 16u * s) >= n) break;
               const uint64_t hi = dvi + ((hb * 8192u + s * 2048u) >> 4), lo = hi + ((2 * M::kVHalf) >> 4);
               const uint32_t c = hb * 32u + s * 8u;
-              mma_bf16_ts(acc, chi + c, hi, kIdAV);
-              mma_bf16_ts(acc, clo + c, hi, kIdAV);
-              mma_bf16_ts(acc, chi + c, lo, kIdAV);
+              mma_bf16_ts(acc, chi + c, hi, kIdAV, 1);
+              mma_bf16_ts(acc, clo + c, hi, kIdAV, 1);
+              mma_bf16_ts(acc, chi + c, lo, kIdAV, 1);
             }
           tc_commit(bar(ACC + (ia & 1)));
           tc_commit(bar(SC_FREE + (ia & 1)));
@@ -289,68 +343,77 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
             mbar_test(bar(SC_FREE + (ig & 1)), ((ig >> 1) & 1) ^ 1)) {
           tc_fence_after();
           const uint32_t b = NB == 1 ? 0u : ig & 1;
-          const uint64_t dA = dQK + (((ig & 1) * 2 * kTile) >> 4);
-#pragma unroll 1
-          for (uint32_t hb = 0; hb <= b; ++hb) {   // K rows of block hb (NB = 1: of the block itself)
-            const uint64_t dB = (NB == 1 ? dA : dQK + ((hb * 2 * kTile) >> 4)) + (8192 >> 4);
+          const uint64_t dA = dQK + (((ig & 1) * M::kBlkQK) >> 4), dB = dQK + ((NB == 1 ? (ig & 1) * M::kBlkQK + 8192u : 8192u) >> 4);
 #pragma unroll
-            for (uint32_t i = 0; i < 8; ++i) {     // k half i >> 2, 32 bytes of k per step
-              const uint32_t off = ((i >> 2) * kTile + (i & 3u) * 32u) >> 4;
-              mma_bf16_ss(tmem + sc_col((int)ig) + 64u * hb, dA + off, dB + off, kIdGram, i);
-            }
+          for (uint32_t i = 0; i < 8; ++i) {   // k half i >> 2, 32 bytes of k per step
+            const uint32_t off = ((i >> 2) * M::kHalfQK + (i & 3u) * 32u) >> 4;
+            mma_bf16_ss(tmem + sc_col((int)ig), dA + off, dB + off, b ? kIdGram2 : kIdGram, i);
           }
           tc_commit(bar(GD + (ig & 1)));
+          if (NB == 1) {
+            tc_commit(bar(QK_FREE + (ig & 1)));
+          } else if (b == 1) {   // block 1's scores read both blocks' keys
+            tc_commit(bar(QK_FREE));
+            tc_commit(bar(QK_FREE + 1));
+          }
           ++ig;
           progress = true;
-        }
-        // X = [Q ; K] S_pre^T, one quarter of k for all blocks of the item
-        if (iu < n_u) {
-          const uint32_t it = iu / kUnits, u = iu % kUnits, g0 = it * NB;
-          bool ready = ig >= g0 + NB && mbar_test(bar(S_SPLIT + u), it & 1);
-          if (ready && u == 0)
-            for (uint32_t b = 0; b < NB; ++b)   // the block that had these columns before has been read out
-              ready = ready && mbar_test(bar(X_FREE + ((g0 + b) & 1)), (((g0 + b) >> 1) & 1) ^ 1);
-          if (ready) {
-            tc_fence_after();
-            const uint64_t dB = dS + ((u * kTile) >> 4);
-#pragma unroll
-            for (uint32_t b = 0; b < NB; ++b) {
-              const uint32_t gb = (g0 + b) & 1;
-              const uint64_t dA = dQK + ((gb * 2 * kTile + (u >> 1) * kTile + (u & 1) * 64u) >> 4);
-#pragma unroll
-              for (uint32_t i = 0; i < 4; ++i)   // hi: k 0..15, 16..31 of the quarter; lo: the same
-                mma_bf16_ss(tmem + kColX + gb * 128u, dA + (((i & 1u) * 32u) >> 4), dB + ((i * 32u) >> 4), kIdX, u | i);
-            }
-            tc_commit(bar(S_FREE + u));
-            if (u == kUnits - 1) {
-              tc_commit(bar(X_DONE + (it & 1)));
-              for (uint32_t b = 0; b < NB; ++b) tc_commit(bar(QK_FREE + ((g0 + b) & 1)));
-            }
-            ++iu;
-            progress = true;
-          }
         }
         if (progress) {
           t_idle = clock64();
           spin = 0;
-        } else if ((++spin & 255u) == 0) {   // the same limit as every other wait of the kernel
-          if (*abort_flag) break;
-          if (clock64() - t_idle > kWaitLimitCycles) {
-            *abort_flag = 1;
-            break;
+        } else {
+          __nanosleep(20);   // four working warps share this one's issue slots
+          if ((++spin & 255u) == 0) {   // the same limit as every other wait of the kernel
+            if (*abort_flag) break;
+            if (clock64() - t_idle > kWaitLimitCycles) {
+              *abort_flag = 1;
+              break;
+            }
           }
         }
+      }
+    } else if (warp == 3 && lane == 0) {
+      // ===================== MMAs: state product =====================
+      constexpr uint32_t kIdX = idesc_bf16(128, false);
+      const uint64_t dQK = desc_kmajor(sbase + M::kOffQK), dS = desc_kmajor(sbase + M::kOffS);
+      bool ok = true;
+      for (uint32_t g = 0; ok && g < n_it * NB; ++g) {
+        const uint32_t it = g / NB, gb = g & 1, ph = (g >> 1) & 1, x = tmem + kColX + gb * 128u;
+        if (!(ok = mbar_wait(bar(M::kCopyA ? A_READY + gb : QK_FULL + gb), ph, abort_flag))) break;
+        if (!(ok = mbar_wait(bar(X_FREE + gb), ph ^ 1, abort_flag))) break;   // what these columns held has been read out
+#pragma unroll 1
+        for (uint32_t u = 0; u < kUnits; ++u) {   // a quarter of k
+          if (!(ok = mbar_wait(bar(S_SPLIT + u), it & 1, abort_flag))) break;
+          tc_fence_after();
+          const uint64_t dB = dS + ((u * kTile) >> 4);
+          const uint64_t dA = dQK + ((gb * M::kBlkQK + (u >> 1) * M::kHalfQK + (u & 1) * 64u) >> 4);
+          const uint32_t aq = tmem + M::kColA + gb * 64u + u * 16u;
+#pragma unroll
+          for (uint32_t i = 0; i < 4; ++i) {   // hi: k 0..15, 16..31 of the quarter; lo: the same
+            if (M::kCopyA) mma_bf16_ts(x, aq + (i & 1u) * 8u, dB + ((i * 32u) >> 4), kIdX, u | i);
+            else mma_bf16_ss(x, dA + (((i & 1u) * 32u) >> 4), dB + ((i * 32u) >> 4), kIdX, u | i);
+          }
+          if (NB == 1 || gb == 1) tc_commit(bar(S_FREE + u));
+        }
+        if (!ok) break;
+        tc_commit(bar(X_DONE + gb));
+        if (!M::kCopyA) tc_commit(bar(QK_FREE + gb));
       }
     } else if (warp == 2) {
       // ===================== metadata =====================
       grid_dependency_wait();   // tree metadata and gates may come from the kernels in front
-      for (uint32_t it = 0; it < n_it; ++it) {
+      // A lane has the nodes lane, lane + 32, ...; the next item's values are on their way while this
+      // one's tables are written.
+      constexpr int NN = 2 * NB;
+      int n = 0, dep[NN], par[NN];
+      float al[NN], be[NN];
+      size_t o0 = 0;               // element offset of the item's first output row
+      auto fetch = [&](uint32_t it) {
         const int item = (int)(blockIdx.x + it * gridDim.x);
-        const uint32_t buf = it % M::kMeta, use = it / M::kMeta;
-        if (!mbar_wait_warp(bar(META_FREE + buf), (use & 1) ^ 1, abort_flag)) break;
-        int n = T, tb = 0;
-        int64_t g0, gstep = 1;   // first gate of the item, step between nodes
-        size_t o0;               // element offset of the item's first output row
+        n = T;
+        int tb = 0;
+        int64_t g0, gstep = 1;     // first gate of the item, step between nodes
         if constexpr (PACKED) {
           const PackedItem pi = packed_item(p.offsets, p.B, p.H, p.Hk, item, p.div);
           n = pi.n;
@@ -364,56 +427,42 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           gstep = p.gate.t;
           o0 = (size_t)((int64_t)lb * p.out.b + (int64_t)h * p.out.h);
         }
-        // all loads first: one trip to memory, not one per table
-        ulonglong2 mk[2 * NB];
-        float al[2 * NB], be[2 * NB];
 #pragma unroll
-        for (int h = 0; h < 2 * NB; ++h) {
+        for (int h = 0; h < NN; ++h) {
           const int nd = lane + 32 * h;
-          mk[h] = make_ulonglong2(0ull, 0ull);
+          dep[h] = -1;
+          par[h] = -1;
           al[h] = 1.f;
           be[h] = 0.f;
           if (nd < n) {
-            mk[h] = __ldg(reinterpret_cast<const ulonglong2*>(p.tree.anc) + (size_t)tb * T + nd);
+            dep[h] = __ldg(p.tree.depth + (size_t)tb * T + nd);
+            par[h] = __ldg(p.tree.parent + (size_t)tb * T + nd);
             al[h] = __ldg(p.alpha + g0 + nd * gstep);
             be[h] = __ldg(p.beta + g0 + nd * gstep);
           }
         }
+      };
+      float2* link = reinterpret_cast<float2*>(sm + M::kOffLink);
+      if (n_it > 0) fetch(0);
+      for (uint32_t it = 0; it < n_it; ++it) {
+        const uint32_t buf = it % M::kMeta, use = it / M::kMeta;
+        if (!mbar_wait_warp(bar(META_FREE + buf), (use & 1) ^ 1, abort_flag)) break;
         float* tab = tab_of(buf);
         uint8_t* paths = sm + M::kOffPath + (buf * kNodes) * 16;
         int8_t* depths = reinterpret_cast<int8_t*>(sm + M::kOffDepth) + buf * kNodes;
+        int slot[NN], j[NN];
+        float P[NN];
 #pragma unroll
-        for (int h = 0; h < 2 * NB; ++h) {
-          tab[lane + 32 * h] = al[h];
-          tab[kNodes + lane + 32 * h] = be[h];
-        }
-        __syncwarp();
-#pragma unroll 1
-        for (int h = 0; h < 2 * NB; ++h) {
+        for (int h = 0; h < NN; ++h) {
           const int nd = lane + 32 * h;
-          // the node's path in slot order: the set bits of (ancestors | self) from the lowest up
-          // (nodes are numbered parent before child); slots past the node's depth name the node itself
-          uint64_t r0 = h == 0 ? mk[0].x : h == 1 ? mk[1].x : NB == 2 ? (h == 2 ? mk[2 * NB - 2].x : mk[2 * NB - 1].x) : 0ull;
-          uint64_t r1 = h == 0 ? mk[0].y : h == 1 ? mk[1].y : NB == 2 ? (h == 2 ? mk[2 * NB - 2].y : mk[2 * NB - 1].y) : 0ull;
-          const int d = __popcll(r0) + __popcll(r1);
-          float P = 1.f;
-          uint32_t w[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-          for (int s = 0; s < kSlots; ++s) {
-            int j = nd;
-            if (r0 != 0ull) {
-              j = __ffsll((long long)r0) - 1;
-              r0 &= r0 - 1;
-            } else if (NB == 2 && r1 != 0ull) {
-              j = 64 + __ffsll((long long)r1) - 1;
-              r1 &= r1 - 1;
-            }
-            w[s >> 2] |= (uint32_t)j << (8 * (s & 3));
-            if (s <= DMAX && s <= d) P *= tab[j];
-          }
-          *reinterpret_cast<uint4*>(paths + nd * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-          depths[nd] = nd < n ? (int8_t)d : (int8_t)-1;
-          tab[2 * kNodes + nd] = P;
+          reinterpret_cast<float2*>(tab)[nd] = make_float2(al[h], be[h]);
+          link[nd] = make_float2(al[h], __int_as_float(par[h]));
+          depths[nd] = (int8_t)dep[h];
+          const uint32_t self = (uint32_t)nd * 0x01010101u;   // slots past the node's depth name the node itself
+          *reinterpret_cast<uint4*>(paths + nd * 16) = make_uint4(self, self, self, self);
+          slot[h] = dep[h];
+          j[h] = nd;
+          P[h] = 1.f;
         }
         if (lane == 0) {
           int32_t* im = item_of(buf);
@@ -422,17 +471,64 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           im[2] = (int32_t)(o0 >> 32);
         }
         __syncwarp();
+        if (it + 1 < n_it) fetch(it + 1);
+        // from every node up: the path in slot order, and P
+#pragma unroll 1
+        for (int e = 0; e <= DMAX; ++e) {
+          bool more = false;
+#pragma unroll
+          for (int h = 0; h < NN; ++h) {
+            if (slot[h] >= 0 && j[h] >= 0) {
+              paths[(lane + 32 * h) * 16 + slot[h]] = (uint8_t)j[h];
+              const float2 y = link[j[h]];
+              P[h] *= y.x;
+              j[h] = __float_as_int(y.y);
+              --slot[h];
+              more = more || slot[h] >= 0;
+            }
+          }
+          if (!__any_sync(0xffffffffu, more)) break;
+        }
+#pragma unroll
+        for (int h = 0; h < NN; ++h) tab[2 * kNodes + lane + 32 * h] = P[h];
+        __syncwarp();
         if (lane == 0) mbar_arrive(bar(META_FULL + buf));
       }
     }
   } else if (warp < 8) {
-    // ===================== state split, V', scaling of X =====================
-    const int quad = warp & 3, row = quad * 32 + lane;   // state row; TMEM lane
-    const int rn = row & 63;                             // node of this tile row within its block
-    const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
+    // ===================== [Q ; K] into tensor memory, state split =====================
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    const int row = (warp & 3) * 32 + lane;
+    const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t swz = (uint32_t)(row & 7);
     bool ok = true;
+    auto copy_qk = [&](uint32_t g) -> bool {
+      const uint32_t gb = g & 1;
+      if (g >= 2 && !mbar_wait_warp(bar(X_DONE + gb), ((g - 2) >> 1) & 1, abort_flag)) return false;   // they were read
+      if (!mbar_wait_warp(bar(QK_FULL + gb), (g >> 1) & 1, abort_flag)) return false;
+      tc_fence_after();
+#pragma unroll 1
+      for (uint32_t h = 0; h < 2; ++h) {   // k half
+        const unsigned char* r = sm + M::kOffQK + gb * M::kBlkQK + h * M::kHalfQK + (uint32_t)row * 128u;
+        uint32_t w[32];
+#pragma unroll
+        for (uint32_t c = 0; c < 8; ++c) {
+          const uint4 x = *reinterpret_cast<const uint4*>(r + ((c ^ swz) << 4));
+          w[4 * c] = x.x; w[4 * c + 1] = x.y; w[4 * c + 2] = x.z; w[4 * c + 3] = x.w;
+        }
+        tmem_st32(tmem + lane_addr + M::kColA + gb * 64u + h * 32u, w);
+      }
+      tmem_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(bar(A_READY + gb));
+        mbar_arrive(bar(QK_FREE + gb));
+      }
+      return true;
+    };
     for (uint32_t it = 0; ok && it < n_it; ++it) {
+      if (M::kCopyA && !(ok = copy_qk(it))) break;
 #pragma unroll 1
       for (int u = 0; u < kUnits; ++u) {
         if (!(ok = mbar_wait_warp(bar(S_FULL + u), it & 1, abort_flag))) break;
@@ -441,12 +537,12 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         uint4 hi[4], lo[4];
 #pragma unroll
         for (uint32_t c = 0; c < 4; ++c) {
-          const float4 a = *reinterpret_cast<const float4*>(r + (((2 * c) ^ swz) << 4));
-          const float4 e = *reinterpret_cast<const float4*>(r + (((2 * c + 1) ^ swz) << 4));
-          split_pair(a.x, a.y, hi[c].x, lo[c].x);
-          split_pair(a.z, a.w, hi[c].y, lo[c].y);
-          split_pair(e.x, e.y, hi[c].z, lo[c].z);
-          split_pair(e.z, e.w, hi[c].w, lo[c].w);
+          const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(r + (((2 * c) ^ swz) << 4));
+          const ulonglong2 e = *reinterpret_cast<const ulonglong2*>(r + (((2 * c + 1) ^ swz) << 4));
+          split_pair(a.x, hi[c].x, lo[c].x);
+          split_pair(a.y, hi[c].y, lo[c].y);
+          split_pair(e.x, hi[c].z, lo[c].z);
+          split_pair(e.y, hi[c].w, lo[c].w);
         }
 #pragma unroll
         for (uint32_t c = 0; c < 4; ++c) {
@@ -457,80 +553,13 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(S_SPLIT + u));
       }
-      if (!ok) break;
-      const uint32_t buf = it % M::kMeta, vb = NB == 1 ? it & 1 : 0;
-      if (!(ok = mbar_wait_warp(bar(META_FULL + buf), (it / M::kMeta) & 1, abort_flag))) break;
-      if (!(ok = mbar_wait_warp(bar(V_FULL + vb), (NB == 1 ? it >> 1 : it) & 1, abort_flag))) break;
-      if (!(ok = mbar_wait_warp(bar(X_DONE + (it & 1)), (it >> 1) & 1, abort_flag))) break;
-      tc_fence_after();
-      const int n = item_of(buf)[0];
-#pragma unroll 1
-      for (int b = 0; b < NB; ++b) {
-        const uint32_t g = it * NB + b;
-        const int nd = kBlk * b + rn;
-        const float P = tab_of(buf)[2 * kNodes + nd];
-        const uint32_t xcol = tmem + lane_addr + kColX + (g & 1) * 128u;
-        if (quad < 2) {
-          // O problem: the prefix term P_i q_i S_pre^T is where the accumulation starts
-          if (kBlk * b + quad * 32 < n) {
-#pragma unroll 1
-            for (int c = 0; c < 4; ++c) {
-              uint32_t x[32];
-              tmem_ld32(xcol + 32u * c, x);
-              tmem_wait_ld();
-#pragma unroll
-              for (int i = 0; i < 32; ++i) x[i] = __float_as_uint(P * __uint_as_float(x[i]));
-              tmem_st32(xcol + 32u * c, x);
-            }
-          }
-        } else {
-          const bool alive = nd < n;
-#pragma unroll 1
-          for (int c = 0; c < 4; ++c) {   // 32 columns: half of dv half c >> 1
-            uint32_t x[32];
-            tmem_ld32(xcol + 32u * c, x);
-            unsigned char* vrow = sm + M::kOffV + vb * M::kVItem + (uint32_t)(c >> 1) * M::kVHalf + (uint32_t)nd * 128u;
-            uint4 v[4];
-#pragma unroll
-            for (uint32_t i = 0; i < 4; ++i)
-              v[i] = *reinterpret_cast<const uint4*>(vrow + ((((uint32_t)(c & 1) * 4 + i) ^ swz) << 4));
-            tmem_wait_ld();
-#pragma unroll
-            for (uint32_t i = 0; i < 4; ++i) {
-              const uint32_t vw[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
-              uint32_t hi[4], lo[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const float a0 = fmaf(-P, __uint_as_float(x[8 * i + 2 * e]), __uint_as_float(vw[e] << 16));
-                const float a1 = fmaf(-P, __uint_as_float(x[8 * i + 2 * e + 1]), __uint_as_float(vw[e] & 0xffff0000u));
-                split_pair(a0, a1, hi[e], lo[e]);
-                hi[e] = alive ? hi[e] : 0u;   // select, never 0 * x: rows past the request may hold anything
-                lo[e] = alive ? lo[e] : 0u;
-              }
-              const uint32_t off = (((uint32_t)(c & 1) * 4 + i) ^ swz) << 4;
-              *reinterpret_cast<uint4*>(vrow + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-              *reinterpret_cast<uint4*>(vrow + 2 * M::kVHalf + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-            }
-#pragma unroll
-            for (int i = 0; i < 32; ++i) x[i] = 0u;   // U problem: the accumulation starts from nothing
-            tmem_st32(xcol + 32u * c, x);
-          }
-          fence_async_smem();
-        }
-        tmem_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(VP + (g & 1)));
-      }
-      if (lane == 0) mbar_arrive(bar(META_FREE + buf));
     }
   } else if (warp < 12) {
     // ===================== path systems =====================
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 144;");
     constexpr int NS = DMAX + 1;            // path slots in use
     const int quad = warp & 3, row = quad * 32 + lane;
     const int rn = row & 63;
-    const int part = row >> 6;              // 0: O problem, 1: U problem
     const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
     float* Gs = reinterpret_cast<float*>(sm + M::kOffGs);
     // 64 bytes of scratch per tile row, seen by its own thread only: values go in by column and come
@@ -543,27 +572,32 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     for (uint32_t it = 0; ok && it < n_it; ++it) {
       const uint32_t buf = it % M::kMeta;
       if (!(ok = mbar_wait_warp(bar(META_FULL + buf), (it / M::kMeta) & 1, abort_flag))) break;
-      const float* al_s = tab_of(buf);
-      const float* be_s = al_s + kNodes;
+      const float2* ab = reinterpret_cast<const float2*>(tab_of(buf));   // alpha, beta
       const int n = item_of(buf)[0];
 #pragma unroll 1
       for (int b = 0; b < NB; ++b) {
         const uint32_t g = it * NB + b;
         const int nd = kBlk * b + rn;
+        const int part = (row >> 6) ^ b;        // 0: O problem, 1: U problem
         const uint4 pw = *reinterpret_cast<const uint4*>(sm + M::kOffPath + (buf * kNodes + nd) * 16);
         const int depth = reinterpret_cast<const int8_t*>(sm + M::kOffDepth)[buf * kNodes + nd];   // -1: no node
         const bool rows_live = kBlk * b + (quad & 1) * 32 < n;     // warp-uniform: some row of the warp is a node
         const bool solves = rows_live && (part == 0 || want_U);    // warp-uniform: its rows carry problems
-        int path[NS];
+        // of every path slot: row of Gs, chunk of 16 score columns, place in the row's scratch
+        int grow[NS], chunk[NS];
+        uint32_t place[NS];
         float al[NS], bt[NS], vec[NS];
         {
           const uint32_t pword[4] = {pw.x, pw.y, pw.z, pw.w};
 #pragma unroll
           for (int s = 0; s < NS; ++s) {
-            path[s] = (int)((pword[s >> 2] >> ((s & 3) * 8)) & 127u);
-            const float a2 = al_s[path[s]], b2 = be_s[path[s]];
-            al[s] = s <= depth ? a2 : 1.f;   // slots past the node count as no decay
-            bt[s] = s <= depth ? b2 : 0.f;
+            const int node = (int)((pword[s >> 2] >> ((s & 3) * 8)) & 127u);
+            grow[s] = node * kLd;
+            chunk[s] = node >> 4;
+            place[s] = word((uint32_t)node & 15u);
+            const float2 y = ab[node];
+            al[s] = s <= depth ? y.x : 1.f;   // slots past the node count as no decay
+            bt[s] = s <= depth ? y.y : 0.f;
             vec[s] = 0.f;
           }
         }
@@ -590,43 +624,34 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
                                 __uint_as_float(r[16 * e + 4 * i + 2]), __uint_as_float(r[16 * e + 4 * i + 3]));
 #pragma unroll
               for (int s = 0; s < NS; ++s)
-                if ((path[s] >> 4) == c + e) vec[s] = *reinterpret_cast<const float*>(srow + word(path[s] & 15));
+                if (chunk[s] == c + e) vec[s] = *reinterpret_cast<const float*>(srow + place[s]);
             }
           }
-          if (part == 1) {
+          // Decay from a path node down to this one: the product of alpha over the slots between, built up
+          // from the node's own slot backwards.
+          //   part 0: C_{i,p_s} = (P_i / P_{p_s}) q_i . k_{p_s}
+          //   part 1: G_{i,p_s} = beta_i (P_i / P_{p_s}) k_i . k_{p_s}, a row of Gs for every row whose path
+          //           leads through this node; its own system is x L = e_d
+          const float be = part == 0 ? 1.f : ab[nd].y;
+          float sfx = 1.f;
 #pragma unroll
-            for (int s = 0; s < NS; ++s) Gs[nd * kLd + s] = vec[s];
+          for (int s = NS - 1; s >= 0; --s) {
+            const float c = vec[s] * (be * sfx);
+            sfx *= al[s];
+            if (part == 1) Gs[nd * kLd + s] = c;
+            vec[s] = part == 1 ? (s == depth ? 1.f : 0.f) : s <= depth ? c : 0.f;
           }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(E1_SYNC));
-        // C_{i,p_s} = (q_i . k_{p_s}) P_i / P_{p_s}: the ratio is the product of alpha over the slots
-        // after s, built up from the node's own slot backwards; x L = e_d for the U problem
-        {
-          float sfx = 1.f;
-#pragma unroll
-          for (int s = NS - 1; s >= 0; --s) {
-            if (part == 0) vec[s] = s <= depth ? vec[s] * sfx : 0.f;
-            else vec[s] = s == depth ? 1.f : 0.f;
-            sfx *= al[s];
-          }
-        }
         if (!(ok = mbar_wait_warp(bar(E1_SYNC), g & 1, abort_flag))) break;
         if (solves) {
-          // w_s = c_s - sum_{t > s} w_t G_{p_t,p_s},  G_{p_t,p_s} = beta_t (P_{p_t} / P_{p_s}) k_t.k_s;
-          // rr[t] holds P_{p_t} / P_{p_s} = alpha_{s+1} ... alpha_t for the current s and grows by one
-          // factor per step.  Slots past the node's depth carry vec = 0 and a deselected G, so nothing
-          // is predicated.
-          float rr[NS];
+          // w_s = c_s - sum_{t > s} w_t G_{p_t,p_s}; slots past the node's depth carry vec = 0
 #pragma unroll
           for (int s = NS - 2; s >= 0; --s) {
             float acc = vec[s];
 #pragma unroll
-            for (int t = s + 1; t < NS; ++t) {
-              rr[t] = t == s + 1 ? al[t] : rr[t] * al[s + 1];
-              const float gts = Gs[path[t] * kLd + s] * (bt[t] * rr[t]);
-              acc = fmaf(-vec[t], t <= depth ? gts : 0.f, acc);
-            }
+            for (int t = s + 1; t < NS; ++t) acc = fmaf(-vec[t], Gs[grow[t] + s], acc);
             if (s < depth) vec[s] = acc;
           }
           // ---- row of [W ; A] = (w or x) D_beta as bf16 hi and lo, into the columns of the scores ----
@@ -643,11 +668,10 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
             uint32_t w[16];
             if (c < nch) {
 #pragma unroll
-              for (uint32_t i = 0; i < 4; ++i) *reinterpret_cast<uint4*>(srow + (i << 4)) = make_uint4(0u, 0u, 0u, 0u);
+              for (uint32_t i = 0; i < 4; ++i) *reinterpret_cast<uint4*>(srow + ((i ^ ssw) << 4)) = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
               for (int s = 0; s < NS; ++s)
-                if (s <= depth && (path[s] >> 4) == c)
-                  *reinterpret_cast<uint32_t*>(srow + word(path[s] & 15)) = __float_as_uint(vec[s]);
+                if (s <= depth && chunk[s] == c) *reinterpret_cast<uint32_t*>(srow + place[s]) = __float_as_uint(vec[s]);
 #pragma unroll
               for (uint32_t i = 0; i < 4; ++i) {
                 const uint4 x = *reinterpret_cast<const uint4*>(srow + ((i ^ ssw) << 4));
@@ -674,12 +698,115 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       }
       if (ok && lane == 0) mbar_arrive(bar(META_FREE + buf));
     }
+  } else if (warp >= 16) {
+    // ===================== V', scaling of X =====================
+    const int quad = warp & 3, row = quad * 32 + lane;   // TMEM lane
+    const int rn = row & 63;                             // node of this tile row within its block
+    const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
+    const uint32_t swz = (uint32_t)(row & 7);
+    bool ok = true;
+    for (uint32_t it = 0; ok && it < n_it; ++it) {
+      const uint32_t buf = it % M::kMeta, vb = NB == 1 ? it & 1 : 0;
+      if (!(ok = mbar_wait_warp(bar(META_FULL + buf), (it / M::kMeta) & 1, abort_flag))) break;
+      if (!(ok = mbar_wait_warp(bar(V_FULL + vb), (NB == 1 ? it >> 1 : it) & 1, abort_flag))) break;
+      const int n = item_of(buf)[0];
+#pragma unroll 1
+      for (int b = 0; b < NB; ++b) {
+        const uint32_t g = it * NB + b;
+        const int nd = kBlk * b + rn;
+        const float P = tab_of(buf)[2 * kNodes + nd];
+        const uint32_t xcol = tmem + lane_addr + kColX + (g & 1) * 128u;
+        if (!(ok = mbar_wait_warp(bar(X_DONE + (g & 1)), (g >> 1) & 1, abort_flag))) break;
+        tc_fence_after();
+        if (((quad >> 1) ^ b) == 0) {
+          // O problem: the prefix term P_i q_i S_pre^T is where the accumulation starts
+          if (kBlk * b + (quad & 1) * 32 < n) {
+#pragma unroll 1
+            for (int c = 0; c < 4; c += 2) {
+              uint32_t x[64];
+              tmem_ld32(xcol + 32u * c, x);
+              tmem_ld32(xcol + 32u * c + 32u, x + 32);
+              tmem_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 64; ++i) x[i] = __float_as_uint(P * __uint_as_float(x[i]));
+              tmem_st32(xcol + 32u * c, x);
+              tmem_st32(xcol + 32u * c + 32u, x + 32);
+            }
+          }
+        } else {
+          const bool alive = nd < n;
+          // rows are multiplied 16 at a time: past the last such group nothing reads them
+          if (kBlk * b + (quad & 1) * 32 < n) {
+            unsigned char* vrow = sm + M::kOffV + vb * M::kVItem + (uint32_t)nd * 128u;
+            // 32 columns (half of dv half d): V is read before anything is stored, and the next columns
+            // of X are on their way meanwhile
+            auto part_of = [&](uint32_t (&x)[32], uint32_t (&next)[32], int d, uint32_t half, bool more) {
+              unsigned char* r = vrow + (uint32_t)d * M::kVHalf;
+              const uint32_t col = xcol + 64u * d + 32u * half;
+              uint4 v[4];
+#pragma unroll
+              for (uint32_t i = 0; i < 4; ++i)
+                v[i] = *reinterpret_cast<const uint4*>(r + (((half * 4 + i) ^ swz) << 4));
+              tmem_wait_ld();
+              if (more) tmem_ld32(col + 32u, next);
+#pragma unroll
+              for (uint32_t i = 0; i < 4; ++i) {
+                const uint32_t vw[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+                uint32_t hi[4], lo[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                  split_pair(fma2(pair(__uint_as_float(x[8 * i + 2 * e]), __uint_as_float(x[8 * i + 2 * e + 1])), pair(-P, -P),
+                                  pair(__uint_as_float(vw[e] << 16), __uint_as_float(vw[e] & 0xffff0000u))),
+                             hi[e], lo[e]);
+                const uint32_t off = ((half * 4 + i) ^ swz) << 4;
+                *reinterpret_cast<uint4*>(r + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                *reinterpret_cast<uint4*>(r + 2 * M::kVHalf + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+              }
+#pragma unroll
+              for (int i = 0; i < 32; ++i) x[i] = 0u;   // U problem: the accumulation starts from nothing
+              tmem_st32(col, x);
+            };
+            uint32_t xa[32], xb[32];
+            tmem_ld32(xcol, xa);
+#pragma unroll 1   // the roles of a CTA share one instruction cache
+            for (int d = 0; d < 2; ++d) {
+              part_of(xa, xb, d, 0, true);
+              part_of(xb, xa, d, 1, d == 0);
+            }
+            if (!alive) {   // rows past the request may hold anything: 0 x that need not be 0
+              const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 1
+              for (uint32_t i = 0; i < 8; ++i)
+#pragma unroll
+                for (uint32_t part = 0; part < 4; ++part)
+                  *reinterpret_cast<uint4*>(vrow + part * M::kVHalf + ((i ^ swz) << 4)) = z;
+            }
+            __syncwarp();
+          }
+          fence_async_smem();
+        }
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(VP + (g & 1)));
+      }
+      if (!ok) break;
+      if (lane == 0) mbar_arrive(bar(META_FREE + buf));
+    }
   } else {
     // ===================== outputs =====================
-    const int quad = warp & 3, part = quad >> 1;
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+    const int quad = warp & 3;
     const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
-    unsigned char* stage = sm + M::kOffOut + (uint32_t)quad * 2048u;
-    const int64_t ostep = PACKED ? 128 : p.out.t;
+    // 32 rows x 32 columns at a time, all or half of the rows through the warp's staging area: a store then
+    // covers whole 128-byte lines (eight lanes per row) where a lane with a row of its own touches 32 lines.
+    // In: lane = row, chunk i at i ^ (row & 7); out: rows (lane >> 3) + 4 i, chunk lane & 7.
+    constexpr int kRows = M::kOutRows;
+    const uint32_t stage = sbase + M::kOffOut + (uint32_t)(quad * kRows * 128);
+    const uint32_t in0 = stage + (uint32_t)(lane % kRows) * 128u + ((uint32_t)(lane & 7) << 4);
+    const uint32_t out0 = stage + (uint32_t)(lane >> 3) * 128u + (((uint32_t)lane & 7u) ^ ((uint32_t)lane >> 3)) * 16u;
+    const uint32_t out1 = (out0 ^ 64u) + 512u;   // rows 4 further have the other half of the swizzle
+    const int64_t step4 = 4 * (PACKED ? (int64_t)128 : p.out.t);
     grid_dependency_wait();   // O and U may still be read by a kernel in front
     // the commit kernel behind this one may be scheduled as SMs drain (it orders itself)
     if (warp == 12 && lane == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -689,44 +816,69 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       if (!(ok = mbar_wait_warp(bar(META_FULL + buf), (it / M::kMeta) & 1, abort_flag))) break;
       const int32_t* im = item_of(buf);
       const int n = im[0];
-      float* out = (part == 0 ? p.O : p.U) + ((size_t)(uint32_t)im[1] | (size_t)(uint32_t)im[2] << 32);
+      const size_t o0 = (size_t)(uint32_t)im[1] | (size_t)(uint32_t)im[2] << 32;
 #pragma unroll 1
       for (int b = 0; b < NB; ++b) {
         const uint32_t g = it * NB + b;
+        const int part = (quad >> 1) ^ b;             // 0: O rows, 1: U rows
+        const int nd0 = kBlk * b + (quad & 1) * 32;   // first node of this warp
+        const uint32_t xcol = tmem + lane_addr + kColX + (g & 1) * 128u;
         if (!(ok = mbar_wait_warp(bar(ACC + (g & 1)), (g >> 1) & 1, abort_flag))) break;
         tc_fence_after();
-        const int nd0 = kBlk * b + (quad & 1) * 32;   // first node of this warp
-        if (nd0 < n && (part == 0 || want_U)) {
-          // 32 rows x 32 columns at a time, 16 rows through the warp's 2 KiB: a store then covers whole
-          // 128-byte lines (eight lanes per row) where a lane with a row of its own touches 32 lines
-#pragma unroll 1
-          for (int c = 0; c < 4; ++c) {
-            uint32_t x[32];
-            tmem_ld32(tmem + lane_addr + kColX + (g & 1) * 128u + 32u * c, x);
-            tmem_wait_ld();
+        const bool stores = nd0 < n && (part == 0 || want_U);   // warp-uniform
+        const int rows = n - nd0 - (lane >> 3);                 // of this lane's rows, those below this are nodes
+        float* o[8];                                            // rows 4 j of this lane
+        o[0] = (part == 0 ? p.O : p.U) + o0 + (int64_t)(nd0 + (lane >> 3)) * (step4 >> 2) + 4 * (lane & 7);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              __syncwarp();
-              if ((lane >> 4) == h) {
+        for (int j = 1; j < 8; ++j) o[j] = o[j - 1] + step4;
+        auto put = [&](const uint32_t (&x)[32], int c) {
 #pragma unroll
-                for (uint32_t i = 0; i < 8; ++i)
-                  *reinterpret_cast<uint4*>(stage + (lane & 15) * 128 + ((i ^ (uint32_t)(lane & 7)) << 4)) =
-                      make_uint4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
-              }
-              __syncwarp();
+          for (int h = 0; h < 32 / kRows; ++h) {
+            __syncwarp();
+            if (lane / kRows == h) {
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const int r = 4 * i + (lane >> 3);
-                const uint4 o4 = *reinterpret_cast<const uint4*>(stage + r * 128 + (((uint32_t)lane ^ (uint32_t)r) & 7u) * 16u);
-                const int nd = nd0 + 16 * h + r;
-                if (nd < n) *reinterpret_cast<uint4*>(out + (int64_t)nd * ostep + 32 * c + 4 * (lane & 7)) = o4;
-              }
+              for (uint32_t i = 0; i < 8; ++i)
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(in0 ^ (i << 4)), "r"(x[4 * i]),
+                             "r"(x[4 * i + 1]), "r"(x[4 * i + 2]), "r"(x[4 * i + 3]) : "memory");
+            }
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < kRows / 16; ++q) {
+              uint4 o4[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                             : "=r"(o4[i].x), "=r"(o4[i].y), "=r"(o4[i].z), "=r"(o4[i].w)
+                             : "r"(((i & 1) ? out1 : out0) + (uint32_t)(q * 2 + (i >> 1)) * 1024u) : "memory");
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                if (16 * (h + q) + 4 * i < rows) *reinterpret_cast<uint4*>(o[4 * (h + q) + i] + 32 * c) = o4[i];
             }
           }
+        };
+        uint32_t xa[32], xb[32];   // the next columns are read under the stores of these
+        auto release = [&]() {   // all of this warp's rows are in registers
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(X_FREE + (g & 1)));
+        };
+        if (!stores) {
+          release();
+          continue;
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(X_FREE + (g & 1)));
+        tmem_ld32(xcol, xa);
+#pragma unroll 1   // the roles of a CTA share one instruction cache
+        for (int d = 0; d < 2; ++d) {
+          tmem_wait_ld();
+          tmem_ld32(xcol + 64u * d + 32u, xb);
+          put(xa, 0);
+          tmem_wait_ld();
+          if (d == 0) tmem_ld32(xcol + 64u, xa);
+          else release();
+          put(xb, 1);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) o[j] += 64;
+        }
       }
       if (ok && lane == 0) mbar_arrive(bar(META_FREE + buf));
     }
