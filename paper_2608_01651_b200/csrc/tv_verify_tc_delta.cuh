@@ -29,7 +29,7 @@
 // each working on a different item or block:
 //     warps 0..3    TMA producer | MMAs of scores and readout | metadata (paths, gates, P of the items to
 //                   come) | MMAs of the state product
-//     warps 4..7    q and k rows into tensor memory, state rows split in place into bf16 hi + lo
+//     warps 4..7    state rows split in place into bf16 hi + lo
 //     warps 8..11   thread = tile row: scores of its path, back-substitution, row of [W ; A]
 //     warps 12..15  finished rows of X to memory
 //     warps 16..19  V' and the scaling of X
@@ -45,9 +45,9 @@
 // state as tf32, operand tiles and staged outputs sharing buffers) and now, us:
 //     items x nodes   512 x 24       512 x 64       2048 x 64       512 x 128      2048 x 128
 //     before          22.7 /  33.9   28.4 /  40.4   89.5 / 139.0    68.0 /  81.2   219 / 271
-//     now             20.6 /  31.8   23.9 /  36.3   78.5 / 133      41.2 /  55.4   133 / 198
+//     now             20.1 /  31.2   23.6 /  36.3   75.2 / 128.5    41.1 /  55.2   132 / 200
 // Error against 64 bits 3e-4 before, 4.4e-6 now.  What is left: the four hops of an item (state product, V',
-// readout, stores) over two sets of columns, with shared memory half busy; without the stores 512 x 128 takes
+// readout, stores) over three or two sets of columns, with shared memory half busy; without the stores 512 x 128 takes
 // 34 us, without V' 40, without the path systems 40.
 // Every wait is a bounded mbarrier wait (status word on expiry); every TMA load is a plain per-CTA copy.
 #pragma once
@@ -74,11 +74,9 @@ struct Map {
   static constexpr uint32_t kHalfQK = NB == 1 ? kTile : 2 * kTile;   // from one k half to the next
   static constexpr uint32_t kOffS = 4 * kTile;       // four units [128 v][32] fp32, after the split [128 v][32 hi | 32 lo] bf16
   static constexpr uint32_t kOffV = 8 * kTile;       // V, then V'_hi in its place, and V'_lo: dv halves of [nodes][64] (NB = 1: two items)
-  // [Q ; K] of the state product: from tensor memory where there is room for two items (columns kColA on; the
-  // next item's q and k then load while this one's product waits for its state), else from shared memory.  One
-  // set of columns, written block by block, was the slower way for NB = 2 (512 x 128: 45.5 against 45.0 us).
-  static constexpr bool kCopyA = NB == 1;
-  static constexpr uint32_t kColA = 384;
+  // Sets of columns of X: blocks between their state product and their stores.  NB = 1, two sets, with [Q ; K] copied
+  // to tensor memory instead: 79.3 / 133 us on 2048 items of 64 nodes, with three 75.2 / 128.5.
+  static constexpr uint32_t kXBufs = NB == 1 ? 3 : 2;
   static constexpr uint32_t kVHalf = kNodes * 128;   // one dv half
   static constexpr uint32_t kVItem = 4 * kVHalf;     // hi, lo
   static constexpr uint32_t kOffRow = 12 * kTile;    // 64 bytes per tile row, private to its thread (warps 8..11)
@@ -98,19 +96,18 @@ struct Map {
 
 // [2]: block g of the CTA (item * NB + row block) uses entry g & 1, in its phase g >> 1
 enum Bar {
-  QK_FULL = 0, QK_FREE = 2, GD = 4, SC_FREE = 6, COEF = 8, VP = 10, ACC = 12, X_FREE = 14,
-  V_FULL = 16, V_FREE = 18,          // [2]: NB = 1 as above, NB = 2 entry 0 per item
-  X_DONE = 20,                       // [2]: as the first
-  S_FULL = 22, S_SPLIT = 26, S_FREE = 30,   // [4]: unit, phase = item
-  META_FULL = 34, META_FREE = 38,    // [kMeta]
-  E1_SYNC = 42,
-  A_READY = 43,                      // [2]: as the first
+  QK_FULL = 0, QK_FREE = 2, GD = 4, SC_FREE = 6, COEF = 8,
+  V_FULL = 10, V_FREE = 12,          // [2]: NB = 1 as above, NB = 2 entry 0 per item
+  VP = 14, X_FREE = 17, ACC = 20, X_DONE = 23,   // [kXBufs]: set of columns of X, phase = its use
+  S_FULL = 26, S_SPLIT = 30, S_FREE = 34,   // [4]: unit, phase = item
+  META_FULL = 38, META_FREE = 41,    // [kMeta]
+  E1_SYNC = 44,
   kNumBars = 45
 };
 static_assert(kNumBars <= 48, "barrier area");
 
-// TMEM columns: X of two blocks, scores (then coefficients), [Q ; K] as packed bf16 (NB = 1: of two items)
-constexpr uint32_t kColX = 0, kColSc = 256;
+// TMEM columns: X from 0 on (three or two sets of 128), then the scores, which become the coefficients (NB = 1: two
+// sets of 64; NB = 2: 64 for block 0, 128 for block 1)
 
 struct Params {
   TreeDev tree;
@@ -195,7 +192,10 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   auto bar = [&](int i) { return sbase + M::kOffBar + 8u * (uint32_t)i; };
   auto tab_of = [&](uint32_t buf) { return reinterpret_cast<float*>(sm + M::kOffTab) + buf * (3 * kNodes); };
   auto item_of = [&](uint32_t buf) { return reinterpret_cast<int32_t*>(sm + M::kOffItem) + buf * 4; };
-  auto sc_col = [](int g) -> uint32_t { return kColSc + (uint32_t)(g & 1) * 64u; };   // NB = 2: block 1 has 128 columns from there
+  auto sc_col = [](int g) -> uint32_t { return M::kXBufs * 128u + (uint32_t)(g & 1) * 64u; };
+  // set of X of block g, and the parity of that use
+  auto x_set = [](uint32_t g) -> uint32_t { return NB == 1 ? g % 3u : g & 1u; };
+  auto x_par = [](uint32_t g) -> uint32_t { return (NB == 1 ? g / 3u : g >> 1) & 1u; };
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int T = p.T;
@@ -213,9 +213,9 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       prefetch_map(&tmV);
     }
     for (int i = lane; i < kNumBars; i += 32) {   // arrivals of a phase: one thread, unless it is four warps
-      const bool warps4 = (i >= COEF && i < ACC) || (i >= X_FREE && i < V_FULL) || (i >= S_SPLIT && i < S_FREE) || i >= E1_SYNC;
+      const bool warps4 = (i >= COEF && i < V_FULL) || (i >= VP && i < ACC) || (i >= S_SPLIT && i < S_FREE) || i == E1_SYNC;
       const bool qk = i >= QK_FREE && i < GD, meta = i >= META_FREE && i < E1_SYNC;
-      mbar_init(bar(i), qk ? (M::kCopyA ? 5 : 2) : meta ? 12 : warps4 ? 4 : 1);
+      mbar_init(bar(i), qk ? 2 : meta ? 12 : warps4 ? 4 : 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -314,10 +314,10 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       while (ia < n_g) {
         bool progress = false;
         // X += [W ; A] V' of block ia
-        if (mbar_test(bar(VP + (ia & 1)), (ia >> 1) & 1) && mbar_test(bar(COEF + (ia & 1)), (ia >> 1) & 1)) {
+        if (mbar_test(bar(VP + x_set(ia)), x_par(ia)) && mbar_test(bar(COEF + (ia & 1)), (ia >> 1) & 1)) {
           tc_fence_after();
           const uint32_t b = NB == 1 ? 0u : ia & 1;
-          const uint32_t acc = tmem + kColX + (ia & 1) * 128u, chi = tmem + sc_col((int)ia), clo = chi + 32u * (b + 1);
+          const uint32_t acc = tmem + x_set(ia) * 128u, chi = tmem + sc_col((int)ia), clo = chi + 32u * (b + 1);
           const uint64_t dvi = dV + (NB == 1 ? ((ia & 1) * M::kVItem) >> 4 : 0u);
           const int n = item_of((ia / NB) % M::kMeta)[0];   // the block's last steps may hold no node
 #pragma unroll 1
@@ -331,7 +331,7 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
               mma_bf16_ts(acc, clo + c, hi, kIdAV, 1);
               mma_bf16_ts(acc, chi + c, lo, kIdAV, 1);
             }
-          tc_commit(bar(ACC + (ia & 1)));
+          tc_commit(bar(ACC + x_set(ia)));
           tc_commit(bar(SC_FREE + (ia & 1)));
           if (NB == 1) tc_commit(bar(V_FREE + (ia & 1)));
           else if (b == 1) tc_commit(bar(V_FREE));
@@ -379,26 +379,23 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       const uint64_t dQK = desc_kmajor(sbase + M::kOffQK), dS = desc_kmajor(sbase + M::kOffS);
       bool ok = true;
       for (uint32_t g = 0; ok && g < n_it * NB; ++g) {
-        const uint32_t it = g / NB, gb = g & 1, ph = (g >> 1) & 1, x = tmem + kColX + gb * 128u;
-        if (!(ok = mbar_wait(bar(M::kCopyA ? A_READY + gb : QK_FULL + gb), ph, abort_flag))) break;
-        if (!(ok = mbar_wait(bar(X_FREE + gb), ph ^ 1, abort_flag))) break;   // what these columns held has been read out
+        const uint32_t it = g / NB, gb = g & 1, xs = x_set(g), x = tmem + xs * 128u;
+        if (!(ok = mbar_wait(bar(QK_FULL + gb), (g >> 1) & 1, abort_flag))) break;
+        if (!(ok = mbar_wait(bar(X_FREE + xs), x_par(g) ^ 1, abort_flag))) break;   // what these columns held has been read out
 #pragma unroll 1
         for (uint32_t u = 0; u < kUnits; ++u) {   // a quarter of k
           if (!(ok = mbar_wait(bar(S_SPLIT + u), it & 1, abort_flag))) break;
           tc_fence_after();
           const uint64_t dB = dS + ((u * kTile) >> 4);
           const uint64_t dA = dQK + ((gb * M::kBlkQK + (u >> 1) * M::kHalfQK + (u & 1) * 64u) >> 4);
-          const uint32_t aq = tmem + M::kColA + gb * 64u + u * 16u;
 #pragma unroll
-          for (uint32_t i = 0; i < 4; ++i) {   // hi: k 0..15, 16..31 of the quarter; lo: the same
-            if (M::kCopyA) mma_bf16_ts(x, aq + (i & 1u) * 8u, dB + ((i * 32u) >> 4), kIdX, u | i);
-            else mma_bf16_ss(x, dA + (((i & 1u) * 32u) >> 4), dB + ((i * 32u) >> 4), kIdX, u | i);
-          }
+          for (uint32_t i = 0; i < 4; ++i)   // hi: k 0..15, 16..31 of the quarter; lo: the same
+            mma_bf16_ss(x, dA + (((i & 1u) * 32u) >> 4), dB + ((i * 32u) >> 4), kIdX, u | i);
           if (NB == 1 || gb == 1) tc_commit(bar(S_FREE + u));
         }
         if (!ok) break;
-        tc_commit(bar(X_DONE + gb));
-        if (!M::kCopyA) tc_commit(bar(QK_FREE + gb));
+        tc_commit(bar(X_DONE + xs));
+        tc_commit(bar(QK_FREE + gb));
       }
     } else if (warp == 2) {
       // ===================== metadata =====================
@@ -496,39 +493,12 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       }
     }
   } else if (warp < 8) {
-    // ===================== [Q ; K] into tensor memory, state split =====================
+    // ===================== state split =====================
     asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
     const int row = (warp & 3) * 32 + lane;
-    const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t swz = (uint32_t)(row & 7);
     bool ok = true;
-    auto copy_qk = [&](uint32_t g) -> bool {
-      const uint32_t gb = g & 1;
-      if (g >= 2 && !mbar_wait_warp(bar(X_DONE + gb), ((g - 2) >> 1) & 1, abort_flag)) return false;   // they were read
-      if (!mbar_wait_warp(bar(QK_FULL + gb), (g >> 1) & 1, abort_flag)) return false;
-      tc_fence_after();
-#pragma unroll 1
-      for (uint32_t h = 0; h < 2; ++h) {   // k half
-        const unsigned char* r = sm + M::kOffQK + gb * M::kBlkQK + h * M::kHalfQK + (uint32_t)row * 128u;
-        uint32_t w[32];
-#pragma unroll
-        for (uint32_t c = 0; c < 8; ++c) {
-          const uint4 x = *reinterpret_cast<const uint4*>(r + ((c ^ swz) << 4));
-          w[4 * c] = x.x; w[4 * c + 1] = x.y; w[4 * c + 2] = x.z; w[4 * c + 3] = x.w;
-        }
-        tmem_st32(tmem + lane_addr + M::kColA + gb * 64u + h * 32u, w);
-      }
-      tmem_wait_st();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(bar(A_READY + gb));
-        mbar_arrive(bar(QK_FREE + gb));
-      }
-      return true;
-    };
     for (uint32_t it = 0; ok && it < n_it; ++it) {
-      if (M::kCopyA && !(ok = copy_qk(it))) break;
 #pragma unroll 1
       for (int u = 0; u < kUnits; ++u) {
         if (!(ok = mbar_wait_warp(bar(S_FULL + u), it & 1, abort_flag))) break;
@@ -715,8 +685,8 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         const uint32_t g = it * NB + b;
         const int nd = kBlk * b + rn;
         const float P = tab_of(buf)[2 * kNodes + nd];
-        const uint32_t xcol = tmem + lane_addr + kColX + (g & 1) * 128u;
-        if (!(ok = mbar_wait_warp(bar(X_DONE + (g & 1)), (g >> 1) & 1, abort_flag))) break;
+        const uint32_t xcol = tmem + lane_addr + x_set(g) * 128u;
+        if (!(ok = mbar_wait_warp(bar(X_DONE + x_set(g)), x_par(g), abort_flag))) break;
         tc_fence_after();
         if (((quad >> 1) ^ b) == 0) {
           // O problem: the prefix term P_i q_i S_pre^T is where the accumulation starts
@@ -788,7 +758,7 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar(VP + (g & 1)));
+        if (lane == 0) mbar_arrive(bar(VP + x_set(g)));
       }
       if (!ok) break;
       if (lane == 0) mbar_arrive(bar(META_FREE + buf));
@@ -822,8 +792,8 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         const uint32_t g = it * NB + b;
         const int part = (quad >> 1) ^ b;             // 0: O rows, 1: U rows
         const int nd0 = kBlk * b + (quad & 1) * 32;   // first node of this warp
-        const uint32_t xcol = tmem + lane_addr + kColX + (g & 1) * 128u;
-        if (!(ok = mbar_wait_warp(bar(ACC + (g & 1)), (g >> 1) & 1, abort_flag))) break;
+        const uint32_t xcol = tmem + lane_addr + x_set(g) * 128u;
+        if (!(ok = mbar_wait_warp(bar(ACC + x_set(g)), x_par(g), abort_flag))) break;
         tc_fence_after();
         const bool stores = nd0 < n && (part == 0 || want_U);   // warp-uniform
         const int rows = n - nd0 - (lane >> 3);                 // of this lane's rows, those below this are nodes
@@ -860,7 +830,7 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         auto release = [&]() {   // all of this warp's rows are in registers
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar(X_FREE + (g & 1)));
+          if (lane == 0) mbar_arrive(bar(X_FREE + x_set(g)));
         };
         if (!stores) {
           release();
