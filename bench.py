@@ -834,11 +834,8 @@ def run_ours(args, wl, rank, world, local_rank):
         "value": value, "unit": "nodes/s", "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "prewarm_steps": prewarm_steps,
         "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": (("bf16 q/k/v, f32 state read by the tensor cores as a bf16 hi+lo pair (16 mantissa bits), "
-                   "f32 accumulate, f32 outputs" if wl.rule_name == "gated" else
-                   "bf16 q/k/v, f32 state read as tf32 by the tensor cores (mean of the cut compensated), "
-                   "f32 accumulate, f32 outputs") if tc
-                  else "f32"),
+        "dtype": ("bf16 q/k/v, f32 state read by the tensor cores as a bf16 hi+lo pair (16 mantissa bits), "
+                  "f32 accumulate, f32 outputs" if tc else "f32"),
         "data": "synthetic",
         "config": {
             "workload": DESCR[wl.name], "layers_per_step": wl.L, "kernel": args.kernel,
