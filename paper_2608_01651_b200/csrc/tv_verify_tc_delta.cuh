@@ -45,7 +45,7 @@
 // state as tf32, operand tiles and staged outputs sharing buffers) and now, us:
 //     items x nodes   512 x 24       512 x 64       2048 x 64       512 x 128      2048 x 128
 //     before          22.7 /  33.9   28.4 /  40.4   89.5 / 139.0    68.0 /  81.2   219 / 271
-//     now             20.1 /  31.2   23.6 /  36.3   75.2 / 128.5    41.1 /  55.2   132 / 200
+//     now             20.0 /  31.1   23.7 /  35.8   75.2 / 128.5    41.0 /  54.3   131 / 195
 // Error against 64 bits 3e-4 before, 4.4e-6 now.  What is left: the four hops of an item (state product, V',
 // readout, stores) over three or two sets of columns, with shared memory half busy; without the stores 512 x 128 takes
 // 34 us, without V' 40, without the path systems 40.
@@ -822,7 +822,9 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
                              : "r"(((i & 1) ? out1 : out0) + (uint32_t)(q * 2 + (i >> 1)) * 1024u) : "memory");
 #pragma unroll
               for (int i = 0; i < 4; ++i)
-                if (16 * (h + q) + 4 * i < rows) *reinterpret_cast<uint4*>(o[4 * (h + q) + i] + 32 * c) = o4[i];
+                if (16 * (h + q) + 4 * i < rows)   // not read here again; cached in L1, rounds of 512 x 64 / 128: 36.3 / 55.3 against 35.8 / 54.3 us
+                  asm volatile("st.global.L1::no_allocate.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(o[4 * (h + q) + i] + 32 * c),
+                               "r"(o4[i].x), "r"(o4[i].y), "r"(o4[i].z), "r"(o4[i].w) : "memory");
             }
           }
         };
