@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 
 #include "tv_internal.h"
+#include "tv_map_cache.h"
 
 namespace tvtc {
 
@@ -253,20 +254,6 @@ inline bool make_map2_plain(CUtensorMap* map, const void* base, CUtensorMapDataT
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// 4-D view of a node-indexed tensor: element (z, h, t, c) at z*sb + h*sh + t*st + c (element
-// strides), c < d contiguous.  z = layer*request for dense and strided layouts, the layer for the
-// planes of a packed forest (t then runs over the plane's `capacity` rows).
-struct NodeView {
-  uint64_t d, T, Hx, Z;
-  int64_t sb, sh, st;
-};
-// Tensor maps want ascending strides: the node and head dimensions go in stride order, and the
-// kernel is told which of the two coordinates comes first.
-inline bool node_first_of(const NodeView& v) { return v.Hx == 1 || v.st <= v.sh; }
-inline uint64_t view_key(const NodeView& v) {
-  return (uint64_t)v.sb * 0x9e3779b97f4a7c15ull ^ (uint64_t)v.sh * 0xc2b2ae3d27d4eb4full ^ (uint64_t)v.st * 0x165667b19e3779f9ull ^
-         (v.T << 20) ^ (v.Hx << 8) ^ v.Z;
-}
 // Box {box_cols, box_rows nodes, 1 head, 1}; 128-byte swizzle, zero fill past the extents.
 inline bool make_map4(CUtensorMap* map, const void* base, CUtensorMapDataType dt, int esize, const NodeView& v,
                       uint32_t box_cols, uint32_t box_rows) {
@@ -370,39 +357,6 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), int grid, int bloc
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
-}
-
-// Tensor maps depend only on base pointers and shapes: a serving loop calls with the same
-// buffers round after round, so the five encodes of a launch are cached per thread.
-struct MapSet {
-  const void* ptr[5];
-  uint64_t items;
-  int32_t T, kind;
-  alignas(64) CUtensorMap map[5];
-};
-
-template <class Make>
-inline const MapSet* cached_maps(const void* const (&ptr)[5], uint64_t items, int32_t T, int32_t kind,
-                                 Make make) {
-  constexpr int kEntries = 16;
-  static thread_local MapSet cache[kEntries];
-  static thread_local int used = 0, next = 0;
-  for (int i = 0; i < used; ++i) {
-    const MapSet& e = cache[i];
-    if (e.items == items && e.T == T && e.kind == kind && e.ptr[0] == ptr[0] && e.ptr[1] == ptr[1] &&
-        e.ptr[2] == ptr[2] && e.ptr[3] == ptr[3] && e.ptr[4] == ptr[4])
-      return &e;
-  }
-  MapSet& e = cache[next];
-  for (int i = 0; i < 5; ++i) e.ptr[i] = ptr[i];
-  e.items = items; e.T = T; e.kind = kind;
-  if (!make(e.map)) {
-    e.items = 0;   // never matches
-    return nullptr;
-  }
-  if (used < kEntries) ++used;
-  next = (next + 1) % kEntries;
-  return &e;
 }
 
 }  // namespace tvtc

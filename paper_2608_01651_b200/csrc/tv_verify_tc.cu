@@ -1087,10 +1087,8 @@ int tv_launch_verify_tc(const VerifyArgs& a, int32_t* status, cudaStream_t strea
     vv = NodeView{128, (uint64_t)cap, (uint64_t)a.H, (uint64_t)a.L, (int64_t)a.H * cap * 128, cap * 128, 128};
     vo = vv;
   }
-  const void* const ptrs[5] = {a.q, a.k, a.v, a.S_pre, a.O};
-  const uint64_t key = view_key(vq) * 3 + view_key(vv) * 5 + view_key(vo) * 7 + items;
   int node_first = 0;
-  const MapSet* ms = cached_maps(ptrs, key, a.T, (packed ? 4 : 0) | (a.Hk << 8), [&](CUtensorMap* m) {
+  const MapSet* ms = cached_maps(MapKey{{a.q, a.k, a.v, a.S_pre, a.O}, {vq, vv, vo}, items, a.T, packed ? 4 : 0}, [&](CUtensorMap* m) {
     return make_map4(&m[0], a.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, vq, 64, rows) &&
            make_map4(&m[1], a.k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, vq, 64, rows) &&
            make_map4(&m[2], a.v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, vv, 64, rows) &&
@@ -1099,8 +1097,7 @@ int tv_launch_verify_tc(const VerifyArgs& a, int32_t* status, cudaStream_t strea
   });
   const MapSet* mo = ms;   // packed forest: output boxes of 32, 16 and 8 rows
   if (packed) {
-    const void* const optrs[5] = {a.O, nullptr, nullptr, nullptr, nullptr};
-    mo = cached_maps(optrs, key, a.T, 5, [&](CUtensorMap* m) {
+    mo = cached_maps(MapKey{{a.O}, {vq, vv, vo}, items, a.T, 5}, [&](CUtensorMap* m) {
       return make_map4(&m[0], a.O, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, vo, 32, 32) &&
              make_map4(&m[1], a.O, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, vo, 32, 16) &&
              make_map4(&m[2], a.O, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, vo, 32, 8);
@@ -1111,8 +1108,7 @@ int tv_launch_verify_tc(const VerifyArgs& a, int32_t* status, cudaStream_t strea
   if (packed) {
     for (int c = 0; c < 2; ++c) {
       const uint32_t r = rows >> (2 - c);
-      const void* const lptrs[5] = {a.q, a.k, a.v, nullptr, nullptr};
-      mh[c] = cached_maps(lptrs, key, a.T, 6 + c, [&](CUtensorMap* m) {
+      mh[c] = cached_maps(MapKey{{a.q, a.k, a.v}, {vq, vv, vo}, items, a.T, 6 + c}, [&](CUtensorMap* m) {
         return make_map4(&m[0], a.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, vq, 64, r) &&
                make_map4(&m[1], a.k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, vq, 64, r) &&
                make_map4(&m[2], a.v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, vv, 64, r);

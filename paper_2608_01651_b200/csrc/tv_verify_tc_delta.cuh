@@ -877,7 +877,6 @@ inline int launch(const VerifyArgs& a, int32_t* status, cudaStream_t stream) {
   if (!supports<NB>(a)) return TV_ERR_UNSUPPORTED;
   const bool packed = a.tree.offsets != nullptr;
   const uint64_t items = (uint64_t)a.L * a.B * a.H;
-  const void* const ptrs[5] = {a.q, a.k, a.v, a.S_pre, nullptr};
   // 4-D views: dense / strided layouts from the resolved strides, packed forests as planes
   NodeView vq, vv;
   if (!packed) {
@@ -889,9 +888,8 @@ inline int launch(const VerifyArgs& a, int32_t* status, cudaStream_t stream) {
     vq = NodeView{128, (uint64_t)cap, (uint64_t)a.Hk, (uint64_t)a.L, (int64_t)a.Hk * cap * 128, cap * 128, 128};
     vv = NodeView{128, (uint64_t)cap, (uint64_t)a.H, (uint64_t)a.L, (int64_t)a.H * cap * 128, cap * 128, 128};
   }
-  const uint64_t key = view_key(vq) * 3 + view_key(vv) * 5 + items;
   // q, k, v in boxes of 64 rows x 64 columns (rows past the tensor read as zero), S_pre in quarters of k
-  const MapSet* ms = cached_maps(ptrs, key, a.T, 9 | (a.Hk << 8), [&](CUtensorMap* m) {
+  const MapSet* ms = cached_maps(MapKey{{a.q, a.k, a.v, a.S_pre}, {vq, vv}, items, a.T, 9}, [&](CUtensorMap* m) {
     return make_map4(&m[0], a.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, vq, 64, 64) &&
            make_map4(&m[1], a.k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, vq, 64, 64) &&
            make_map4(&m[2], a.v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, vv, 64, 64) &&

@@ -250,3 +250,26 @@ def test_device_built_metadata_bit_exact(name):
     anc_d2, depth_d2 = tree.meta_device()
     anc_h2, depth_h2, _ = tree.meta()
     assert anc_d2.tobytes() == anc_h2.tobytes() and depth_d2.tobytes() == depth_h2.tobytes()
+
+
+@pytest.mark.parametrize("rule,H,T,small,large", [("delta", 8, 64, 4, 132), ("delta", 8, 96, 1, 129), ("gated", 15, 64, 1, 129),
+                                                  ("gated", 9, 24, 2, 162), ("delta", 24, 40, 64, 128)])
+def test_batches_that_share_the_largest_ones_buffers(rule, H, T, small, large):
+    """A server keeps buffers for its largest batch and works on the front of them: a small batch, then
+    a large one at the same addresses, gives what fresh buffers give (bit for bit)."""
+    wl = inputs.workload("c4" if rule == "delta" else "c3", B=large, H=H, T=T, tree="frontier", seed=H)
+    parents, _ = inputs.make_trees(wl)
+    t = {n: None if x is None else x.cuda() for n, x in inputs.make_tensors(wl).items()}
+    O = torch.zeros(large, H, T, 128, device="cuda")
+
+    def run(tens, out, B):
+        tree = tv.tree_build(parents[:B]).upload()
+        x = [None if tens[n] is None else tens[n][:B] for n in ("S_pre", "q", "k", "v", "alpha", "beta")]
+        tv.tree_verify(tree, *x, rule=wl.rule, O=out[:B], impl=tv.IMPL_TC)
+        tree.device_status()
+        return out[:B]
+
+    fresh = run({n: None if x is None else x.clone() for n, x in t.items()}, torch.zeros_like(O), large)
+    for B in (small, large, small, large):
+        O.fill_(7.0)
+        assert torch.equal(run(t, O, B), fresh[:B]), B
