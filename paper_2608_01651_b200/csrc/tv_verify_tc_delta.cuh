@@ -486,8 +486,14 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           }
           if (!__any_sync(0xffffffffu, more)) break;
         }
+        // V' holds P and meets every node of the item in a dense product, whose zero coefficients do not stop a NaN:
+        // where a gate leaves P not finite, V' is zero instead (V' group) and the node's beta a NaN, which reaches
+        // the rows of the node and of its descendants alone.
 #pragma unroll
-        for (int h = 0; h < NN; ++h) tab[2 * kNodes + lane + 32 * h] = P[h];
+        for (int h = 0; h < NN; ++h) {
+          tab[2 * kNodes + lane + 32 * h] = P[h];
+          if (!isfinite(P[h])) tab[2 * (lane + 32 * h) + 1] = __int_as_float(0x7fffffff);
+        }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(META_FULL + buf));
       }
@@ -704,7 +710,7 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
             }
           }
         } else {
-          const bool alive = nd < n;
+          const bool alive = nd < n && isfinite(P);
           // rows are multiplied 16 at a time: past the last such group nothing reads them
           if (kBlk * b + (quad & 1) * 32 < n) {
             unsigned char* vrow = sm + M::kOffV + vb * M::kVItem + (uint32_t)nd * 128u;
@@ -743,7 +749,7 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
               part_of(xa, xb, d, 0, true);
               part_of(xb, xa, d, 1, d == 0);
             }
-            if (!alive) {   // rows past the request may hold anything: 0 x that need not be 0
+            if (!alive) {   // rows past the request may hold anything: 0 x that need not be 0 (nor 0 x P that is not finite)
               const uint4 z = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
               for (uint32_t i = 0; i < 8; ++i)

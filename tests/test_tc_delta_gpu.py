@@ -76,3 +76,31 @@ def test_non_finite_rows_stay_in_their_request(n_max, sizes):
                 assert torch.isnan(O[:, rows]).all()
             else:
                 assert torch.equal(O[:, rows], O0[:, rows]) and torch.equal(U[:, rows], U0[:, rows])
+
+
+@pytest.mark.parametrize("T,tree", [(1, "chain"), (15, "chain"), (40, "frontier"), (64, "frontier"), (100, "spine"), (128, "frontier")])
+@pytest.mark.parametrize("gate,value", [("alpha", float("nan")), ("alpha", float("inf")), ("beta", float("nan"))])
+def test_non_finite_gate_reaches_its_subtree_alone(T, tree, gate, value):
+    # a node's output depends on its root path: a gate elsewhere, whatever it is, does not change it
+    wl = dataclasses.replace(inputs.workload("c4"), B=2, H=2, T=T, tree=tree, seed=11)
+    parents, _ = inputs.make_trees(wl)
+    t = {n: x.cuda() for n, x in inputs.make_tensors(wl).items()}
+    tree_h = tv.tree_build(parents).upload()
+    anc, _, _ = tree_h.meta()
+
+    def run(t):
+        return tv.tree_verify(tree_h, *[t[n] for n in ("S_pre", "q", "k", "v", "alpha", "beta")], rule=tv.DELTA, want_U=True,
+                              impl=tv.IMPL_TC)
+
+    O0, U0 = run(t)
+    for node in sorted({0, T // 3, T // 2, T - 1}):
+        x = dict(t)
+        x[gate] = t[gate].clone()
+        x[gate][1, 0, node] = value
+        O, U = run(x)
+        tree_h.device_status()
+        hit = np.array([i == node or bool(int(anc[1, i, node >> 6]) >> (node & 63) & 1) for i in range(T)])
+        free = torch.from_numpy(~hit).cuda()
+        assert torch.isnan(O[1, 0][~free]).all() and torch.isnan(U[1, 0][~free]).all()
+        assert torch.equal(O[1, 0][free], O0[1, 0][free]) and torch.equal(U[1, 0][free], U0[1, 0][free])
+        assert torch.equal(O[0], O0[0]) and torch.equal(O[1, 1], O0[1, 1]) and torch.equal(U[0], U0[0]) and torch.equal(U[1, 1], U0[1, 1])
