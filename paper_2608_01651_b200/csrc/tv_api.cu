@@ -315,7 +315,7 @@ TV_API int tv_tree_upload(tv_tree* t, void* stream) {
     off_mapped = (const int32_t*)((const char*)t->h_stage_dev + slot * L.slot_b + L.i32_b);
   }
   st = tv_launch_tree_meta((const int32_t*)((const char*)t->h_stage_dev + slot * L.slot_b), t->n_trees, t->n,
-                           t->d_anc_w, t->d_depth_w, t->d_parent_w, t->d_status, off_mapped, t->d_offsets_w, t->n,
+                           t->d_anc_w, t->d_depth_w, t->d_parent_w, t->d_status, off_mapped, t->d_offsets_w, -1, t->n,
                            next_gen(t), s);
   if (st != TV_OK) return st;
   TV_CUDA_TRY(cudaEventRecord(t->staged[slot], s));
@@ -335,7 +335,7 @@ TV_API int tv_forest_upload_device(tv_tree* t, const int32_t* parent_padded, con
   int st = ensure_device(t, L);
   if (st != TV_OK) return st;
   st = tv_launch_tree_meta(parent_padded, t->n_trees, t->n, t->d_anc_w, t->d_depth_w, t->d_parent_w, t->d_status,
-                           offsets, t->d_offsets_w, max_depth_bound, next_gen(t), (cudaStream_t)stream);
+                           offsets, t->d_offsets_w, t->capacity, max_depth_bound, next_gen(t), (cudaStream_t)stream);
   if (st != TV_OK) return st;
   t->max_depth_all = max_depth_bound;
   t->uploaded = true;
@@ -362,7 +362,7 @@ TV_API int tv_tree_device_status(tv_tree* t, void* stream) {
   TV_CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream));
   if (st[0] == TV_ERR_CUDA) return TV_ERR_CUDA;   // a kernel refused its shared-memory window
   if (st[0] != 0) return TV_ERR_DEVICE_TIMEOUT;
-  if (st[1] != 0 && st[1] == t->upload_gen) return TV_ERR_UNSUPPORTED;   // trees deeper than the stated bound
+  if (st[1] != 0 && st[1] == t->upload_gen) return TV_ERR_UNSUPPORTED;   // trees deeper than the stated bound, offsets out of place
   return TV_OK;
 }
 

@@ -11,7 +11,7 @@ __global__ void __launch_bounds__(TV_MAX_NODES)
 tree_meta_kernel(const int32_t* __restrict__ parent, int32_t n, uint64_t* __restrict__ anc,
                  int32_t* __restrict__ depth, int32_t* __restrict__ parent_dev, int32_t* status,
                  const int32_t* __restrict__ offsets, int32_t* __restrict__ offsets_dev,
-                 int32_t depth_bound, int32_t generation) {
+                 int32_t capacity, int32_t depth_bound, int32_t generation) {
   __shared__ int32_t par_s[TV_MAX_NODES];
   const int t = blockIdx.x, i = threadIdx.x;
   // This kernel is itself launched as a dependent of the kernels in front of it.  The parents and
@@ -37,7 +37,18 @@ tree_meta_kernel(const int32_t* __restrict__ parent, int32_t n, uint64_t* __rest
     off0 = offsets[t];
     if (last_tree) off1 = offsets[t + 1];
   }
-  __syncthreads();
+  // Offsets that come from the device (capacity >= 0) have not been validated either, and every kernel
+  // addresses its rows and its tables by them: any one out of place -- descending, a request longer than its
+  // slab, rows past a plane -- and the upload is a forest of empty requests, marked as failed.  Every CTA
+  // looks at all of them, so all agree.
+  bool misplaced = false;
+  if (capacity >= 0)
+    for (int b = i; b < (int)gridDim.x; b += TV_MAX_NODES) {
+      const int32_t from = offsets[b], to = offsets[b + 1];
+      misplaced = misplaced || from < 0 || to < from || to > capacity || to - from > n;
+    }
+  misplaced = __syncthreads_or(misplaced);
+  if (misplaced) off0 = off1 = 0;
   uint64_t w0 = 0, w1 = 0;
   int d = 0;
   // -1 <= parent[j] < j holds by now, so the walk ends within n steps.  The caller's depth bound
@@ -56,7 +67,7 @@ tree_meta_kernel(const int32_t* __restrict__ parent, int32_t n, uint64_t* __rest
     if (last_tree) offsets_dev[t + 1] = off1;
   }
   if (i >= n) return;
-  if (p >= 0) atomicExch(status + 1, generation);
+  if (p >= 0 || misplaced) atomicExch(status + 1, generation);
   const size_t o = (size_t)t * n + i;
   anc[2 * o] = w0;
   anc[2 * o + 1] = w1;
@@ -143,8 +154,9 @@ int tv_launch_tree_meta_params(const int32_t* parent_host, int32_t n_trees, int3
 
 int tv_launch_tree_meta(const int32_t* parent_mapped, int32_t n_trees, int32_t n, uint64_t* anc,
                         int32_t* depth, int32_t* parent_dev, int32_t* status, const int32_t* offsets_mapped,
-                        int32_t* offsets_dev, int32_t depth_bound, int32_t generation, cudaStream_t stream) {
+                        int32_t* offsets_dev, int32_t capacity, int32_t depth_bound, int32_t generation,
+                        cudaStream_t stream) {
   TV_CUDA_TRY(tvtc::launch_dependent(tree_meta_kernel, n_trees, TV_MAX_NODES, 0, stream, parent_mapped, n, anc, depth,
-                                     parent_dev, status, offsets_mapped, offsets_dev, depth_bound, generation));
+                                     parent_dev, status, offsets_mapped, offsets_dev, capacity, depth_bound, generation));
   return TV_OK;
 }

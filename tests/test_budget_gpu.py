@@ -222,3 +222,60 @@ def test_depth_bound_is_checked_on_the_device():
     forest.upload_device(par_d, offsets, max_depth_bound=2)
     forest.rebuild_forest([c for c in chains]).upload()
     forest.device_status()
+
+
+@pytest.mark.parametrize("n_max", [40, 100])
+def test_offsets_are_checked_on_the_device(n_max):
+    """Offsets in device memory that leave their bounds (a request longer than its slab, rows past the
+    planes, descending, negative): the upload is a forest of empty requests and is reported, so nothing is
+    read or written at them; the next upload with offsets in place clears the report."""
+    B, H, W = 5, 2, 4
+    counts = [7, n_max, 1, 20, 13]
+    good = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    cap = int(good[-1])
+    par = np.tile(np.concatenate([[-1], (np.arange(1, n_max) - 1) // 2]).astype(np.int32), (B, 1))
+    par_d = torch.from_numpy(par).to(DEV)
+    wl = inputs.workload("c4", B=1, H=H, T=cap, seed=7)
+    t = {n: x[0].to(DEV) for n, x in inputs.make_tensors(wl).items()}
+    S = inputs.make_tensors(inputs.workload("c4", B=B, H=H, T=1, seed=8))["S_pre"].to(DEV)
+    acc = torch.zeros(B, dtype=torch.int32, device=DEV)
+    x = torch.randn(cap, H * 3 * 128, device=DEV).bfloat16()
+    ctx = torch.randn(B, W - 1, H * 3 * 128, device=DEV).bfloat16()
+    weight = torch.randn(H * 3 * 128, W, device=DEV)
+    forest = tv.forest_build([np.array([-1], dtype=np.int32)] * B, n_max=n_max, capacity=cap)
+
+    def round_(offsets):
+        forest.upload_device(par_d, torch.from_numpy(np.asarray(offsets, dtype=np.int32)).to(DEV), max_depth_bound=7)
+        outs = []
+        for rule in (tv.DELTA, tv.GATED):
+            for impl in (tv.IMPL_TC, tv.IMPL_SIMT):
+                O = torch.full((H, cap, 128), 7.0, device=DEV)
+                U = torch.full_like(O, 7.0)
+                beta = t["beta"] if rule == tv.DELTA else None
+                tv.tree_verify(forest, S, t["q"], t["k"], t["v"], t["alpha"], beta, rule=rule, O=O, U=U, impl=impl)
+                Sn = tv.commit_path(forest, acc, S, t["k"], t["v"], t["alpha"], beta, rule=rule, U=U,
+                                    S_new=torch.zeros_like(S))
+                outs += [O, U, Sn]
+        y = [torch.full((H, cap, 128), 7.0, device=DEV).bfloat16() for _ in range(3)]
+        tv.tree_conv(forest, x, ctx, weight, H=H, dk=128, dv=128, q=y[0], k=y[1], v=y[2])
+        new = tv.conv_commit(forest, acc, x, ctx, H=H, dk=128, dv=128, ctx_new=torch.zeros_like(ctx))
+        return outs, y, new
+
+    ref, ref_y, ref_ctx = round_(good)
+    forest.device_status()
+    assert all(torch.isfinite(o).all() for o in ref) and not torch.equal(ref[2], S)
+    long_last = good.copy(); long_last[4] = good[5] - n_max - 1; long_last[3] = min(long_last[3], long_last[4])
+    bad = [long_last, [0, 0, 0, 0, 0, cap + 1], [0, 10, 5, 20, 30, 40], [-1, 5, 6, 7, 8, 9], [0, 1, 2, 3, 4, 2 ** 30],
+           [0, n_max + 1, n_max + 1, n_max + 1, n_max + 1, n_max + 1]]
+    for offsets in bad:
+        outs, y, new = round_(offsets)
+        with pytest.raises(tv.TreeVerifyError) as e:
+            forest.device_status()
+        assert e.value.status == -3
+        for i, o in enumerate(outs):
+            assert torch.equal(o, S) if i % 3 == 2 else bool((o == 7.0).all()), (offsets, i)
+        assert all(bool((z == 7.0).all()) for z in y) and torch.equal(new, ctx)
+        outs, y, new = round_(good)      # and in place again
+        forest.device_status()
+        assert all(torch.equal(a, b) for a, b in zip(outs, ref)) and torch.equal(new, ref_ctx)
+        assert all(torch.equal(a, b) for a, b in zip(y, ref_y))
