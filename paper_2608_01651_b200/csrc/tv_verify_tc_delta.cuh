@@ -144,6 +144,12 @@ __device__ __forceinline__ uint32_t pack_rn(float lo_elem, float hi_elem) {
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi_elem), "f"(lo_elem));
   return r;
 }
+// The same, finite values never rounded to infinity: what is left over then stays for a second piece.
+__device__ __forceinline__ uint32_t pack_sat(float lo_elem, float hi_elem) {
+  uint32_t r;
+  asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi_elem), "f"(lo_elem));
+  return r;
+}
 // Two fp32 in a register pair; a * b + c in both halves with one instruction.
 __device__ __forceinline__ uint64_t pair(float x0, float x1) {
   uint64_t r;
@@ -160,10 +166,10 @@ __device__ __forceinline__ float2 halves(uint64_t a) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
   return r;
 }
-// A pair of fp32 as bf16 hi (rounded to nearest) and lo (the exact remainder, rounded to nearest)
+// A pair of fp32 as bf16 hi (rounded to nearest, within bf16's range) and lo (the exact remainder, rounded to nearest)
 __device__ __forceinline__ void split_pair(uint64_t x, uint32_t& hi, uint32_t& lo) {
   const float2 v = halves(x);
-  hi = pack_rn(v.x, v.y);
+  hi = pack_sat(v.x, v.y);
   const float2 r = halves(fma2(pair(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), pair(-1.f, -1.f), x));
   lo = pack_rn(r.x, r.y);
 }

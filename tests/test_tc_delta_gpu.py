@@ -104,3 +104,20 @@ def test_non_finite_gate_reaches_its_subtree_alone(T, tree, gate, value):
         assert torch.isnan(O[1, 0][~free]).all() and torch.isnan(U[1, 0][~free]).all()
         assert torch.equal(O[1, 0][free], O0[1, 0][free]) and torch.equal(U[1, 0][free], U0[1, 0][free])
         assert torch.equal(O[0], O0[0]) and torch.equal(O[1, 1], O0[1, 1]) and torch.equal(U[0], U0[0]) and torch.equal(U[1, 1], U0[1, 1])
+
+
+@pytest.mark.parametrize("T", [40, 100])
+def test_states_beyond_the_largest_bf16(T):
+    # the largest fp32 numbers round to infinity in bf16; the two pieces together must still hold them
+    wl = dataclasses.replace(inputs.workload("c4"), B=1, H=2, T=T, tree="frontier", seed=3)
+    parents, accepted = inputs.make_trees(wl)
+    t = inputs.make_tensors(wl)
+    t["S_pre"][0, 0, 5, 7] = 3.4e38
+    t["S_pre"][0, 1, 9, 7] = -3.4028234e38
+    t["k"][..., 7] = 0                      # the keys leave the entry alone, the queries read a part of it
+    t["q"] = t["q"] * 2.0 ** -20
+    O, U, Sn, tree_h = gpu_round(wl, parents, accepted, t, impl=tv.IMPL_TC)
+    tree_h.device_status()
+    ver, com = oracle_round(wl, parents, accepted, t)
+    eO, eU, eS = compare(wl, O, U, Sn, ver, com)
+    assert eO < BOUND and eU < BOUND and eS < BOUND, (eO, eU, eS)
