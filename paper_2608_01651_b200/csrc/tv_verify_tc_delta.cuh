@@ -729,7 +729,7 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
 #pragma unroll
               for (uint32_t i = 0; i < 4; ++i)
                 v[i] = *reinterpret_cast<const uint4*>(r + (((half * 4 + i) ^ swz) << 4));
-              tmem_wait_ld();
+              tmem_wait_ld(x);
               if (more) tmem_ld32(col + 32u, next);
 #pragma unroll
               for (uint32_t i = 0; i < 4; ++i) {
@@ -754,6 +754,7 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
             for (int d = 0; d < 2; ++d) {
               part_of(xa, xb, d, 0, true);
               part_of(xb, xa, d, 1, d == 0);
+              tmem_wait_ld(xa);   // no load in flight from one pass to the next
             }
             if (!alive) {   // rows past the request may hold anything: 0 x that need not be 0 (nor 0 x P that is not finite)
               const uint4 z = make_uint4(0u, 0u, 0u, 0u);
@@ -851,15 +852,16 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           continue;
         }
         tmem_ld32(xcol, xa);
+        tmem_wait_ld(xa);
 #pragma unroll 1   // the roles of a CTA share one instruction cache
         for (int d = 0; d < 2; ++d) {
-          tmem_wait_ld();
           tmem_ld32(xcol + 64u * d + 32u, xb);
           put(xa, 0);
-          tmem_wait_ld();
+          tmem_wait_ld(xb);
           if (d == 0) tmem_ld32(xcol + 64u, xa);
           else release();
           put(xb, 1);
+          tmem_wait_ld(xa);   // no load in flight from one pass to the next
 #pragma unroll
           for (int j = 0; j < 8; ++j) o[j] += 64;
         }
