@@ -348,6 +348,30 @@ __device__ __forceinline__ int request_of(int item, int B, const ItemDiv& d) {
   return lb - (int)fdiv((uint32_t)lb, d.dB) * B;
 }
 
+// Registers a thread of a group of four warps, from here on (all four warps together).
+template <int N>
+__device__ __forceinline__ void set_registers_down() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void set_registers_up() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
+// Shared memory and registers of a kernel, settled before its first launch on a device.  An increase waits, without
+// a limit, for registers that other groups give up, out of those the block was launched with: `shares` (of all
+// groups, those that keep what they have left out) must not exceed what the compiler gave that many groups.
+template <class Kernel>
+inline int allow_kernel(Kernel kernel, uint32_t smem, int shares, int groups) {
+  cudaFuncAttributes at;
+  TV_CUDA_TRY(cudaFuncGetAttributes(&at, kernel));
+  if (shares > groups * at.numRegs) {
+    tv_set_cuda_error(cudaErrorLaunchOutOfResources);
+    return TV_ERR_CUDA;
+  }
+  TV_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  return TV_OK;
+}
+
 // Programmatic dependent launch: the kernel may start while the kernel in front of it on the
 // stream is still running, provided that kernel released its dependents early; whatever reads
 // that kernel's output first passes grid_dependency_wait().

@@ -63,6 +63,7 @@ constexpr int kComputeWarps = 8;
 constexpr int kFirstComputeWarp = 4;
 constexpr int kFirstSplitWarp = 12;
 constexpr int kSplitWarps = 4;
+constexpr int kServiceRegs = 64, kComputeRegs = 168, kSplitRegs = 104;   // a thread, after the split of 4 x 128
 
 // Shared memory map (byte offsets from the 1024-aligned base).  An MMA with M = 128 reads 128
 // rows of its A tile whatever T is: with 64-row boxes the rows 64..127 it reads are the bytes
@@ -337,7 +338,7 @@ verify_tc_gated_kernel(const __grid_constant__ LoadMaps lm, const __grid_constan
   const uint32_t tmem = *tmem_slot;
   // registers: 128 per thread at launch; the compute warps take what the others give up
   if (warp < kFirstComputeWarp) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    set_registers_down<kServiceRegs>();
   if (warp == 0) {
     // ===================== TMA producer =====================
     // Three independent load streams (q+k, v, S_pre), each in item order and each gated by the
@@ -665,7 +666,7 @@ verify_tc_gated_kernel(const __grid_constant__ LoadMaps lm, const __grid_constan
   }
   } else if (warp >= kFirstSplitWarp) {
     // ===================== operand warps: q rows into TMEM, state split =====================
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
+    set_registers_down<kSplitRegs>();
     const int row = tid - kFirstSplitWarp * 32;   // state row v, and node i for the q copy
     const int pw = warp - kFirstSplitWarp;        // = TMEM lane window of this warp
     const uint32_t lane_addr = (uint32_t)(pw * 32) << 16;
@@ -723,7 +724,7 @@ verify_tc_gated_kernel(const __grid_constant__ LoadMaps lm, const __grid_constan
     }
   } else {
     // ===================== compute warps =====================
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
+    set_registers_up<kComputeRegs>();
     const int cw = warp - kFirstComputeWarp;
     const int quad = warp & 3;          // TMEM lane window of this warp
     const int hc = cw >> 2;             // column half handled by this warp
@@ -1038,27 +1039,22 @@ extern "C" __attribute__((visibility("default"))) int tv_selftest_wait_timeout(i
   return TV_OK;
 }
 
-// Allows every form of the gated kernel its shared memory on the current device (which loads them).
-static int allow_shared_memory() {
-  TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<false, false, 128>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<false>::kSmemBytes));
-  TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<true, false, 128>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<false>::kSmemBytes));
-  TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<false, true, 128>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<true>::kSmemBytes));
-  TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<true, true, 128>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<true>::kSmemBytes));
-  TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<false, false, 64>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<false>::kSmemBytes));
-  TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_gated_kernel<false, true, 64>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lay<true>::kSmemBytes));
-  return TV_OK;
+// Settles every form of the gated kernel on the current device (which loads them).
+static int allow_kernels() {
+  constexpr int shares = kServiceRegs + 2 * kComputeRegs + kSplitRegs;
+  int st = allow_kernel(verify_tc_gated_kernel<false, false, 128>, Lay<false>::kSmemBytes, shares, 4);
+  if (st == TV_OK) st = allow_kernel(verify_tc_gated_kernel<true, false, 128>, Lay<false>::kSmemBytes, shares, 4);
+  if (st == TV_OK) st = allow_kernel(verify_tc_gated_kernel<false, true, 128>, Lay<true>::kSmemBytes, shares, 4);
+  if (st == TV_OK) st = allow_kernel(verify_tc_gated_kernel<true, true, 128>, Lay<true>::kSmemBytes, shares, 4);
+  if (st == TV_OK) st = allow_kernel(verify_tc_gated_kernel<false, false, 64>, Lay<false>::kSmemBytes, shares, 4);
+  if (st == TV_OK) st = allow_kernel(verify_tc_gated_kernel<false, true, 64>, Lay<true>::kSmemBytes, shares, 4);
+  return st;
 }
 
 int tv_prepare_verify_tc() {
   cudaFuncAttributes at;
   TV_CUDA_TRY(cudaFuncGetAttributes(&at, widen_rows_kernel));
-  return allow_shared_memory();
+  return allow_kernels();
 }
 
 bool tv_verify_tc_supports(const VerifyArgs& a) {
@@ -1129,7 +1125,7 @@ int tv_launch_verify_tc(const VerifyArgs& a, int32_t* status, cudaStream_t strea
   int dev = 0;
   TV_CUDA_TRY(cudaGetDevice(&dev));
   if (configured_dev != dev) {
-    const int st = allow_shared_memory();
+    const int st = allow_kernels();
     if (st != TV_OK) return st;
     TV_CUDA_TRY(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
     configured_dev = dev;

@@ -62,6 +62,8 @@ constexpr int kSlots = 16;     // path slots per node: depth <= 15
 constexpr int kBlk = 64;       // nodes per row block
 constexpr int kLd = 17;        // row stride of the table of G (floats): conflict-free per slot
 constexpr int kUnits = 4;      // quarters of k, ring slots of the state
+// registers a thread, by group, out of 96 at launch; the V' group keeps its 96
+constexpr int kServiceRegs = 64, kSplitRegs = 64, kPathRegs = 144, kOutRegs = 112;
 
 template <int NB>
 struct Map {
@@ -237,7 +239,7 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
 
   // registers: 96 per thread at launch, moved to where the long rows are held
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    set_registers_down<kServiceRegs>();
     if (warp == 0 && lane == 0) {
       // ===================== TMA producer =====================
       grid_dependency_wait();   // inputs may come from the kernel in front (dependent launch)
@@ -506,7 +508,7 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     }
   } else if (warp < 8) {
     // ===================== state split =====================
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    set_registers_down<kSplitRegs>();
     const int row = (warp & 3) * 32 + lane;
     const uint32_t swz = (uint32_t)(row & 7);
     bool ok = true;
@@ -538,7 +540,7 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     }
   } else if (warp < 12) {
     // ===================== path systems =====================
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 144;");
+    set_registers_up<kPathRegs>();
     constexpr int NS = DMAX + 1;            // path slots in use
     const int quad = warp & 3, row = quad * 32 + lane;
     const int rn = row & 63;
@@ -778,7 +780,7 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     }
   } else {
     // ===================== outputs =====================
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+    set_registers_up<kOutRegs>();
     const int quad = warp & 3;
     const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
     // 32 rows x 32 columns at a time, all or half of the rows through the warp's staging area: a store then
@@ -915,10 +917,12 @@ inline int launch(const VerifyArgs& a, int32_t* status, cudaStream_t stream) {
   int dev = 0;
   TV_CUDA_TRY(cudaGetDevice(&dev));
   if (configured_dev != dev) {
-    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_delta_kernel<NB, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_delta_kernel<NB, 15, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_delta_kernel<NB, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    TV_CUDA_TRY(cudaFuncSetAttribute(verify_tc_delta_kernel<NB, 15, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    constexpr int shares = kServiceRegs + kSplitRegs + kPathRegs + kOutRegs;
+    int st = allow_kernel(verify_tc_delta_kernel<NB, 8, false>, smem, shares, 4);
+    if (st == TV_OK) st = allow_kernel(verify_tc_delta_kernel<NB, 15, false>, smem, shares, 4);
+    if (st == TV_OK) st = allow_kernel(verify_tc_delta_kernel<NB, 8, true>, smem, shares, 4);
+    if (st == TV_OK) st = allow_kernel(verify_tc_delta_kernel<NB, 15, true>, smem, shares, 4);
+    if (st != TV_OK) return st;
     configured_dev = dev;
   }
   const int sm_count = tv_sm_count();
