@@ -942,16 +942,13 @@ inline int launch(const VerifyArgs& a, int32_t* status, cudaStream_t stream) {
   p.gate = a.lay.gate;
   p.out = a.lay.out;
   p.node_first = (node_first_of(vq) ? 1 : 0) | (node_first_of(vv) ? 2 : 0);
-  // With a few items per CTA, as many CTAs as give every one the same number of items (512 items
-  // on 148 SMs: 128 CTAs of 4 rather than 148 of 3 or 4 -- the launch takes four item periods
-  // either way, and the CTAs that run share the memory system with fewer others: 512 items of 128
-  // nodes 48.3 us against 48.6).  With many items per CTA an idle SM costs more than the balance
-  // gains, so the rule stops at eight.
+  // One CTA per SM.  NB = 1 with up to two items per SM: as many CTAs as give every one the same number of items,
+  // which share the memory system with fewer others (200 items 13.4 us against 13.7, 260 13.7 against 13.9; 160 and
+  // 296 the same).  With more items the SMs left out cost more than that gains (300 items 17.9 us against 16.8, 460
+  // 23.5 against 22.7, 600 28.2 against 26.4; 512 the same), with two row blocks always (160 items 23.2 us against 22.5,
+  // 300 32.5 against 30.8, 600 49.9 against 47.8; 200 and 512 the same).
   int grid = (int)(items < (uint64_t)sm_count ? items : (uint64_t)sm_count);
-  if (items > (uint64_t)sm_count) {
-    const uint64_t rounds = (items + sm_count - 1) / sm_count;
-    if (rounds <= 8) grid = (int)((items + rounds - 1) / rounds);
-  }
+  if (NB == 1 && items > (uint64_t)sm_count && items <= 2 * (uint64_t)sm_count) grid = (int)((items + 1) / 2);
   const bool shallow = a.tree.max_depth_all <= 8;
   auto go = [&](auto kernel) {
     return launch_dependent(kernel, grid, kThreads, smem, stream, ms->map[0], ms->map[1], ms->map[2], ms->map[3], p);
