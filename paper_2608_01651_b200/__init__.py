@@ -428,12 +428,6 @@ def tree_verify(tree: Tree, S_pre, q, k, v, alpha, beta=None, *, rule=GATED, O=N
     Tensors are CUDA, contiguous, in the layout of ``tree_verify.h``.  Returns
     ``O`` or ``(O, U)``.
     """
-    if O is None or (U is None and want_U):
-        import torch
-        if O is None:
-            O = torch.empty(*v.shape[:-1], v.shape[-1], device=v.device, dtype=torch.float32)
-        if U is None and want_U:
-            U = torch.empty_like(O)
     key = (tree_verify, tree.n, tree.capacity, type(rule), rule, type(impl), impl, _form(S_pre), _form(q), _form(k), _form(v),
            _form(alpha), _form(beta), _form(O), _form(U))
     d = _forms.get(key)
@@ -444,6 +438,13 @@ def tree_verify(tree: Tree, S_pre, q, k, v, alpha, beta=None, *, rule=GATED, O=N
             _require(t, n, torch.float32, strided=True)
         for t, n in ((q, "q"), (k, "k"), (v, "v")):
             _require(t, n, k.dtype, strided=True)
+    if O is None or (U is None and want_U):   # allocated outputs are contiguous, as those of the call that was checked
+        import torch
+        if O is None:
+            O = torch.empty(*v.shape[:-1], v.shape[-1], device=v.device, dtype=torch.float32)
+        if U is None and want_U:
+            U = torch.empty_like(O)
+    if d is None:
         _require(O, "O", torch.float32, strided=True)
         _require(U, "U", torch.float32, strided=True)
         d = _keep_form(key, ctypes.byref(_dims(S_pre, k, v, rule, impl, tree, q=q, gates=(alpha, beta), outs=(O, U))))
@@ -572,8 +573,10 @@ def _conv_dims(x, H, dk, dv, W, normalize_qk, eps, tree=None, impl=IMPL_AUTO) ->
 
 def _conv_args(tree, x, ctx, weight, bias, H, dk, dv, gate_a, gate_b, A_log, dt_bias, normalize_qk, eps,
                q, k, v, alpha, beta, stream, impl=IMPL_AUTO):
-    key = (_conv_args, tree.n, tree.n_trees, tree.capacity, type(H), H, type(dk), dk, type(dv), dv, type(impl), impl,
-           type(normalize_qk), normalize_qk, type(eps), eps, _form(x), _form(ctx), _form(weight), _form(bias),
+    # the values, not the objects: a tensor or an array of one element may change between calls
+    impl, normalize_qk, eps = int(impl), bool(normalize_qk), float(eps)
+    key = (_conv_args, tree.n, tree.n_trees, tree.capacity, type(H), H, type(dk), dk, type(dv), dv, impl, normalize_qk,
+           eps, _form(x), _form(ctx), _form(weight), _form(bias),
            _form(gate_a), _form(gate_b), _form(A_log), _form(dt_bias), _form(q), _form(k), _form(v), _form(alpha), _form(beta))
     found = _forms.get(key)
     if found is None:

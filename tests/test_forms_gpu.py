@@ -1,6 +1,7 @@
 """Calls whose form (shapes, strides, types) was seen before: same results, same refusals."""
 import dataclasses
 
+import numpy as np
 import pytest
 import torch
 
@@ -24,11 +25,12 @@ def test_repeated_forms_agree_and_refuse_as_before():
     args = [t[n] for n in ("S_pre", "q", "k", "v", "alpha", "beta")]
     strided = [t["S_pre"]] + [_token_major(t[n], 4) for n in ("q", "k", "v")] + [_token_major(t[n], 3) for n in ("alpha", "beta")]
     first = tv.tree_verify(tree, *args, rule=tv.DELTA, want_U=True)
+    first_S = tv.commit_path(tree, acc, args[0], *args[2:], rule=tv.DELTA, U=first[1], S_new=torch.empty_like(args[0]))
     for x in (args, strided, args, strided):          # alternating forms, new buffers each time
         O, U = tv.tree_verify(tree, *[y.clone(memory_format=torch.preserve_format) for y in x], rule=tv.DELTA, want_U=True)
         assert torch.equal(O, first[0]) and torch.equal(U, first[1])
         Sn = tv.commit_path(tree, acc, x[0], *x[2:], rule=tv.DELTA, U=first[1], S_new=torch.empty_like(x[0]))
-        assert torch.isfinite(Sn).all()
+        assert torch.equal(Sn, first_S)
     S, q, k, v, al, be = args
     O, U = first
     bad = [(S.double(), q, k, v, al, be), (S, q.float(), k, v, al, be), (S, q, k, v, al.bfloat16(), be),
@@ -51,3 +53,42 @@ def test_repeated_forms_agree_and_refuse_as_before():
             tv.tree_verify(other, *args, rule=tv.DELTA, O=O, U=U)
         with pytest.raises(TypeError):
             tv.tree_verify(tree, *args, rule=1.0, O=O, U=U)
+
+
+
+def test_front_end_values_are_read_anew():
+    # sizes and switches of one element that are not plain numbers: their value counts, in every call
+    wl = dataclasses.replace(inputs.workload("c4"), B=2, H=2, T=12, seed=4)
+    parents, _ = inputs.make_trees(wl)
+    g = {n: x.cuda() for n, x in inputs.make_conv_inputs(wl, device="cpu", W=4).items()}
+    tree = tv.tree_build(parents).upload()
+
+    def conv(**kw):
+        return tv.tree_conv(tree, g["x"], g["ctx"], g["weight"], g["bias"], H=2, dk=128, dv=128, **kw)[:2]
+
+    eps, norm = torch.tensor(1e-6), torch.tensor(True)
+    for value, on in ((1e-6, True), (3.0, True), (3.0, False), (1e-6, True)):
+        eps.fill_(value)
+        norm.fill_(on)
+        want = conv(eps=value, normalize_qk=on)
+        for e, n in ((eps, norm), (np.array(value), np.array(on)), (np.float64(value), int(on))):
+            got = conv(eps=e, normalize_qk=n)
+            assert all(torch.equal(a, b) for a, b in zip(got, want)), (value, on)
+    a, b = conv(eps=1e-6, normalize_qk=True), conv(eps=3.0, normalize_qk=True)
+    assert not torch.equal(a[0], b[0])
+
+
+def test_refused_inputs_allocate_no_outputs():
+    wl = dataclasses.replace(inputs.workload("c4"), B=2, H=2, T=12, seed=4)
+    parents, _ = inputs.make_trees(wl)
+    t = inputs.make_tensors(wl, device="cuda")
+    tree = tv.tree_build(parents).upload()
+    args = [t[n] for n in ("S_pre", "q", "k", "v", "alpha", "beta")]
+    tv.tree_verify(tree, *args, rule=tv.DELTA)
+    torch.cuda.synchronize()
+    for bad in ([args[0].double()] + args[1:], args[:3] + [t["v"].cpu()] + args[4:], args[:1] + [t["q"].float()] + args[2:]):
+        held = torch.cuda.memory_allocated()
+        torch.cuda.reset_peak_memory_stats()
+        with pytest.raises(ValueError):
+            tv.tree_verify(tree, *bad, rule=tv.DELTA, want_U=True)
+        assert torch.cuda.max_memory_allocated() == held
