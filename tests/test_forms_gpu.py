@@ -92,3 +92,74 @@ def test_refused_inputs_allocate_no_outputs():
         with pytest.raises(ValueError):
             tv.tree_verify(tree, *bad, rule=tv.DELTA, want_U=True)
         assert torch.cuda.max_memory_allocated() == held
+
+
+def test_other_calls_repeat_and_refuse_by_form():
+    # alternating forms of the calls without strides: every result as from a table that holds nothing
+    wls = [dataclasses.replace(inputs.workload("c4"), B=B, H=2, T=T, seed=T) for B, T in ((3, 12), (2, 12), (3, 13))]
+    cases = []
+    for i, wl in enumerate(wls):
+        parents, accepted = inputs.make_trees(wl)
+        t = inputs.make_tensors(wl, device="cuda")
+        W = 4 if i else 3
+        g = {n: x.cuda() for n, x in inputs.make_conv_inputs(wl, device="cpu", W=W).items()}
+        cases.append((wl, tv.tree_build(parents).upload(), torch.from_numpy(parents).cuda(), torch.from_numpy(accepted).cuda(), t, g))
+
+    def calls(case, one_tree, norm, eps):
+        wl, tree, par, acc, t, g = case
+        args = [t[n] for n in ("S_pre", "q", "k", "v", "alpha", "beta")]
+        O = torch.zeros(wl.B, wl.H, wl.T, 128, device="cuda")
+        U = torch.zeros_like(O)
+        tv.tree_verify_static(par[0] if one_tree else par, *args, rule=tv.DELTA, O=O, U=U)
+        dims = dict(H=wl.H, dk=128, dv=128)
+        y = tv.tree_conv(tree, g["x"], g["ctx"], g["weight"], g["bias"], gate_a=g["gate_a"], gate_b=g["gate_b"],
+                         A_log=g["A_log"], dt_bias=g["dt_bias"], normalize_qk=norm, eps=eps, **dims)
+        ctx = tv.conv_commit(tree, acc, g["x"], g["ctx"], ctx_new=torch.zeros_like(g["ctx"]), **dims)
+        return [O, U, *y, ctx]
+
+    variants = [(c, one, norm, eps) for c in cases for one in (False, True) for norm, eps in ((True, 1e-6), (True, 0.5), (False, 1e-6))]
+    want = []
+    for v in variants:
+        tv._forms.clear()
+        want.append(calls(*v))
+    for v, w in list(zip(variants, want)) * 2:
+        assert all(torch.equal(a, b) for a, b in zip(calls(*v), w))
+    # a neighbour of an accepted form is refused, before and after
+    wl, tree, par, acc, t, g = cases[0]
+    args = [t[n] for n in ("S_pre", "q", "k", "v", "alpha", "beta")]
+    O = torch.zeros(wl.B, wl.H, wl.T, 128, device="cuda")
+    for _ in range(2):
+        for bad in (par[:2], par[:, :-1].contiguous(), par.long(), par.t().contiguous(), par.cpu()):
+            with pytest.raises(ValueError):
+                tv.tree_verify_static(bad, *args, rule=tv.DELTA, O=O)
+        with pytest.raises(ValueError):
+            tv.tree_verify_static(par, *args, rule=tv.DELTA, O=O.transpose(1, 2).contiguous().transpose(1, 2))
+        with pytest.raises(ValueError):
+            tv.tree_conv(tree, g["x"], g["ctx"][:, :-1].contiguous(), g["weight"], H=wl.H, dk=128, dv=128)
+        with pytest.raises(ValueError):
+            tv.tree_conv(tree, g["x"], g["ctx"], g["weight"], H=wl.H, dk=64, dv=128)
+        with pytest.raises(ValueError):
+            tv.conv_commit(tree, acc.long(), g["x"], g["ctx"], H=wl.H, dk=128, dv=128)
+        with pytest.raises(ValueError):
+            tv.conv_commit(tree, acc, g["x"], g["ctx"], H=wl.H + 1, dk=128, dv=128)
+
+
+def test_more_forms_than_the_table_keeps():
+    S = torch.randn(4, 2, 128, 128, device="cuda") * 0.05
+    rows = {n: (torch.randn(4, 2, 128, 128, device="cuda") / 8).bfloat16() for n in ("q", "k", "v")}
+    gates = torch.rand(2, 4, 2, 128, device="cuda")
+    trees = {}
+
+    def verify(B, T):
+        if (B, T) not in trees:
+            trees[B, T] = tv.tree_build(np.tile(np.concatenate([[-1], np.arange(T - 1) // 2]).astype(np.int32), (B, 1))).upload()
+        cut = lambda x: x[:B, :, :T].contiguous()
+        return tv.tree_verify(trees[B, T], S[:B], *[cut(rows[n]) for n in ("q", "k", "v")], cut(gates[0]), cut(gates[1]),
+                              rule=tv.DELTA)
+
+    sizes = [(B, T) for T in range(1, 129) for B in (1, 2, 4)]
+    assert len(sizes) > tv._FORMS_KEPT
+    first = [verify(*s) for s in sizes]
+    assert len(tv._forms) <= tv._FORMS_KEPT
+    for s, x in zip(sizes, first):
+        assert torch.equal(verify(*s), x)
