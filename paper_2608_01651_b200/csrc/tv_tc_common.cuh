@@ -164,6 +164,14 @@ __device__ __forceinline__ void mma_bf16_ss(uint32_t d, uint64_t a, uint64_t b, 
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
 }
+// the same with A in tensor memory
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t idesc,
+                                            uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -202,6 +210,36 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[32]) {
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
+// Two fp32 in one register pair: one instruction for both, rounded as two scalar ones.
+struct Pair {
+  uint64_t v;
+};
+__device__ __forceinline__ Pair pack(float a, float b) {
+  Pair r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack(Pair a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+  return r;
+}
+__device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c) {
+  Pair r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ Pair mul2(Pair a, Pair b) {
+  Pair r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ Pair add2(Pair a, Pair b) {
+  Pair r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
 }
 
 // Shared-memory matrix descriptors, 128-byte swizzle, 1024-byte swizzle atoms.
@@ -307,19 +345,7 @@ __device__ __forceinline__ uint32_t fdiv(uint32_t n, const FastDiv& f) { return 
 struct PackedItem {
   int b, plane_v, plane_qk, row0, n;
 };
-__device__ __forceinline__ PackedItem packed_item(const int32_t* offsets, int B, int H, int Hk, int item) {
-  PackedItem r;
-  const int lb = item / H, h = item - lb * H;
-  const int l = lb / B;
-  r.b = lb - l * B;
-  r.plane_v = l * H + h;
-  r.plane_qk = l * Hk + (Hk == H ? h : h / (H / Hk));
-  r.row0 = offsets[r.b];
-  r.n = offsets[r.b + 1] - r.row0;
-  return r;
-}
-
-// The same with the divisions by H, B and the q/k group size H / Hk done as multiply-shift.
+// Divisions by H, B and the q/k group size H / Hk as multiply-shift.
 struct ItemDiv {
   FastDiv dH, dB, dG;
 };

@@ -86,37 +86,15 @@ __device__ __forceinline__ uint4 lds16(uint32_t addr) {
   return r;
 }
 
-// Two fp32 channels in one register pair.  The row loop is bound by instruction issue, and the packed
-// multiply and add of sm_100 do two channels with one instruction (same roundings as two scalar ones):
-// 20.5 -> 18.9 us on 16 requests of 64 nodes and 12288 bf16 channels.
-struct Pair {
-  uint64_t v;
-};
-__device__ __forceinline__ Pair pack(float a, float b) {
-  Pair r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float2 unpack(Pair a) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
-  return r;
-}
-__device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c) {
-  Pair r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-  return r;
-}
-__device__ __forceinline__ Pair mul2(Pair a, Pair b) {
-  Pair r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-  return r;
-}
-__device__ __forceinline__ Pair add2(Pair a, Pair b) {
-  Pair r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-  return r;
-}
+// The row loop is bound by instruction issue, and the packed multiply and add of sm_100 do two channels with one
+// instruction (same roundings as two scalar ones): 20.5 -> 18.9 us on 16 requests of 64 nodes and 12288 bf16
+// channels.
+using tvtc::Pair;
+using tvtc::pack;
+using tvtc::unpack;
+using tvtc::fma2;
+using tvtc::mul2;
+using tvtc::add2;
 
 // The eight staged values of this lane for one tap row; a0 / a1 are the shared-memory byte
 // addresses of the lane's two channel groups in that row (bf16 reads both with one load).

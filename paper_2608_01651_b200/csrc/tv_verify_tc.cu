@@ -111,14 +111,6 @@ constexpr uint32_t kColQb = 0, kColSc = 128, kColAcc0 = 256, kColAcc1 = 384;
 constexpr uint32_t kIdescKK128 = idesc_bf16(128, false);
 constexpr uint32_t kIdescKK64 = idesc_bf16(64, false);
 
-__device__ __forceinline__ void mma_bf16_ts(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t idesc,
-                                            uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
-}
-
 // Eight fp32 values -> bf16 hi and lo parts (hi = upper 16 bits, lo = the exact remainder cut to
 // its upper 16 bits: hi + lo carries 16 mantissa bits), stored as two 16-byte chunks.
 __device__ __forceinline__ void store_split8(unsigned char* chi, unsigned char* clo, uint32_t off,

@@ -129,12 +129,6 @@ struct Params {
   int32_t node_first;
 };
 
-__device__ __forceinline__ void mma_bf16_ts(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
-}
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
@@ -152,27 +146,11 @@ __device__ __forceinline__ uint32_t pack_sat(float lo_elem, float hi_elem) {
   asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi_elem), "f"(lo_elem));
   return r;
 }
-// Two fp32 in a register pair; a * b + c in both halves with one instruction.
-__device__ __forceinline__ uint64_t pair(float x0, float x1) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x0), "f"(x1));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ float2 halves(uint64_t a) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
-  return r;
-}
 // A pair of fp32 as bf16 hi (rounded to nearest, within bf16's range) and lo (the exact remainder, rounded to nearest)
-__device__ __forceinline__ void split_pair(uint64_t x, uint32_t& hi, uint32_t& lo) {
-  const float2 v = halves(x);
+__device__ __forceinline__ void split_pair(Pair x, uint32_t& hi, uint32_t& lo) {
+  const float2 v = unpack(x);
   hi = pack_sat(v.x, v.y);
-  const float2 r = halves(fma2(pair(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), pair(-1.f, -1.f), x));
+  const float2 r = unpack(fma2(pack(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), pack(-1.f, -1.f), x));
   lo = pack_rn(r.x, r.y);
 }
 
@@ -523,10 +501,10 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         for (uint32_t c = 0; c < 4; ++c) {
           const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(r + (((2 * c) ^ swz) << 4));
           const ulonglong2 e = *reinterpret_cast<const ulonglong2*>(r + (((2 * c + 1) ^ swz) << 4));
-          split_pair(a.x, hi[c].x, lo[c].x);
-          split_pair(a.y, hi[c].y, lo[c].y);
-          split_pair(e.x, hi[c].z, lo[c].z);
-          split_pair(e.y, hi[c].w, lo[c].w);
+          split_pair(Pair{a.x}, hi[c].x, lo[c].x);
+          split_pair(Pair{a.y}, hi[c].y, lo[c].y);
+          split_pair(Pair{e.x}, hi[c].z, lo[c].z);
+          split_pair(Pair{e.y}, hi[c].w, lo[c].w);
         }
 #pragma unroll
         for (uint32_t c = 0; c < 4; ++c) {
@@ -739,8 +717,8 @@ verify_tc_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
                 uint32_t hi[4], lo[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                  split_pair(fma2(pair(__uint_as_float(x[8 * i + 2 * e]), __uint_as_float(x[8 * i + 2 * e + 1])), pair(-P, -P),
-                                  pair(__uint_as_float(vw[e] << 16), __uint_as_float(vw[e] & 0xffff0000u))),
+                  split_pair(fma2(pack(__uint_as_float(x[8 * i + 2 * e]), __uint_as_float(x[8 * i + 2 * e + 1])), pack(-P, -P),
+                                  pack(__uint_as_float(vw[e] << 16), __uint_as_float(vw[e] & 0xffff0000u))),
                              hi[e], lo[e]);
                 const uint32_t off = ((half * 4 + i) ^ swz) << 4;
                 *reinterpret_cast<uint4*>(r + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);

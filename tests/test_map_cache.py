@@ -12,6 +12,7 @@ PROGRAM = r"""
 using namespace tvtc;
 
 static long made = 0;
+static bool fails = false;   // of the encode
 // a set of maps that says what it was made from
 static void stamp(CUtensorMap* m, const MapKey& k) {
   std::memcpy(&m[0], &k.view[0], sizeof(NodeView));
@@ -20,7 +21,7 @@ static void stamp(CUtensorMap* m, const MapKey& k) {
   std::memcpy(&m[3], k.ptr, sizeof(k.ptr));
 }
 static bool serves(const MapKey& k) {
-  const MapSet* s = cached_maps(k, [&](CUtensorMap* m) { stamp(m, k); ++made; return true; });
+  const MapSet* s = cached_maps(k, [&](CUtensorMap* m) { stamp(m, k); ++made; return !fails; });
   CUtensorMap want[5];
   std::memset(want, 0, sizeof(want));
   stamp(want, k);
@@ -65,8 +66,11 @@ int main() {
   // an encode that fails is not kept
   MapKey f = k;
   f.kind = 77;
-  for (int i = 0; i < 2; ++i) bad += cached_maps(f, [](CUtensorMap*) { return false; }) != nullptr;
-  bad += !serves(f);
+  fails = true;
+  for (int i = 0; i < 2; ++i) { before = made; bad += serves(f) + 1000 * (made != before + 1); }
+  fails = false;
+  before = made;
+  bad += !serves(f) + 1000 * (made != before + 1) + !serves(k);
   std::printf("%ld lookups, %ld bad\n", calls, bad);
   return bad != 0;
 }
