@@ -920,13 +920,18 @@ inline int launch(const VerifyArgs& a, int32_t* status, cudaStream_t stream) {
   p.gate = a.lay.gate;
   p.out = a.lay.out;
   p.node_first = (node_first_of(vq) ? 1 : 0) | (node_first_of(vv) ? 2 : 0);
-  // One CTA per SM.  NB = 1 with up to two items per SM: as many CTAs as give every one the same number of items,
-  // which share the memory system with fewer others (200 items 13.4 us against 13.7, 260 13.7 against 13.9; 160 and
-  // 296 the same).  With more items the SMs left out cost more than that gains (300 items 17.9 us against 16.8, 460
-  // 23.5 against 22.7, 600 28.2 against 26.4; 512 the same), with two row blocks always (160 items 23.2 us against 22.5,
-  // 300 32.5 against 30.8, 600 49.9 against 47.8; 200 and 512 the same).
+  // One CTA per SM, or as many as give every one the same number of items: they share the memory system with fewer
+  // others, and the commit behind finds SMs free.  With two items a CTA always, with three or four where that
+  // leaves out few SMs, never with more (us, equal shares / all SMs):
+  //     items, 64 nodes     160          200          260          300          400          512          600          800
+  //     back to back        13.2 / 13.1  13.3 / 13.7  13.7 / 13.9  17.9 / 16.8  18.7 / 18.7  23.7 / 23.5  28.2 / 26.4  33.6 / 33.0
+  //     in rounds           19.8 / 20.6  20.7 / 21.3  21.9 / 22.1  26.5 / 26.7  29.8 / 29.9  36.0 / 36.4  42.0 / 41.5  52.9 / 52.1
+  //     items, 128 nodes
+  //     back to back        23.2 / 22.5  23.2 / 23.1  23.7 / 23.9  32.5 / 30.8  32.3 / 32.4  41.2 / 41.2  49.9 / 47.8  59.0 / 58.5
+  //     in rounds           30.0 / 30.6  30.7 / 31.5  31.9 / 32.6  40.5 / 41.1  44.4 / 44.8  54.3 / 54.8  64.9 / 65.2  83.1 / 82.5
   int grid = (int)(items < (uint64_t)sm_count ? items : (uint64_t)sm_count);
-  if (NB == 1 && items > (uint64_t)sm_count && items <= 2 * (uint64_t)sm_count) grid = (int)((items + 1) / 2);
+  const int each = (int)((items + sm_count - 1) / sm_count), even = (int)((items + each - 1) / each);
+  if (each == 2 || (each <= 4 && 20 * even >= 17 * sm_count)) grid = even;
   const bool shallow = a.tree.max_depth_all <= 8;
   auto go = [&](auto kernel) {
     return launch_dependent(kernel, grid, kThreads, smem, stream, ms->map[0], ms->map[1], ms->map[2], ms->map[3], p);
