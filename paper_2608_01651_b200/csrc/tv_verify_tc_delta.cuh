@@ -44,11 +44,15 @@
 // Measured, back to back / in rounds of upload, verify and commit, before (one chain of phases over eight warps,
 // state as tf32, operand tiles and staged outputs sharing buffers) and now, us:
 //     items x nodes   512 x 24       512 x 64       2048 x 64       512 x 128      2048 x 128
-//     before          22.7 /  33.9   28.4 /  40.4   89.5 / 139.0    68.0 /  81.2   219 / 271
-//     now             20.0 /  31.1   23.7 /  35.8   75.2 / 128.5    41.0 /  54.3   131 / 195
+//     before          22.7 /  34.1   28.6 /  40.5   90.3 / 140.1    68.3 /  81.4   220 / 275
+//     now             20.1 /  31.4   23.9 /  36.0   74.1 / 132.7    41.4 /  54.7   132 / 205
 // Error against 64 bits 3e-4 before, 4.4e-6 now.  What is left: the four hops of an item (state product, V',
-// readout, stores) over three or two sets of columns, with shared memory half busy; without the stores 512 x 128 takes
-// 34 us, without V' 40, without the path systems 40.
+// readout, stores) over three or two sets of columns, with shared memory half busy.  Parts left out in a scratch
+// build, all waits intact, 512 x 64 / 512 x 128: the output group's reads, staging and stores 19.9 / 32.9 us, its
+// global stores alone 21.5 / 38.6, V' 22.1 / 38.7, scores and path systems 20.9 / 37.7.
+//
+// Values that are not finite: a gate's reaches the rows of its node's subtree (see the metadata warp); a q row's its own
+// output row; a k or v row's or a state entry's every node of the (request, head), the entry's in its value column.
 // Every wait is a bounded mbarrier wait (status word on expiry); every TMA load is a plain per-CTA copy.
 #pragma once
 #include "tv_tc_common.cuh"
