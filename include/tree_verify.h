@@ -159,10 +159,10 @@ int tv_tree_meta_device(tv_tree* tree, uint64_t* anc, int32_t* depth, void* stre
  * core completion that never came): TV_OK or TV_ERR_DEVICE_TIMEOUT.  After a
  * timeout the outputs of that launch are undefined; the context stays usable.
  * TV_ERR_UNSUPPORTED: the trees of the last tv_forest_upload_device were deeper
- * than the bound that call was given, or its offsets out of place.  TV_ERR_CUDA: a tensor-core kernel (or
- * tv_tree_conv, whose row boxes arrive by TMA) found its shared-memory window
- * off the boundary its tiles need and left without computing (outputs
- * undefined, as after a timeout).                                             */
+ * than the bound that call was given, or its offsets out of place.
+ * TV_ERR_CUDA: a tensor-core kernel (or tv_tree_conv, whose row boxes arrive by
+ * TMA) found its shared-memory window off the boundary its tiles need and left
+ * without computing (outputs undefined, as after a timeout).                  */
 int tv_tree_device_status(tv_tree* tree, void* stream);
 /* Self-test of that mechanism: launches one CTA that waits, with a limit of a
  * few milliseconds, on a barrier nothing ever signals, and writes what the
@@ -228,11 +228,11 @@ int tv_forest_rebuild(tv_tree* forest, const int32_t* parent_flat /*host*/,
  * of them, so every kernel stays within its tables, the results of that round
  * are not the tree's, and tv_tree_device_status returns TV_ERR_UNSUPPORTED
  * until the next upload.  The offsets are checked there as well (0 <= offsets[r]
- * <= offsets[r+1] <= capacity, at most n_max nodes per request): if one is out of
- * place every request of that round is empty -- no output row is written, no
- * state changes -- and the status is the same.  After it the handle's host-side metadata is stale:
- * tv_tree_meta and tv_tree_path return TV_ERR_UNSUPPORTED until the next
- * tv_forest_rebuild + tv_tree_upload.                                          */
+ * <= offsets[r+1] <= capacity, at most n_max nodes per request): if one is out
+ * of place every request of that round is empty -- no output row is written, no
+ * state changes -- and the status is the same.  After the call the handle's
+ * host-side metadata is stale: tv_tree_meta and tv_tree_path return
+ * TV_ERR_UNSUPPORTED until the next tv_forest_rebuild + tv_tree_upload.        */
 size_t tv_budget_workspace_bytes(int32_t n_req, int32_t n_cand);
 int tv_budget_select(const int32_t* parent /*dev*/, const float* p_draft /*dev*/, int32_t n_req,
                      int32_t n_cand, int32_t budget, float* rho, int32_t* counts, int32_t* offsets,
