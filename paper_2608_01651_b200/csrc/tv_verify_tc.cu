@@ -379,8 +379,12 @@ verify_tc_gated_kernel(const __grid_constant__ LoadMaps lm, const __grid_constan
           progress = true;
         }
         // (two stages: the second item's state is not asked for before the first item's operands
-        // have landed -- at the start of a launch every CTA's first loads share the memory system)
-        if (i_s < n_it && (!SMALL || i_s != 1 || (poll(bar(S_FULL0), 0) && poll(bar(QK_FULL), 0))) &&
+        // have landed -- at the start of a launch every CTA's first loads share the memory system.
+        // QK_FULL is only asked until the first scores are issued: where the state comes later than
+        // the second item's q and k, that barrier has gone on to a phase of the same parity, and a
+        // CTA of two items would wait for a third one's.)
+        if (i_s < n_it &&
+            (!SMALL || i_s != 1 || (poll(bar(S_FULL0), 0) && (i_sc > 0 || poll(bar(QK_FULL), 0)))) &&
             poll(bar(S_FREE0 + s_stage(i_s)), s_phase(i_s) ^ 1)) {
           const int sj = s_stage(i_s);
           const int item = (int)(blockIdx.x + i_s * gridDim.x);
