@@ -91,7 +91,9 @@ typedef struct tv_dims {
   int32_t impl;        /* TV_IMPL_AUTO picks a tensor-core kernel when the
                           shape allows it (bf16, dk = dv = 128; gated rule
                           also dk = dv = 64 in dense layouts; delta rule: tree
-                          depth <= 15) and the SIMT fp32 kernel otherwise;
+                          depth <= 15), else, for 17 to 64 nodes and widths of
+                          64 and 128, one of fp32 accuracy where that is the
+                          faster, and the SIMT fp32 kernel otherwise;
                           TV_IMPL_TC returns TV_ERR_UNSUPPORTED instead of
                           falling back                                          */
   int32_t Hk;          /* grouped key heads (Section IV-D: a K factor shared by

@@ -467,6 +467,7 @@ TV_API int tv_tree_verify(const tv_tree* tree, const tv_dims* d, const float* S_
     if (tc_gated) return tv_launch_verify_tc(a, tree->d_status, (cudaStream_t)stream);
     if (tc_delta) return tv_launch_verify_tc_delta(a, tree->d_status, (cudaStream_t)stream);
     if (tc_delta128) return tv_launch_verify_tc_delta128(a, tree->d_status, (cudaStream_t)stream);
+    if (tv_verify_exact_takes(a)) return tv_launch_verify_exact(a, tree->d_status, (cudaStream_t)stream);
   }
   return tv_launch_verify_simt(a, (cudaStream_t)stream);
 }

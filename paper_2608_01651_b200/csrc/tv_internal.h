@@ -181,6 +181,9 @@ int tv_launch_tree_meta_params(const int32_t* parent_host, int32_t n_trees, int3
                                int32_t* offsets_dev, cudaStream_t stream);
 bool tv_verify_tc_supports(const VerifyArgs& a);
 int tv_launch_verify_tc(const VerifyArgs& a, int32_t* status, cudaStream_t stream);
+bool tv_verify_exact_takes(const VerifyArgs& a);
+int tv_launch_verify_exact(const VerifyArgs& a, int32_t* status, cudaStream_t stream);
+int tv_prepare_verify_exact();
 bool tv_verify_tc_delta_supports(const VerifyArgs& a);
 int tv_launch_verify_tc_delta(const VerifyArgs& a, int32_t* status, cudaStream_t stream);
 bool tv_verify_tc_delta128_supports(const VerifyArgs& a);   // 64 < T <= 128

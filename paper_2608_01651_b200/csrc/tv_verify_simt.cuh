@@ -1,6 +1,6 @@
 // Tree verification, general fp32 kernels (any T <= 128, dk, dv <= 128, f32 or bf16 operands, gated
-// and delta rules).  All arithmetic is fp32 FMA, so they serve the all-fp32 workloads, the delta
-// rule on trees deeper than the tensor-core kernels' tables, and every shape those refuse.
+// and delta rules).  All arithmetic is fp32 FMA, so they serve every shape that the tensor-core kernels
+// refuse, the calls where they are ahead of the one of fp32 accuracy (tv_verify_exact.cu), and TV_IMPL_SIMT.
 //
 // One CTA per (layer, request, head) and chunk of value columns, following Theorem 1 (Eq. 2) in the
 // factorised form of Eq. 4 / Lemma 2 (Eq. 5):

@@ -92,7 +92,7 @@ unsigned char* scratch_address(int dev, cudaError_t* err) {
     cudaFuncAttributes at;
     if ((*err = cudaFuncGetAttributes(&at, tree_meta_static_kernel)) != cudaSuccess) return nullptr;
     if ((*err = cudaFuncGetAttributes(&at, forward_status_kernel)) != cudaSuccess) return nullptr;
-    if (tv_prepare_verify_simt() != TV_OK || tv_prepare_verify_tc() != TV_OK) {
+    if (tv_prepare_verify_simt() != TV_OK || tv_prepare_verify_tc() != TV_OK || tv_prepare_verify_exact() != TV_OK) {
       *err = (cudaError_t)tv_last_cuda_error();
       return nullptr;
     }
@@ -167,6 +167,7 @@ int tv_tree_verify_static(const int32_t* parent, int32_t n_trees, const tv_dims*
   TV_CUDA_TRY(cudaGetLastError());
   int st;
   if (tc_gated && d->impl != TV_IMPL_SIMT) st = tv_launch_verify_tc(a, scratch_status, s);
+  else if (d->impl == TV_IMPL_AUTO && tv_verify_exact_takes(a)) st = tv_launch_verify_exact(a, scratch_status, s);
   else st = tv_launch_verify_simt(a, s);
   if (st != TV_OK) return st;
   if (status) {

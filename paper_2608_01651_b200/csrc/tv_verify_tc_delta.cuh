@@ -133,23 +133,6 @@ struct Params {
   int32_t node_first;
 };
 
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-               : "memory");
-}
-// Two fp32 -> one word of two bf16, rounded to nearest even (first argument in the low half).
-__device__ __forceinline__ uint32_t pack_rn(float lo_elem, float hi_elem) {
-  uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi_elem), "f"(lo_elem));
-  return r;
-}
-// The same, finite values never rounded to infinity: what is left over then stays for a second piece.
-__device__ __forceinline__ uint32_t pack_sat(float lo_elem, float hi_elem) {
-  uint32_t r;
-  asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi_elem), "f"(lo_elem));
-  return r;
-}
 // A pair of fp32 as bf16 hi (rounded to nearest, within bf16's range) and lo (the exact remainder, rounded to nearest)
 __device__ __forceinline__ void split_pair(Pair x, uint32_t& hi, uint32_t& lo) {
   const float2 v = unpack(x);

@@ -1,0 +1,159 @@
+"""The verify kernels at fp32 accuracy on the tensor cores (what `auto` takes for f32 operands, for the delta
+rule on trees deeper than the other tensor-core kernels hold, and for 64-wide heads): blocks of 16 nodes, path
+and block form, one or two halves of the value columns, several items on a CTA.
+
+Tolerances: 1e-5 per node as everywhere for all-fp32 operands.  Whole tensors: 1.5e-7.  An operand in three
+bf16 pieces is exact to 2^-24; a product drops three of nine piece products, each below 2^-24 of it; the sums are
+fp32, four truncated steps on top of smaller ones in two halves, 2^-23 each at most and half of that on average, then
+at most four roundings: 1.4e-7 of the result's norm where partial sums are no larger than it."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2608_01651_b200 as tv
+from oracle import tree_oracle as orc
+from paper_2608_01651_b200 import inputs
+from tests import parity_util as pu
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(B, H, T, rule, tree, dtype, dk=128, dv=128, seed=0):
+    wl = inputs.workload("c4", B=B, H=H, T=T, dk=dk, dv=dv, rule=rule, tree=tree, qkv_dtype=dtype, seed=seed + T)
+    tens = inputs.make_tensors(wl)
+    if dtype == inputs.F32:
+        tens["k"] = tens["k"] * (8.0 / dk ** 0.5)
+    return (wl,) + inputs.make_trees(wl) + (tens,)
+
+
+def _check(wl, parents, accepted, tens, whole=1.5e-7):
+    O, U, Sn, tree = pu.gpu_round(wl, parents, accepted, tens, impl=tv.IMPL_AUTO, commit_with_U=True)
+    tree.device_status()
+    n = wl.B * wl.H
+    items = sorted({(i // wl.H, i % wl.H) for i in (0, 1, n // 2, n - 1, min(n - 1, 148), min(n - 1, 149))})
+    ver, com = pu.oracle_round(wl, parents, accepted, tens, items=items)
+    errs = pu.compare(wl, O, U, Sn, ver, com)
+    assert max(errs) <= 1e-5, errs
+    for x, which in ((O, 0),) + (((U, 1),) if wl.rule == inputs.DELTA else ()):
+        got, ref = (np.stack(y) for y in ([x[i] for i in items], [ver[i][which] for i in items]))
+        assert pu.rel_fro(got, ref) <= whole
+
+
+@pytest.mark.parametrize("tree", ["frontier", "chain"])
+@pytest.mark.parametrize("T", [17, 32, 33, 48, 49, 63, 64])
+def test_delta(T, tree):
+    # 6 items: halves; 80: whole columns; 200: two items on a CTA
+    for B, H in ((2, 3), (10, 8), (25, 8)):
+        if tree == "chain" or T > 32 or (B == 10 or T == 32 and B == 2):   # others: the general kernel's
+            _check(*_inputs(B, H, T, inputs.DELTA, tree, inputs.F32, seed=B))
+    if tree == "chain":
+        for B, H in ((2, 3), (25, 8)):
+            _check(*_inputs(B, H, T, inputs.DELTA, tree, inputs.BF16, seed=B))
+
+
+@pytest.mark.parametrize("T", [49, 64])
+@pytest.mark.parametrize("tree", ["frontier", "chain"])
+def test_gated(T, tree):
+    for B, H in ((5, 8), (10, 8), (25, 8)):
+        _check(*_inputs(B, H, T, inputs.GATED, tree, inputs.F32, seed=B))
+
+
+@pytest.mark.parametrize("dk,dv", [(64, 64), (64, 128), (128, 64)])
+@pytest.mark.parametrize("dtype", [inputs.F32, inputs.BF16])
+@pytest.mark.parametrize("rule", [inputs.GATED, inputs.DELTA])
+def test_other_widths(rule, dtype, dk, dv):
+    if dtype == inputs.BF16 and rule == inputs.GATED and dk == dv:
+        pytest.skip("a kernel of its own")
+    for T, tree in ((31, "chain"), (50, "frontier"), (64, "chain")):
+        for B, H in ((3, 2), (10, 8), (25, 8)):
+            if rule == inputs.GATED and (T < 49 or B == 3 or B == 25 and dv == 64):   # the general kernel's
+                continue
+            _check(*_inputs(B, H, T, rule, tree, dtype, dk=dk, dv=dv, seed=B))
+
+
+@pytest.mark.parametrize("depth", [15, 16])
+def test_the_depth_where_the_forms_change(depth):
+    rng = np.random.default_rng(depth)
+    for T in (25, 40, 64):
+        wl, _, _, tens = _inputs(5, 4, T, inputs.DELTA, "frontier", inputs.F32)
+        parents = np.stack([inputs.tree_frontier(T, rng, max_depth=depth, spine=depth + 1) for _ in range(5)])
+        accepted = np.array([depth, T - 1, -1, 0, depth], dtype=np.int32)
+        _check(wl, parents, accepted, tens)
+
+
+def test_more_items_than_a_cta_keeps_a_record_of():
+    wl, parents, accepted, tens = _inputs(160, 32, 33, inputs.DELTA, "frontier", inputs.F32, dk=64, dv=64)
+    _check(wl, parents, accepted, tens)
+
+
+def test_packed_forest_and_strides():
+    """Requests of 1 to 64 nodes, shallow and deep; grouped key heads and token-major rows against dense ones."""
+    rng = np.random.default_rng(3)
+    H = 4
+    par = [inputs.tree_chain(64), inputs.tree_frontier(40, rng), inputs.tree_chain(17),
+           inputs.tree_frontier(1, rng), inputs.tree_frontier(64, rng)]
+    forest = tv.forest_build(par, n_max=64).upload()
+    N = int(forest.offsets[-1])
+    t = _inputs(1, H, N, inputs.DELTA, "chain", inputs.F32)[3]
+    S = inputs.make_tensors(inputs.workload("c4", B=len(par), H=H, T=1, seed=78))["S_pre"]
+    dev = {n: t[n][0].cuda() for n in ("q", "k", "v", "alpha", "beta")}
+    O, U = tv.tree_verify(forest, S.cuda(), *dev.values(), rule=tv.DELTA, want_U=True)
+    forest.device_status()
+    for b, p in enumerate(par):
+        lo, hi = int(forest.offsets[b]), int(forest.offsets[b + 1])
+        cut = {n: inputs.to_f64(t[n][:, :, lo:hi]) for n in dev}
+        ver = orc.verify_batch(inputs.to_f64(S[b:b + 1]), *cut.values(), p[None], "delta")
+        for h in range(H):
+            assert pu.rel_l2_rows(inputs.to_f64(O[h, lo:hi]), ver[(0, h)][0]) <= 1e-5
+            assert pu.rel_l2_rows(inputs.to_f64(U[h, lo:hi]), ver[(0, h)][1]) <= 1e-5
+    for dtype, rule in ((inputs.F32, tv.GATED), (inputs.F32, tv.DELTA), (inputs.BF16, tv.DELTA)):
+        wl, parents, _, t = _inputs(20, 10, 50, rule, "chain", dtype)
+        x = {n: y.cuda() if y is not None else None for n, y in t.items()}
+        x["q"], x["k"] = x["q"][:, ::2].contiguous(), x["k"][:, ::2].contiguous()
+        tree = tv.tree_build(parents).upload()
+        names = ("S_pre", "q", "k", "v", "alpha", "beta")
+        dense = tv.tree_verify(tree, *[x[n] for n in names], rule=rule, want_U=True)
+        token = lambda y: y if y is None else y.transpose(1, 2).contiguous().transpose(1, 2)
+        moved = [x["S_pre"]] + [token(x[n]) for n in names[1:]]
+        out = [token(torch.zeros_like(dense[0])) for _ in range(2)]
+        tv.tree_verify(tree, *moved, rule=rule, O=out[0], U=out[1])
+        assert torch.equal(out[0], dense[0]) and torch.equal(out[1], dense[1])
+
+
+@pytest.mark.parametrize("what", ["v", "k", "alpha", "beta", "zero gate", "state"])
+@pytest.mark.parametrize("rule", [inputs.GATED, inputs.DELTA])
+@pytest.mark.parametrize("T,tree", [(50, "frontier"), (49, "chain")])
+def test_values_that_are_not_finite(T, tree, rule, what):
+    """They reach the rows that the recurrence takes them to -- a node's subtree, an entry of the state its value
+    column -- and change no bit of any other row, whatever the coefficients between them."""
+    if what == "beta" and rule == inputs.GATED:
+        pytest.skip("no beta")
+    wl, parents, accepted, tens = _inputs(20, 8, T, rule, tree, inputs.F32)
+    bad = T // 3
+    if what == "zero gate":
+        tens["alpha"][3][:, torch.from_numpy(parents[3] == bad)] = 0.0
+    run = lambda: pu.gpu_round(wl, parents, accepted, tens, impl=tv.IMPL_AUTO)[:2]
+    O0, U0 = run()
+    if what == "state":
+        tens["S_pre"][3, 2, 5, 7] = float("inf")
+    elif what == "zero gate":
+        tens["v"][3, 2, bad] = float("nan")
+    else:
+        tens[what][3, 2, bad] = float("nan")
+    O, U = run()
+    hit = np.array([bad in orc.path_to(parents[3], i) for i in range(T)])
+    O_is, U_is = np.ones_like(O, dtype=bool), np.ones_like(O, dtype=bool)   # where nothing may change
+    if what == "state":
+        O_is[3, 2, :, 5] = U_is[3, 2, :, 5] = False
+        assert not np.isfinite(O[3, 2, :, 5]).any()
+    else:
+        O_is[3, 2, hit] = False
+        U_is[3, 2, hit] = False
+        if not (what == "k" and rule == inputs.GATED and hit.sum() == 1):
+            assert np.isnan(O[3, 2, hit]).all()
+    if what == "state":   # every row of the item is worked out again, in fp32
+        np.testing.assert_allclose(O[3, 2][O_is[3, 2]], O0[3, 2][O_is[3, 2]], rtol=0, atol=1e-5 * np.abs(O0[3, 2]).max())
+        O_is[3, 2] = U_is[3, 2] = False
+    assert np.array_equal(O[O_is], O0[O_is])
+    if rule == inputs.DELTA:
+        assert np.array_equal(U[U_is], U0[U_is])
