@@ -9,8 +9,8 @@
 //   budget_rho_kernel     one CTA per request: rho_i = rho_parent * p_i in float32, level by level
 //                         (parent before child, one rounding per edge), and a 32-bit sort key
 //   budget_choose_kernel  one CTA per request: every CTA finds the budget-th largest key of the batch
-//                         for itself (all keys in its registers, two bits of the threshold per step),
-//                         counts what the requests in front of its own keep, then compacts its own
+//                         for itself (all keys in its registers, two bits of the threshold per step,
+//                         until exactly as many keys reach it as are wanted), counts what the requests in front of its own keep, then compacts its own
 //                         request in order and renumbers the parents; ties go in (request, node) order
 // Everything else takes three launches:
 //   budget_rho_kernel, then
@@ -19,11 +19,16 @@
 //   budget_pack_kernel    one CTA per request: order-preserving compaction and parent renumbering
 // The sizes are tiny (at most a few 10^4 candidates): what counts is the chain of launches and of
 // steps inside them.  A whole device-built round of 2048 candidates (32 requests, budget 1234) took 69.8 us
-// with three ordinary launches and takes 61.7 us with these two.
+// with three ordinary launches, 61.2 us with these two and 60.0 us since the search ends early.  The search
+// is steps of compares, one reduction and one barrier (some 0.25 us each): 16 of them to the last bit, 9 for 2048 spread
+// probabilities, all 16 where ties decide.  Four warps of 16 keys a thread, three counts in one word and so one
+// reduction a step, against eight warps with two reductions and all steps: 7.6 -> 5.45 us a selection of 2048 candidates
+// in 16 or 32 requests, 7.3 -> 4.8 of 64 in one, 7.7 -> 7.7 where ties decide.  One launch for everything, every CTA
+// working out all scores, was slower: 8.7 us, and 37 on chains (7.6 and 12.4).
 // Every request's CTA of the two-launch form searches all keys: its work is requests x candidates.  Device
-// time of a selection, two launches against three: 2048 candidates in 16 / 148 / 300 / 1024 requests 7.5 / 7.7 /
-// 11.5 / 21.7 us against 10.4 / 10.9 / 10.3 / 10.5, 512 in 200 / 256 requests 8.9 / 10.4 against 8.9 / 9.2: up to
-// one CTA per SM.  With 32 keys per thread, which 2049 to 8192 candidates need, it was slower at any number of
+// time of a selection, two launches (before the early end) against three: 2048 candidates in 16 / 148 / 300 / 1024
+// requests 7.5 / 7.7 / 11.5 / 21.7 us against 10.4 / 10.9 / 10.3 / 10.5, 512 in 200 / 256 requests 8.9 / 10.4 against
+// 8.9 / 9.2: up to one CTA per SM.  With 32 keys per thread, which 2049 to 8192 candidates need, it was slower at any number of
 // requests: 4096 candidates in 32 / 1024 requests 14.5 / 64 us against 11.4 / 11.4.
 #include "tv_internal.h"
 #include "tv_tc_common.cuh"
@@ -101,67 +106,57 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* t
   return warp_tot[warp] + incl - v;
 }
 
-constexpr int kChooseThreads = 256;
+constexpr int kChooseThreads = 128, kChooseWarps = kChooseThreads / 32;
+constexpr int KPT = 16;   // keys per thread, consecutive ones
 
-// Sum over the CTA; the same answer in all threads.  A buffer is used again only after another barrier.
-__device__ __forceinline__ uint32_t block_sum(uint32_t x, uint32_t* buf) {
-  x = __reduce_add_sync(0xffffffffu, x);
-  if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = x;
-  __syncthreads();
-  uint32_t t = 0;
-#pragma unroll
-  for (int w = 0; w < kChooseThreads / 32; ++w) t += buf[w];
-  return t;
-}
-
-constexpr int KPT = 8;   // keys per thread, consecutive ones.  Counts stay below 65536: two of them share a word.
 __global__ void __launch_bounds__(kChooseThreads)
-budget_choose_kernel(const uint32_t* __restrict__ key, const int32_t* __restrict__ parent, int32_t N, int32_t K,
+budget_choose_kernel(const uint32_t* __restrict__ key, const int32_t* parent, int32_t N, int32_t K,
                      int32_t B, int32_t Tc, int32_t budget, int32_t* __restrict__ counts, int32_t* __restrict__ offsets,
-                     int32_t* __restrict__ parent_packed, int32_t* __restrict__ node_id) {
-  static_assert(KPT * kChooseThreads < 65536, "counts of 16 bits");
-  __shared__ uint32_t buf[2][2 * kChooseThreads / 32];
-  __shared__ int rank_s[TV_MAX_NODES];
-  __shared__ unsigned ballot_s[2][TV_MAX_NODES / 32];
+                     int32_t* parent_packed, int32_t* __restrict__ node_id) {
+  static_assert(KPT * 32 < 1024 && KPT * kChooseThreads <= 2048, "counts of a warp in 10 bits, of the CTA in 12");
+  static_assert(kChooseThreads == TV_MAX_NODES && kChooseWarps == 4, "a thread per node; four words are read at once");
+  __shared__ __align__(16) uint32_t turn_s[2][kChooseWarps];
+  __shared__ __align__(16) uint32_t front_s[2][kChooseWarps];
+  __shared__ __align__(16) unsigned ballot_s[2][kChooseWarps];
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   tvtc::grid_dependency_wait();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int i0 = tid * KPT;
   uint32_t k[KPT];
 #pragma unroll
-  for (int x = 0; x < KPT; ++x) k[x] = i0 + x < N ? key[i0 + x] : 0u;
+  for (int x = 0; x < KPT; x += 4) {   // (keys lie on 16-byte boundaries)
+    if (i0 + x + 4 <= N) {
+      const uint4 y = *reinterpret_cast<const uint4*>(key + i0 + x);
+      k[x] = y.x, k[x + 1] = y.y, k[x + 2] = y.z, k[x + 3] = y.w;
+    } else {
+#pragma unroll
+      for (int z = 0; z < 4; ++z) k[x + z] = i0 + x + z < N ? key[i0 + x + z] : 0u;
+    }
+  }
   const bool node = tid < Tc;
   const uint32_t own = node ? key[(size_t)b * Tc + tid] : 0u;
-  int par = node ? parent[(size_t)b * Tc + tid] : -1;
+  int par = node ? parent[(size_t)b * Tc + tid] : -1;   // (parent_packed may be the same buffer: read before any write)
   if (par < -1 || par >= tid) par = -1;
 
-  // the largest tau that at least K keys reach: from the top, two bits at a time (the places past N hold
-  // zero and every candidate is at least one)
+  // the largest tau that at least K keys reach, or any that exactly K reach: from the top, two bits at a
+  // time (the places past N hold zero and every candidate is at least one).  Three counts share a word.
   uint32_t tau = 0;
 #pragma unroll 1
   for (int shift = 30; shift >= 0; shift -= 2) {
     const uint32_t c1 = tau | 1u << shift, c2 = tau | 2u << shift, c3 = tau | 3u << shift;
-    uint32_t n12 = 0, n3 = 0;
+    uint32_t n = 0;
 #pragma unroll
-    for (int x = 0; x < KPT; ++x) {
-      n12 += (k[x] >= c1 ? 1u : 0u) + (k[x] >= c2 ? 0x10000u : 0u);
-      n3 += k[x] >= c3 ? 1u : 0u;
-    }
-    uint32_t* turn = buf[(shift >> 1) & 1];   // used again two steps on: one barrier per step is enough
-    n12 = __reduce_add_sync(0xffffffffu, n12);
-    n3 = __reduce_add_sync(0xffffffffu, n3);
-    if (lane == 0) {
-      turn[2 * warp] = n12;
-      turn[2 * warp + 1] = n3;
-    }
+    for (int x = 0; x < KPT; ++x) n += (k[x] >= c1 ? 1u : 0u) + (k[x] >= c2 ? 1u << 10 : 0u) + (k[x] >= c3 ? 1u << 20 : 0u);
+    n = __reduce_add_sync(0xffffffffu, n);
+    uint32_t* turn = turn_s[(shift >> 1) & 1];   // used again two steps on: one barrier per step is enough
+    if (lane == 0) turn[warp] = n;
     __syncthreads();
-    n12 = n3 = 0;
-#pragma unroll
-    for (int w = 0; w < kChooseThreads / 32; ++w) {
-      n12 += turn[2 * w];
-      n3 += turn[2 * w + 1];
-    }
-    tau = (int)n3 >= K ? c3 : (int)(n12 >> 16) >= K ? c2 : (int)(n12 & 0xffffu) >= K ? c1 : tau;
+    const uint4 w = *reinterpret_cast<const uint4*>(turn);
+    const int n1 = (int)((w.x & 1023u) + (w.y & 1023u) + (w.z & 1023u) + (w.w & 1023u));
+    const int n2 = (int)((w.x >> 10 & 1023u) + (w.y >> 10 & 1023u) + (w.z >> 10 & 1023u) + (w.w >> 10 & 1023u));
+    const int n3 = (int)((w.x >> 20) + (w.y >> 20) + (w.z >> 20) + (w.w >> 20));
+    tau = n3 >= K ? c3 : n2 >= K ? c2 : n1 >= K ? c1 : tau;
+    if (n3 == K || n2 == K || n1 == K) break;   // (then tau is that one, and no lower bit changes the set)
   }
   // keys above tau, in the batch and in front of this request; keys equal to it in front of this request
   uint32_t above = 0, ties = 0;
@@ -172,32 +167,48 @@ budget_choose_kernel(const uint32_t* __restrict__ key, const int32_t* __restrict
     above += k[x] > tau ? (front ? 0x10001u : 1u) : 0u;
     ties += k[x] == tau && front ? 1u : 0u;
   }
-  above = block_sum(above, buf[1]);
-  ties = block_sum(ties, buf[0]);
+  above = __reduce_add_sync(0xffffffffu, above);
+  ties = __reduce_add_sync(0xffffffffu, ties);
+  const bool tie = node && own == tau;
+  const unsigned tie_ballot = __ballot_sync(0xffffffffu, tie);
+  if (lane == 0) {
+    front_s[0][warp] = above;
+    front_s[1][warp] = ties;
+    ballot_s[0][warp] = tie_ballot;
+  }
+  __syncthreads();
+  above = ties = 0;
+#pragma unroll
+  for (int w = 0; w < kChooseWarps; ++w) {
+    above += front_s[0][w];
+    ties += front_s[1][w];
+  }
   const int need = K - (int)(above & 0xffffu);      // keys equal to tau to take, in index order
   const int offset = (int)(above >> 16) + min(need, (int)ties);
 
   // this request's nodes
-  const bool tie = node && own == tau;
-  const unsigned tie_ballot = __ballot_sync(0xffffffffu, tie);
-  if (lane == 0 && warp < TV_MAX_NODES / 32) ballot_s[0][warp] = tie_ballot;
-  __syncthreads();
   int before = (int)ties + __popc(tie_ballot & ((1u << lane) - 1u));
-  for (int w = 0; w < warp && w < TV_MAX_NODES / 32; ++w) before += __popc(ballot_s[0][w]);
+#pragma unroll
+  for (int w = 0; w < kChooseWarps; ++w)
+    if (w < warp) before += __popc(ballot_s[0][w]);
   const bool flag = node && (own > tau || (tie && before < need));
   const unsigned ballot = __ballot_sync(0xffffffffu, flag);
-  if (lane == 0 && warp < TV_MAX_NODES / 32) ballot_s[1][warp] = ballot;
+  if (lane == 0) ballot_s[1][warp] = ballot;
   __syncthreads();
-  int rank = __popc(ballot & ((1u << lane) - 1u)), count = 0;
-  for (int w = 0; w < TV_MAX_NODES / 32; ++w) {
-    const int c = __popc(ballot_s[1][w]);
+  int rank = __popc(ballot & ((1u << lane) - 1u)), count = 0, above_par = 0;
+  unsigned par_word = 0;
+#pragma unroll
+  for (int w = 0; w < kChooseWarps; ++w) {
+    const unsigned kept = ballot_s[1][w];
+    const int c = __popc(kept);
     if (w < warp) rank += c;
+    if (w < par >> 5) above_par += c;
+    if (w == par >> 5) par_word = kept;
     count += c;
   }
-  if (node) rank_s[tid] = flag ? rank : -1;
-  __syncthreads();
   if (flag) {
-    parent_packed[(size_t)b * Tc + rank] = par < 0 ? -1 : rank_s[par];   // -1 also if the parent was dropped
+    const unsigned bit = 1u << (par & 31);   // (-1 has no word: it stays without a parent, as one that was dropped)
+    parent_packed[(size_t)b * Tc + rank] = par_word & bit ? above_par + __popc(par_word & (bit - 1u)) : -1;
     node_id[offset + rank] = b * Tc + tid;
   }
   if (node && tid >= count) parent_packed[(size_t)b * Tc + tid] = -1;    // padding of the slab

@@ -53,6 +53,42 @@ def test_select_matches_oracle_bit_for_bit(case):
     assert np.array_equal(node_id[:K], ref["node_id"][:K]) and (node_id[K:] == -1).all()
 
 
+REGISTERS = [  # B, Tc, budget, tree: all keys in every CTA's registers, thresholds that exactly K keys reach and ties
+    (1, 128, 77, "chain"), (16, 128, 1000, "chain"), (17, 120, 1200, "frontier"), (33, 62, 1023, "frontier"),
+    (32, 64, 2048, "frontier"), (32, 64, 2047, "star"), (64, 32, 65, "chain"), (148, 13, 700, "frontier"),
+    (128, 16, 128, "frontier"), (40, 51, 999, "ties"), (7, 1, 7, "frontier"), (2, 96, 50, "zeros"),
+]
+
+
+@pytest.mark.parametrize("shared", [False, True])
+@pytest.mark.parametrize("case", REGISTERS)
+def test_batches_of_up_to_2048_candidates(case, shared):
+    """Bit for bit as the oracle, with results of their own and with the scores and the packed parents
+    written over the candidates."""
+    B, Tc, budget, tree = case
+    par, p = candidates(B, Tc, seed=B + 1000 * Tc, ties=tree == "ties")
+    if tree == "chain":
+        par[:] = np.arange(Tc) - 1
+    if tree == "star":
+        par[:, 1:] = 0
+    if tree == "zeros":
+        p[:, 3:] = 0
+    ref = bo.select(par, p, budget)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    dpar, dp = torch.from_numpy(par).to(DEV), torch.from_numpy(p).to(DEV)
+    out = tv.budget_select(dpar.clone(), dp.clone(), budget)
+    if shared:
+        out["rho"], out["parent_packed"] = dp, dpar
+    for x in ("counts", "offsets", "node_id"):
+        out[x].fill_(-77)
+    got = tv.budget_select(dpar, dp, budget, status=status, out=out)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert np.array_equal(got["rho"].cpu().numpy().view(np.uint32), ref["rho"].view(np.uint32))
+    for x in ("counts", "offsets", "parent_packed", "node_id"):
+        assert np.array_equal(got[x].cpu().numpy(), ref[x]), x
+
+
 def test_invalid_parent_is_reported_not_followed():
     par, p = candidates(4, 16, seed=5)
     par[2, 7] = 9          # parent after child
