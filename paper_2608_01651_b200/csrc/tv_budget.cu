@@ -10,8 +10,9 @@
 //                         (parent before child, one rounding per edge), and a 32-bit sort key
 //   budget_choose_kernel  one CTA per request: every CTA finds the budget-th largest key of the batch
 //                         for itself (all keys in its registers, two bits of the threshold per step,
-//                         until exactly as many keys reach it as are wanted), counts what the requests in front of its own keep, then compacts its own
-//                         request in order and renumbers the parents; ties go in (request, node) order
+//                         until exactly as many keys reach it as are wanted), counts what the requests in
+//                         front of its own keep, then compacts its own request in order and renumbers the
+//                         parents; ties go in (request, node) order
 // Everything else takes three launches:
 //   budget_rho_kernel, then
 //   budget_select_kernel  one CTA: 4-pass radix select of the budget-th largest key, then per-request
@@ -26,10 +27,12 @@
 // in 16 or 32 requests, 7.3 -> 4.8 of 64 in one, 7.7 -> 7.7 where ties decide.  One launch for everything, every CTA
 // working out all scores, was slower: 8.7 us, and 37 on chains (7.6 and 12.4).
 // Every request's CTA of the two-launch form searches all keys: its work is requests x candidates.  Device
-// time of a selection, two launches (before the early end) against three: 2048 candidates in 16 / 148 / 300 / 1024
-// requests 7.5 / 7.7 / 11.5 / 21.7 us against 10.4 / 10.9 / 10.3 / 10.5, 512 in 200 / 256 requests 8.9 / 10.4 against
-// 8.9 / 9.2: up to one CTA per SM.  With 32 keys per thread, which 2049 to 8192 candidates need, it was slower at any number of
-// requests: 4096 candidates in 32 / 1024 requests 14.5 / 64 us against 11.4 / 11.4.
+// time of a selection of about 2000 candidates, two launches against three: 160 / 200 / 256 / 300 / 400 / 512 / 1024
+// requests 7.2 / 6.5 / 6.6 / 8.7 / 10.7 / 11.5 / 12.9 us against 9.6 / 10.9 / 10.7 / 10.7 / 10.7 / 10.2 / 10.6, where ties
+// decide 256 / 400 / 1024 requests 8.6 / 14.9 / 20.7 against 10.6 / 10.9 / 10.8.  The line stays at one CTA
+// per SM (tests/test_budget_choose_gpu.py holds it there); up to two would be ahead.  With 32
+// keys per thread, which 2049 to 8192 candidates need, it was slower at any number of requests (on eight warps, searching
+// to the last bit): 4096 candidates in 32 / 1024 requests 14.5 / 64 us against 11.4 / 11.4.
 #include "tv_internal.h"
 #include "tv_tc_common.cuh"
 
