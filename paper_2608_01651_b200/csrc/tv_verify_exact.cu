@@ -30,17 +30,18 @@ int tv_exact_bf16_prepare();
 //     24 nodes, f32, chain, 128 wide  9.2 / 10.3  12.4 / 10.7  16.8 / 13.5  26.6 / 23.2  27.6 / 24.1  39.9 / 34.7  52.0 / 45.4
 //     33 nodes, f32, chain, 64 x 64  10.6 / 10.9  10.9 / 11.0  13.9 / 11.6  18.1 / 19.9  18.9 / 20.8  31.0 / 30.1  36.9 / 39.9
 //     64 nodes, f32, chain, 64 x 64  14.0 / 14.4  14.4 / 14.5  19.2 / 15.0  26.8 / 26.4                42.7 / 39.1  53.3 / 51.0
-//     56 nodes, f32, gated, 128 x 64  9.9 / 10.9  10.1 / 10.9  15.3 / 12.5  (64 x 64 chains of 64, 72 items: 8.9 / 9.5, 96: 11.5 / 9.7;
-//      from half an SM per item on the general kernel no longer splits the value columns)
+//     56 nodes, f32, gated, 128 x 64  9.9 / 10.9  10.1 / 10.9  15.3 / 12.5
+//     (64 nodes, f32, gated, chain, 64 x 64: 72 items 8.9 / 9.5, 96 11.5 / 9.7; beyond half an item per SM the
+//     general kernel no longer splits 64 value columns over two CTAs)
 // (600, 800, 1024 items of 17 nodes, bf16, chain, 64 x 64: 28.5 / 27.3, 32.8 / 33.5, 40.0 / 39.0.)
 bool tv_verify_exact_takes(const VerifyArgs& a) {
-  if (a.T > 64 || (a.dk != 64 && a.dk != 128) || (a.dv != 64 && a.dv != 128)) return false;
+  if (a.T > 64 || a.T <= (a.rule == TV_GATED_DELTA ? 16 : 48)) return false;
+  if ((a.dk != 64 && a.dk != 128) || (a.dv != 64 && a.dv != 128)) return false;
   const int64_t items = (int64_t)a.L * a.B * a.H;
   const int sms = tv_sm_count();
   const bool wide = a.dk == 128 && a.dv == 128, narrow = a.dk == 64 && a.dv == 64;
   if (a.rule != TV_GATED_DELTA)
-    return a.T > 48 && (a.bf16 || (a.dv == 128 ? items > 32 : 2 * items > sms && items <= sms));
-  if (a.T <= 16) return false;
+    return a.bf16 || (a.dv == 128 ? items > 32 : 2 * items > sms && items <= sms);
   if (a.bf16) {
     if (a.T > 32) return true;
     if (narrow) return items <= 2 * sms || (items > 3 * sms && items <= 4 * sms);
