@@ -10,7 +10,10 @@
 // (PATHS), or, for trees of any depth, in blocks of 16 columns.
 //
 // Accuracy.  An fp32 operand is three bf16 pieces of 8 mantissa bits each, so a product of two is six products of
-// pieces (the other three lie below 2^-24 of it); bf16 operands are their own only piece.  The tensor core adds into
+// pieces (the other three lie below 2^-24 of it); bf16 operands are their own only piece.  The pieces are those of
+// 2^16 times the value, and the sums are brought back where they are read: bf16 ends at 2^-133, fp32 at 2^-149, and
+// without the factor a value of 2^-120 keeps 14 of its bits.  Values of 2^112 and sums of 2^96 and more leave fp32's range
+// by it and take the way of values that are not finite (below), in fp32 throughout.  The tensor core adds into
 // its fp32 accumulator without rounding to nearest, so the products of the lower pieces go in first, the
 // leading ones on top of them, and the two halves of a contraction over 128 have an accumulator each, added here.
 // Error of a 128 x 128 x 128 product of normal / positive numbers against 64 bits 0.75e-7 / 0.75e-7; one chain of
@@ -43,6 +46,7 @@ using namespace tvtc;
 constexpr int kNodes = 64;
 constexpr int kMaxItems = 32;   // of a CTA
 constexpr int kPath = 16;       // entries of a path list
+constexpr float kUp = 65536.f;  // on every operand that is split into pieces
 
 constexpr int kWorkers = 16;                    // warps; four more: products, tables (two), requests to L2
 constexpr int kThreads = 32 * (kWorkers + 4);
@@ -61,6 +65,8 @@ struct Cfg {
   static constexpr int NR = BF16 && !DELTA ? 1 : 3;     // pieces of R
   static constexpr int KH = DK / 64;                    // halves of the contraction over dk
   static constexpr int NQ = BF16 ? 2 : 1;               // sets of q and k rows
+  static constexpr float kXDown = NP == 3 ? 1.f / (kUp * kUp) : 1.f / kUp;      // the sums, back
+  static constexpr float kLastDown = NR == 3 ? 1.f / (kUp * kUp) : 1.f / kUp;
   static constexpr int CW = DVC / 4;                    // columns of a tile row that a worker thread has
   static constexpr int SU = DVC / 32;                   // 16-byte chunks of the state per thread and half
   // bytes from the 1024-aligned base
@@ -123,9 +129,11 @@ __device__ __forceinline__ float4 ldg_stream(const float* p) {
                : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "l"(p) : "memory");
   return r;
 }
-// A pair of fp32 as three words of two bf16: every piece rounded to nearest, every remainder exact.
+// kUp times a pair of fp32 as three words of two bf16: every piece rounded to nearest, every remainder exact, for any
+// number that the factor does not take past fp32's range (infinite or NaN pieces there).
 __device__ __forceinline__ void split3(Pair x, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
   const Pair minus = pack(-1.f, -1.f);
+  x = mul2(x, pack(kUp, kUp));
   float2 v = unpack(x);
   hi = pack_sat(v.x, v.y);
   x = fma2(pack(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), minus, x);
@@ -608,6 +616,7 @@ verify_exact_kernel(const __grid_constant__ VerifyArgs a, int n_units, int n_spl
             for (int e = 0; e < 4; ++e) {
               float s = __uint_as_float(x[4 * q + e]);
               s += __uint_as_float(y[4 * q + e]);
+              if (!BF16) s *= C::kXDown;   // (q and k both split)
               s *= __uint_as_float(w[e]);
               if (key) s *= be;
               v[e] = (bits >> (4 * q + e)) & 1 ? s : 0.f;   // select, never 0 * x
@@ -800,9 +809,12 @@ verify_exact_kernel(const __grid_constant__ VerifyArgs a, int n_units, int n_spl
           }
           if (!key) {
 #pragma unroll
-            for (int e = 0; e < 16; ++e) {
-              const float s = __uint_as_float(x[e]) + __uint_as_float(y[e]);
-              y[e] = __float_as_uint(P * s);
+            for (int e = 0; e < 16; e += 2) {
+              Pair s = add2(pack(__uint_as_float(x[e]), __uint_as_float(x[e + 1])), pack(__uint_as_float(y[e]), __uint_as_float(y[e + 1])));
+              s = mul2(mul2(s, pack(C::kXDown, C::kXDown)), pack(P, P));
+              const float2 s2 = unpack(s);
+              y[e] = __float_as_uint(s2.x);
+              y[e + 1] = __float_as_uint(s2.y);
             }
           } else {
 #pragma unroll
@@ -815,7 +827,7 @@ verify_exact_kernel(const __grid_constant__ VerifyArgs a, int n_units, int n_spl
                                : pack(__uint_as_float(vv[n % NV]), __uint_as_float(vv[(n + 1) % NV]));
                 if (DELTA) {
                   Pair s = pack(__uint_as_float(x[n]), __uint_as_float(x[n + 1]));
-                  s = add2(s, pack(__uint_as_float(y[n]), __uint_as_float(y[n + 1])));
+                  s = mul2(add2(s, pack(__uint_as_float(y[n]), __uint_as_float(y[n + 1]))), pack(C::kXDown, C::kXDown));
                   rr = mul2(fma2(s, pack(-P, -P), rr), pack(be, be));
                 }
                 if (!node) rr = pack(0.f, 0.f);
@@ -913,7 +925,7 @@ verify_exact_kernel(const __grid_constant__ VerifyArgs a, int n_units, int n_spl
             for (int e = 0; e < 2; ++e) {
               const int k = 4 * g + 2 * e;
               z[e] = pack(__uint_as_float(y[k]), __uint_as_float(y[k + 1]));
-              if (DELTA || !key) z[e] = add2(z[e], pack(__uint_as_float(x[k]), __uint_as_float(x[k + 1])));
+              if (DELTA || !key) z[e] = fma2(pack(__uint_as_float(x[k]), __uint_as_float(x[k + 1])), pack(C::kLastDown, C::kLastDown), z[e]);
               seen = watch(seen, z[e]);
             }
             const float2 z0 = unpack(z[0]), z1 = unpack(z[1]);

@@ -125,6 +125,41 @@ def test_packed_forest_and_strides():
         assert torch.equal(out[0], dense[0]) and torch.equal(out[1], dense[1])
 
 
+@pytest.mark.parametrize("what", ["q", "coefficients", "state and v", "v", "large q", "large state and v"])
+@pytest.mark.parametrize("rule,dtype,T,tree", [(inputs.DELTA, inputs.F32, 64, "frontier"), (inputs.DELTA, inputs.F32, 50, "chain"),
+                                               (inputs.GATED, inputs.F32, 64, "frontier"), (inputs.DELTA, inputs.BF16, 40, "chain")])
+def test_numbers_near_the_ends_of_the_range(rule, dtype, T, tree, what):
+    """The recurrence is linear in q and in (S_pre, v): a power of two on them is the same power on the outputs, and changes no
+    other bit of any sum as long as its terms are normal numbers.  Results down here are some 2^-120; a last place lost
+    to subnormal numbers is 2^-149, less than 2^-24 of a tensor's norm.  bf16 operands are used as they are: 2^-108 on
+    q leaves their scores normal.  What passes 2^112 is worked out row by row in fp32: the tolerance per node."""
+    wl, parents, accepted, tens = _inputs(10, 8, T, rule, tree, dtype)
+    if what in ("coefficients", "v"):
+        tens["S_pre"].zero_()
+    up = {"q": -116, "coefficients": -116, "state and v": -114, "v": -114, "large q": 113, "large state and v": 113}[what]
+    if dtype == inputs.BF16 and up == -116:
+        up = -108
+    if dtype == inputs.BF16:   # nothing that the power leaves with fewer than its 8 bits
+        for n in ("q", "v"):
+            tens[n] = tens[n] * (tens[n].abs() >= 2.0 ** -11)
+    moved = dict(tens)
+    for n in ("q",) if what in ("q", "coefficients", "large q") else ("S_pre", "v"):
+        moved[n] = tens[n] * 2.0 ** up
+        assert torch.isfinite(moved[n]).all()
+    O0, U0 = pu.gpu_round(wl, parents, accepted, tens, impl=tv.IMPL_AUTO)[:2]
+    O, U, _, tree = pu.gpu_round(wl, parents, accepted, moved, impl=tv.IMPL_AUTO)
+    tree.device_status()
+    items = [(0, 0), (4, 3), (9, 7)]
+    f = {n: inputs.to_f64(x) for n, x in moved.items()}
+    ver = orc.verify_batch(f["S_pre"], f["q"], f["k"], f["v"], f["alpha"], f["beta"], parents, wl.rule_name, memo=True, items=items)
+    by_q = what in ("q", "coefficients", "large q")
+    for x, x0, which in ((O, O0, 0),) + (((U, U0, 1),) if rule == inputs.DELTA else ()):
+        got, ref = (np.stack(y) for y in ([x[i] for i in items], [ver[i][which] for i in items]))
+        assert pu.rel_l2_rows(got, ref) <= 1e-5
+        if up < 0:
+            assert pu.rel_fro(x, x0 * (1.0 if by_q and which else 2.0 ** up)) <= 2.0 ** -24
+
+
 @pytest.mark.parametrize("what", ["v", "k", "alpha", "beta", "zero gate", "state"])
 @pytest.mark.parametrize("rule", [inputs.GATED, inputs.DELTA])
 @pytest.mark.parametrize("T,tree", [(50, "frontier"), (49, "chain")])
