@@ -996,9 +996,10 @@ inline int launch(const VerifyArgs& a, int sms, int32_t* status, cudaStream_t st
   const int n_split = a.dv / DVC;
   const int64_t units = (int64_t)a.L * a.B * a.H * n_split;
   if (units > 0x7fffffffLL) return TV_ERR_UNSUPPORTED;
-  // one CTA per SM, more only where one would have more items than it keeps a record of
-  const int64_t fewest = (units + kMaxItems - 1) / kMaxItems;
-  const int64_t grid = units < sms ? units : fewest > sms ? fewest : sms;
+  // One CTA per SM, more only where one would have more items than it keeps a record of: then the same number for every
+  // SM, as no two run on one at the same time (4768 fp32 items of 33 nodes, 64 x 64: 462 us with 149 CTAs, 242 with 296).
+  const int64_t waves = (units + (int64_t)kMaxItems * sms - 1) / ((int64_t)kMaxItems * sms);
+  const int64_t grid = units < sms ? units : waves * sms;
   TV_CUDA_TRY(launch_dependent(verify_exact_kernel<BF16, DELTA, DK, DVC, PATHS>, (int)grid, kThreads,
                                Cfg<BF16, DELTA, DK, DVC>::kSmem, stream, a, (int)units, n_split, status));
   return TV_OK;

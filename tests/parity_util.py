@@ -87,3 +87,33 @@ def compare(wl, O, U, Sn, ver, com, layer=None):
             eU = max(eU, rel_l2_rows(U[idx], Ur))
         eS = max(eS, rel_fro(Sn[idx], com[(b, h)]))
     return eO, eU, eS
+
+
+def kernels_of(call):
+    """(name, blocks) of every kernel that `call` launches, from a captured graph that is not run."""
+    import ctypes
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    drv = ctypes.CDLL("libcuda.so.1")
+
+    class Params(ctypes.Structure):   # CUDA_KERNEL_NODE_PARAMS
+        _fields_ = ([("func", ctypes.c_void_p)] + [(n, ctypes.c_uint) for n in ("gx", "gy", "gz", "bx", "by", "bz", "smem")] +
+                    [(n, ctypes.c_void_p) for n in ("args", "extra", "kern", "ctx")])
+
+    g, n = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t()
+    assert drv.cuGraphGetNodes(g, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert drv.cuGraphGetNodes(g, nodes, ctypes.byref(n)) == 0
+    out = []
+    for node in nodes:
+        kind = ctypes.c_int()
+        assert drv.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value:   # CU_GRAPH_NODE_TYPE_KERNEL is 0
+            continue
+        p, name = Params(), ctypes.c_char_p()
+        assert drv.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)) == 0
+        get, of = (drv.cuFuncGetName, p.func) if p.func else (drv.cuKernelGetName, p.kern)
+        assert get(ctypes.byref(name), ctypes.c_void_p(of)) == 0
+        out.append((name.value.decode(), p.gx * p.gy * p.gz))
+    return out

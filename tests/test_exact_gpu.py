@@ -91,6 +91,22 @@ def test_more_items_than_a_cta_keeps_a_record_of():
     _check(wl, parents, accepted, tens)
 
 
+@pytest.mark.parametrize("full,more", [(0, 1), (1, 0), (1, 1), (32, 0), (32, 1), (33, 5), (64, 0), (64, 1)])
+def test_every_sm_gets_as_many_ctas_as_the_others(full, more):
+    """A CTA takes at most 32 items and an SM to itself; a few CTAs beyond a multiple of the SMs would run alone at the end."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = full * sms + more
+    t = {x: torch.empty(n, 1, 64, d, device="cuda") for x, d in (("S_pre", 64), ("q", 64), ("k", 64), ("v", 64), ("O", 64), ("U", 64))}
+    gates = torch.empty(n, 1, 64, device="cuda")
+    tree = tv.tree_build(np.stack([inputs.tree_chain(64)])).upload()
+    call = lambda: tv.tree_verify(tree, *[t[x] for x in ("S_pre", "q", "k", "v")], gates, gates, rule=tv.DELTA, O=t["O"], U=t["U"])
+    if n < 33:   # the general kernel's
+        tree = tv.tree_build(np.stack([inputs.tree_frontier(64, np.random.default_rng(1))])).upload()
+    (name, grid), = pu.kernels_of(call)
+    assert "verify_exact_kernel" in name
+    assert grid == (n if n < sms else sms * -(-n // (32 * sms)))
+
+
 def test_packed_forest_and_strides():
     """Requests of 1 to 64 nodes, shallow and deep; grouped key heads and token-major rows against dense ones."""
     rng = np.random.default_rng(3)
