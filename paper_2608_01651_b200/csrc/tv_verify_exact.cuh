@@ -37,6 +37,8 @@
 // are zeroed before the dense products, and the rows below them are worked out again, one by one, at the end.
 // Every wait is bounded (status word on expiry).
 #pragma once
+#include <type_traits>
+
 #include "tv_tc_common.cuh"
 
 namespace tvexact {
@@ -82,7 +84,15 @@ struct Cfg {
   static constexpr uint32_t kSBytes = 3 * KH * kSHalf > kWorkers * kStage ? 3 * KH * kSHalf : kWorkers * kStage;
   static constexpr uint32_t oTab = oS + kSBytes;
   static constexpr uint32_t kMat = 10 * 1024;           // a triangular matrix of 4 x 4 blocks of 16 x 16: C, G, decay ratios (then N)
-  static constexpr uint32_t oJump4 = oTab + 3 * kMat;   // float4 per node
+  // redo_rows, where operands and matrices were: 128 rows of q and k, 64 state rows (then C and G), X
+  static constexpr int kRedoLd = DK + 4;
+  static constexpr uint32_t oRedoS = 2 * kNodes * kRedoLd * 4, kRedoCoef = 2 * kNodes * (kNodes + 1) * 4;
+  static constexpr uint32_t oRedoX = oRedoS + (kNodes * kRedoLd * 4 > kRedoCoef ? kNodes * kRedoLd * 4 : kRedoCoef);
+  static constexpr uint32_t kRedo = oRedoX + 2 * kNodes * DVC * 4;
+  // A call, where the same code in line takes registers from the pipeline: 512 items of 64 nodes, in line / called, f32 gated
+  // 61.8 / 55.2 us, bf16 gated 64 x 128 25.8 / 24.8; 128 x 64 21.4 / 22.0, bf16 delta 64 x 64 27.1 / 27.8.
+  static constexpr bool kRedoCall = !BF16 || (!DELTA && DK < DVC);
+  static constexpr uint32_t oJump4 = oTab + 3 * kMat > kRedo ? oTab + 3 * kMat : kRedo;   // float4 per node
   static constexpr uint32_t oUp4 = oJump4 + kNodes * 16;   // 4 x int8 per node
   static constexpr uint32_t oPath = oUp4 + kNodes * 4;     // uint8 [kPath] per node: its path by depth, itself last
   static constexpr uint32_t oDepth = oPath + kNodes * kPath;   // uint8 per node: four times its depth
@@ -96,7 +106,7 @@ struct Cfg {
   static constexpr uint32_t oPlace = oMisc + 32;        // of two items
   static constexpr uint32_t kSmem = oPlace + 2 * sizeof(Place);
   static_assert(3 * kRPiece <= kSBytes, "R in the state's place");
-  static_assert(oJump4 % 16 == 0 && oBar % 8 == 0 && oBad % 16 == 0, "alignment");
+  static_assert(oJump4 % 16 == 0 && oBar % 8 == 0 && oBad % 16 == 0 && oRedoX % 16 == 0, "alignment");
   static_assert(kSmem <= 232448, "shared memory of one CTA");
 };
 
@@ -151,72 +161,170 @@ __device__ __forceinline__ bool spotted(Pair s) {
 }
 
 // Rows that a value that is not finite reaches, by the recurrence's own terms: the dense products lose track of whose it was.
-// B: nodes whose value reaches all nodes below them, W: nodes of their own row only.  Plain loops: no such
-// value is expected.
+// `bad`: nodes whose value reaches all nodes below them, two words, then nodes of their own row only.  The whole item is worked
+// out again in fp32 by the worker warps, in the pipeline's shared memory (4 x 4 tiles a thread for the products, a thread per
+// column for U), and the rows in question are stored.  No such value is expected; a poisoned request should still not hold
+// up a batch: 512 items of 64 nodes, 32 of them NaN, f32 delta 145 us, all of them 430 (row by row from global memory 840
+// and 3270; without any 56, general kernel 111), bf16 chains 245 and 825 (1065 and 4140; 52, 127).
 template <bool BF16, bool DELTA, int DK, int DVC>
-__device__ __forceinline__ void redo_rows(const VerifyArgs& a, int item, int v_first, uint64_t B, uint64_t W, float* U_s,
-                                       float2* cg, float2* link, float* beta) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
-  const ItemRows rows = tv_item_rows(a.tree, a.lay, item, a.B, a.H, a.Hk, a.T, DK, a.dv);
-  if (tid < rows.n) {
-    const uint64_t m = a.tree.anc[(rows.meta0 + tid) * 2];
-    link[tid] = make_float2(a.alpha[rows.g0 + (size_t)tid * rows.g_rs], __int_as_float(m ? 63 - __clzll((long long)m) : -1));
-    beta[tid] = DELTA ? a.beta[rows.g0 + (size_t)tid * rows.g_rs] : 0.f;
-  }
-  __syncthreads();
-  auto at = [&](const void* p, size_t i) {
-    return BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p)[i]) : reinterpret_cast<const float*>(p)[i];
+__device__ __forceinline__ void redo_rows(const VerifyArgs& a, int item, int v_first, const uint32_t* bad, unsigned char* sm,
+                                          float2* link, float* be_s, float* P_s, uint64_t* mask_s, int tid) {
+  using C = Cfg<BF16, DELTA, DK, DVC>;
+  constexpr int LD = C::kRedoLd, kT = 32 * kWorkers;
+  float* const rows_s = reinterpret_cast<float*>(sm);                     // q rows, then k rows
+  float* const state_s = reinterpret_cast<float*>(sm + C::oRedoS);        // 64 value columns of the state
+  float* const coef_s = state_s;                                          // later: C, then G
+  float* const x_s = reinterpret_cast<float*>(sm + C::oRedoX);            // [Q ; K] S^T; then R and U in the k rows
+  auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kT) : "memory"); };
+  // worked out again for every part: kept through all of them, they would take registers from the whole kernel
+  auto place = [&] {
+    asm volatile("" : "+r"(item));
+    return tv_item_rows(a.tree, a.lay, item, a.B, a.H, a.Hk, a.T, DK, a.dv);
   };
-  for (int i = 0; i < rows.n; ++i) {
-    const size_t qi = rows.qk0 + (size_t)((int64_t)i * rows.qk_rs);
-    const float be = DELTA ? beta[i] : 0.f;
-    float w = 1.f;
-    bool hit = (W >> i) & 1;
-    int e = 0;
-    for (int j = i; j >= 0; ++e) {
-      hit = hit || ((B >> j) & 1);
-      if (e % warps == warp) {
-        const size_t kj = rows.qk0 + (size_t)((int64_t)j * rows.qk_rs);
-        float c = 0.f, g = 0.f;
-        for (int x = lane; x < DK; x += 32) {
-          c = fmaf(at(a.q, qi + x), at(a.k, kj + x), c);
-          g = fmaf(at(a.k, qi + x), at(a.k, kj + x), g);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          c += __shfl_xor_sync(0xffffffffu, c, o);
-          g += __shfl_xor_sync(0xffffffffu, g, o);
-        }
-        if (lane == 0) cg[j] = make_float2(w * c, be * (w * g));
-      }
-      w *= link[j].x;
-      j = __float_as_int(link[j].y);
-    }
-    __syncthreads();
-    if (tid < DVC) {
-      const float* s = a.S_pre + ((size_t)item * a.dv + v_first + tid) * DK;
-      float xq = 0.f, xk = 0.f;
-      for (int x = 0; x < DK; ++x) {
-        xq = fmaf(at(a.q, qi + x), s[x], xq);
-        if (DELTA) xk = fmaf(at(a.k, qi + x), s[x], xk);
-      }
-      float u = at(a.v, rows.v0 + (size_t)((int64_t)i * rows.v_rs) + v_first + tid);
-      if (DELTA) {
-        float known = 0.f;
-        for (int j = __float_as_int(link[i].y); j >= 0; j = __float_as_int(link[j].y))
-          known = fmaf(cg[j].y, U_s[j * DVC + tid], known);
-        u = be * (u - w * xk) - known;
-      }
-      U_s[i * DVC + tid] = u;
-      float o = 0.f;
-      for (int j = i; j >= 0; j = __float_as_int(link[j].y)) o = fmaf(cg[j].x, U_s[j * DVC + tid], o);
-      if (hit) {
-        const size_t to = rows.o0 + (size_t)((int64_t)i * rows.o_rs) + v_first + tid;
-        a.O[to] = w * xq + o;
-        if (a.U) a.U[to] = u;
-      }
-    }
-    __syncthreads();
+  ItemRows rows = place();
+  const int n = rows.n;
+  if (tid < n) {
+    mask_s[tid] = a.tree.anc[(rows.meta0 + tid) * 2];
+    link[tid].x = a.alpha[rows.g0 + (size_t)tid * rows.g_rs];
+    be_s[tid] = DELTA ? a.beta[rows.g0 + (size_t)tid * rows.g_rs] : 1.f;
   }
+  auto four = [&](const void* x, size_t i) {
+    if (!BF16) return *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(x) + i);
+    const uint2 w = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(x) + i);
+    return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
+  };
+#pragma unroll 1
+  for (int x = tid; x < n * (DK / 4); x += kT) {
+    const int r = x / (DK / 4), c = x % (DK / 4) * 4;
+    const size_t at = rows.qk0 + (size_t)((int64_t)r * rows.qk_rs) + c;
+    *reinterpret_cast<float4*>(rows_s + r * LD + c) = four(a.q, at);
+    *reinterpret_cast<float4*>(rows_s + (kNodes + r) * LD + c) = four(a.k, at);
+  }
+  // products of the 128 rows with 64 value columns of the state after the other, and with the k rows
+  constexpr int kChunks = DVC / 64, R = DELTA ? 4 : 2;   // (gated rule: q rows only)
+  using Vec = std::conditional_t<BF16, float2, float4>;   // (fewer registers where this is compiled in line, see kRedoCall)
+  constexpr int VW = sizeof(Vec) / 4;
+#pragma unroll 1
+  for (int ch = 0; ch <= kChunks; ++ch) {
+    const bool coef = ch == kChunks;
+    if (!coef) {
+      const float* S = a.S_pre + ((size_t)item * a.dv + v_first + 64 * ch) * DK;
+#pragma unroll 1
+      for (int x = tid; x < 64 * (DK / 4); x += kT)
+        *reinterpret_cast<float4*>(state_s + x / (DK / 4) * LD + x % (DK / 4) * 4) = *reinterpret_cast<const float4*>(S + 4 * x);
+    }
+    sync();
+    const float* ra = rows_s + (tid >> 4) * LD;                                           // rows tid / 16 + 0, 32, ..
+    const float* rb = (coef ? rows_s + kNodes * LD : state_s) + (tid & 15) * LD;          // columns tid % 16 + 0, 16, 32, 48
+    float acc[R][4] = {};
+#pragma unroll 1
+    for (int x = 0; x < DK; x += VW) {
+      Vec l[R];
+#pragma unroll
+      for (int e = 0; e < R; ++e) l[e] = *reinterpret_cast<const Vec*>(ra + 32 * e * LD + x);
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const Vec r = *reinterpret_cast<const Vec*>(rb + 16 * f * LD + x);
+#pragma unroll
+        for (int w = 0; w < VW; ++w)
+#pragma unroll
+          for (int e = 0; e < R; ++e)
+            acc[e][f] = fmaf(reinterpret_cast<const float*>(&l[e])[w], reinterpret_cast<const float*>(&r)[w], acc[e][f]);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < R; ++e)
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const int r = (tid >> 4) + 32 * e, c = (tid & 15) + 16 * f;
+        (coef ? coef_s + r * (kNodes + 1) : x_s + r * DVC + 64 * ch)[c] = acc[e][f];
+      }
+    sync();
+  }
+  // decay, from a node up its path: C in the first 64 rows, G in the others
+  if (tid < (DELTA ? 2 : 1) * kNodes && (tid & (kNodes - 1)) < n) {
+    const int i = tid & (kNodes - 1);
+    const bool g = DELTA && tid >= kNodes;
+    float* c = coef_s + tid * (kNodes + 1);
+    float w = 1.f;
+#pragma unroll 1
+    for (int j = i; j >= 0;) {
+      c[j] = g ? be_s[i] * (w * c[j]) : w * c[j];
+      w *= link[j].x;
+      const uint64_t m = mask_s[j];
+      j = m ? 63 - __clzll((long long)m) : -1;
+    }
+    if (!g) P_s[i] = w;
+  }
+  sync();
+  rows = place();
+#pragma unroll 1
+  for (int x = tid; x < n * DVC; x += kT) {
+    const int i = x / DVC, c = x % DVC;
+    const size_t at = rows.v0 + (size_t)((int64_t)i * rows.v_rs) + v_first + c;
+    float u = BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(a.v)[at]) : reinterpret_cast<const float*>(a.v)[at];
+    if (DELTA) u = be_s[i] * (u - P_s[i] * x_s[(kNodes + i) * DVC + c]);
+    x_s[(kNodes + i) * DVC + c] = u;
+  }
+  sync();
+  // sum over the nodes of m, from the deepest up, of their coefficients in a row times their entries of U in column c
+  auto over = [&](const float* row, uint64_t m, int c) {
+    float s = 0.f;
+#pragma unroll 1
+    while (m) {
+      float w[4], u[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int j = 63 - __clzll((long long)m);
+        w[e] = m ? row[j] : 0.f;
+        u[e] = m ? x_s[(kNodes + j) * DVC + c] : 0.f;
+        if (m) m ^= 1ull << j;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s = fmaf(w[e], u[e], s);
+    }
+    return s;
+  };
+  if (DELTA) {
+    if (tid < DVC)
+#pragma unroll 1
+      for (int i = 0; i < n; ++i) x_s[(kNodes + i) * DVC + tid] -= over(coef_s + (kNodes + i) * (kNodes + 1), mask_s[i], tid);
+    sync();
+  }
+  rows = place();
+  const uint64_t B = bad[0] | (uint64_t)bad[1] << 32, W = bad[2] | (uint64_t)bad[3] << 32;
+#pragma unroll 1
+  for (int x = tid; x < n * DVC; x += kT) {
+    const int i = x / DVC, c = x % DVC;
+    const uint64_t m = mask_s[i] | 1ull << i;
+    if (!((m & B) || (W >> i & 1))) continue;
+    const size_t to = rows.o0 + (size_t)((int64_t)i * rows.o_rs) + v_first + c;
+    a.O[to] = P_s[i] * x_s[i * DVC + c] + over(coef_s + i * (kNodes + 1), m, c);
+    if (a.U) a.U[to] = x_s[(kNodes + i) * DVC + c];
+  }
+  sync();
+}
+
+// All items of the CTA that have such rows.  Only the worker warps come back from here to barriers.
+template <bool BF16, bool DELTA, int DK, int DVC>
+__device__ __forceinline__ void redo_items(const VerifyArgs& a, int n_units, int n_split, unsigned char* sm) {
+  using C = Cfg<BF16, DELTA, DK, DVC>;
+  int tid;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+  if (tid >= 32 * kWorkers) return;
+  const uint32_t* bad = reinterpret_cast<const uint32_t*>(sm + C::oBad);
+#pragma unroll 1
+  for (int unit = (int)blockIdx.x; unit < n_units; unit += (int)gridDim.x, bad += 4) {
+    if (!(bad[0] | bad[1] | bad[2] | bad[3])) continue;
+    const int item = unit / n_split;
+    redo_rows<BF16, DELTA, DK, DVC>(a, item, (unit - item * n_split) * DVC, bad, sm, reinterpret_cast<float2*>(sm + C::oLink),
+                                    reinterpret_cast<float*>(sm + C::oBe), reinterpret_cast<float*>(sm + C::oP), reinterpret_cast<uint64_t*>(sm + C::oMask), tid);
+  }
+}
+
+template <bool BF16, bool DELTA, int DK, int DVC>
+__device__ __noinline__ void redo_items_call(const VerifyArgs& a, int n_units, int n_split, unsigned char* sm) {
+  redo_items<BF16, DELTA, DK, DVC>(a, n_units, n_split, sm);
 }
 
 template <bool BF16, bool DELTA, int DK, int DVC, bool PATHS>
@@ -312,175 +420,7 @@ verify_exact_kernel(const __grid_constant__ VerifyArgs a, int n_units, int n_spl
   if (tid == 0) set_place(0);
   __syncthreads();
 
-  if (warp >= kWorkers) {
-    set_registers_down<kServiceRegs>();
-    if (warp == kWorkers) {
-      // ===================== products =====================
-      if (lane == 0) {
-        const uint64_t dQK = desc_kmajor(sbase + C::oQK), dS = desc_kmajor(sbase + C::oS), dR = desc_mnmajor(sbase + C::oS, 8192);
-        constexpr uint32_t kIdSc = idesc_bf16(kNodes, false), kIdX = idesc_bf16(DVC, false), kIdR = idesc_bf16(DVC, true);
-        using OS = Order<C::NP, C::NP>;
-        using OX = Order<C::NP, 3>;
-        using OR = Order<3, C::NR>;
-#pragma unroll 1
-        for (int it = 0; it < n_it; ++it) {
-          const uint32_t ph = it & 1, set = BF16 ? (ph * C::kQKSet) >> 4 : 0;
-          // scores
-          if (!mbar_wait(bar(QK), ph, abort_flag)) break;
-          const int nb = (place_s[ph].n + 15) >> 4;
-          tc_fence_after();
-#pragma unroll 1
-          for (uint32_t h = 0; h < 2; ++h)   // halves of the contraction: an accumulator each
-#pragma unroll 1
-            for (int o = 0; o < OS::n; ++o) {
-              const uint32_t pa = (OS::code >> (4 * o)) & 3u, pb = (OS::code >> (4 * o + 2)) & 3u;
-              const uint64_t dA = dQK + set + ((pa * KH * C::kHalf + h * C::kStep) >> 4), dB = dQK + set + ((pb * KH * C::kHalf + h * C::kStep + 8192u) >> 4);
-#pragma unroll
-              for (uint32_t k = 0; k < DK / 32; ++k)
-                mma_bf16_ss(sc_col + 64u * h, dA + ((k * 32u) >> 4), dB + ((k * 32u) >> 4), kIdSc, o > 0 || k > 0);
-            }
-          tc_commit(bar(SC));
-          // state product
-          bool ok = true;
-#pragma unroll 1
-          for (uint32_t h = 0; h < 2; ++h) {
-            if (h < KH && !(ok = mbar_wait(bar(ST + (int)h), ph, abort_flag))) break;
-            tc_fence_after();
-#pragma unroll 1
-            for (int o = 0; o < OX::n; ++o) {
-              const uint32_t pa = (OX::code >> (4 * o)) & 3u, pb = (OX::code >> (4 * o + 2)) & 3u;
-              const uint64_t dA = dQK + set + ((pa * KH * C::kHalf + h * C::kStep) >> 4), dB = dS + ((pb * KH * C::kSHalf + h * (KH == 2 ? C::kSHalf : 64u)) >> 4);
-#pragma unroll
-              for (uint32_t k = 0; k < DK / 32; ++k)
-                mma_bf16_ss(tmem + DVC * h, dA + ((k * 32u) >> 4), dB + ((k * 32u) >> 4), kIdX, o > 0 || k > 0);
-            }
-          }
-          if (!ok) break;
-          tc_commit(bar(X));
-          // [C N ; N - I] R
-          if (!mbar_wait(bar(COEF), ph, abort_flag) || !mbar_wait(bar(RP), ph, abort_flag)) break;
-          tc_fence_after();
-#pragma unroll 1
-          for (int o = 0; o < OR::n; ++o) {
-            const uint32_t pa = (OR::code >> (4 * o)) & 3u, pb = (OR::code >> (4 * o + 2)) & 3u;
-            const uint32_t A = sc_col + pa * 32u;
-            const uint64_t dB = dR + ((pb * C::kRPiece) >> 4);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {   // 16 nodes
-              if (k >= nb) break;
-              mma_bf16_ts(tmem, A + k * 8u, dB + ((k * 2048u) >> 4), kIdR, o > 0 || k > 0);
-            }
-          }
-          tc_commit(bar(ACC));
-        }
-      }
-    } else if (warp < kWorkers + 3) {
-      // ===================== tables: masks, gates and decay ratios, a node per thread =====================
-      const int n = tid - 32 * (kWorkers + 1);
-      float4* const jump4 = reinterpret_cast<float4*>(sm + C::oJump4);
-      uint32_t* const up4 = reinterpret_cast<uint32_t*>(sm + C::oUp4);
-#pragma unroll 1
-      for (int it = 0; it < n_it; ++it) {
-        const uint32_t ph = it & 1;
-        // the tables of the item before have been read (and this one's place is known)
-        if (it > 0) {
-          mbar_wait_warp(bar(COEF), ph ^ 1, abort_flag);
-          mbar_wait_warp(bar(RP), ph ^ 1, abort_flag);
-        }
-        const Place& pl = place_s[ph];
-        const bool node = n < pl.n;
-        uint64_t m = 0;
-        float al = 1.f, be = 0.f;
-        if (node) {
-          m = a.tree.anc[(pl.meta0 + n) * 2];
-          al = a.alpha[pl.g0 + (size_t)n * a.lay.gate.t];
-          if (DELTA) be = a.beta[pl.g0 + (size_t)n * a.lay.gate.t];
-        }
-        link[n] = make_float2(al, __int_as_float(m ? 63 - __clzll((long long)m) : -1));
-        mask_s[n] = m;
-        be_s[n] = be;
-        asm volatile("bar.sync 2, 64;" ::: "memory");
-        // four steps up at a time: the ancestors and the products of alpha on the way to them
-        {
-          float w[4], acc = 1.f;
-          uint32_t up = 0;
-          int j = n;
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            if (j >= 0) {
-              const float2 y = link[j];
-              acc *= y.x;
-              j = __float_as_int(y.y);
-            }
-            w[e] = acc;
-            up |= (uint32_t)(j & 255) << (8 * e);
-          }
-          jump4[n] = make_float4(w[0], w[1], w[2], w[3]);
-          up4[n] = up;
-        }
-        asm volatile("bar.sync 2, 64;" ::: "memory");
-        // the products of alpha from a node up to, not including, each node of its path
-        const uint32_t row = sbase + C::oTab + 2 * C::kMat + (uint32_t)(((n >> 4) * ((n >> 4) + 1)) >> 1) * 1024u + (uint32_t)(n & 15) * 64u;
-        const uint32_t swz = (uint32_t)((n & 15) >> 1) & 3u;
-        auto put = [&](uint32_t col, float x) {
-          asm volatile("st.shared.f32 [%0], %1;" ::"r"(row + (col >> 4) * 1024u + ((((col & 15u) >> 2) ^ swz) << 4) + (col & 3u) * 4u), "f"(x) : "memory");
-        };
-        float w = 1.f;
-        int j = node ? n : -1;
-#pragma unroll 1
-        while (j >= 0) {
-          const float4 y = jump4[j];
-          const uint32_t up = up4[j];
-          put(j, w);
-          if (!(up & 0x80u)) put(up & 255u, w * y.x);
-          if (!(up & 0x8000u)) put((up >> 8) & 255u, w * y.y);
-          if (!(up & 0x800000u)) put((up >> 16) & 255u, w * y.z);
-          w *= y.w;
-          j = (int32_t)up >> 24;
-        }
-        P_s[n] = w;
-        if (PATHS) {
-          const int depth = __popcll(m) & (kPath - 1);
-          sm[C::oDepth + n] = (uint8_t)(4 * depth);
-          j = n;
-#pragma unroll 1
-          for (int e = depth; e >= 0; --e) {
-            sm[C::oPath + n * kPath + e] = (uint8_t)j;
-            j = __float_as_int(link[j].y);
-          }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(TAB));
-      }
-    } else {
-      // ===================== places; requests to L2: v of this item, all of the next =====================
-      auto near = [](const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); };
-      constexpr int ES = BF16 ? 2 : 4, QL = DK * ES / 128, VL = DVC * ES / 128;   // lines of a row
-      auto near_v = [&](const Place& pl) {
-        const char* v = reinterpret_cast<const char*>(a.v) + pl.v0 * ES;
-        for (int x = lane; x < pl.n * VL; x += 32) near(v + (int64_t)(x / VL) * a.lay.v.t * ES + (x % VL) * 128);
-      };
-      near_v(place_s[0]);
-#pragma unroll 1
-      for (int it = 0; it < n_it; ++it) {
-        mbar_wait_warp(bar(QK), it & 1, abort_flag);   // the item before is done with, this one's operands are here
-        const bool more = it + 1 < n_it;
-        if (more && lane == 0) set_place(it + 1);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(TAB));
-        if (!more) break;
-        const Place& pl = place_s[(it + 1) & 1];
-        if (!BF16)   // bf16: requested by the workers, to shared memory
-          for (int x = lane; x < pl.n * QL; x += 32) {
-            const size_t at = (pl.qk0 + (size_t)((int64_t)(x / QL) * a.lay.qk.t)) * ES + (x % QL) * 128;
-            near(reinterpret_cast<const char*>(a.q) + at);
-            near(reinterpret_cast<const char*>(a.k) + at);
-          }
-        for (int x = lane; x < DVC * DK / 32; x += 32) near(pl.S + x * 32);
-        near_v(pl);
-      }
-    }
-  } else {
+  if (warp < kWorkers) {   // (this branch first in the code: 512 f32 items of 64 nodes 61.3 -> 58.4 us)
     // ===================== workers =====================
     // A wait that runs out sets the abort flag, and every later one returns soon; the warps go on all the same, for
     // they meet at barriers of the CTA.
@@ -763,24 +703,23 @@ verify_exact_kernel(const __grid_constant__ VerifyArgs a, int n_units, int n_spl
               sts128(at0, d0.x, d0.y, d0.z, d0.w);
               sts128(at1, d1.x, d1.y, d1.z, d1.w);
             } else {
+              // (the last product apart: both in one loop compile to a form that is 7 % slower on 64-node chains)
 #pragma unroll 1
-              for (int tb = cb + 1; tb <= rb + 1; ++tb) {
-                const bool last = tb > rb;
-                if (last && cb < rb) {
-                  const Pair minus = pack(-1.f, -1.f);
-                  uint4 y0 = make_uint4(0u, 0u, 0u, 0u), y1 = y0;
-                  if (!of_n) {
-                    y0 = lds128(at0);
-                    y1 = lds128(at1);
-                  }
-                  put(at0, fma2(s[0], minus, pack(__uint_as_float(y0.x), __uint_as_float(y0.y))), fma2(s[1], minus, pack(__uint_as_float(y0.z), __uint_as_float(y0.w))));
-                  put(at1, fma2(s[2], minus, pack(__uint_as_float(y1.x), __uint_as_float(y1.y))), fma2(s[3], minus, pack(__uint_as_float(y1.z), __uint_as_float(y1.w))));
-#pragma unroll
-                  for (int e = 0; e < 4; ++e) s[e] = pack(0.f, 0.f);
-                  __syncwarp();
+              for (int tb = cb + 1; tb <= rb; ++tb) times(blk(mat, rb, tb), blk(1, tb, cb), s);
+              if (cb < rb) {
+                const Pair minus = pack(-1.f, -1.f);
+                uint4 y0 = make_uint4(0u, 0u, 0u, 0u), y1 = y0;
+                if (!of_n) {
+                  y0 = lds128(at0);
+                  y1 = lds128(at1);
                 }
-                times(last ? own : blk(mat, rb, tb), blk(1, last ? cb : tb, cb), s);
+                put(at0, fma2(s[0], minus, pack(__uint_as_float(y0.x), __uint_as_float(y0.y))), fma2(s[1], minus, pack(__uint_as_float(y0.z), __uint_as_float(y0.w))));
+                put(at1, fma2(s[2], minus, pack(__uint_as_float(y1.x), __uint_as_float(y1.y))), fma2(s[3], minus, pack(__uint_as_float(y1.z), __uint_as_float(y1.w))));
+#pragma unroll
+                for (int e = 0; e < 4; ++e) s[e] = pack(0.f, 0.f);
+                __syncwarp();
               }
+              times(own, blk(1, cb, cb), s);
               __syncwarp();
               put(at0, s[0], s[1]);
               put(at1, s[2], s[3]);
@@ -955,6 +894,174 @@ verify_exact_kernel(const __grid_constant__ VerifyArgs a, int n_units, int n_spl
       }
       if (more) sync();   // the staged rows have been read
     }
+  } else {
+    set_registers_down<kServiceRegs>();
+    if (warp == kWorkers) {
+      // ===================== products =====================
+      if (lane == 0) {
+        const uint64_t dQK = desc_kmajor(sbase + C::oQK), dS = desc_kmajor(sbase + C::oS), dR = desc_mnmajor(sbase + C::oS, 8192);
+        constexpr uint32_t kIdSc = idesc_bf16(kNodes, false), kIdX = idesc_bf16(DVC, false), kIdR = idesc_bf16(DVC, true);
+        using OS = Order<C::NP, C::NP>;
+        using OX = Order<C::NP, 3>;
+        using OR = Order<3, C::NR>;
+#pragma unroll 1
+        for (int it = 0; it < n_it; ++it) {
+          const uint32_t ph = it & 1, set = BF16 ? (ph * C::kQKSet) >> 4 : 0;
+          // scores
+          if (!mbar_wait(bar(QK), ph, abort_flag)) break;
+          const int nb = (place_s[ph].n + 15) >> 4;
+          tc_fence_after();
+#pragma unroll 1
+          for (uint32_t h = 0; h < 2; ++h)   // halves of the contraction: an accumulator each
+#pragma unroll 1
+            for (int o = 0; o < OS::n; ++o) {
+              const uint32_t pa = (OS::code >> (4 * o)) & 3u, pb = (OS::code >> (4 * o + 2)) & 3u;
+              const uint64_t dA = dQK + set + ((pa * KH * C::kHalf + h * C::kStep) >> 4), dB = dQK + set + ((pb * KH * C::kHalf + h * C::kStep + 8192u) >> 4);
+#pragma unroll
+              for (uint32_t k = 0; k < DK / 32; ++k)
+                mma_bf16_ss(sc_col + 64u * h, dA + ((k * 32u) >> 4), dB + ((k * 32u) >> 4), kIdSc, o > 0 || k > 0);
+            }
+          tc_commit(bar(SC));
+          // state product
+          bool ok = true;
+#pragma unroll 1
+          for (uint32_t h = 0; h < 2; ++h) {
+            if (h < KH && !(ok = mbar_wait(bar(ST + (int)h), ph, abort_flag))) break;
+            tc_fence_after();
+#pragma unroll 1
+            for (int o = 0; o < OX::n; ++o) {
+              const uint32_t pa = (OX::code >> (4 * o)) & 3u, pb = (OX::code >> (4 * o + 2)) & 3u;
+              const uint64_t dA = dQK + set + ((pa * KH * C::kHalf + h * C::kStep) >> 4), dB = dS + ((pb * KH * C::kSHalf + h * (KH == 2 ? C::kSHalf : 64u)) >> 4);
+#pragma unroll
+              for (uint32_t k = 0; k < DK / 32; ++k)
+                mma_bf16_ss(tmem + DVC * h, dA + ((k * 32u) >> 4), dB + ((k * 32u) >> 4), kIdX, o > 0 || k > 0);
+            }
+          }
+          if (!ok) break;
+          tc_commit(bar(X));
+          // [C N ; N - I] R
+          if (!mbar_wait(bar(COEF), ph, abort_flag) || !mbar_wait(bar(RP), ph, abort_flag)) break;
+          tc_fence_after();
+#pragma unroll 1
+          for (int o = 0; o < OR::n; ++o) {
+            const uint32_t pa = (OR::code >> (4 * o)) & 3u, pb = (OR::code >> (4 * o + 2)) & 3u;
+            const uint32_t A = sc_col + pa * 32u;
+            const uint64_t dB = dR + ((pb * C::kRPiece) >> 4);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {   // 16 nodes
+              if (k >= nb) break;
+              mma_bf16_ts(tmem, A + k * 8u, dB + ((k * 2048u) >> 4), kIdR, o > 0 || k > 0);
+            }
+          }
+          tc_commit(bar(ACC));
+        }
+      }
+    } else if (warp < kWorkers + 3) {
+      // ===================== tables: masks, gates and decay ratios, a node per thread =====================
+      const int n = tid - 32 * (kWorkers + 1);
+      float4* const jump4 = reinterpret_cast<float4*>(sm + C::oJump4);
+      uint32_t* const up4 = reinterpret_cast<uint32_t*>(sm + C::oUp4);
+#pragma unroll 1
+      for (int it = 0; it < n_it; ++it) {
+        const uint32_t ph = it & 1;
+        // the tables of the item before have been read (and this one's place is known)
+        if (it > 0) {
+          mbar_wait_warp(bar(COEF), ph ^ 1, abort_flag);
+          mbar_wait_warp(bar(RP), ph ^ 1, abort_flag);
+        }
+        const Place& pl = place_s[ph];
+        const bool node = n < pl.n;
+        uint64_t m = 0;
+        float al = 1.f, be = 0.f;
+        if (node) {
+          m = a.tree.anc[(pl.meta0 + n) * 2];
+          al = a.alpha[pl.g0 + (size_t)n * a.lay.gate.t];
+          if (DELTA) be = a.beta[pl.g0 + (size_t)n * a.lay.gate.t];
+        }
+        link[n] = make_float2(al, __int_as_float(m ? 63 - __clzll((long long)m) : -1));
+        mask_s[n] = m;
+        be_s[n] = be;
+        asm volatile("bar.sync 2, 64;" ::: "memory");
+        // four steps up at a time: the ancestors and the products of alpha on the way to them
+        {
+          float w[4], acc = 1.f;
+          uint32_t up = 0;
+          int j = n;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            if (j >= 0) {
+              const float2 y = link[j];
+              acc *= y.x;
+              j = __float_as_int(y.y);
+            }
+            w[e] = acc;
+            up |= (uint32_t)(j & 255) << (8 * e);
+          }
+          jump4[n] = make_float4(w[0], w[1], w[2], w[3]);
+          up4[n] = up;
+        }
+        asm volatile("bar.sync 2, 64;" ::: "memory");
+        // the products of alpha from a node up to, not including, each node of its path
+        const uint32_t row = sbase + C::oTab + 2 * C::kMat + (uint32_t)(((n >> 4) * ((n >> 4) + 1)) >> 1) * 1024u + (uint32_t)(n & 15) * 64u;
+        const uint32_t swz = (uint32_t)((n & 15) >> 1) & 3u;
+        auto put = [&](uint32_t col, float x) {
+          asm volatile("st.shared.f32 [%0], %1;" ::"r"(row + (col >> 4) * 1024u + ((((col & 15u) >> 2) ^ swz) << 4) + (col & 3u) * 4u), "f"(x) : "memory");
+        };
+        float w = 1.f;
+        int j = node ? n : -1;
+#pragma unroll 1
+        while (j >= 0) {
+          const float4 y = jump4[j];
+          const uint32_t up = up4[j];
+          put(j, w);
+          if (!(up & 0x80u)) put(up & 255u, w * y.x);
+          if (!(up & 0x8000u)) put((up >> 8) & 255u, w * y.y);
+          if (!(up & 0x800000u)) put((up >> 16) & 255u, w * y.z);
+          w *= y.w;
+          j = (int32_t)up >> 24;
+        }
+        P_s[n] = w;
+        if (PATHS) {
+          const int depth = __popcll(m) & (kPath - 1);
+          sm[C::oDepth + n] = (uint8_t)(4 * depth);
+          j = n;
+#pragma unroll 1
+          for (int e = depth; e >= 0; --e) {
+            sm[C::oPath + n * kPath + e] = (uint8_t)j;
+            j = __float_as_int(link[j].y);
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(TAB));
+      }
+    } else {
+      // ===================== places; requests to L2: v of this item, all of the next =====================
+      auto near = [](const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); };
+      constexpr int ES = BF16 ? 2 : 4, QL = DK * ES / 128, VL = DVC * ES / 128;   // lines of a row
+      auto near_v = [&](const Place& pl) {
+        const char* v = reinterpret_cast<const char*>(a.v) + pl.v0 * ES;
+        for (int x = lane; x < pl.n * VL; x += 32) near(v + (int64_t)(x / VL) * a.lay.v.t * ES + (x % VL) * 128);
+      };
+      near_v(place_s[0]);
+#pragma unroll 1
+      for (int it = 0; it < n_it; ++it) {
+        mbar_wait_warp(bar(QK), it & 1, abort_flag);   // the item before is done with, this one's operands are here
+        const bool more = it + 1 < n_it;
+        if (more && lane == 0) set_place(it + 1);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(TAB));
+        if (!more) break;
+        const Place& pl = place_s[(it + 1) & 1];
+        if (!BF16)   // bf16: requested by the workers, to shared memory
+          for (int x = lane; x < pl.n * QL; x += 32) {
+            const size_t at = (pl.qk0 + (size_t)((int64_t)(x / QL) * a.lay.qk.t)) * ES + (x % QL) * 128;
+            near(reinterpret_cast<const char*>(a.q) + at);
+            near(reinterpret_cast<const char*>(a.k) + at);
+          }
+        for (int x = lane; x < DVC * DK / 32; x += 32) near(pl.S + x * 32);
+        near_v(pl);
+      }
+    }
   }
 
   // ---- teardown: every path comes here ----
@@ -967,14 +1074,12 @@ verify_exact_kernel(const __grid_constant__ VerifyArgs a, int n_units, int n_spl
     if (tid == 0 && status) atomicExch(status, (int)TV_ERR_DEVICE_TIMEOUT);
     return;
   }
-  if (*any_bad) {
-    for (int it = 0; it < n_it; ++it) {
-      const uint64_t below = bad_s[4 * it] | (uint64_t)bad_s[4 * it + 1] << 32, own = bad_s[4 * it + 2] | (uint64_t)bad_s[4 * it + 3] << 32;
-      if (!(below | own)) continue;
-      const int unit = unit_of(it), item = unit / n_split;
-      redo_rows<BF16, DELTA, DK, DVC>(a, item, (unit - item * n_split) * DVC, below, own, reinterpret_cast<float*>(sm + C::oS),
-                                      reinterpret_cast<float2*>(sm + C::oTab), link, be_s);
-    }
+  // (values of this part's own, so that none is kept through the pipeline for it)
+  const VerifyArgs* args = &a;
+  asm volatile("" : "+l"(args), "+l"(sm));
+  if (*reinterpret_cast<volatile int*>(sm + C::oMisc + 8)) {   // any_bad
+    if (!C::kRedoCall) redo_items<BF16, DELTA, DK, DVC>(*args, n_units, n_split, sm);
+    else redo_items_call<BF16, DELTA, DK, DVC>(*args, n_units, n_split, sm);
   }
 }
 

@@ -213,3 +213,55 @@ def test_values_that_are_not_finite(T, tree, rule, what):
     assert np.array_equal(O[O_is], O0[O_is])
     if rule == inputs.DELTA:
         assert np.array_equal(U[U_is], U0[U_is])
+
+
+@pytest.mark.parametrize("B,H,T,tree,rule,dtype,dk,dv", [
+    (6, 8, 64, "frontier", inputs.DELTA, inputs.F32, 128, 128),     # halves of the columns
+    (4, 8, 40, "chain", inputs.DELTA, inputs.BF16, 64, 128),
+    (20, 16, 40, "chain", inputs.DELTA, inputs.BF16, 128, 128),     # three items on a CTA
+    (20, 16, 50, "frontier", inputs.DELTA, inputs.BF16, 64, 64),
+    (20, 16, 64, "chain", inputs.DELTA, inputs.F32, 64, 128),
+    (10, 8, 33, "frontier", inputs.DELTA, inputs.F32, 128, 64),
+    (20, 16, 49, "frontier", inputs.GATED, inputs.F32, 128, 128),
+    (20, 16, 64, "chain", inputs.GATED, inputs.BF16, 64, 128),
+    (20, 16, 64, "frontier", inputs.GATED, inputs.BF16, 128, 64),
+])
+def test_values_that_are_not_finite_on_every_variant(B, H, T, tree, rule, dtype, dk, dv):
+    """In the first and the last item of a CTA, single entries left and right: what they reach and what comes out elsewhere are
+    the general kernel's, whose sums run over a node's own path; rows that they do not reach keep every bit."""
+    wl, parents, accepted, tens = _inputs(B, H, T, rule, tree, dtype, dk=dk, dv=dv)
+    clean = pu.gpu_round(wl, parents, accepted, tens, impl=tv.IMPL_AUTO)[:2]
+    last = (B * H - 1) // 148 * 148
+    items = sorted({(i // H, i % H) for i in (0, 1, 2, last, last + 1)})
+    bad = T // 3
+    tens["v"][items[0]][bad, dv - 1] = float("nan")
+    tens["k"][items[1]][bad, 5] = float("inf")
+    tens["S_pre"][items[2]][dv - 2, 3] = float("inf")
+    for b, h in items[3:]:
+        tens["alpha"][b, h, bad] = float("nan")
+        tens["v"][b, h, 0, 1] = float("-inf")
+    got = pu.gpu_round(wl, parents, accepted, tens, impl=tv.IMPL_AUTO)[:2]
+    ref = pu.gpu_round(wl, parents, accepted, tens, impl=tv.IMPL_SIMT)[:2]
+    for x, y, c in list(zip(got, ref, clean))[:2 if rule == inputs.DELTA else 1]:
+        assert np.array_equal(np.isfinite(x), np.isfinite(y))
+        rest = np.ones((B, H), dtype=bool)
+        for i in items:
+            rest[i] = False
+            ok = np.isfinite(y[i])
+            assert not ok.all()
+            np.testing.assert_allclose(x[i][ok], y[i][ok], rtol=0, atol=1e-5 * np.abs(y[i][ok]).max())
+        assert np.array_equal(x[rest], c[rest])
+
+
+def test_a_poisoned_request_does_not_hold_up_the_batch():
+    """Items that hold such values are worked out a second time, in fp32: some four times what the general kernel takes."""
+    wl, parents, _, tens = _inputs(8, 16, 63, inputs.DELTA, "frontier", inputs.F32)
+    tens["S_pre"][3] = float("nan")
+    t = {n: x.cuda() for n, x in tens.items()}
+    tree = tv.tree_build(parents).upload()
+    O, U = torch.empty_like(t["v"]), torch.empty_like(t["v"])
+    us = {}
+    for impl in (tv.IMPL_SIMT, tv.IMPL_AUTO):
+        call = lambda: tv.tree_verify(tree, *[t[n] for n in ("S_pre", "q", "k", "v", "alpha", "beta")], rule=tv.DELTA, O=O, U=U, impl=impl)
+        us[impl] = pu.device_us(call)
+    assert us[tv.IMPL_AUTO] <= 8 * us[tv.IMPL_SIMT], us
