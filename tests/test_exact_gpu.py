@@ -107,6 +107,25 @@ def test_every_sm_gets_as_many_ctas_as_the_others(full, more):
     assert grid == (n if n < sms else sms * -(-n // (32 * sms)))
 
 
+@pytest.mark.parametrize("rule,dtype,tree,T,dk,dv,line", [
+    (inputs.DELTA, inputs.F32, "chain", 24, 64, 64, "half"), (inputs.DELTA, inputs.F32, "chain", 32, 128, 64, "half"),
+    (inputs.DELTA, inputs.F32, "chain", 17, 64, 128, "quarter"), (inputs.DELTA, inputs.F32, "chain", 32, 128, 128, "quarter"),
+    (inputs.GATED, inputs.F32, "chain", 56, 64, 128, "quarter"), (inputs.GATED, inputs.F32, "frontier", 64, 128, 128, "quarter"),
+    (inputs.GATED, inputs.F32, "chain", 49, 128, 64, "half"), (inputs.DELTA, inputs.F32, "frontier", 29, 128, 128, 2),
+    (inputs.DELTA, inputs.F32, "frontier", 32, 64, 64, 2)])
+def test_the_general_kernel_keeps_few_items(rule, dtype, tree, T, dk, dv, line):
+    """As long as the general kernel has an SM for every part of an item's columns (four of 128, two of 64), and on one or
+    two small trees, it is the faster one: 7.7 us against 8.6 on 64 chains of 24 nodes, 64 x 64."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = {"half": sms // 2, "quarter": sms // 4}.get(line, line)
+    trees = tv.tree_build(np.stack([inputs.tree_chain(T) if tree == "chain" else inputs.tree_frontier(T, np.random.default_rng(T))])).upload()
+    for items, name in ((n, "verify_simt"), (n + 1, "verify_exact")):
+        t = [torch.empty(items, 1, r, d, device="cuda") for r, d in ((dv, dk), (T, dk), (T, dk), (T, dv))]
+        gates, O = torch.empty(items, 1, T, device="cuda"), torch.empty(items, 1, T, dv, device="cuda")
+        launched = pu.kernels_of(lambda: tv.tree_verify(trees, *t, gates, gates if rule else None, rule=rule, O=O))
+        assert len(launched) == 1 and name in launched[0][0], (items, launched)
+
+
 def test_packed_forest_and_strides():
     """Requests of 1 to 64 nodes, shallow and deep; grouped key heads and token-major rows against dense ones."""
     rng = np.random.default_rng(3)
