@@ -46,6 +46,7 @@ bool tv_verify_exact_takes(const VerifyArgs& a) {
   const int64_t items = (int64_t)a.L * a.B * a.H;
   const int sms = tv_sm_count();
   const bool wide = a.dk == 128 && a.dv == 128, narrow = a.dk == 64 && a.dv == 64;
+  if (a.bf16 && wide && (a.rule != TV_GATED_DELTA || a.tree.max_depth_all < 16)) return false;   // the gated and the delta kernel's
   const bool crowded = a.dv == 128 ? 4 * items > sms : 2 * items > sms;   // more CTAs of the general kernel than SMs
   if (a.rule != TV_GATED_DELTA) return a.bf16 || (crowded && (a.dv == 128 || items <= sms));
   if (a.bf16) {

@@ -1110,6 +1110,10 @@ inline int launch(const VerifyArgs& a, int sms, int32_t* status, cudaStream_t st
   return TV_OK;
 }
 
+// bf16 operands at 128 x 128 come here for deep trees under the delta rule only: other kernels take the rest.
+template <bool BF16, bool DELTA, bool PATHS>
+constexpr bool kHasWide = !BF16 || (DELTA && !PATHS);
+
 template <bool BF16, bool DELTA, bool PATHS>
 inline int launch_width(const VerifyArgs& a, int32_t* status, cudaStream_t stream) {
   const int sms = tv_sm_count();
@@ -1118,7 +1122,9 @@ inline int launch_width(const VerifyArgs& a, int32_t* status, cudaStream_t strea
   const bool halves = a.dv == 64 || 2 * (int64_t)a.L * a.B * a.H <= sms;
   if (a.dk == 64)
     return halves ? launch<BF16, DELTA, 64, 64, PATHS>(a, sms, status, stream) : launch<BF16, DELTA, 64, 128, PATHS>(a, sms, status, stream);
-  return halves ? launch<BF16, DELTA, 128, 64, PATHS>(a, sms, status, stream) : launch<BF16, DELTA, 128, 128, PATHS>(a, sms, status, stream);
+  if (halves) return launch<BF16, DELTA, 128, 64, PATHS>(a, sms, status, stream);
+  if constexpr (kHasWide<BF16, DELTA, PATHS>) return launch<BF16, DELTA, 128, 128, PATHS>(a, sms, status, stream);
+  return TV_ERR_UNSUPPORTED;
 }
 template <bool BF16>
 inline int launch_any(const VerifyArgs& a, int32_t* status, cudaStream_t stream) {
@@ -1130,7 +1136,8 @@ inline int prepare_width() {
   int st = prepare<BF16, DELTA, 64, 64, PATHS>();
   if (st == TV_OK) st = prepare<BF16, DELTA, 64, 128, PATHS>();
   if (st == TV_OK) st = prepare<BF16, DELTA, 128, 64, PATHS>();
-  if (st == TV_OK) st = prepare<BF16, DELTA, 128, 128, PATHS>();
+  if constexpr (kHasWide<BF16, DELTA, PATHS>)
+    if (st == TV_OK) st = prepare<BF16, DELTA, 128, 128, PATHS>();
   return st;
 }
 // The callers of tv_prepare_verify_exact do not know the depth.

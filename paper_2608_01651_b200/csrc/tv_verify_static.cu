@@ -34,8 +34,10 @@ tree_meta_static_kernel(const int32_t* __restrict__ parent, int32_t n, uint64_t*
   __shared__ int32_t par_s[TV_MAX_NODES];
   __shared__ int32_t max_s;
   const int t = blockIdx.x, i = threadIdx.x;
-  // a verify kernel launched behind this one may be scheduled now and set itself up; it waits
-  // for this grid to finish before it reads global memory
+  // A verify kernel launched behind this one may be scheduled now and set itself up.  It waits for this grid to
+  // finish before it reads anything that this one writes; the state, which the general kernel and those on the tensor
+  // cores ask for earlier, is safe to read because this grid is an ordinary launch: it starts only when all older work
+  // on the stream is done.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   bool bad = false;
   if (i == 0) max_s = 0;
