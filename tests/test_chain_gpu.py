@@ -9,6 +9,7 @@ import torch
 
 import paper_2608_01651_b200 as tv
 from paper_2608_01651_b200 import inputs
+from tests import parity_util as pu
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -78,8 +79,9 @@ def test_unsynchronised_rounds_equal_synchronised_ones(name, B, H, T, rule, impl
 
 
 @pytest.mark.parametrize("rule", [tv.GATED, tv.DELTA])
-@pytest.mark.parametrize("d,T", [(64, 64), (128, 64), (64, 128), (128, 128)])
-def test_commit_that_rejects_every_request_keeps_the_order(d, T, rule):
+@pytest.mark.parametrize("d,T,impl", [(64, 64, tv.IMPL_SIMT), (128, 64, tv.IMPL_SIMT), (64, 128, tv.IMPL_SIMT), (128, 128, tv.IMPL_SIMT),
+                                      (64, 64, tv.IMPL_AUTO), (128, 64, tv.IMPL_AUTO)])
+def test_commit_that_rejects_every_request_keeps_the_order(d, T, impl, rule):
     """verify -> in-place commit in which no request accepts anything -> other trees -> verify, queued
     without synchronisation.  The commit has nothing to do, and must still not end before the verify in
     front of it: the upload behind it waits for the commit only and then overwrites the masks."""
@@ -98,7 +100,7 @@ def test_commit_that_rejects_every_request_keeps_the_order(d, T, rule):
         for r in range(2):
             tree.rebuild(trees[r]).upload(); pause()
             tv.tree_verify(tree, S, t["q"], t["k"], t["v"], t["alpha"], t["beta"], rule=rule, O=outs[2 * r],
-                           U=outs[2 * r + 1], impl=tv.IMPL_SIMT); pause()
+                           U=outs[2 * r + 1], impl=impl); pause()
             tv.commit_path(tree, none, S, t["k"], t["v"], t["alpha"], t["beta"], rule=rule, U=outs[2 * r + 1]); pause()
         tree.rebuild(trees[0]).upload()      # over the masks of the last verify
         torch.cuda.synchronize()
@@ -139,10 +141,36 @@ def test_queued_rounds_of_the_general_kernel(tree, T, d, dtype, B, H, rule):
     _compare(_round_calls(wl, rule, tv.IMPL_SIMT))
 
 
+@pytest.mark.parametrize("tree,T,dk,dv,dtype,B,H,rule", [
+    ("frontier", 63, 128, 128, inputs.F32, 9, 16, tv.DELTA),     # path form, whole columns
+    ("frontier", 63, 128, 128, inputs.F32, 16, 16, tv.DELTA),    # two items on a CTA
+    ("frontier", 40, 128, 128, inputs.F32, 4, 16, tv.DELTA),     # halves
+    ("chain", 40, 128, 128, inputs.BF16, 9, 16, tv.DELTA),       # block form; the state goes to registers before the wait
+    ("chain", 40, 128, 128, inputs.BF16, 28, 16, tv.DELTA),      # four items on a CTA
+    ("chain", 24, 128, 128, inputs.BF16, 4, 8, tv.DELTA),
+    ("chain", 50, 64, 64, inputs.F32, 12, 16, tv.DELTA),
+    ("chain", 40, 64, 64, inputs.BF16, 12, 16, tv.DELTA),
+    ("frontier", 64, 64, 128, inputs.BF16, 12, 16, tv.DELTA),
+    ("frontier", 63, 128, 128, inputs.F32, 12, 16, tv.GATED),
+    ("chain", 64, 64, 128, inputs.BF16, 12, 16, tv.GATED),
+])
+def test_queued_rounds_of_the_kernel_of_fp32_accuracy(tree, T, dk, dv, dtype, B, H, rule):
+    """It asks for the state before its wait and releases the commit behind it at once, and runs between an in-place commit
+    and an upload that overwrites its masks."""
+    wl = inputs.workload("c4", B=B, H=H, T=T, dk=dk, dv=dv, tree=tree, qkv_dtype=dtype, rule=rule, seed=T + dk)
+    t = {n: None if x is None else x.to(DEV) for n, x in inputs.make_tensors(wl).items()}
+    trees = tv.tree_build(inputs.make_trees(wl)[0]).upload()
+    O = torch.empty(B, H, T, dv, device=DEV)
+    (name, _), = pu.kernels_of(lambda: tv.tree_verify(trees, *[t[n] for n in ("S_pre", "q", "k", "v", "alpha", "beta")], rule=rule, O=O))
+    assert "verify_exact_kernel" in name
+    _compare(_round_calls(wl, rule, tv.IMPL_AUTO))
+
+
 @pytest.mark.parametrize("B,Tc,rule,dtype", [
     (32, 64, tv.GATED, inputs.BF16),    # 2048 candidates
     (32, 64, tv.DELTA, inputs.BF16),
     (24, 100, tv.DELTA, inputs.F32),    # 2400, general verify kernel
+    (24, 60, tv.DELTA, inputs.F32),     # the verify kernel of fp32 accuracy
     (100, 90, tv.GATED, inputs.BF16),   # 9000
     (700, 3, tv.GATED, inputs.F32),     # many small requests
 ])

@@ -26,7 +26,17 @@ def _inputs(B, H, T, rule, tree, dtype, dk=128, dv=128, seed=0):
     return (wl,) + inputs.make_trees(wl) + (tens,)
 
 
+def _takes(wl, parents, tens):
+    """The call goes to this kernel: with another rule the cases here would test another one."""
+    t = {n: None if x is None else x.cuda() for n, x in tens.items()}
+    tree = tv.tree_build(parents).upload()
+    O = torch.empty(t["v"].shape, device="cuda")
+    launched = pu.kernels_of(lambda: tv.tree_verify(tree, *[t[n] for n in ("S_pre", "q", "k", "v", "alpha", "beta")], rule=wl.rule, O=O))
+    return len(launched) == 1 and "verify_exact_kernel" in launched[0][0]
+
+
 def _check(wl, parents, accepted, tens, whole=1.5e-7):
+    assert _takes(wl, parents, tens)
     O, U, Sn, tree = pu.gpu_round(wl, parents, accepted, tens, impl=tv.IMPL_AUTO, commit_with_U=True)
     tree.device_status()
     n = wl.B * wl.H
@@ -74,6 +84,44 @@ def test_other_widths(rule, dtype, dk, dv):
             if rule == inputs.DELTA and dtype == inputs.BF16 and T < 33 and B == 3 and dk < dv:
                 continue
             _check(*_inputs(B, H, T, rule, tree, dtype, dk=dk, dv=dv, seed=B))
+
+
+@pytest.mark.parametrize("rule,dtype,dk,dv,T,tree,B", [
+    (inputs.DELTA, inputs.BF16, 128, 128, 40, "chain", 80),      # 640 items: four and five a CTA, q and k in two sets of rows
+    (inputs.DELTA, inputs.BF16, 64, 128, 50, "frontier", 80),
+    (inputs.DELTA, inputs.BF16, 64, 64, 33, "chain", 63),        # 504
+    (inputs.DELTA, inputs.F32, 128, 128, 64, "chain", 57),       # 456
+    (inputs.GATED, inputs.F32, 64, 128, 49, "frontier", 57),
+    (inputs.GATED, inputs.BF16, 128, 64, 64, "chain", 57),
+    (inputs.GATED, inputs.BF16, 64, 128, 49, "frontier", 1),     # 8: halves
+    (inputs.GATED, inputs.BF16, 64, 128, 64, "chain", 1)])
+def test_many_items_and_few(rule, dtype, dk, dv, T, tree, B):
+    _check(*_inputs(B, 8, T, rule, tree, dtype, dk=dk, dv=dv, seed=B))
+
+
+def test_packed_forest_of_64_wide_heads_under_the_gated_rule():
+    """bf16 operands: dense batches of these have a kernel of their own, packed ones come here."""
+    rng = np.random.default_rng(4)
+    H, d = 6, 64
+    par = [inputs.tree_chain(64), inputs.tree_frontier(40, rng), inputs.tree_frontier(1, rng), inputs.tree_frontier(64, rng), inputs.tree_chain(49)]
+    forest = tv.forest_build(par, n_max=64).upload()
+    N = int(forest.offsets[-1])
+    t = _inputs(1, H, N, inputs.GATED, "chain", inputs.BF16, dk=d, dv=d)[3]
+    S = inputs.make_tensors(inputs.workload("c4", B=len(par), H=H, T=1, dk=d, dv=d, seed=78))["S_pre"]
+    dev = [S.cuda()] + [t[n][0].cuda() for n in ("q", "k", "v", "alpha")] + [None]
+    O, U = torch.full((H, N, d), 7.0, device="cuda"), torch.full((H, N, d), 7.0, device="cuda")
+    call = lambda: tv.tree_verify(forest, *dev, rule=tv.GATED, O=O, U=U)
+    (name, _), = pu.kernels_of(call)
+    assert "verify_exact_kernel" in name
+    call()
+    forest.device_status()
+    for b, p in enumerate(par):
+        lo, hi = int(forest.offsets[b]), int(forest.offsets[b + 1])
+        cut = {n: inputs.to_f64(t[n][:, :, lo:hi]) for n in ("q", "k", "v", "alpha")}
+        ver = orc.verify_batch(inputs.to_f64(S[b:b + 1]), *cut.values(), None, p[None], "gated")
+        for h in range(H):
+            assert pu.rel_l2_rows(inputs.to_f64(O[h, lo:hi]), ver[(0, h)][0]) <= 1e-5
+            assert torch.equal(U[h, lo:hi].cpu(), t["v"][0, h, lo:hi].float())
 
 
 @pytest.mark.parametrize("depth", [15, 16])
