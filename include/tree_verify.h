@@ -93,7 +93,12 @@ typedef struct tv_dims {
                           also dk = dv = 64 in dense layouts; delta rule: tree
                           depth <= 15), else, for 17 to 64 nodes and widths of
                           64 and 128, one of fp32 accuracy where that is the
-                          faster, and the SIMT fp32 kernel otherwise;
+                          faster, and the SIMT fp32 kernel otherwise.  Where it
+                          is depends on the number of items (L * B * H), the
+                          number of SMs and the deepest tree of the call, so the
+                          order of a request's sums, and with it the last bits
+                          of its outputs (some 1e-7), can depend on what else is
+                          in the call; TV_IMPL_SIMT keeps to the general one.
                           TV_IMPL_TC returns TV_ERR_UNSUPPORTED instead of
                           falling back                                          */
   int32_t Hk;          /* grouped key heads (Section IV-D: a K factor shared by

@@ -24,13 +24,15 @@
 // is steps of compares, one reduction and one barrier (some 0.25 us each): 16 of them to the last bit, 9 for 2048 spread
 // probabilities, all 16 where ties decide.  Four warps of 16 keys a thread, three counts in one word and so one
 // reduction a step, against eight warps with two reductions and all steps: 7.6 -> 5.45 us a selection of 2048 candidates
-// in 16 or 32 requests, 7.3 -> 4.8 of 64 in one, 7.7 -> 7.7 where ties decide.  One launch for everything, every CTA
+// in 16 or 32 requests, 7.3 -> 4.8 of 64 in one, 7.7 -> 7.7 where ties decide.  The early end is all of it: without
+// it the four warps take 7.6 us, and 7.2 on 64 in one request.  One launch for everything, every CTA
 // working out all scores, was slower: 8.7 us, and 37 on chains (7.6 and 12.4).
 // Every request's CTA of the two-launch form searches all keys: its work is requests x candidates.  Device
 // time of a selection of about 2000 candidates, two launches against three: 160 / 200 / 256 / 300 / 400 / 512 / 1024
 // requests 7.2 / 6.5 / 6.6 / 8.7 / 10.7 / 11.5 / 12.9 us against 9.6 / 10.9 / 10.7 / 10.7 / 10.7 / 10.2 / 10.6, where ties
-// decide 256 / 400 / 1024 requests 8.6 / 14.9 / 20.7 against 10.6 / 10.9 / 10.8.  The line stays at one CTA
-// per SM (tests/test_budget_choose_gpu.py holds it there); up to two would be ahead.  With 32
+// decide 256 / 400 / 1024 requests 8.6 / 14.9 / 20.7 against 10.6 / 10.9 / 10.8.  The line is at one CTA per SM,
+// where it was set when the search took all its steps (7.7 / 11.5 us on 148 / 300 requests against 10.9 / 10.3); since
+// the shorter search two CTAs per SM would still be ahead, by 2 to 4 us, and nobody has moved it.  With 32
 // keys per thread, which 2049 to 8192 candidates need, it was slower at any number of requests (on eight warps, searching
 // to the last bit): 4096 candidates in 32 / 1024 requests 14.5 / 64 us against 11.4 / 11.4.
 #include "tv_internal.h"

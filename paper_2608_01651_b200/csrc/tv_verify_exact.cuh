@@ -24,17 +24,18 @@
 // (masks, gates, products of alpha from each node up its path, four steps at a time), one works out where the next item
 // lies and brings it near.  f32 q, k and state pass through registers into their pieces; bf16 q and k are copied, an item
 // ahead.  Beside the general fp32 kernel, whose state product alone is 13 of 27 us on 128 items (fp32 FMA rate: 8.6):
-//     128 items of 63 nodes, f32, delta          29.6 -> 17.7 us        512 of 64   109 -> 61.3
-//     256 items, chains of 40 nodes, bf16        48.0 -> 23.4           512 of 64   130 -> 56.0
-//     256 items of 24 nodes, bf16, depth unknown 25.3 -> 17.0
+//     128 items of 63 nodes, f32, delta          29.6 -> 17.0 us        512 of 64   109 -> 58.6
+//     256 items, chains of 40 nodes, bf16        48.0 -> 22.7           512 of 64   130 -> 54.3
+//     256 items of 24 nodes, bf16, depth unknown 25.3 -> 16.8
 // What bounds it: the phases of an item one after the other (128 items of 63 nodes, thousands of cycles: operands 8, of
 // which 6 at the copy rate; scores 2; C and G 1; state product behind them 4; R 2; last product 3; outputs 3), and code
 // of 70 KiB that runs once per item through an instruction cache smaller than that: loops stay rolled, and one kernel
-// that held both forms of the systems was 10 % slower on chains.  The SM's four quarters matter too: the warps of the q
+// that held both forms of the systems was 10 % slower on chains.  The f32 variants of 128 value columns spill (124 to 184 bytes
+// of stores and 176 to 236 of loads a thread): two batches of operands on their way take 64 registers of it.  The SM's four quarters matter too: the warps of the q
 // rows sit on two of them (a warp reads the tensor memory lanes of its number mod 4).
 //
 // Values that are not finite reach the rows that the recurrence takes them to and no others: rows of R and G that hold any
-// are zeroed before the dense products, and the rows below them are worked out again, one by one, at the end.
+// are zeroed before the dense products, and the rows below them are worked out again at the end, in fp32 (redo_rows).
 // Every wait is bounded (status word on expiry).
 #pragma once
 #include <type_traits>
